@@ -26,6 +26,7 @@
 #include <mutex>
 
 #include "../../include/usp.h"
+#include "usp_sums.cuh"
 
 // Scratch: 20 FP64 sums for each of up to USP_NOALLOC_MAX_CELLS cells
 // (20 x 8192 x 8 B = 1.25 MiB on every device that loads the library).
@@ -33,8 +34,7 @@ static __device__ __align__(256) double g_na_scratch[20 * USP_NOALLOC_MAX_CELLS]
 
 namespace {
 
-constexpr int kNaAcc = 20;     // accumulators per cell
-constexpr int kNaBlock = 256;
+constexpr int kNaAcc = usp::kRawN;   // accumulators per cell
 constexpr double kNaKB = 1.380649e-23;  // Boltzmann constant [J/K]
 
 // what the moments need of the species: R = k_B / m and Theta_vib
@@ -59,81 +59,44 @@ __global__ void na_clear(double* acc, int n) {
     acc[i] = 0.0;
 }
 
-__device__ __forceinline__ double na_warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// pass 0: sum c, sum eps, sum I; pass 1: central sums about the cell mean.
-// acc layout per cell: [0..2] sum c, [3] sum eps, [4] sum I, [5..10] sum CC,
-// [11..13] sum C^2 C / 2, [14..16] sum C eps, [17..19] sum C I.
-__global__ void __launch_bounds__(kNaBlock)
-na_pass(int pass, int ncell, const int64_t* __restrict__ off, const double* __restrict__ cx,
+// Raw sums of every cell about its reference velocity (usp_sums.cuh), one
+// pass; blockIdx.y walks the cells.  Bound by the FP64 pipe (22 to 26
+// operations per particle, 2 lanes per clock and SM).
+__global__ void __launch_bounds__(usp::kRawBlock)
+na_sums(int ncell, int chunk_min, const int64_t* __restrict__ off, const double* __restrict__ cx,
         const double* __restrict__ cy, const double* __restrict__ cz,
-        const double* __restrict__ er, const int32_t* __restrict__ lev, double* __restrict__ acc) {
-  __shared__ double red[kNaBlock / 32][15];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        const double* __restrict__ er, const int32_t* __restrict__ lev, double* __restrict__ acc,
+        double* __restrict__ out) {
   for (int c = blockIdx.y; c < ncell; c += gridDim.y) {
-    const long long b = off[c], e = off[c + 1];
-    const double N = (double)(e - b);
-    double mean[3] = {0.0, 0.0, 0.0};
-    if (pass == 1 && N > 0.0)
-      for (int i = 0; i < 3; ++i) mean[i] = acc[(size_t)c * kNaAcc + i] / N;
-    double a[15];
-    for (int i = 0; i < 15; ++i) a[i] = 0.0;
-    for (long long k = b + (long long)blockIdx.x * blockDim.x + threadIdx.x; k < e;
-         k += (long long)gridDim.x * blockDim.x) {
-      const double ep = er[k], li = (double)lev[k];
-      if (pass == 0) {
-        a[0] += cx[k]; a[1] += cy[k]; a[2] += cz[k]; a[3] += ep; a[4] += li;
-      } else {
-        const double C0 = cx[k] - mean[0], C1 = cy[k] - mean[1], C2 = cz[k] - mean[2];
-        const double q = 0.5 * (C0 * C0 + C1 * C1 + C2 * C2);
-        a[0] += C0 * C0; a[1] += C1 * C1; a[2] += C2 * C2;
-        a[3] += C0 * C1; a[4] += C0 * C2; a[5] += C1 * C2;
-        a[6] += q * C0; a[7] += q * C1; a[8] += q * C2;
-        a[9] += C0 * ep; a[10] += C1 * ep; a[11] += C2 * ep;
-        a[12] += C0 * li; a[13] += C1 * li; a[14] += C2 * li;
-      }
-    }
-    const int na = pass == 0 ? 5 : 15;
-    for (int i = 0; i < na; ++i) {
-      const double s = na_warp_sum(a[i]);
-      if (lane == 0) red[wid][i] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < na) {
-      double s = 0.0;
-      for (int w = 0; w < kNaBlock / 32; ++w) s += red[w][threadIdx.x];
-      atomicAdd(&acc[(size_t)c * kNaAcc + (pass == 0 ? 0 : 5) + threadIdx.x], s);
-    }
-    __syncthreads();
+    const long long b = off[c], n = off[c + 1] - b;
+    usp::raw_cell(b, n, chunk_min, [&] { return usp::raw_reference(b, n, cx, cy, cz); }, cx, cy,
+                  cz, er, lev, acc + (size_t)c * kNaAcc, out + ncell + c, ncell);
   }
 }
 
+// one thread per cell; na_sums left the reference velocities in the rows of U
 __global__ void na_assemble(NaGas gas, int ncell, const int64_t* __restrict__ off,
                             const double* __restrict__ acc, double* __restrict__ out) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
   const double R = gas.R;
-  const double N = (double)(off[c + 1] - off[c]);
-  const double* a = acc + (size_t)c * kNaAcc;
-  if (N <= 0.0) {
+  const long long n = off[c + 1] - off[c];
+  if (n <= 0) {
     for (int f = 0; f < USP_NMOM; ++f) out[(size_t)f * ncell + c] = 0.0;
     return;
   }
-  const double inv = 1.0 / N;
-  out[c] = N;
-  for (int i = 0; i < 3; ++i) out[(size_t)(1 + i) * ncell + c] = a[i] * inv;
-  out[(size_t)4 * ncell + c] = (a[5] + a[6] + a[7]) * inv / (3.0 * R);
-  out[(size_t)5 * ncell + c] = a[3] * inv / R;
-  out[(size_t)6 * ncell + c] = na_T_vib(gas, a[4] * inv);
-  for (int i = 0; i < 6; ++i) out[(size_t)(7 + i) * ncell + c] = a[5 + i] * inv;
+  const double w[3] = {out[ncell + c], out[2 * (size_t)ncell + c], out[3 * (size_t)ncell + c]};
+  const usp::RawMoments m = usp::raw_moments(acc + (size_t)c * kNaAcc, (double)n, w);
+  out[c] = (double)n;
+  for (int i = 0; i < 3; ++i) out[(size_t)(1 + i) * ncell + c] = m.U[i];
+  out[(size_t)4 * ncell + c] = (m.P[0] + m.P[1] + m.P[2]) / (3.0 * R);
+  out[(size_t)5 * ncell + c] = m.eps / R;
+  out[(size_t)6 * ncell + c] = na_T_vib(gas, m.lev);
+  for (int i = 0; i < 6; ++i) out[(size_t)(7 + i) * ncell + c] = m.P[i];
   for (int i = 0; i < 3; ++i) {
-    out[(size_t)(13 + i) * ncell + c] = a[11 + i] * inv;
-    out[(size_t)(16 + i) * ncell + c] = a[14 + i] * inv;
-    out[(size_t)(19 + i) * ncell + c] = a[17 + i] * inv * R * gas.theta_v;
+    out[(size_t)(13 + i) * ncell + c] = m.qt[i];
+    out[(size_t)(16 + i) * ncell + c] = m.qr[i];
+    out[(size_t)(19 + i) * ncell + c] = m.ql[i] * R * gas.theta_v;
   }
 }
 
@@ -176,13 +139,10 @@ extern "C" int usp_moments_noalloc(const usp_species* sp, int n_cells, const int
   const int nacc = kNaAcc * n_cells;
   na_clear<<<(nacc + 255) / 256, 256, 0, st>>>(acc, nacc);
   if (cudaGetLastError() != cudaSuccess) return USP_ECUDA;
-  const dim3 grid(8, n_cells < 65535 ? n_cells : 65535);
-  for (int pass = 0; pass < 2; ++pass) {
-    na_pass<<<grid, kNaBlock, 0, st>>>(pass, n_cells, d_offsets, d_cx, d_cy, d_cz, d_erot,
-                                       d_lev, acc);
-    if (cudaGetLastError() != cudaSuccess) return USP_ECUDA;
-  }
-  na_assemble<<<(n_cells + 127) / 128, 128, 0, st>>>(gas, n_cells, d_offsets, acc, d_out);
+  na_sums<<<dim3(usp::raw_blocks(n_cells), n_cells), usp::kRawBlock, 0, st>>>(
+      n_cells, usp::raw_chunk(n_cells), d_offsets, d_cx, d_cy, d_cz, d_erot, d_lev, acc, d_out);
+  if (cudaGetLastError() != cudaSuccess) return USP_ECUDA;
+  na_assemble<<<(n_cells + 63) / 64, 64, 0, st>>>(gas, n_cells, d_offsets, acc, d_out);
   if (cudaGetLastError() != cudaSuccess) return USP_ECUDA;
   return USP_OK;
 }
