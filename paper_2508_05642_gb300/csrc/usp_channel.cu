@@ -746,7 +746,7 @@ int ch_step_t(ChannelCtx* h, const ChEnv& env, ch_prof_fn prof) {
       if (prof) prof(env.owner, 0, 1);
       ch_collide_fpm<T><<<wb, 128, 0, s>>>(h->ny, cells, h->fpmrec, cx, cy, cz, er, h->lv[b],
                                            h->pd[b], sums, h->dstep,
-                                           philox_round_keys(env.k0, env.k1), env.flags);
+                                           env.rk, env.flags);
     }
   }
   if (!h->fpmrec) {
@@ -759,7 +759,7 @@ int ch_step_t(ChannelCtx* h, const ChEnv& env, ch_prof_fn prof) {
   if (prof) prof(env.owner, 0, 1);
   ch_collide<T, S><<<wb, 128, 0, s>>>(h->ny, cells, (const ChParams<T>*)h->prm, y, cx, cy, cz,
                                       er, h->lv[b], h->pd[b], sums, h->dstep,
-                                      philox_round_keys(env.k0, env.k1), env.flags, env.counters);
+                                      env.rk, env.flags, env.counters);
   }
   CHK(cudaGetLastError());
   if (prof) prof(env.owner, 0, 0);

@@ -16,6 +16,7 @@ struct ChEnv {
   unsigned long long* counters;
   usp::Species sp;
   uint32_t k0, k1;            // Philox key
+  usp::PhiloxRoundKeys rk;    // its round keys, with the tables of the FP64 draws
   int precision;              // USP_FP32 or USP_FP64
   void* (*alloc)(void* owner, size_t bytes);   // owner-tracked device allocation
   void (*release)(void* owner, void* p);       // give an allocation back early

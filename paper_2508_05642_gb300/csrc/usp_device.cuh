@@ -72,11 +72,20 @@ __device__ __forceinline__ U4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c
 // The ten round keys of one key, computed once on the host: kernels take
 // them as a by-value parameter, so each round reads its key from the
 // parameter bank instead of advancing it per thread.
+// FP64 forms of kTabledParticles particles or more also carry the tables of
+// the collision draws (draw_tables_kernel): the Box-Muller radius of each of
+// the 2^23 radius uniforms and the direction (cosine, sine) of each of the
+// 2^18 angles; null otherwise.
 struct PhiloxRoundKeys {
   uint32_t k0[10], k1[10];
+  const double* radius;
+  const double2* direction;
 };
+constexpr int kRadiusBits = 23, kAngleBits = 18;
 inline PhiloxRoundKeys philox_round_keys(uint32_t k0, uint32_t k1) {
   PhiloxRoundKeys rk;
+  rk.radius = nullptr;
+  rk.direction = nullptr;
   for (int r = 0; r < 10; ++r) {
     rk.k0[r] = k0;
     rk.k1[r] = k1;
@@ -144,7 +153,23 @@ __device__ __forceinline__ float sqrt_fast(float x) {
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-__device__ __forceinline__ double sqrt_fast(double x) { return sqrt(x); }
+// FP64: the hardware reciprocal square root (about 2^-20), one Goldschmidt
+// step for the root and its half reciprocal together and Markstein's residual
+// correction (P. Markstein, "IA-64 and Elementary Functions", 2000), five
+// multiply-adds in all; the library function outside exponents +-900, which
+// also answers zero, negative values, infinities and NaN.
+__device__ __forceinline__ double sqrt_fast(double x) {
+  const int hi = __double2hiint(x);
+  if ((unsigned)(hi - (123 << 20)) > (unsigned)(1800 << 20)) return sqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double g = x * y;
+  double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));   // y / 2
+  const double r = fma(-g, h, 0.5);
+  g = fma(g, r, g);
+  h = fma(h, r, h);
+  return fma(fma(-g, g, x), h, g);
+}
 
 // Box-Muller pair: G_a = sqrt(-2 ln u_a) cos(2 pi u_b), G_b = ... sin(2 pi u_b).
 // The float version takes -2 ln u = -2 ln 2 log2 u with the hardware base-2
@@ -225,11 +250,20 @@ __device__ __forceinline__ void particle_draws(uint32_t pid, uint32_t step,
                                                double& g2, double& g3, uint32_t& j5,
                                                uint32_t& j6) {
   const U4 w = philox4x32_10(pid, step, PTAG_NORMALS, 0u, rk);
-  box_muller(uniform23_d(w.x), angle_uniform18_d(w.x, w.y), g0, g1);
-  box_muller(uniform23_d(w.y), angle_uniform18_d(w.z, w.w), g2, g3);
+  if (rk.radius) {
+    const double ra = __ldg(rk.radius + (w.x >> 9)), rb = __ldg(rk.radius + (w.y >> 9));
+    const double2 da = __ldg(rk.direction + angle_bits18(w.x, w.y));
+    const double2 db = __ldg(rk.direction + angle_bits18(w.z, w.w));
+    g0 = ra * da.x; g1 = ra * da.y;
+    g2 = rb * db.x; g3 = rb * db.y;
+  } else {
+    box_muller(uniform23_d(w.x), angle_uniform18_d(w.x, w.y), g0, g1);
+    box_muller(uniform23_d(w.y), angle_uniform18_d(w.z, w.w), g2, g3);
+  }
   j5 = w.z;
   j6 = w.w;
 }
+
 
 // ---------------------------------------------------------------------------
 // Jump samplers of Eq. update_evib: sequential inversion with one uniform,

@@ -25,7 +25,7 @@
 //                    under the affine rescale: U' = U, Pi' = s^2 Pi*,
 //                    e_rot' = r e_rot*), and the next step's coefficients
 //                    (Sec. 3.A) in FP64.
-//   jumptable_kernel (FP32 form) the per-cell inversion tables of the
+//   jumptable_kernel the per-cell inversion tables of the
 //                    vibrational jump samplers for the next step.
 // The rescale is never written back as a separate pass: it rides along with
 // the next collide pass, or with usp_moments / usp_get_particles.
@@ -91,7 +91,7 @@ struct Tile {
 };
 
 // ---------------------------------------------------------------------------
-// Jump tables of the FP32 form.  In a homogeneous cell p_NB and p_B are cell
+// Jump tables.  In a homogeneous cell p_NB and p_B are cell
 // constants, so the cumulative values the sequential inversion would compute
 // for a given r = I + 1 (or n = I) are the same for every particle of the
 // cell.  jumptable_kernel computes them once per cell and step with exactly
@@ -100,70 +100,89 @@ struct Tile {
 // cumulative sum and the end of the binomial support become +inf entries, an
 // underflowed P(0) marks the row (-1) and sends the particle to the
 // sequential search, as does a search running past the row.
+// The FP64 form's rows are computed in FP64 and hold, for each cumulative
+// value, the least of the 2^23 jump uniforms that is not below it (+inf:
+// none): a uniform passes the entry exactly when it passes the value, and
+// the uniforms are floats in both forms, so the same search serves both.
+// FP64 contexts with kTabledCell particles per cell or more take the tables:
+// a particle then needs no FP64 operation for its jump (some 20 to 50
+// before), a cell's rows cost about as much as 400 particles' inversions.
 // ---------------------------------------------------------------------------
 constexpr int kJR = 32;   // rows: NB r = 1..32, B n = 0..31
 constexpr int kJK = 48;   // cumulative values per row (rows 16-byte aligned)
+constexpr long long kTabledCell = 512;
 
 // The pmf ratios of the rows, the same for every cell: (k + r) / (k + 1) of
 // the NB row r (index r - 1) and (n - k) / (k + 1) of the binomial row n,
-// each the correctly rounded float quotient that the sequential inversion
+// each the correctly rounded quotient that the sequential inversion
 // forms; filled once per context by jratio_kernel.
-__device__ float g_jratio[2][kJR][kJK];
+template <typename T>
+__device__ T g_jratio[2][kJR][kJK];
 
+template <typename T>
 __global__ void jratio_kernel() {
   for (int e = threadIdx.x; e < kJR * kJK; e += blockDim.x) {
     const int a = e / kJK, k = e % kJK;
-    g_jratio[0][a][k] = rn_div(rn_i2f(k + a + 1, 0.0f), rn_i2f(k + 1, 0.0f));
-    g_jratio[1][a][k] = k < a ? rn_div(rn_i2f(a - k, 0.0f), rn_i2f(k + 1, 0.0f)) : 0.0f;
+    g_jratio<T>[0][a][k] = rn_div(rn_i2f(k + a + 1, T(0)), rn_i2f(k + 1, T(0)));
+    g_jratio<T>[1][a][k] = k < a ? rn_div(rn_i2f(a - k, T(0)), rn_i2f(k + 1, T(0))) : T(0);
   }
 }
 
-__device__ void nb_row(int r, float p, float* T) {
-  const float q = rn_sub(1.0f, p);
-  float P = powi_rn(p, r);
-  if (P < 1.17549435e-38f) { T[0] = -1.0f; return; }
-  float cdf = P;
-  T[0] = cdf;
-  bool stop = false;
-  for (int j = 1; j < kJK; ++j) {
-    if (!stop) {
-      const int k = j - 1;
-      const float t = g_jratio[0][r - 1][k];   // (k + r) / (k + 1)
-      P = rn_mul(P, t);
-      P = rn_mul(P, q);
-      const float nc = rn_add(cdf, P);
-      if (nc == cdf) stop = true;
-      else cdf = nc;
-    }
-    T[j] = stop ? __int_as_float(0x7f800000) : cdf;
-  }
+// the entry of a cumulative value: itself (FP32), or the least jump uniform
+// (2 k + 1) 2^-24 that is not below it (FP64; +inf: none).  k = ceil((2^24 cdf -
+// 1) / 2), every operation exact.
+__device__ __forceinline__ float row_entry(float cdf) { return cdf; }
+__device__ __forceinline__ float row_entry(double cdf) {
+  const double k = fmax(ceil(0.5 * (16777216.0 * cdf - 1.0)), 0.0);
+  return k < 8388608.0 ? __fmaf_rn((float)k, 0x1p-23f, 0x1p-24f) : __int_as_float(0x7f800000);
+}
+__device__ __forceinline__ float pmf_least(float) { return 1.17549435e-38f; }
+__device__ __forceinline__ double pmf_least(double) { return 2.2250738585072014e-308; }
+
+// the entries after the last finite one
+__device__ __forceinline__ void row_end(float* T, int j) {
+  for (; j < kJK; ++j) T[j] = __int_as_float(0x7f800000);
 }
 
-// p here is the binomial parameter after the p > 1/2 flip
-__device__ void b_row(int n, float p, float* T) {
-  const float q = rn_sub(1.0f, p);
-  float P = powi_rn(q, n);
-  if (P < 1.17549435e-38f) { T[0] = -1.0f; return; }
-  const float pq = rn_div(p, q);
-  float cdf = P;
-  T[0] = cdf;
-  bool stop = false;
-  for (int j = 1; j < kJK; ++j) {
-    if (!stop) {
-      if (j >= n) {
-        stop = true;   // the search ends at k = n whatever u is
-      } else {
-        const int k = j - 1;
-        const float t = g_jratio[1][n][k];       // (n - k) / (k + 1)
-        P = rn_mul(P, t);
-        P = rn_mul(P, pq);
-        const float nc = rn_add(cdf, P);
-        if (nc == cdf) stop = true;
-        else cdf = nc;
-      }
-    }
-    T[j] = stop ? __int_as_float(0x7f800000) : cdf;
+template <typename F>
+__device__ void nb_row(int r, F p, float* T) {
+  const F q = rn_sub(F(1), p);
+  F P = powi_rn(p, r);
+  if (P < pmf_least(P)) { T[0] = -1.0f; return; }
+  F cdf = P;
+  T[0] = row_entry(cdf);
+  int j = 1;
+  for (; j < kJK; ++j) {
+    P = rn_mul(P, g_jratio<F>[0][r - 1][j - 1]);   // (k + r) / (k + 1), k = j - 1
+    P = rn_mul(P, q);
+    const F nc = rn_add(cdf, P);
+    if (nc == cdf) break;
+    cdf = nc;
+    T[j] = row_entry(cdf);
   }
+  row_end(T, j);
+}
+
+// p here is the binomial parameter after the p > 1/2 flip; the search ends at
+// k = n whatever u is
+template <typename F>
+__device__ void b_row(int n, F p, float* T) {
+  const F q = rn_sub(F(1), p);
+  F P = powi_rn(q, n);
+  if (P < pmf_least(P)) { T[0] = -1.0f; return; }
+  const F pq = rn_div(p, q);
+  F cdf = P;
+  T[0] = row_entry(cdf);
+  int j = 1;
+  for (; j < kJK && j < n; ++j) {
+    P = rn_mul(P, g_jratio<F>[1][n][j - 1]);       // (n - k) / (k + 1), k = j - 1
+    P = rn_mul(P, pq);
+    const F nc = rn_add(cdf, P);
+    if (nc == cdf) break;
+    cdf = nc;
+    T[j] = row_entry(cdf);
+  }
+  row_end(T, j);
 }
 
 // Guide tables (the indexed search of Chen & Asau): per row, one byte for
@@ -204,38 +223,40 @@ __device__ __forceinline__ int guided_search(const float* __restrict__ T, unsign
 }
 
 // The general path of the two samplers (the guide byte of u's bin gv)
-__device__ __forceinline__ int nb_tab(const float* __restrict__ T, unsigned gv, int r, float p,
+template <typename F>
+__device__ __forceinline__ int nb_tab(const float* __restrict__ T, unsigned gv, int r, F p,
                                       float u, uint32_t& fl) {
-  if (r <= 0 || !(p < 1.0f)) return 0;
-  if (r > kJR) return nb_inv(r, p, u, fl);
+  if (r <= 0 || !(p < F(1))) return 0;
+  if (r > kJR) return nb_inv(r, p, (F)u, fl);
   if (guide_outcome(gv) < (unsigned)kJK) return (int)guide_outcome(gv);
   const int k = guided_search(T, gv, u);
-  return k < kJK ? k : nb_inv(r, p, u, fl);
+  return k < kJK ? k : nb_inv(r, p, (F)u, fl);
 }
 
 // npb counts the draws clamped at p_B > 1
-__device__ __forceinline__ int b_tab(const float* __restrict__ T, unsigned gv, int n, float p,
+template <typename F>
+__device__ __forceinline__ int b_tab(const float* __restrict__ T, unsigned gv, int n, F p,
                                      float u, uint32_t& fl, int& npb) {
   if (n <= 0) return 0;
-  if (p >= 1.0f) {
-    if (p > 1.0f) {
+  if (p >= F(1)) {
+    if (p > F(1)) {
       fl |= F_PB_CLAMP;
       ++npb;
     }
     return n;
   }
-  if (!(p > 0.0f)) return 0;
-  const bool flip = p > 0.5f;
+  if (!(p > F(0))) return 0;
+  const bool flip = p > F(0.5);
   if (n < kJR) {
     if (guide_outcome(gv) < (unsigned)kJK) return (int)guide_outcome(gv);
     const int k = guided_search(T, gv, u);   // T[n] = +inf: k <= n < kJK
     if (k < kJK) return flip ? n - k : k;
   }
-  const int k = binv(n, flip ? rn_sub(1.0f, p) : p, u, fl);
+  const int k = binv(n, flip ? rn_sub(F(1), p) : p, (F)u, fl);
   return flip ? n - k : k;
 }
 
-// the per-cell jump tables and their guides (FP32 form)
+// the per-cell jump tables and their guides (null: an FP64 context without)
 struct JumpTabs {
   const float* nb;
   const float* b;
@@ -259,12 +280,13 @@ __device__ __forceinline__ void collide_one(const CollideParams<T>& P, uint32_t 
   T g0, g1, g2, g3;
   uint32_t j5, j6;
   particle_draws(pid, P.step, rk, g0, g1, g2, g3, j5, j6);
-  // FP32 form: the guide bytes of the particle's two rows (NB r = I + 1 is
+  // the guide bytes of the particle's two rows (NB r = I + 1 is
   // row I, binomial n = I is row I) are loaded here, so that their latency
   // passes under the arithmetic below
+  const bool tabled = METHOD == 0 && (sizeof(T) == 4 || jt.nb);
   size_t row = 0;
   unsigned gv5 = 0, gv6 = 0;
-  if constexpr (sizeof(T) == 4 && METHOD == 0) {
+  if (tabled) {
     row = (size_t)(I < kJR ? I : 0);
     gv5 = guide_byte(jt.gnb + row * kGB, j5);
     gv6 = guide_byte(jt.gb + row * kGB, j6);
@@ -281,7 +303,6 @@ __device__ __forceinline__ void collide_one(const CollideParams<T>& P, uint32_t 
   const T root = sqrt_fast(er) * P.ar + P.sqrt_a * g3;
   er = P.a_rot + root * root;
   // I' = I + NB(I + 1, p_NB) - B(I, p_B)
-  const T u5 = jump_uniform<T>(j5), u6 = jump_uniform<T>(j6);
   if constexpr (METHOD == 1) {
     // plain FPM method: Gillespie's direct method (Sec. 2.C)
     uint32_t f1 = 0;
@@ -290,7 +311,7 @@ __device__ __forceinline__ void collide_one(const CollideParams<T>& P, uint32_t 
     fl |= f1;
   } else {
     int up, dn;
-    if constexpr (sizeof(T) == 4) {
+    if (tabled) {
       // both guide bytes hold their outcome (every cell case included):
       // one test decides the jump
       const unsigned o5 = guide_outcome(gv5), o6 = guide_outcome(gv6);
@@ -298,13 +319,13 @@ __device__ __forceinline__ void collide_one(const CollideParams<T>& P, uint32_t 
         up = (int)o5;
         dn = (int)o6;
       } else {
-        up = nb_tab(jt.nb + row * kJK, gv5, I + 1, P.p_nb, u5, fl);
-        dn = b_tab(jt.b + row * kJK, gv6, I, P.p_b, u6, fl, npb);
+        up = nb_tab(jt.nb + row * kJK, gv5, I + 1, P.p_nb, uniform_open<float>(j5), fl);
+        dn = b_tab(jt.b + row * kJK, gv6, I, P.p_b, uniform_open<float>(j6), fl, npb);
       }
     } else {
       uint32_t f1 = 0;
-      up = sample_nb<T>(I + 1, P.p_nb, u5, f1);
-      dn = sample_b<T>(I, P.p_b, u6, f1);
+      up = sample_nb<T>(I + 1, P.p_nb, jump_uniform<T>(j5), f1);
+      dn = sample_b<T>(I, P.p_b, jump_uniform<T>(j6), f1);
       npb += (f1 & F_PB_CLAMP) ? 1 : 0;
       fl |= f1;
     }
@@ -316,6 +337,28 @@ __device__ __forceinline__ void collide_one(const CollideParams<T>& P, uint32_t 
   acc[6] += r0 * r1; acc[7] += r0 * r2; acc[8] += r1 * r2;
   acc[9] += er;
   accI += lv;
+}
+
+// The tables of the FP64 collision draws: entry i of radius is the radius of
+// the uniform (2 i + 1) 2^-24, entry a of direction the cosine and sine of
+// 2 pi (2 a + 1) 2^-19, by the functions the direct path calls, so that a draw
+// is the same number either way.  The FP64 pipe of this chip has 2 lanes per SM
+// and clock; a logarithm takes 35 lane-operations, a sine-cosine pair 33, a
+// square root 10, so the two pairs of a particle were half of the FP64 collision
+// pass.  Gathers of 8 bytes from 64 MB run at 290 billion per second (one
+// 32-byte sector of L2 each), 1/8 of that time.  Filling takes 0.7 ms, the
+// work of 4 million particle-steps, hence the least count.
+constexpr long long kTabledParticles = 1 << 16;
+__global__ void draw_tables_kernel(double* __restrict__ radius,
+                                          double2* __restrict__ direction) {
+  const int n = gridDim.x * blockDim.x, t = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int i = t; i < 1 << kRadiusBits; i += n)
+    radius[i] = sqrt(-2.0 * log(uniform23_d((uint32_t)i << 9)));
+  for (int a = t; a < 1 << kAngleBits; a += n) {
+    double s, c;
+    sincospi(2.0 * ((2.0 * (double)a + 1.0) * 1.9073486328125e-06), &s, &c);
+    direction[a] = make_double2(c, s);
+  }
 }
 
 template <typename T>
@@ -591,8 +634,10 @@ collide_warp_kernel(const Tile* __restrict__ tiles, int ntiles,
       int* Lv = reinterpret_cast<int*>(b + 4 * kWT * sizeof(T));
       const uint32_t pid0 = P.pid0 + (uint32_t)tl.start;
       const size_t tc = (size_t)tl.cell * kJR;
-      const JumpTabs jt{tabs.nb + tc * kJK, tabs.b + tc * kJK, tabs.gnb + tc * kGB,
-                        tabs.gb + tc * kGB};
+      const JumpTabs jt = sizeof(T) == 4 || tabs.nb
+                              ? JumpTabs{tabs.nb + tc * kJK, tabs.b + tc * kJK,
+                                         tabs.gnb + tc * kGB, tabs.gb + tc * kGB}
+                              : tabs;
 #pragma unroll 1
       for (int k = lane; k < tl.count; k += 32) {
         T x = X[k], y = X[k + kWT], z = X[k + 2 * kWT], e = X[k + 3 * kWT];
@@ -782,8 +827,10 @@ collide_kernel(const Tile* __restrict__ tiles, int ntiles,
       int* Lv = sb_l<T>(buf);
       const uint32_t pid0 = P.pid0 + (uint32_t)tl.start;
       const size_t tc = (size_t)tl.cell * kJR;
-      const JumpTabs jt{tabs.nb + tc * kJK, tabs.b + tc * kJK, tabs.gnb + tc * kGB,
-                        tabs.gb + tc * kGB};
+      const JumpTabs jt = sizeof(T) == 4 || tabs.nb
+                              ? JumpTabs{tabs.nb + tc * kJK, tabs.b + tc * kJK,
+                                         tabs.gnb + tc * kGB, tabs.gb + tc * kGB}
+                              : tabs;
 #pragma unroll 1
       for (int k = tid; k < tl.count; k += kBlock) {
         T x = X[k], y = X[k + kTileMax], z = X[k + 2 * kTileMax], e = X[k + 3 * kTileMax];
@@ -847,17 +894,19 @@ collide_kernel(const Tile* __restrict__ tiles, int ntiles,
 }
 
 
-// Jump-table rows of every cell for the coming step (FP32 form), one block of
+// Jump-table rows of every cell for the coming step, one block of
 // kJT threads per cell: thread j < kJR builds the NB row r = j + 1, thread
 // kJR + n the binomial row n, for the rows the cell's levels can reach; then
 // every row's guide is built by kGP threads.
 constexpr int kJT = 8 * kJR;
 
-__device__ __forceinline__ bool nb_row_used(int j, int rows, float p_nb) {
-  return j + 1 <= rows && p_nb < 1.0f;
+template <typename F>
+__device__ __forceinline__ bool nb_row_used(int j, int rows, F p_nb) {
+  return j + 1 <= rows && p_nb < F(1);
 }
-__device__ __forceinline__ bool b_row_used(int n, int rows, float p_b) {
-  return n >= 1 && n <= rows - 1 && p_b < 1.0f && p_b > 0.0f;
+template <typename F>
+__device__ __forceinline__ bool b_row_used(int n, int rows, F p_b) {
+  return n >= 1 && n <= rows - 1 && p_b < F(1) && p_b > F(0);
 }
 
 // bins [q kQ, (q + 1) kQ) of the guide of row T (the guide tables above),
@@ -913,22 +962,24 @@ __host__ __device__ inline void guide_part(const float* T, uint8_t* __restrict__
   }
 }
 
+template <typename F>
 __global__ void __launch_bounds__(kJT)
-jumptable_kernel(int c0, int c1, const CollideParams<float>* __restrict__ prm,
+jumptable_kernel(int c0, int c1, const CollideParams<F>* __restrict__ prm,
                  const CellState* __restrict__ cells, float* __restrict__ tab_nb,
                  float* __restrict__ tab_b, uint8_t* __restrict__ gd_nb,
                  uint8_t* __restrict__ gd_b) {
   const int c = c0 + blockIdx.x;
   const int j = threadIdx.x;
   if (c >= c1) return;                       // uniform over the block
-  const CollideParams<float>& P = prm[c];
+  const CollideParams<F>& P = prm[c];
   if (!P.active) return;                     // uniform over the block
-  // the rows are built in shared memory, copied out coalesced, and the
+  // the rows are built in shared memory (one word of padding each: the threads
+  // build one row each, entry by entry), copied out coalesced, and the
   // guides read them there
-  __shared__ float rs[2][kJR][kJK];
+  __shared__ float rs[2][kJR][kJK + 1];
   const int rows = min(kJR, cells[c].maxI + 1);
-  float pb = P.p_b;
-  if (pb > 0.5f && pb < 1.0f) pb = rn_sub(1.0f, pb);
+  F pb = P.p_b;
+  if (pb > F(0.5) && pb < F(1)) pb = rn_sub(F(1), pb);
   if (j < kJR) {
     if (nb_row_used(j, rows, P.p_nb)) nb_row(j + 1, P.p_nb, rs[0][j]);
   } else if (j < 2 * kJR) {
@@ -952,13 +1003,13 @@ jumptable_kernel(int c0, int c1, const CollideParams<float>* __restrict__ prm,
   } else {
     const int n = row - kJR;
     uint8_t* g = gd_b + ((size_t)c * kJR + n) * kGB;
-    const float p = P.p_b;
+    const F p = P.p_b;
     if (b_row_used(n, rows, p))
-      guide_part(rs[1][n], g, q, p > 0.5f ? n : -1);
+      guide_part(rs[1][n], g, q, p > F(0.5) ? n : -1);
     else if (n < rows)
       // n = 0 or p_B <= 0: no jump down; p_B = 1: n; p_B > 1: the general
       // path, which flags the clamp
-      guide_fill(g, q, n >= 1 && p >= 1.0f ? (p > 1.0f ? 0x7fu : 0x80u | (uint32_t)n) : 0x80u);
+      guide_fill(g, q, n >= 1 && p >= F(1) ? (p > F(1) ? 0x7fu : 0x80u | (uint32_t)n) : 0x80u);
   }
 }
 
@@ -1577,6 +1628,8 @@ struct usp_ctx {
   float* tab_b;
   uint8_t* gd_nb;           // their guide tables
   uint8_t* gd_b;
+  double* radius;           // tables of the FP64 collision draws (null: computed)
+  double2* direction;
   uint32_t* flags;
   unsigned long long* counters;
   std::vector<long long> h_uoff;
@@ -1675,6 +1728,32 @@ void dev_release(usp_ctx* c, void* p) {
 void* env_alloc(void* owner, size_t bytes) { return dev_alloc((usp_ctx*)owner, bytes); }
 void env_release(void* owner, void* p) { dev_release((usp_ctx*)owner, p); }
 
+PhiloxRoundKeys round_keys(const usp_ctx* c) {
+  PhiloxRoundKeys rk = philox_round_keys(key0(c), key1(c));
+  rk.radius = c->radius;
+  rk.direction = c->direction;
+  return rk;
+}
+
+// Memory for the tables of the FP64 collision draws of a context of n
+// particles, and their contents once the context has its stream.
+int alloc_draw_tables(usp_ctx* c, long long n) {
+  if ((c->precision != USP_FP64 && c->precision != USP_FP64_TANGENT) || n < kTabledParticles)
+    return USP_OK;
+  const size_t nr = (size_t)1 << kRadiusBits, na = (size_t)1 << kAngleBits;
+  c->radius = (double*)dev_alloc(c, nr * sizeof(double) + na * sizeof(double2));
+  if (!c->radius) return USP_ENOMEM;
+  c->direction = (double2*)(c->radius + nr);
+  return USP_OK;
+}
+int fill_draw_tables(usp_ctx* c) {
+  if (!c->radius) return USP_OK;
+  draw_tables_kernel<<<1024, 256, 0, c->stream>>>(c->radius, c->direction);
+  CK(cudaGetLastError());
+  c->launches += 1;
+  return USP_OK;
+}
+
 ChEnv make_env(usp_ctx* c) {
   ChEnv e;
   e.stream = c->stream;
@@ -1683,6 +1762,7 @@ ChEnv make_env(usp_ctx* c) {
   e.sp = c->sp;
   e.k0 = key0(c);
   e.k1 = key1(c);
+  e.rk = round_keys(c);
   e.precision = c->precision;
   e.alloc = env_alloc;
   e.release = env_release;
@@ -1810,7 +1890,7 @@ int launch_collide_m(usp_ctx* c, int warp_tiles, int minb, int grid, void* cx, v
   const size_t smem = collide_smem<T>(warp_tiles);
   const CollideParams<T>* prm = (const CollideParams<T>*)c->prm;
   T* x = (T*)cx; T* y = (T*)cy; T* z = (T*)cz; T* e = (T*)er;
-  const PhiloxRoundKeys rk = philox_round_keys(key0(c), key1(c));
+  const PhiloxRoundKeys rk = round_keys(c);
   const JumpTabs tb{c->tab_nb, c->tab_b, c->gd_nb, c->gd_b};
   if (warp_tiles) {
     const Tile* tiles = c->wtiles + r.w0;
@@ -1852,19 +1932,25 @@ int launch_collide(usp_ctx* c, int warp_tiles, int minb, int grid, void* cx, voi
                                       counters, r);
 }
 
-// jump tables for the coming step (FP32 form only)
-int launch_tables(usp_ctx* c, const CellRange& r) {
-  if (c->precision != USP_FP32 || c->sp.method != 0 || r.c1 <= r.c0) return USP_OK;
+bool has_tables(const usp_ctx* c) { return c->tab_nb && c->sp.method == 0; }
+
+// jump tables for the coming step
+template <typename T>
+int launch_tables_t(usp_ctx* c, const CellRange& r) {
+  if (!has_tables(c) || r.c1 <= r.c0) return USP_OK;
   if (!c->jratio_ready) {
-    jratio_kernel<<<1, 256, 0, c->stream>>>();
+    jratio_kernel<T><<<1, 256, 0, c->stream>>>();
     CK(cudaGetLastError());
     c->jratio_ready = true;
   }
-  jumptable_kernel<<<r.c1 - r.c0, kJT, 0, c->stream>>>(
-      r.c0, r.c1, (const CollideParams<float>*)c->prm, c->cells, c->tab_nb, c->tab_b, c->gd_nb,
+  jumptable_kernel<T><<<r.c1 - r.c0, kJT, 0, c->stream>>>(
+      r.c0, r.c1, (const CollideParams<T>*)c->prm, c->cells, c->tab_nb, c->tab_b, c->gd_nb,
       c->gd_b);
   CK(cudaGetLastError());
   return USP_OK;
+}
+int launch_tables(usp_ctx* c, const CellRange& r) {
+  return c->precision == USP_FP32 ? launch_tables_t<float>(c, r) : launch_tables_t<double>(c, r);
 }
 
 // one step of the cells of r
@@ -1896,7 +1982,7 @@ int launch_step(usp_ctx* c, const CellRange& r) {
 int kernels_per_step(const usp_ctx* c) {
   if (c->kind == 1) return ch_kernels_per_step(c->ch);
   if (c->kind == 2) return pl_kernels_per_step(c->pl);
-  return c->precision == USP_FP32 && c->sp.method == 0 ? 4 : 3;
+  return has_tables(c) ? 4 : 3;
 }
 
 int step_once(usp_ctx* c) {
@@ -1961,7 +2047,7 @@ int init_params(usp_ctx* c, const CellRange& r) {
   CK(cudaGetLastError());
   c->launches += 2;
   if ((rc = launch_tables(c, r))) return rc;
-  c->launches += c->precision == USP_FP32 && c->sp.method == 0 ? 1 : 0;
+  c->launches += has_tables(c) ? 1 : 0;
   return USP_OK;
 }
 template <typename T>
@@ -2312,13 +2398,14 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
   c->tab_b = nullptr;
   c->gd_nb = nullptr;
   c->gd_b = nullptr;
-  if (c->precision == USP_FP32) {
+  if (c->precision == USP_FP32 || (cfg->method == USP_METHOD_USP_FPM && n >= kTabledCell * n_cells)) {
     c->tab_nb = (float*)dev_alloc(c, sizeof(float) * (size_t)n_cells * kJR * kJK);
     c->tab_b = (float*)dev_alloc(c, sizeof(float) * (size_t)n_cells * kJR * kJK);
     c->gd_nb = (uint8_t*)dev_alloc(c, (size_t)n_cells * kJR * kGB);
     c->gd_b = (uint8_t*)dev_alloc(c, (size_t)n_cells * kJR * kGB);
     if (!c->tab_nb || !c->tab_b || !c->gd_nb || !c->gd_b) return fail(USP_ENOMEM);
   }
+  if (alloc_draw_tables(c, n) != USP_OK) return fail(USP_ENOMEM);
   c->flags = (uint32_t*)dev_alloc(c, 256);
   c->counters = (unsigned long long*)dev_alloc(c, 256);
   if (!c->cx || !c->cy || !c->cz || !c->er || !c->lev || !c->cells || !c->prm || !c->sums ||
@@ -2346,6 +2433,7 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
       cudaMemcpyAsync(c->uoff, c->h_uoff.data(), sizeof(long long) * (n_cells + 1),
                       cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
     return fail(USP_ECUDA);
+  if (fill_draw_tables(c) != USP_OK) return fail(USP_ECUDA);
   // the particle pass stages fixed tiles of kTileMax; smaller tiles (tests)
   // split cells more finely but use the same staging buffers
   const int tile = cfg->tile > 0 ? std::min(kTileMax, (cfg->tile + kAlign - 1) / kAlign * kAlign)
@@ -2449,10 +2537,11 @@ int usp_init_channel(usp_ctx** out, const usp_species* sp, const usp_config* cfg
   };
   c->flags = (uint32_t*)dev_alloc(c, 256);
   c->counters = (unsigned long long*)dev_alloc(c, 256);
-  if (!c->flags || !c->counters) return fail(USP_ENOMEM);
+  if (!c->flags || !c->counters || alloc_draw_tables(c, n) != USP_OK) return fail(USP_ENOMEM);
   if (cudaMemsetAsync(c->flags, 0, 256, c->stream) != cudaSuccess ||
       cudaMemsetAsync(c->counters, 0, 256, c->stream) != cudaSuccess)
     return fail(USP_ECUDA);
+  if (fill_draw_tables(c) != USP_OK) return fail(USP_ECUDA);
   const int rc = ch_create(&c->ch, make_env(c), ch, dt, n, cfg->step0, h_y, h_cx, h_cy, h_cz,
                            h_erot, h_lev, h_pid);
   if (rc != USP_OK) return fail(rc);
@@ -2516,10 +2605,11 @@ int usp_init_plane(usp_ctx** out, const usp_species* sp, const usp_config* cfg,
   };
   c->flags = (uint32_t*)dev_alloc(c, 256);
   c->counters = (unsigned long long*)dev_alloc(c, 256);
-  if (!c->flags || !c->counters) return fail(USP_ENOMEM);
+  if (!c->flags || !c->counters || alloc_draw_tables(c, n) != USP_OK) return fail(USP_ENOMEM);
   if (cudaMemsetAsync(c->flags, 0, 256, c->stream) != cudaSuccess ||
       cudaMemsetAsync(c->counters, 0, 256, c->stream) != cudaSuccess)
     return fail(USP_ECUDA);
+  if (fill_draw_tables(c) != USP_OK) return fail(USP_ECUDA);
   const int rc = pl_create(&c->pl, make_env(c), pl, dt, area_frac, n, capacity, cfg->step0, h_x,
                            h_y, h_cx, h_cy, h_cz, h_erot, h_lev, h_pid);
   if (rc != USP_OK) return fail(rc);
@@ -2758,7 +2848,7 @@ int homog_segments(usp_ctx* c, void** ptr, size_t* bytes) {
   ptr[k] = c->cells; bytes[k++] = sizeof(CellState) * c->ncell;
   ptr[k] = c->prm; bytes[k++] = pb * c->ncell;
   ptr[k] = c->sums; bytes[k++] = sizeof(CellSums) * c->ncell;
-  if (c->tab_nb) {
+  if (c->precision == USP_FP32) {   // the FP64 form's are built again on loading
     ptr[k] = c->tab_nb; bytes[k++] = sizeof(float) * (size_t)c->ncell * kJR * kJK;
     ptr[k] = c->tab_b; bytes[k++] = sizeof(float) * (size_t)c->ncell * kJR * kJK;
     ptr[k] = c->gd_nb; bytes[k++] = (size_t)c->ncell * kJR * kGB;
@@ -2873,6 +2963,10 @@ int usp_load(usp_ctx* c, const void* buf, int buf_is_device) {
     for (int i = 0; i < k; ++i) {
       CK(cudaMemcpyAsync(p[i], b, sz[i], b2d, c->stream));
       b += sz[i];
+    }
+    if (c->precision != USP_FP32) {
+      const int rc = launch_tables(c, all_cells(c));
+      if (rc) return rc;
     }
   }
   c->step = h.step;

@@ -1721,11 +1721,11 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
   if (fpm)
     pl_collide<T, 1><<<h->grid_col, kBlk, pl_collide_smem<T>(), s>>>(
         ncell, h->cells, (const PlParams<T>*)h->prm, x, y, cx, cy, cz, er, h->lv[b], h->pd[b],
-        h->sums, h->dstep, philox_round_keys(env.k0, env.k1), env.flags, env.counters);
+        h->sums, h->dstep, env.rk, env.flags, env.counters);
   else
     pl_collide<T, 0><<<h->grid_col, kBlk, pl_collide_smem<T>(), s>>>(
         ncell, h->cells, (const PlParams<T>*)h->prm, x, y, cx, cy, cz, er, h->lv[b], h->pd[b],
-        h->sums, h->dstep, philox_round_keys(env.k0, env.k1), env.flags, env.counters);
+        h->sums, h->dstep, env.rk, env.flags, env.counters);
   CHK(cudaGetLastError());
   if (prof) prof(env.owner, 0, 0);
   if (prof) prof(env.owner, 1, 1);
