@@ -10,6 +10,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "usp_math.cuh"
+
 namespace usp {
 
 constexpr double kB = 1.380649e-23;  // Boltzmann constant [J/K]
@@ -47,6 +49,7 @@ struct Species {
   // derived on the host: T_ref^omega, pi d_ref^2 / sigma_vib, R = k_B / m,
   // and the VSS mu_ref and tau_c / (mu / p) at this omega
   double Tref_w, zv_ht, R, mu_ref0, tauf0;
+  double iT_ref, iR, iRtheta;   // 1 / T_ref, 1 / R, 1 / (R Theta_v)
   int method;   // 0 USP-FPM (Sec. 3, 4), 1 the plain FPM method (Sec. 2.C)
 };
 
@@ -478,12 +481,73 @@ __device__ __forceinline__ void collision_numbers(const Species& s, const S& Ttr
   zv = (s.C1 / (s.Tref_w * xw)) * exp(s.C2 / cbrt(Ttr)) + s.zv_ht * sqrt(Ttr / s.T_ref) / xw;
 }
 
+// The fixed point x = F(x) of Sec. 3.A.1's implicit c_v,vib(T_1): with T_check(x) =
+// T_tr + (g_rot c_rot (T_rot - T_tr) + g_vib x (T_vib - T_tr)) / den(x),
+// F is the secant of e_vib between T_check and T_vib, or c_v,vib(T_vib) where
+// the two differ by less than 1e-9.  Newton's method: F' = -g_vib (c_v,vib(T_check) -
+// F) / den needs no function that F does not, and the passes are first made
+// in FP32 from c_v,vib(T_tr); one FP64 pass then usually ends it, where the
+// plain iteration took six to eight at 4,500 cycles each.  A pass that moves
+// x by ch leaves an error of at most (g_vib ch)^2 / x (the curvature of F is
+// of order g_vib^2 / x): the passes end when g_vib ch <= 1e-8 x, or when ch is
+// below the rounding of the secant, whose numerator cancels near equilibrium.
+// evT, cvT: e_vib and c_v,vib at T_vib.
+__device__ __forceinline__ double solve_cv_T1(double Rtheta, double theta, double R, double gr,
+                                              double gv, double Ttr, double Trot, double Tvib,
+                                              double evT, double cvT) {
+  const double D = 1.5 * R + gr * R, a0 = gr * R * (Trot - Ttr), dT = Tvib - Ttr;
+  double x;
+  {
+    const float th = (float)theta, Rf = (float)R, gvf = (float)gv, Df = (float)D, a0f = (float)a0;
+    const float Tt = (float)Ttr, Tv = (float)Tvib, dTf = (float)dT, evf = (float)evT,
+                cvf = (float)cvT;
+    auto cv32 = [&](float T, float& e) {
+      const float xx = fminf(__fdividef(th, T), 80.0f), iE = __frcp_rn(expm1f(xx));
+      e = Rf * th * iE;
+      return Rf * xx * xx * iE * (1.0f + iE);
+    };
+    float ef, xf = cv32(fmaxf(Tt, 1.0f), ef);
+    for (int it = 0; it < 4; ++it) {
+      const float iden = __frcp_rn(fmaf(gvf, xf, Df));
+      const float Tc = fmaf(fmaf(gvf * xf, dTf, a0f), iden, Tt), d = Tc - Tv;
+      float F, dF = 0.0f;
+      if (!(Tc > 1.0f) || !(fabsf(d) > 1e-6f * Tv)) {
+        F = cvf;
+      } else if (fabsf(d) < 0.02f * Tv) {
+        F = cv32(0.5f * (Tc + Tv), ef);
+      } else {
+        const float cv = cv32(Tc, ef);
+        F = __fdividef(ef - evf, d);
+        dF = -gvf * (cv - F) * iden;
+      }
+      const float step = __fdividef(F - xf, 1.0f - dF);
+      xf += step;
+      if (fabsf(step) <= 1e-6f * fabsf(xf)) break;
+    }
+    x = (double)xf;
+  }
+  for (int it = 0; it < 50; ++it) {
+    const double iden = d_rcp(fma(gv, x, D));
+    const double Tc = fma(fma(gv * x, dT, a0), iden, Ttr), d = Tc - Tvib;
+    const double xx = theta * d_rcp(Tc), iE = d_rcp(d_expm1(xx));
+    const bool cold = !(Tc > 0.0);
+    const double ec = cold ? 0.0 : Rtheta * iE, cvc = cold ? 0.0 : R * (xx * xx) * (iE * (1.0 + iE));
+    const bool near = fabs(d) <= 1e-9 * fmax(fabs(Tc), fabs(Tvib));
+    const double id = d_rcp(d), F = near ? cvT : (ec - evT) * id;
+    const double dF = near ? 0.0 : -gv * (cvc - F) * iden;
+    const double step = (F - x) * d_rcp(1.0 - dF), ch = fabs(step);
+    x += step;
+    if (gv * ch <= 1e-8 * fabs(x)) break;
+    // rounding of the secant
+    if (!near && ch <= 4.0 * 0x1p-52 * (fabs(ec) + fabs(evT)) * fabs(id)) break;
+  }
+  return x;
+}
+
 // Per-cell coefficients of Sec. 3.A: alpha = A^(1/3) (the real cube root,
 // negative when dt >= 2 mu / (p Pr)), nu, the gamma
-// coefficients with the implicit c_v,vib(T_1) (fixed point started at
-// c_v,vib(T_tr), relative tolerance 1e-14 or the secant's own rounding,
-// whichever is larger, at most 50 passes), and the second-order energy
-// targets.
+// coefficients with the implicit c_v,vib(T_1) (solve_cv_T1), and the
+// second-order energy targets.
 template <typename S>
 struct CellCoeffsT {
   S mu_p, Pr, A, B, alpha, nu_ref;
@@ -528,26 +592,24 @@ __device__ inline CellCoeffsT<S> cell_coeffs_t(const Species& s, const S& omega,
   const S gr = dt / (dt + 2.0 * tau_rot);
   const S gv = dt / (dt + 2.0 * tau_vib);
   const S evT = e_vib_T<S>(s, Tvib);
-  S x = cv_vib_T<S>(s, Ttr);
-  for (int it = 0; it < 50; ++it) {
-    // T_check = T_tr + (gamma_tr-rot/2 (T_rot - T_tr) + gamma_tr-vib/2 (T_vib - T_tr)) / c_tr
-    // with gamma / 2 c_tr = g c / den: one division per pass
-    const S idn = 1.0 / (ctr + gr * crot + gv * x);
-    const S Tc = Ttr + (gr * crot * (Trot - Ttr) + gv * x * (Tvib - Ttr)) * idn;
-    const S scale = fmax(fabs(Tc), fabs(Tvib));
-    S xn;
-    double noise = 0.0;   // rounding of the secant (its numerator cancels near equilibrium)
-    if (fabs(Tc - Tvib) <= 1e-9 * scale) {
-      xn = cv_vib_T<S>(s, Tvib);
+  // the value of the fixed point, then its derivatives: those of F at that
+  // value, over 1 - F'
+  const double xv = solve_cv_T1(R * s.theta_v, s.theta_v, R, (double)gr, (double)gv, (double)Ttr,
+                                (double)Trot, (double)Tvib, (double)evT,
+                                cv_vib_T<double>(s, (double)Tvib));
+  S x(xv);
+  if constexpr (sizeof(S) != sizeof(double)) {
+    const S iden = 1.0 / (ctr + gr * crot + gv * xv);
+    const S Tc = Ttr + (gr * crot * (Trot - Ttr) + gv * xv * (Tvib - Ttr)) * iden;
+    if (!(fabs(Tc - Tvib) <= 1e-9 * fmax(fabs(Tc), fabs(Tvib)))) {
+      const S F = (e_vib_T<S>(s, Tc) - evT) / (Tc - Tvib);
+      const double dF = -(double)gv * (cv_vib_T<double>(s, (double)Tc) - xv) * (double)iden;
+      const double k = 1.0 / (1.0 - dF);
+      for (int i = 0; i < 3; ++i) x.d[i] = F.d[i] * k;
     } else {
-      const S ec = e_vib_T<S>(s, Tc);
-      xn = (ec - evT) / (Tc - Tvib);
-      noise = 4.0 * 0x1p-52 * (::fabs((double)ec) + ::fabs((double)evT)) /
-              ::fabs((double)(Tc - Tvib));
+      const S F = cv_vib_T<S>(s, Tvib);
+      for (int i = 0; i < 3; ++i) x.d[i] = F.d[i];
     }
-    const S ch = fabs(xn - x);
-    x = xn;
-    if (ch <= 1e-14 * fabs(xn) || ch <= noise) break;
   }
   const S idn = 1.0 / (ctr + gr * crot + gv * x);
   c.g_tr_rot = 2.0 * gr * ctr * crot * idn;
@@ -565,21 +627,66 @@ __device__ inline CellCoeffsT<S> cell_coeffs_t(const Species& s, const S& omega,
 
 typedef CellCoeffsT<double> CellCoeffs;
 
+// A cell's vibrational state from its mean level: L = Theta / T_vib = log(1 +
+// 1/ebar), so that exp(L) - 1 = 1/ebar and T_vib, e_vib = R Theta ebar, c_v,vib and
+// the Eucken fraction x / (exp x - 1) take one logarithm.
+struct VibState {
+  double Tvib, ev, cv, xi;
+};
+__device__ __forceinline__ VibState vib_state(const Species& s, double ebar) {
+  const bool cold = !(ebar > 0.0);
+  const double L = d_log1p_inv(cold ? 1.0 : ebar);
+  return cold ? VibState{0.0, 0.0, 0.0, 0.0}
+              : VibState{d_div(s.theta_v, L), s.R * s.theta_v * ebar,
+                         s.R * (L * L) * (ebar * (1.0 + ebar)), L * ebar};
+}
+
+// cell_coeffs_t for plain FP64 on the functions of usp_math.cuh, with the
+// cell's mean level in place of T_vib.  One thread's chain: 37 us with the
+// library's functions and the plain T_1 iteration (the cell update of one
+// cell), 9 us now.
 __device__ inline CellCoeffs cell_coeffs(const Species& s, double n, double dt, double Ttr,
-                                         double Trot, double Tvib) {
-  return cell_coeffs_t<double>(s, s.omega, s.Z_rot, n, dt, Ttr, Trot, Tvib);
+                                         double Trot, const VibState& v) {
+  CellCoeffs c;
+  const double R = s.R, ctr = 1.5 * R;
+  const double lt = d_log(Ttr * s.iT_ref);
+  const double xw = d_exp(s.omega * lt);
+  c.mu_p = s.mu_ref0 * xw * d_rcp(n * kB * Ttr);
+  const double tau_c = s.tauf0 * c.mu_p;
+  double zr, zv;
+  collision_numbers<double>(s, Ttr, xw, s.Z_rot, zr, zv);
+  c.Pr = d_div(fma(2.0, v.xi, 14.0), fma(2.0, v.xi, 19.0));
+  const double m2 = 2.0 * c.mu_p, pd = c.Pr * dt;
+  c.A = d_div(m2 - pd, m2 + pd);
+  c.B = d_div(m2 - dt, m2 + dt);
+  const double gr = d_div(dt, fma(2.0 * zr, tau_c, dt)), gv = d_div(dt, fma(2.0 * zv, tau_c, dt));
+  c.ok = c.A > -1.0 && c.A < 1.0;
+  c.alpha = c.ok ? d_cbrt(c.A) : 0.0;
+  const double a2 = c.alpha * c.alpha;
+  c.nu_ref = d_div(c.B - a2, 1.0 - a2);
+  const double x = solve_cv_T1(R * s.theta_v, s.theta_v, R, gr, gv, Ttr, Trot, v.Tvib, v.ev, v.cv);
+  const double idn = d_rcp(fma(gv, x, fma(gr, R, ctr)));
+  c.g_tr_rot = 2.0 * gr * ctr * R * idn;
+  c.g_tr_vib = 2.0 * gv * ctr * x * idn;
+  c.g_rot_vib = 2.0 * gr * gv * R * x * idn;
+  c.e_rot_tgt = R * Trot + c.g_tr_rot * (Ttr - Trot) - c.g_rot_vib * (Trot - v.Tvib);
+  c.e_vib_tgt = v.ev + c.g_tr_vib * (Ttr - v.Tvib) + c.g_rot_vib * (Trot - v.Tvib);
+  c.tgt_clamped = false;
+  if (c.e_rot_tgt < 0.0) { c.e_rot_tgt = 0.0; c.tgt_clamped = true; }
+  if (c.e_vib_tgt < 0.0) { c.e_vib_tgt = 0.0; c.tgt_clamped = true; }
+  return c;
 }
 
 // Relaxation temperatures (Eqs. T_tr_USP, T_rot_USP, T_vib_USP) for a given
 // alpha; negative values are clamped to 0 and reported.
 __device__ __forceinline__ void relax_temps(const Species& s, const CellCoeffs& c, double alpha,
-                                            double Ttr, double Trot, double Tvib, double& ttr,
-                                            double& trot, double& evr, bool& clamped) {
-  const double R = gasR(s);
-  const double oma2 = 1.0 - alpha * alpha;
-  ttr = Ttr - (c.g_tr_rot * (Ttr - Trot) + c.g_tr_vib * (Ttr - Tvib)) / (oma2 * 1.5 * R);
-  trot = Trot + (c.g_tr_rot * (Ttr - Trot) - c.g_rot_vib * (Trot - Tvib)) / (oma2 * R);
-  evr = e_vib_T(s, Tvib) + (c.g_tr_vib * (Ttr - Tvib) + c.g_rot_vib * (Trot - Tvib)) / oma2;
+                                            double Ttr, double Trot, double Tvib, double ev,
+                                            double& ttr, double& trot, double& evr,
+                                            bool& clamped) {
+  const double io = d_rcp(1.0 - alpha * alpha), ioR = io * s.iR;
+  ttr = Ttr - (c.g_tr_rot * (Ttr - Trot) + c.g_tr_vib * (Ttr - Tvib)) * (ioR * (2.0 / 3.0));
+  trot = Trot + (c.g_tr_rot * (Ttr - Trot) - c.g_rot_vib * (Trot - Tvib)) * ioR;
+  evr = ev + (c.g_tr_vib * (Ttr - Tvib) + c.g_rot_vib * (Trot - Tvib)) * io;
   clamped = false;
   if (ttr < 0.0) { ttr = 0.0; clamped = true; }
   if (trot < 0.0) { trot = 0.0; clamped = true; }
@@ -599,6 +706,21 @@ __device__ __forceinline__ bool chol3(const T* M, T* L) {
   const T d2 = M[2] - l20 * l20 - l21 * l21;
   if (!(d2 > T(0))) return false;
   L[0] = l00; L[1] = l10; L[2] = l11; L[3] = l20; L[4] = l21; L[5] = sqrt(d2);
+  return true;
+}
+
+// the same for a per-cell matrix, by reciprocal square roots (usp_math.cuh)
+__device__ __forceinline__ bool chol3_cell(const double* M, double* L) {
+  if (!(M[0] > 0.0)) return false;
+  const double r0 = d_rsqrt(M[0]);
+  const double l10 = M[3] * r0, l20 = M[4] * r0;
+  const double d1 = M[1] - l10 * l10;
+  if (!(d1 > 0.0)) return false;
+  const double r1 = d_rsqrt(d1);
+  const double l21 = (M[5] - l20 * l10) * r1;
+  const double d2 = M[2] - l20 * l20 - l21 * l21;
+  if (!(d2 > 0.0)) return false;
+  L[0] = M[0] * r0; L[1] = l10; L[2] = d1 * r1; L[3] = l20; L[4] = l21; L[5] = d_sqrt(d2);
   return true;
 }
 
@@ -737,23 +859,23 @@ struct FpmCell {
 };
 
 __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const double* Pi,
-                                   double Ttr, double Trot, double Tvib) {
+                                   double Ttr, double Trot, const VibState& v) {
   FpmCell o;
   o.fixed = o.nu_zero = o.failed = o.clamped = false;
   const double R = gasR(s);
   const double p = n * kB * Ttr;
-  const double xw = exp(s.omega * log(Ttr / s.T_ref));
-  const double mu = s.mu_ref0 * xw;
-  const double tau_c = s.tauf0 * mu / p;
+  const double xw = d_exp(s.omega * d_log(Ttr * s.iT_ref));
+  const double mu_p = s.mu_ref0 * xw * d_rcp(p);
+  const double tau_c = s.tauf0 * mu_p;
   double zr, zv;
   collision_numbers<double>(s, Ttr, xw, s.Z_rot, zr, zv);
-  const double Pr = prandtl_T<double>(s, Tvib);
-  const double nu0 = 1.0 - 3.0 / (2.0 * Pr);
-  const double tau = 2.0 * mu * (1.0 - nu0) / p;
+  // nu = 1 - 3 / (2 Pr), Pr = (14 + 2 xi) / (19 + 2 xi)
+  const double nu0 = 1.0 - d_div(1.5 * fma(2.0, v.xi, 19.0), fma(2.0, v.xi, 14.0));
+  const double tau = 2.0 * mu_p * (1.0 - nu0), itau = d_rcp(tau);
   o.ok = tau > 0.0;
-  o.alpha = o.ok ? exp(-dt / tau) : 0.0;
-  const double grot = tau / (2.0 * zr * tau_c), gvib = tau / (2.0 * zv * tau_c);
-  const double ev = e_vib_T<double>(s, Tvib), evt = e_vib_T<double>(s, Ttr);
+  o.alpha = o.ok ? d_exp(-dt * itau) : 0.0;
+  const double grot = d_div(tau, 2.0 * zr * tau_c), gvib = d_div(tau, 2.0 * zv * tau_c);
+  const double ev = v.ev, evt = R * s.theta_v * d_rcp(d_expm1(s.theta_v * d_rcp(Ttr)));
   double etr = 1.5 * R * Ttr + grot * (R * Trot - R * Ttr) + gvib * (ev - evt);
   double erot = R * Trot + grot * (R * Ttr - R * Trot);
   double evib = ev + gvib * (evt - ev);
@@ -761,10 +883,10 @@ __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const 
   if (erot < 0.0) { erot = 0.0; o.clamped = true; }
   if (evib < 0.0) { evib = 0.0; o.clamped = true; }
   const double RT = R * Ttr, RTrel = etr / 1.5;
-  o.Trot_rel = erot / R;
-  const double ebar = evib / (R * s.theta_v);
-  o.lam_up = 2.0 * dt * ebar / tau;
-  o.lam_dn = 2.0 * dt * (1.0 + ebar) / tau;
+  o.Trot_rel = erot * s.iR;
+  const double ebar = evib * s.iRtheta;
+  o.lam_up = 2.0 * dt * ebar * itau;
+  o.lam_dn = 2.0 * dt * (1.0 + ebar) * itau;
   const double a2 = o.alpha * o.alpha;
   o.e_rot_tgt = erot + (R * Trot - erot) * a2;
   o.e_vib_tgt = evib + (ev - evib) * a2;
@@ -778,7 +900,7 @@ __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const 
     M[5] = nu_ * Pi[5];
   };
   fill(nu);
-  if (chol3(M, o.L)) return o;
+  if (chol3_cell(M, o.L)) return o;
   o.fixed = true;
   double lmin, lmax;
   sym3_minmax(Pi, lmin, lmax);
@@ -789,7 +911,7 @@ __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const 
   }
   nu = nu * (1.0 - 1e-6);
   fill(nu);
-  if (chol3(M, o.L)) return o;
+  if (chol3_cell(M, o.L)) return o;
   o.nu_zero = true;
   const double sq = RTrel > 0.0 ? sqrt(RTrel) : 0.0;
   o.failed = !(RTrel > 0.0);
@@ -832,14 +954,16 @@ struct DriftDiff {
 };
 
 __device__ inline DriftDiff drift_diffusion(const Species& s, const CellCoeffs& c, double dt,
-                                            const double* Pi, double Ttr, double Trot, double Tvib) {
+                                            const double* Pi, double Ttr, double Trot,
+                                            const VibState& v) {
+  const double Tvib = v.Tvib;
   DriftDiff o;
   const double R = gasR(s);
   o.alpha = c.alpha;
   o.fixed = false;
   o.nu_zero = false;
   o.failed = false;
-  relax_temps(s, c, o.alpha, Ttr, Trot, Tvib, o.Ttr_rel, o.Trot_rel, o.evib_rel, o.clamped);
+  relax_temps(s, c, o.alpha, Ttr, Trot, Tvib, v.ev, o.Ttr_rel, o.Trot_rel, o.evib_rel, o.clamped);
   double nu = c.nu_ref;
   double M[6];
   auto fill = [&](double nu_) {
@@ -851,7 +975,7 @@ __device__ inline DriftDiff drift_diffusion(const Species& s, const CellCoeffs& 
     M[5] = nu_ * Pi[5];
   };
   fill(nu);
-  if (chol3(M, o.L)) return o;
+  if (chol3_cell(M, o.L)) return o;
   o.fixed = true;
   double lmin, lmax;
   sym3_minmax(Pi, lmin, lmax);
@@ -871,10 +995,10 @@ __device__ inline DriftDiff drift_diffusion(const Species& s, const CellCoeffs& 
     const double prm = 2.0 * c.mu_p * (1.0 - am * am * am) / (dt * (1.0 + am * am * am));
     o.alpha = (fabs(prm - c.Pr) < fabs(prp - c.Pr)) ? am : ap;
     bool cl;
-    relax_temps(s, c, o.alpha, Ttr, Trot, Tvib, o.Ttr_rel, o.Trot_rel, o.evib_rel, cl);
+    relax_temps(s, c, o.alpha, Ttr, Trot, Tvib, v.ev, o.Ttr_rel, o.Trot_rel, o.evib_rel, cl);
     o.clamped = o.clamped || cl;
     fill(nu);
-    ok = chol3(M, o.L);
+    ok = chol3_cell(M, o.L);
   }
   if (!ok) {
     // nu = 0 with alpha^2 = B (Eq. alpha_USP_positivity_1 at nu = 0): inside
@@ -886,7 +1010,7 @@ __device__ inline DriftDiff drift_diffusion(const Species& s, const CellCoeffs& 
     const double prm = 2.0 * c.mu_p * (1.0 - am * am * am) / (dt * (1.0 + am * am * am));
     o.alpha = (fabs(prm - c.Pr) < fabs(prp - c.Pr)) ? am : ap;
     bool cl;
-    relax_temps(s, c, o.alpha, Ttr, Trot, Tvib, o.Ttr_rel, o.Trot_rel, o.evib_rel, cl);
+    relax_temps(s, c, o.alpha, Ttr, Trot, Tvib, v.ev, o.Ttr_rel, o.Trot_rel, o.evib_rel, cl);
     o.clamped = o.clamped || cl;
     o.failed = !(o.Ttr_rel > 0.0);
     const double sq = o.failed ? 0.0 : sqrt(R * o.Ttr_rel);

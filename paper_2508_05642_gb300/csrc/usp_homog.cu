@@ -1029,11 +1029,11 @@ __device__ void write_params(const Species& sp, CellState& cs, CollideParams<T>&
   P.method = sp.method;
   P.pad_ = 0;
   if (!cs.active) return;
-  const double Tvib = T_vib_of_level(sp, cs.ebar);
+  const VibState vib = vib_state(sp, cs.ebar);
   if (sp.method == 1) {
     // the plain FPM method (Sec. 2.C): Gorji's velocity update and the
     // Milstein square form with alpha = exp(-dt/tau), Gillespie levels
-    const FpmCell f = fpm_cell(sp, cs.ndens, cs.dt, cs.Pi, cs.Ttr, cs.Trot, Tvib);
+    const FpmCell f = fpm_cell(sp, cs.ndens, cs.dt, cs.Pi, cs.Ttr, cs.Trot, vib);
     if (!f.ok) {
       atomicOr(flags, (uint32_t)F_A_NONPOS);
       cs.active = 0;
@@ -1049,18 +1049,18 @@ __device__ void write_params(const Species& sp, CellState& cs, CollideParams<T>&
       atomicOr(flags, (uint32_t)F_TREL_CLAMP);
       atomicAdd(&counters[C_TREL_CLAMP], 1ull);
     }
-    const double a = f.alpha, oma2 = 1.0 - a * a, sq = sqrt(oma2);
+    const double a = f.alpha, oma2 = 1.0 - a * a, sq = sqrt_fast(oma2);
     P.as = (T)(a * cs.s);
-    P.ar = (T)(a * sqrt(cs.r));
+    P.ar = (T)(a * sqrt_fast(cs.r));
     for (int i = 0; i < 6; ++i) P.Lp[i] = (T)(sq * f.L[i]);
     const double arot = R * f.Trot_rel * oma2 / 2.0;
     P.a_rot = (T)arot;
-    P.sqrt_a = (T)sqrt(arot);
+    P.sqrt_a = (T)sqrt_fast(arot);
     P.p_nb = (T)f.lam_up;
     P.p_b = (T)f.lam_dn;
     return;
   }
-  const CellCoeffs c = cell_coeffs(sp, cs.ndens, cs.dt, cs.Ttr, cs.Trot, Tvib);
+  const CellCoeffs c = cell_coeffs(sp, cs.ndens, cs.dt, cs.Ttr, cs.Trot, vib);
   if (!c.ok) {
     atomicOr(flags, (uint32_t)F_A_NONPOS);
     cs.active = 0;
@@ -1075,7 +1075,7 @@ __device__ void write_params(const Species& sp, CellState& cs, CollideParams<T>&
   }
   // homogeneous cell: the fields at every particle are the cell values, so
   // D_tr, its Cholesky factor and the relaxation temperatures are per cell
-  const DriftDiff dd = drift_diffusion(sp, c, cs.dt, cs.Pi, cs.Ttr, cs.Trot, Tvib);
+  const DriftDiff dd = drift_diffusion(sp, c, cs.dt, cs.Pi, cs.Ttr, cs.Trot, vib);
   if (dd.fixed) atomicAdd(&counters[C_CHOL_FIX], 1ull);
   if (dd.nu_zero) atomicAdd(&counters[C_NU_ZERO], 1ull);
   if (dd.failed) atomicOr(flags, (uint32_t)F_CHOL_FAIL_AFTER_FIX);
@@ -1083,15 +1083,15 @@ __device__ void write_params(const Species& sp, CellState& cs, CollideParams<T>&
     atomicOr(flags, (uint32_t)F_TREL_CLAMP);
     atomicAdd(&counters[C_TREL_CLAMP], 1ull);
   }
-  const double a = dd.alpha, oma2 = 1.0 - a * a, sq = sqrt(oma2);
+  const double a = dd.alpha, oma2 = 1.0 - a * a, sq = sqrt_fast(oma2);
   P.as = (T)(a * cs.s);
-  P.ar = (T)(a * sqrt(cs.r));
+  P.ar = (T)(a * sqrt_fast(cs.r));
   for (int i = 0; i < 6; ++i) P.Lp[i] = (T)(sq * dd.L[i]);
   const double arot = R * dd.Trot_rel * oma2 / 2.0;
   P.a_rot = (T)arot;
-  P.sqrt_a = (T)sqrt(arot);
-  const double eb = dd.evib_rel / (R * sp.theta_v);
-  P.p_nb = (T)(1.0 / (1.0 + eb * oma2));
+  P.sqrt_a = (T)sqrt_fast(arot);
+  const double eb = dd.evib_rel * sp.iRtheta;
+  P.p_nb = (T)d_rcp(1.0 + eb * oma2);
   P.p_b = (T)((1.0 + eb) * oma2);
 }
 
@@ -1283,11 +1283,11 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
   const double R = gasR(sp);
   const double Rth = R * sp.theta_v;
   const CellSums S = sums[c];
-  const double invN = 1.0 / (double)cs.N;
+  const double invN = d_rcp((double)cs.N);
   const double sumI = (double)((long long)S.I + S.net);
   // rotational scaling
   const double er_star = S.v[9] * invN;
-  const double r = er_star > 0.0 ? cs.e_rot_tgt / er_star : 1.0;
+  const double r = er_star > 0.0 ? d_div(cs.e_rot_tgt, er_star) : 1.0;
   const double e_rot_new = r * er_star;
   const double e_vib_new = Rth * sumI * invN;
   // velocity scaling about the post-collision mean
@@ -1303,7 +1303,7 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
   const double e_tr_n = 0.5 * (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]);
   const double e_rot_n = R * cs.Trot;
   const double e_vib_n = Rth * cs.ebar;
-  const double rad = (e_tr_n + e_rot_n + e_vib_n - e_rot_new - e_vib_new) / etr_star;
+  const double rad = d_div(e_tr_n + e_rot_n + e_vib_n - e_rot_new - e_vib_new, etr_star);
   double s;
   double Un[3] = {cs.U[0], cs.U[1], cs.U[2]};
   double Us[3] = {cs.U[0] + m0, cs.U[1] + m1, cs.U[2] + m2};
@@ -1313,12 +1313,12 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
     s = 1.0;  // velocities stay as collided: c = U* + (c* - U*)
     for (int i = 0; i < 3; ++i) Un[i] = Us[i];
   } else {
-    s = sqrt(rad);
+    s = d_sqrt(rad);
   }
   for (int i = 0; i < 3; ++i) { cs.U[i] = Un[i]; cs.Us[i] = Us[i]; }
   for (int i = 0; i < 6; ++i) cs.Pi[i] = s * s * Ps[i];
-  cs.Ttr = (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]) / (3.0 * R);
-  cs.Trot = e_rot_new / R;
+  cs.Ttr = (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]) * (sp.iR * (1.0 / 3.0));
+  cs.Trot = e_rot_new * sp.iR;
   cs.ebar = sumI * invN;
   cs.s = s;
   cs.r = r;
@@ -1706,6 +1706,9 @@ Species to_dev(const usp_species* s) {
   d.Tref_w = std::pow(s->T_ref, s->omega);
   d.zv_ht = s->sigma_vib > 0 ? kPi * s->d_ref * s->d_ref / s->sigma_vib : 0.0;
   d.R = kB / s->m;
+  d.iT_ref = 1.0 / s->T_ref;
+  d.iR = 1.0 / d.R;
+  d.iRtheta = 1.0 / (d.R * s->theta_v);
   const double ca = s->c_alpha, w = s->omega;
   d.mu_ref0 = 5.0 * (ca + 1.0) * (ca + 2.0) * std::sqrt(s->m * kB * s->T_ref / kPi) /
               (4.0 * ca * (5.0 - 2.0 * w) * (7.0 - 2.0 * w) * s->d_ref * s->d_ref);

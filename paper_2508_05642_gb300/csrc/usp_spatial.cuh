@@ -707,8 +707,11 @@ __global__ void ch_coeffs(int ny, double F_num, double vol, const double* __rest
       continue;
     }
     cs.n = (double)cs.N * F_num / v;
-    const CellCoeffsT<S> k =
-        cell_coeffs_t<S>(sp, omega, zrot, cs.n, dt, cs.Ttr, cs.Trot, S(cs.Tvib));
+    CellCoeffsT<S> k;
+    if constexpr (std::is_same<S, double>::value)
+      k = cell_coeffs(sp, cs.n, dt, cs.Ttr, cs.Trot, vib_state(sp, cs.ebar));
+    else
+      k = cell_coeffs_t<S>(sp, omega, zrot, cs.n, dt, cs.Ttr, cs.Trot, S(cs.Tvib));
     if (!k.ok) {
       tally_or(tal, (uint32_t)F_A_NONPOS);
       cs.active = 0;
@@ -888,7 +891,7 @@ __global__ void ch_coeffs_fpm(int ncell, double F_num, double vol, const double*
       continue;
     }
     cs.n = (double)cs.N * F_num / v;
-    const FpmCell f = fpm_cell(sp, cs.n, dt, cs.Pi, cs.Ttr, cs.Trot, cs.Tvib);
+    const FpmCell f = fpm_cell(sp, cs.n, dt, cs.Pi, cs.Ttr, cs.Trot, vib_state(sp, cs.ebar));
     if (!f.ok) {
       tally_or(tal, (uint32_t)F_A_NONPOS);
       cs.active = 0;
