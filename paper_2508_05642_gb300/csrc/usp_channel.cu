@@ -672,6 +672,7 @@ struct ChannelCtx {
   double* fpmrec;           // the plain FPM method: kFpmRec per-cell constants (else null)
   double* prof;             // time-averaged profiles (USP_NPROF x ny per block)
   double* grad;             // the objective's gradient (3 doubles, gradient form)
+  double* hstage;           // read-back buffer (null: none kept)
 };
 
 namespace {
@@ -980,8 +981,11 @@ int ch_get_particles(ChannelCtx* h, const ChEnv& env, double* y, double* cx, dou
   const long long n = h->n;
   if (n == 0) return USP_OK;
   cudaStream_t s = env.stream;
-  double* tmp = (double*)env.alloc(env.owner, 5 * n * sizeof(double));
+  // a small buffer is kept for the next call, a large one given back
+  double* tmp = h->hstage;
+  if (!tmp) tmp = (double*)env.alloc(env.owner, 5 * n * sizeof(double));
   if (!tmp) return USP_ENOMEM;
+  if (n * 5 * (long long)sizeof(double) <= (64ll << 20)) h->hstage = tmp;
   const int b = h->cur;
   const int nb = (int)((n + 255) / 256);
   if (env.precision == USP_FP32)
@@ -1000,20 +1004,19 @@ int ch_get_particles(ChannelCtx* h, const ChEnv& env, double* y, double* cx, dou
     ch_to_host_layout<double, double><<<nb, 256, 0, s>>>(n, h->keycell,
         (const ChCellT<double>*)h->cells, (double*)h->st[b][0], (double*)h->st[b][1],
         (double*)h->st[b][2], (double*)h->st[b][3], (double*)h->st[b][4], tmp);
-  std::vector<double> hl(5 * n);
   bool ok = cudaGetLastError() == cudaSuccess;
-  ok = ok && cudaMemcpyAsync(hl.data(), tmp, 5 * n * sizeof(double), cudaMemcpyDeviceToHost, s) ==
-                 cudaSuccess;
+  double* const out[5] = {y, cx, cy, cz, erot};
+  for (int f = 0; f < 5; ++f)
+    if (out[f])
+      ok = ok && cudaMemcpyAsync(out[f], tmp + f * n, n * sizeof(double), cudaMemcpyDeviceToHost,
+                                 s) == cudaSuccess;
   ok = ok && cudaMemcpyAsync(lev, h->lv[b], n * 4, cudaMemcpyDeviceToHost, s) == cudaSuccess;
   if (pid)
     ok = ok && cudaMemcpyAsync(pid, h->pd[b], n * 4, cudaMemcpyDeviceToHost, s) == cudaSuccess;
   ok = ok && cudaStreamSynchronize(s) == cudaSuccess;
-  env.release(env.owner, tmp);
+  if (!ok) cudaStreamSynchronize(s);   // copies to the caller's arrays may be in flight
+  if (!h->hstage) env.release(env.owner, tmp);
   if (!ok) return USP_ECUDA;
-  for (long long j = 0; j < n; ++j) {
-    if (y) y[j] = hl[j];
-    cx[j] = hl[n + j]; cy[j] = hl[2 * n + j]; cz[j] = hl[3 * n + j]; erot[j] = hl[4 * n + j];
-  }
   return USP_OK;
 }
 
