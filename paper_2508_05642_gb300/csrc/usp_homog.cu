@@ -2267,13 +2267,16 @@ int autotune(usp_ctx* c) {
   const int last_cell = c->ncell - 1;
   const long long end = c->h_poff[last_cell] +
       ((c->h_uoff[last_cell + 1] - c->h_uoff[last_cell]) + kAlign - 1) / kAlign * kAlign;
-  const size_t bytes = (size_t)end * (4 * es + 4);
-  unsigned char* scratch = (unsigned char*)dev_alloc(c, bytes + sizeof(CellSums) * c->ncell + 512);
+  // the state's copy, rounded up to where the sums begin, the sums, and
+  // 256 bytes each of flags and counters
+  const size_t state_bytes = ((size_t)end * (4 * es + 4) + 255) & ~(size_t)255;
+  const size_t bytes = state_bytes + sizeof(CellSums) * c->ncell + 512;
+  unsigned char* scratch = (unsigned char*)dev_alloc(c, bytes);
   if (!scratch) return USP_ENOMEM;
   void* sx = scratch; void* sy = scratch + end * es; void* sz = scratch + 2 * end * es;
   void* se = scratch + 3 * end * es;
   int* sl = (int*)(scratch + 4 * end * es);
-  CellSums* ssum = (CellSums*)(scratch + ((bytes + 255) & ~(size_t)255));
+  CellSums* ssum = (CellSums*)(scratch + state_bytes);
   uint32_t* sflags = (uint32_t*)((unsigned char*)ssum + sizeof(CellSums) * c->ncell);
   unsigned long long* scnt = (unsigned long long*)((unsigned char*)sflags + 256);
   auto fresh = [&]() -> int {
@@ -2320,7 +2323,7 @@ int autotune(usp_ctx* c) {
   if (!c->cfg.alloc) cudaFree(scratch);
   else if (c->cfg.free_) c->cfg.free_(scratch, c->cfg.alloc_user);
   c->owned.erase(std::find(c->owned.begin(), c->owned.end(), (void*)scratch));
-  c->device_bytes -= (long long)(((bytes + sizeof(CellSums) * c->ncell + 512) + 255) & ~(size_t)255);
+  c->device_bytes -= (long long)((bytes + 255) & ~(size_t)255);
   return USP_OK;
 }
 
