@@ -383,7 +383,8 @@ __global__ void ch_collide(int ny, const ChCellT<S>* __restrict__ cells,
       ++nfb;
     }
     T v0 = cx[j], v1 = cy[j], v2 = cz[j], en = er[j];
-    const int ln = collide_particle_t(P, f, v0, v1, v2, en, lev[j], pid[j], step, rk, tl);
+    const int ln = collide_particle_t<std::is_same<T, double>::value>(P, f, v0, v1, v2, en, lev[j],
+                                                                      pid[j], step, rk, tl);
     cx[j] = v0; cy[j] = v1; cz[j] = v2; er[j] = en;
     lev[j] = ln;
     maxI = max(maxI, ln);

@@ -232,9 +232,14 @@ __device__ __forceinline__ double uniform23_d(uint32_t x) {
   return (2.0 * (double)(x >> 9) + 1.0) * 5.9604644775390625e-08;             // 2^-24
 }
 
-// the jump-sampler uniform of a word, in the working type
+// the jump-sampler uniform of a word, in the working type: in FP64 the float
+// uniform (normal, exact) with its bits moved, which spares the FP64 pipe a
+// conversion and a multiply-add
 template <typename T>
-__device__ __forceinline__ T jump_uniform(uint32_t x) { return T(uniform23_d(x)); }
+__device__ __forceinline__ T jump_uniform(uint32_t x) {
+  const uint32_t u = __float_as_uint(uniform_open<float>(x));
+  return T(__hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29)));
+}
 template <>
 __device__ __forceinline__ float jump_uniform<float>(uint32_t x) { return uniform_open<float>(x); }
 
@@ -267,6 +272,41 @@ __device__ __forceinline__ void particle_draws(uint32_t pid, uint32_t step,
   j6 = w.w;
 }
 
+
+// Warp totals of the N values in a[] by recursive halving: in every round the
+// lanes of a pair exchange the halves that the other one keeps, N/2 + N/4 + ...
+// additions and shuffles per lane in place of 5 N.  The additions of one total
+// are those of a butterfly sum with the offsets 16, 8, 4, 2, 1, so the totals
+// are the same bit for bit.  Afterwards a[0] is the total of value `index`
+// (-1: this lane holds none).
+template <int N, int O, typename T>
+__device__ __forceinline__ void halve_rounds(T* a, int& base, int& count) {
+  if constexpr (O > 0) {
+    if constexpr (N == 1) {
+      a[0] += __shfl_xor_sync(0xffffffffu, a[0], O);
+      if (threadIdx.x & O) count = 0;   // the lower lane of each pair reports it
+      halve_rounds<1, O / 2>(a, base, count);
+    } else {
+      constexpr int H = (N + 1) / 2;
+      const bool up = threadIdx.x & O;
+#pragma unroll
+      for (int i = 0; i < H; ++i) {
+        const T hi = i + H < N ? a[i + H] : T(0);
+        const T send = up ? a[i] : hi, keep = up ? hi : a[i];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+      }
+      base += up ? H : 0;
+      count = up ? count - H : (count < H ? count : H);
+      halve_rounds<H, O / 2>(a, base, count);
+    }
+  }
+}
+template <int N, typename T>
+__device__ __forceinline__ int halve_totals(T* a) {
+  int base = 0, count = N;
+  halve_rounds<N, 16>(a, base, count);
+  return count > 0 ? base : -1;
+}
 
 // ---------------------------------------------------------------------------
 // Jump samplers of Eq. update_evib: sequential inversion with one uniform,
@@ -394,6 +434,8 @@ __device__ __forceinline__ int binv(int n, double p, double u, uint32_t& fl) {
 template <typename T>
 __device__ __forceinline__ int sample_nb(int r, T p, T u, uint32_t& fl) {
   if (r <= 0 || !(p < T(1))) return 0;
+  // the ground state's common outcome: P(0) = p > u (u > 2^-25, so p is normal)
+  if (r == 1 && u < p) return 0;
   return nb_inv(r, p, u, fl);
 }
 // B(n, p); p >= 1 gives n (and flags p > 1).

@@ -554,15 +554,13 @@ template <typename T>
 __device__ __forceinline__ void flush_sums_warp(const T* acc, int accI, int maxI,
                                                 CellSums* dst) {
   const int lane = threadIdx.x & 31;
-  double mine = 0.0;
+  T tot[10];
 #pragma unroll
-  for (int i = 0; i < 10; ++i) {
-    const T s = warp_sum(acc[i]);
-    if (lane == i) mine = (double)s;
-  }
-  const int sI = warp_sum(accI);
+  for (int i = 0; i < 10; ++i) tot[i] = acc[i];
+  const int at = halve_totals<10>(tot);
+  const int sI = __reduce_add_sync(0xffffffffu, accI);
   const int mI = __reduce_max_sync(0xffffffffu, maxI);
-  if (lane < 10) atomicAdd(&dst->v[lane], mine);
+  if (at >= 0) atomicAdd(&dst->v[at], (double)tot[0]);
   if (lane == 10) atomicAdd(&dst->I, (unsigned long long)(long long)sI);
   if (lane == 11 && mI > 0) atomicMax(&dst->maxI, mI);
 }

@@ -1167,7 +1167,7 @@ __global__ void __launch_bounds__(kBlk, 2) pl_collide(int ncell, const ChCellT<d
             for (int q = 0; q < kNF; ++q) f[q] = P.F[q];
             ++nfb;
           }
-          ln = collide_particle_t<sizeof(T) == 4>(P, f, v0, v1, v2, en, l0, id, step, rk, tl);
+          ln = collide_particle_t<true>(P, f, v0, v1, v2, en, l0, id, step, rk, tl);
         }
         cx[j] = v0; cy[j] = v1; cz[j] = v2; er[j] = en;
         lev[j] = ln;
@@ -1179,20 +1179,16 @@ __global__ void __launch_bounds__(kBlk, 2) pl_collide(int ncell, const ChCellT<d
         acc[9] += en;
         accI += ln;
       }
-      // warp totals; lane i < 10 converts total i (one FP64 conversion per warp)
-      T mine = T(0);
-#pragma unroll
-      for (int i = 0; i < 10; ++i) {
-        const T t = wsum(acc[i]);
-        mine = lane == i ? t : mine;
-      }
-      const double sv = (double)mine;
-      const long long sI = wsum((long long)accI);
+      // warp totals, each converted by the lane that holds it (one FP64
+      // conversion per warp)
+      const int at = halve_totals<10>(acc);
+      const double sv = (double)acc[0];
+      const int sI = __reduce_add_sync(0xffffffffu, accI);
       const int mI = __reduce_max_sync(0xffffffffu, maxI);
       ChSumsT<double>& sm = sums[c];
-      if (lane < 10) sm.v[lane] = sv;
+      if (at >= 0) sm.v[at] = sv;
       if (lane == 0) {
-        sm.I = (unsigned long long)sI;
+        sm.I = (unsigned long long)(long long)sI;
         sm.net = 0;
         sm.maxI = mI;
       }

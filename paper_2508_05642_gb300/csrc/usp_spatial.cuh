@@ -150,6 +150,39 @@ __device__ __forceinline__ void relax_fast(const P_& P, float alpha, const float
   if (evr < 0.f) { evr = 0.f; cl = true; }
 }
 
+// FP64: the same on the functions of usp_math.cuh.  The library's divisions,
+// square roots and expm1 were two thirds of the FP64 operations of a particle
+// (0.77 million particles on 240 x 160 cells: the plane's FP64 collision pass
+// 1.47 ms).
+__device__ __forceinline__ bool chol3_fast(const double* M, double* L) {
+  return chol3_cell(M, L);
+}
+template <typename P_>
+__device__ __forceinline__ void relax_fast(const P_& P, double alpha, const double* f, double& ttr,
+                                           double& trot, double& evr, bool& cl) {
+  const double io = d_rcp(1.0 - alpha * alpha), ioR = io * d_rcp(P.R);
+  const double x = P.gtr * (f[3] - f[4]), y = P.gtv * (f[3] - f[5]), z = P.grv * (f[4] - f[5]);
+  ttr = f[3] - (x + y) * (ioR * (2.0 / 3.0));
+  trot = f[4] + (x - z) * ioR;
+  const double ev =
+      f[5] > 0.0 ? P.R * P.theta * d_rcp(d_expm1(P.theta * d_rcp(f[5]))) : 0.0;
+  evr = ev + (y + z) * io;
+  cl = false;
+  if (ttr < 0.0) { ttr = 0.0; cl = true; }
+  if (trot < 0.0) { trot = 0.0; cl = true; }
+  if (evr < 0.0) { evr = 0.0; cl = true; }
+}
+
+// the square roots and reciprocals of the collision: FP32 as the form always
+// took them, FP64 on usp_math.cuh
+template <bool kFast, typename T>
+__device__ __forceinline__ T root_sel(const T& x) {
+  if constexpr (kFast && sizeof(T) == 8) return sqrt_fast(x);
+  else return sqrt(x);
+}
+__device__ __forceinline__ float rcp_fast(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ double rcp_fast(double x) { return d_rcp(x); }
+
 template <bool kFast, typename T, typename P_>
 __device__ __forceinline__ void relax_sel(const P_& P, T alpha, const T* f, T& ttr, T& trot,
                                           T& evr, bool& cl) {
@@ -178,7 +211,7 @@ template <bool kFast = false, typename T, typename P_>
 __device__ __forceinline__ int collide_particle_t(const P_& P, const T* f, T& vx, T& vy, T& vz,
                                                   T& e, int I, uint32_t id, uint32_t step,
                                                   const PhiloxRoundKeys& rk, CollideTally& t) {
-  static_assert(!kFast || sizeof(T) == 4, "the fast forms are FP32");
+  static_assert(!kFast || sizeof(T) == 4 || sizeof(T) == 8, "float or double");
   T alpha = P.alpha, nu = P.nu_ref, ttr, trot, evr;
   bool cl;
   relax_sel<kFast>(P, alpha, f, ttr, trot, evr, cl);
@@ -238,20 +271,20 @@ __device__ __forceinline__ int collide_particle_t(const P_& P, const T* f, T& vx
   uint32_t j5, j6;
   particle_draws(id, step, rk, g0, g1, g2, g3, j5, j6);
   // Eq. update_ci about the interpolated bulk velocity
-  const T a2 = alpha * alpha, sq = sqrt(T(1) - a2);
+  const T a2 = alpha * alpha, sq = root_sel<kFast>(T(1) - a2);
   const T v0 = f[0] + alpha * (vx - f[0]) + sq * (L[0] * g0);
   const T v1 = f[1] + alpha * (vy - f[1]) + sq * (L[1] * g0 + L[2] * g1);
   const T v2 = f[2] + alpha * (vz - f[2]) + sq * (L[3] * g0 + L[4] * g1 + L[5] * g2);
   vx = v0; vy = v1; vz = v2;
   // Eq. update_erot
   const T a = P.R * trot * (T(1) - a2) / T(2);
-  const T root = sqrt(e) * alpha + sqrt(a) * g3;
+  const T root = root_sel<kFast>(e) * alpha + root_sel<kFast>(a) * g3;
   e = a + root * root;
   // Eq. update_evib
   T eb, p_nb;
   if constexpr (kFast) {
-    eb = evr * __frcp_rn(P.R * P.theta);
-    p_nb = __frcp_rn(T(1) + eb * (T(1) - a2));
+    eb = evr * rcp_fast(P.R * P.theta);
+    p_nb = rcp_fast(T(1) + eb * (T(1) - a2));
   } else {
     eb = evr / (P.R * P.theta);
     p_nb = T(1) / (T(1) + eb * (T(1) - a2));
@@ -619,7 +652,15 @@ __global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
       for (long long j = b + 32 + lane; j < e; j += 32) {
         a0 += cx[j]; a1 += cy[j]; a2 += cz[j]; ae += er[j]; al += lev[j];
       }
-      const T t0 = wsum(a0), t1 = wsum(a1), t2 = wsum(a2), te = wsum(ae);
+      T t0, t1, t2, te;
+      if constexpr (sizeof(T) <= 8) {
+        T tot[4] = {a0, a1, a2, ae};
+        halve_totals<4>(tot);   // totals 0, 1, 2, 3 end on lanes 0, 8, 16, 24
+        t0 = __shfl_sync(0xffffffffu, tot[0], 0); t1 = __shfl_sync(0xffffffffu, tot[0], 8);
+        t2 = __shfl_sync(0xffffffffu, tot[0], 16); te = __shfl_sync(0xffffffffu, tot[0], 24);
+      } else {
+        t0 = wsum(a0); t1 = wsum(a1); t2 = wsum(a2); te = wsum(ae);
+      }
       const long long sl = wsum(al);
       // the reference mean of the second pass (an FP32 state keeps FP32)
       T m0, m1, m2;
@@ -642,7 +683,14 @@ __global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
         p[3] += C0 * C1; p[4] += C0 * C2; p[5] += C1 * C2;
       }
       T q[6];
-      for (int i = 0; i < 6; ++i) q[i] = wsum(p[i]);
+      if constexpr (sizeof(T) <= 8) {
+        halve_totals<6>(p);     // totals 0 .. 5 end on lanes 0, 4, 8, 16, 20, 24
+        constexpr int at[6] = {0, 4, 8, 16, 20, 24};
+#pragma unroll
+        for (int i = 0; i < 6; ++i) q[i] = __shfl_sync(0xffffffffu, p[0], at[i]);
+      } else {
+        for (int i = 0; i < 6; ++i) q[i] = wsum(p[i]);
+      }
       if (lane == g) {
         k0 = t0; k1 = t1; k2 = t2; ke = te; kl = sl; kb = b; kN = N;
         for (int i = 0; i < 6; ++i) kq[i] = q[i];
@@ -936,7 +984,7 @@ __device__ __forceinline__ int fpm_particle(const T* U, T a, const T* Lp, T a_ro
   v0 = U[0] + a * d0 + Lp[0] * g0;
   v1 = U[1] + a * d1 + (Lp[1] * g0 + Lp[2] * g1);
   v2 = U[2] + a * d2 + (Lp[3] * g0 + Lp[4] * g1 + Lp[5] * g2);
-  const T root = sqrt(en) * a + sqrt_a * g3;
+  const T root = root_sel<sizeof(T) == 8>(en) * a + sqrt_a * g3;
   en = a_rot + root * root;
   return gillespie<T>(l0, lam_up, lam_dn, id, step, rk, fl);
 }

@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+#include "usp_device.cuh"
+
 namespace usp {
 
 // S_k = sum d_k | Q = sum d_i d_j (xx yy zz xy xz yz) | T_k = sum |d|^2 d_k |
@@ -32,44 +34,6 @@ __device__ __forceinline__ void raw_add(double* a, long long& aI, double d0, dou
     a[kRL + 2] = fma(d2, li, a[kRL + 2]);
     aI += l;
   }
-}
-
-// Warp totals of the 20 sums by recursive halving: the lanes split the sums
-// between them in every round, 21 additions per lane instead of the 100 of
-// twenty butterfly sums (the FP64 pipe issues one warp instruction per 16
-// cycles, and a warp here holds few particles).  Returns the total of sum
-// `index` (-1: this lane holds none).
-__device__ __forceinline__ double raw_warp_total(const double* a, int& index) {
-  const int lane = threadIdx.x & 31;
-  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2, b0 = lane & 1;
-  double r1[10], r2[5], r3[3], r4[2];
-#pragma unroll
-  for (int i = 0; i < 10; ++i) {
-    const double send = b4 ? a[i] : a[i + 10], keep = b4 ? a[i + 10] : a[i];
-    r1[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const double send = b3 ? r1[i] : r1[i + 5], keep = b3 ? r1[i + 5] : r1[i];
-    r2[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const double hi = i + 3 < 5 ? r2[i + 3] : 0.0;
-    const double send = b2 ? r2[i] : hi, keep = b2 ? hi : r2[i];
-    r3[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const double hi = i + 2 < 3 ? r3[i + 2] : 0.0;
-    const double send = b1 ? r3[i] : hi, keep = b1 ? hi : r3[i];
-    r4[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-  }
-  const double send = b0 ? r4[0] : r4[1], keep = b0 ? r4[1] : r4[0];
-  const int g = (b1 ? 2 : 0) + (b0 ? 1 : 0);          // place among 3 (b2 = 0) or 2
-  const bool ok = b2 ? g < 2 : g < 3;
-  index = ok ? (b4 ? 10 : 0) + (b3 ? 5 : 0) + (b2 ? 3 : 0) + g : -1;
-  return keep + __shfl_xor_sync(0xffffffffu, send, 1);
 }
 
 // The reference velocity of a cell of n particles: the FP32 mean of 32 of them
@@ -168,7 +132,11 @@ __device__ __forceinline__ void raw_cell(long long b, long long n, int chunk_min
     for (long long k = b + k0 + lane; k < b + k1; k += 32)
       raw_add(a, aI, cx[k] - w.w[0], cy[k] - w.w[1], cz[k] - w.w[2], er[k], lev[k]);
     a[kRI] = (double)aI;
-    mine = raw_warp_total(a, index);
+    // 21 additions per lane instead of the 100 of twenty butterfly sums: the
+    // FP64 pipe issues one warp instruction per 16 cycles, and a warp here
+    // holds few particles
+    index = halve_totals<kRawN>(a);
+    mine = a[0];
   }
   __syncthreads();                                            // the previous cell's readers
   if (lane < kRawN) red[wid][lane] = 0.0;
