@@ -19,36 +19,53 @@
 
 #include <cmath>
 
+#include "usp_device.cuh"
+
 namespace usp {
 namespace dual {
 
 constexpr int kND = 3;
 
-// elementary functions of the value type
-__host__ __device__ inline float vsqrt(float x) { return sqrtf(x); }
-__host__ __device__ inline double vsqrt(double x) { return ::sqrt(x); }
-__host__ __device__ inline float vlog(float x) { return logf(x); }
-__host__ __device__ inline double vlog(double x) { return ::log(x); }
-__host__ __device__ inline float vlog1p(float x) { return log1pf(x); }
-__host__ __device__ inline double vlog1p(double x) { return ::log1p(x); }
-__host__ __device__ inline float vexp(float x) { return expf(x); }
-__host__ __device__ inline double vexp(double x) { return ::exp(x); }
-__host__ __device__ inline float vexpm1(float x) { return expm1f(x); }
-__host__ __device__ inline double vexpm1(double x) { return ::expm1(x); }
-__host__ __device__ inline float vsinh(float x) { return sinhf(x); }
-__host__ __device__ inline double vsinh(double x) { return ::sinh(x); }
-__host__ __device__ inline float vcosh(float x) { return coshf(x); }
-__host__ __device__ inline double vcosh(double x) { return ::cosh(x); }
-__host__ __device__ inline float vcos(float x) { return cosf(x); }
-__host__ __device__ inline double vcos(double x) { return ::cos(x); }
-__host__ __device__ inline float vsin(float x) { return sinf(x); }
-__host__ __device__ inline double vsin(double x) { return ::sin(x); }
-__host__ __device__ inline float vacos(float x) { return acosf(x); }
-__host__ __device__ inline double vacos(double x) { return ::acos(x); }
-__host__ __device__ inline float vcbrt(float x) { return cbrtf(x); }
-__host__ __device__ inline double vcbrt(double x) { return ::cbrt(x); }
-__host__ __device__ inline float vpow(float x, float y) { return powf(x, y); }
-__host__ __device__ inline double vpow(double x, double y) { return ::pow(x, y); }
+// elementary functions of the value type: FP32 the library's, FP64 those of
+// usp_math.cuh (a derivative number's division took four divisions by the
+// same value, 38 FP64 operations of a particle's lane; now 17)
+__device__ inline float vsqrt(float x) { return sqrtf(x); }
+__device__ inline double vsqrt(double x) { return sqrt_fast(x); }
+__device__ inline float vlog(float x) { return logf(x); }
+__device__ inline double vlog(double x) { return d_log(x); }
+__device__ inline float vlog1p(float x) { return log1pf(x); }
+__device__ inline double vlog1p(double x) { return ::log1p(x); }
+__device__ inline float vexp(float x) { return expf(x); }
+__device__ inline double vexp(double x) { return d_exp(x); }
+// exp(x) - 1 and its derivative
+__device__ inline float vexpm1(float x, float& df) { df = expf(x); return expm1f(x); }
+__device__ inline double vexpm1(double x, double& df) {
+  const double e = d_expm1(x);
+  df = e + 1.0;
+  return e;
+}
+__device__ inline float vsinh(float x) { return sinhf(x); }
+__device__ inline double vsinh(double x) { return ::sinh(x); }
+__device__ inline float vcosh(float x) { return coshf(x); }
+__device__ inline double vcosh(double x) { return ::cosh(x); }
+__device__ inline float vcos(float x) { return cosf(x); }
+__device__ inline double vcos(double x) { return ::cos(x); }
+__device__ inline float vsin(float x) { return sinf(x); }
+__device__ inline double vsin(double x) { return ::sin(x); }
+__device__ inline float vacos(float x) { return acosf(x); }
+__device__ inline double vacos(double x) { return ::acos(x); }
+__device__ inline float vcbrt(float x) { return cbrtf(x); }
+__device__ inline double vcbrt(double x) { return d_cbrt(x); }
+__device__ inline float vpow(float x, float y) { return powf(x, y); }
+__device__ inline double vpow(double x, double y) { return ::pow(x, y); }
+// a / b, and the quotients d_i / b of the derivatives
+__device__ inline float vdiv(float a, float b) { return a / b; }
+__device__ inline double vdiv(double a, double b) { return d_div(a, b); }
+__device__ inline void vdiv3(float* d, float b) { for (int i = 0; i < kND; ++i) d[i] = d[i] / b; }
+__device__ inline void vdiv3(double* d, double b) {
+  const double y = d_rcp(b);
+  for (int i = 0; i < kND; ++i) d[i] *= y;
+}
 
 template <typename V>
 struct Dual {
@@ -82,9 +99,10 @@ struct Dual {
     v *= b.v;
     return *this;
   }
-  __host__ __device__ Dual& operator/=(const Dual& b) {
-    const V q = v / b.v;
-    for (int i = 0; i < kND; ++i) d[i] = (d[i] - q * b.d[i]) / b.v;
+  __device__ Dual& operator/=(const Dual& b) {
+    const V q = vdiv(v, b.v);
+    for (int i = 0; i < kND; ++i) d[i] = d[i] - q * b.d[i];
+    vdiv3(d, b.v);
     v = q;
     return *this;
   }
@@ -100,7 +118,7 @@ __host__ __device__ inline Dual<V> operator-(Dual<V> a, const Dual<V>& b) { retu
 template <typename V>
 __host__ __device__ inline Dual<V> operator*(Dual<V> a, const Dual<V>& b) { return a *= b; }
 template <typename V>
-__host__ __device__ inline Dual<V> operator/(Dual<V> a, const Dual<V>& b) { return a /= b; }
+__device__ inline Dual<V> operator/(Dual<V> a, const Dual<V>& b) { return a /= b; }
 template <typename V>
 __host__ __device__ inline Dual<V> operator+(Dual<V> a, double b) { a.v += V(b); return a; }
 template <typename V>
@@ -124,14 +142,14 @@ __host__ __device__ inline Dual<V> operator*(Dual<V> a, double b) {
 template <typename V>
 __host__ __device__ inline Dual<V> operator*(double b, Dual<V> a) { return a * b; }
 template <typename V>
-__host__ __device__ inline Dual<V> operator/(Dual<V> a, double b) {
+__device__ inline Dual<V> operator/(Dual<V> a, double b) {
   const V c = V(b);
-  a.v /= c;
-  for (int i = 0; i < kND; ++i) a.d[i] /= c;
+  a.v = vdiv(a.v, c);
+  vdiv3(a.d, c);
   return a;
 }
 template <typename V>
-__host__ __device__ inline Dual<V> operator/(double b, const Dual<V>& a) { return Dual<V>(b) / a; }
+__device__ inline Dual<V> operator/(double b, const Dual<V>& a) { return Dual<V>(b) / a; }
 template <typename V>
 __host__ __device__ inline Dual<V> operator-(const Dual<V>& a) {
   Dual<V> r;
@@ -169,10 +187,10 @@ __host__ __device__ inline Dual<V> chain(const Dual<V>& a, V fv, V df) {
 template <typename V>
 __device__ inline Dual<V> sqrt(const Dual<V>& a) {
   const V s = vsqrt(a.v);
-  return chain(a, s, s > V(0) ? V(0.5) / s : V(0));
+  return chain(a, s, s > V(0) ? vdiv(V(0.5), s) : V(0));
 }
 template <typename V>
-__device__ inline Dual<V> log(const Dual<V>& a) { return chain(a, vlog(a.v), V(1) / a.v); }
+__device__ inline Dual<V> log(const Dual<V>& a) { return chain(a, vlog(a.v), vdiv(V(1), a.v)); }
 template <typename V>
 __device__ inline Dual<V> log1p(const Dual<V>& a) {
   return chain(a, vlog1p(a.v), V(1) / (V(1) + a.v));
@@ -183,7 +201,11 @@ __device__ inline Dual<V> exp(const Dual<V>& a) {
   return chain(a, e, e);
 }
 template <typename V>
-__device__ inline Dual<V> expm1(const Dual<V>& a) { return chain(a, vexpm1(a.v), vexp(a.v)); }
+__device__ inline Dual<V> expm1(const Dual<V>& a) {
+  V df;
+  const V e = vexpm1(a.v, df);
+  return chain(a, e, df);
+}
 template <typename V>
 __device__ inline Dual<V> sinh(const Dual<V>& a) { return chain(a, vsinh(a.v), vcosh(a.v)); }
 template <typename V>
@@ -196,7 +218,7 @@ __device__ inline Dual<V> acos(const Dual<V>& a) {
 template <typename V>
 __device__ inline Dual<V> cbrt(const Dual<V>& a) {
   const V c = vcbrt(a.v);
-  return chain(a, c, c != V(0) ? c / (V(3) * a.v) : V(0));
+  return chain(a, c, c != V(0) ? vdiv(c, V(3) * a.v) : V(0));
 }
 template <typename V>
 __device__ inline Dual<V> fabs(const Dual<V>& a) { return a.v < V(0) ? -a : a; }
