@@ -7,20 +7,30 @@
 //   ch_advect      pending conservation rescale of the previous step, ballistic
 //                  flight with the body force, diffuse-wall re-emission
 //                  (full accommodation at T_wall, flight continued for the
-//                  rest of the step), new cell key
-//   radix passes   stable LSD radix sort of (cell key, index), 8-bit digits
-//   ch_gather      state permuted into cell order
-//   ch_offsets     cell segment starts from the sorted keys
-//   ch_moments     per-cell moments (Sec. 2.A), one warp per cell
-//   ch_coeffs      per-cell coefficients alpha, nu, gamma, targets (Sec. 3.A)
-//   ch_recon       first-order reconstruction of Sec. 3.B: per cell the field
-//                  values and the slopes used on each side of the centroid
-//   ch_collide     per particle: interpolated fields, relaxation temperatures,
-//                  tau D_tr and its Cholesky factor with the Sec. 3.A.3 fix,
-//                  Eqs. update_ci / update_erot / update_evib; cell sums
-//   ch_levelfix    vibrational +-1 correction of Sec. 4.C (warp per cell)
-//   ch_update      rescale factors of Sec. 4.C, kept pending for the next move
-//   ch_sample      (while sampling) time-average sums of the post-step state
+//                  rest of the step), new cell key; on the placed path also
+//                  the block's count of every cell
+//   ch_place       (few cells and particles) stable counting sort in one pass:
+//                  every block finds its particles' places from the counts
+//                  and moves their state there; cell segment starts
+//   radix passes, ch_gather, ch_offsets  (otherwise) stable LSD radix sort of
+//                  (cell key, index), state permuted into cell order
+//   ch_prepare     per-cell moments (Sec. 2.A) and coefficients alpha, nu,
+//                  gamma, targets (Sec. 3.A), one warp per cell
+//   ch_collide     blocks of one cell: the first-order reconstruction of Sec.
+//                  3.B (field values and the slopes on each side of the
+//                  centroid, in shared memory), then per particle the
+//                  interpolated fields, relaxation temperatures, tau D_tr
+//                  and its Cholesky factor with the Sec. 3.A.3 fix, Eqs.
+//                  update_ci / update_erot / update_evib
+//   ch_finish      one block per cell: cell sums, the vibrational +-1
+//                  correction and the rescale factors of Sec. 4.C (kept
+//                  pending for the next move), while sampling the time
+//                  averages of the post-step state; the last block advances
+//                  the step
+// A channel of some 10,000 particles is all latency: 17 launches of 1 to 30 us
+// took 123 us a step at 64 cells x 200 particles (FP32, sampling on).  The
+// passes above spread each cell's particles over a block and its per-cell
+// chains over all SMs.
 #include <cuda_runtime.h>
 
 #include <type_traits>
@@ -94,6 +104,10 @@ __device__ __forceinline__ int sample_b<D3>(int n, D3 p, D3 u, uint32_t& fl) {
 namespace {
 
 
+// limits of the one-pass sort
+constexpr int kPlaceCells = 256, kPlaceBlocks = 128;
+constexpr int kAB = 128;   // threads per block of the move
+
 template <typename T>
 struct ChParams {
   T alpha, nu_ref, B, mu_p, Pr, gtr, gtv, grv;
@@ -127,15 +141,17 @@ __device__ void wall_emit(const Species& sp, uint32_t pid, uint32_t step, int hi
   const double u2 = (double)value(uniform_open<T>(w.z));
   const double u3 = (double)value(uniform_open<T>(w.w));
   const double u4 = (double)value(uniform_open<T>(v.x));
-  const S vn = sqrt(-2.0 * R * Tw * log(u0));
+  const S vn = sqrt(-2.0 * R * Tw * d_log(u0));
   vy = into_pos ? vn : -vn;
-  double g1, g2;
-  box_muller(u1, u2, g1, g2);
+  double sn, cn;
+  const double rad = sqrt_fast(-2.0 * d_log(u1));
+  sincospi(2.0 * u2, &sn, &cn);
+  const double g1 = rad * cn, g2 = rad * sn;
   const S s = sqrt(R * Tw);
   vx = s * g1;
   vz = s * g2;
-  e = -R * Tw * log(u3);
-  l = (int)floor(-log(u4) * value(Tw) / sp.theta_v);
+  e = -R * Tw * d_log(u3);
+  l = (int)floor(-d_log(u4) * value(Tw) / sp.theta_v);
 }
 
 template <typename T, typename S>
@@ -146,9 +162,15 @@ __global__ void ch_advect(long long n, int ny, double L, double dy, S Tw, double
                           const uint32_t* __restrict__ pid, int* __restrict__ keyout,
                           int* __restrict__ idxout, const long long* __restrict__ dstep, Species sp,
                           uint32_t k0, uint32_t k1, double* wallmom, uint32_t* flags,
-                          unsigned long long* counters) {
+                          unsigned long long* counters, int* __restrict__ counts) {
+  // placed path: the block's count of every cell (counts: ny per block)
+  __shared__ int hist[kPlaceCells];
   const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
+  if (counts) {
+    for (int d = threadIdx.x; d < ny; d += blockDim.x) hist[d] = 0;
+    __syncthreads();
+  }
+  if (j < n) {
   const uint32_t step = (uint32_t)*dstep;
   const ChCellT<S>& cc = cells[keycell[j]];
   // pending conservation rescale of the previous step
@@ -200,7 +222,74 @@ __global__ void ch_advect(long long n, int ny, double L, double dy, S Tw, double
   int k = cell_index(yy, dy);
   k = k < 0 ? 0 : (k >= ny ? ny - 1 : k);
   keyout[j] = k;
-  idxout[j] = (int)j;
+  if (counts) atomicAdd(&hist[k], 1);
+  else idxout[j] = (int)j;
+  }
+  if (counts) {
+    __syncthreads();
+    for (int d = threadIdx.x; d < ny; d += blockDim.x)
+      counts[(size_t)blockIdx.x * ny + d] = hist[d];
+  }
+}
+
+// ---------------------------------------------------------------------------
+// stable counting sort by cell in one pass (at most kPlaceCells cells and
+// kPlaceBlocks blocks of 256 particles): a particle's place is its cell's
+// start, plus the cell's particles in earlier blocks, plus those before it in
+// its block.  Each block sums the columns of the counts itself (at most
+// kPlaceBlocks values per cell, read coalesced from L2).
+// ---------------------------------------------------------------------------
+template <typename T>
+__global__ void __launch_bounds__(256)
+ch_place(int n, int ny, const int* __restrict__ counts, const int* __restrict__ key,
+         const T* __restrict__ y0, const T* __restrict__ x0, const T* __restrict__ vy0,
+         const T* __restrict__ z0, const T* __restrict__ e0, const int* __restrict__ l0,
+         const uint32_t* __restrict__ p0, T* __restrict__ y1, T* __restrict__ x1,
+         T* __restrict__ vy1, T* __restrict__ z1, T* __restrict__ e1, int* __restrict__ l1,
+         uint32_t* __restrict__ p1, int* __restrict__ keycell, long long* __restrict__ off) {
+  __shared__ int base[kPlaceCells];
+  __shared__ int cnt[8][kPlaceCells];
+  __shared__ int wtot[8];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int j = blockIdx.x * 256 + t;
+  const int k = j < n ? key[j] : -1;
+  int before = 0, total = 0;
+  if (t < ny) {
+    const int nb = (n + kAB - 1) / kAB, me = blockIdx.x * (256 / kAB);
+#pragma unroll 8
+    for (int b = 0; b < nb; ++b) {
+      const int v = counts[(size_t)b * ny + t];
+      total += v;
+      before += b < me ? v : 0;
+    }
+  }
+  for (int q = 0; q < 8; ++q) cnt[q][t] = 0;
+  // exclusive scan of the totals over the cells
+  int v = total;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += u;
+  }
+  if (lane == 31) wtot[w] = v;
+  __syncthreads();
+  int start = v - total;
+  for (int q = 0; q < w; ++q) start += wtot[q];
+  if (t < ny) base[t] = start + before;
+  if (blockIdx.x == 0 && t < ny) {
+    off[t] = start;
+    if (t == ny - 1) off[ny] = start + total;
+  }
+  const unsigned peers = __match_any_sync(0xffffffffu, k);
+  const int rank = __popc(peers & lane_lt());
+  if (k >= 0 && rank == 0) cnt[w][k] = __popc(peers);
+  __syncthreads();
+  if (k < 0) return;
+  int at = base[k] + rank;
+  for (int q = 0; q < w; ++q) at += cnt[q][k];
+  y1[at] = y0[j]; x1[at] = x0[j]; vy1[at] = vy0[j]; z1[at] = z0[j]; e1[at] = e0[j];
+  l1[at] = l0[j]; p1[at] = p0[j];
+  keycell[at] = k;
 }
 
 // ---------------------------------------------------------------------------
@@ -309,106 +398,98 @@ __global__ void ch_offsets(long long n, int ny, const int* __restrict__ key,
 }
 
 // ---------------------------------------------------------------------------
-// per-cell moments, coefficients, reconstruction
+// per-particle collision, several blocks of kCB threads per cell
 // ---------------------------------------------------------------------------
+constexpr int kCB = 128;
+
 // Sec. 3.B in one dimension: the line through the cell average at the
 // centroid and the neighbour's average at its centroid, the neighbour on the
 // particle's side, or on the other side when that one is a wall or holds
-// fewer than two particles.
+// fewer than two particles.  The block's threads form the record of cell c in
+// shared memory, a field each.
 template <typename T, typename S>
-__global__ void ch_recon(int ny, double dy, int recon, double dt,
-                         const ChCellT<S>* __restrict__ cells, ChParams<T>* __restrict__ prm,
-                         Species sp) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ny) return;
+__device__ void ch_recon(int c, int ny, double dy, int recon, double dt,
+                         const ChCellT<S>* __restrict__ cells, ChParams<T>& P, const Species& sp) {
   const ChCellT<S>& cs = cells[c];
-  ChParams<T> P;
-  P.active = cs.active;
-  P.pad = 0;
-  P.alpha = (T)cs.alpha; P.nu_ref = (T)cs.nu_ref; P.B = (T)cs.B; P.mu_p = (T)cs.mu_p;
-  P.Pr = (T)cs.Pr; P.gtr = (T)cs.gtr; P.gtv = (T)cs.gtv; P.grv = (T)cs.grv;
-  P.R = (T)gasR(sp); P.theta = (T)sp.theta_v; P.dt = (T)dt;
-  P.yc = (T)((c + 0.5) * dy);
-  S f[kNF];
-  cell_fields(cs, f);
+  const int t = threadIdx.x;
   auto valid = [&](int k) { return k >= 0 && k < ny && cells[k].active; };
   const int up = valid(c + 1) ? c + 1 : (valid(c - 1) ? c - 1 : -1);
   const int dn = valid(c - 1) ? c - 1 : (valid(c + 1) ? c + 1 : -1);
-  S fu[kNF], fd[kNF];
-  if (up >= 0) cell_fields(cells[up], fu);
-  if (dn >= 0) cell_fields(cells[dn], fd);
-  for (int i = 0; i < kNF; ++i) {
-    P.F[i] = (T)f[i];
-    P.Sp[i] = (recon && up >= 0) ? (T)((fu[i] - f[i]) / ((up - c) * dy)) : T(0);
-    P.Sm[i] = (recon && dn >= 0) ? (T)((fd[i] - f[i]) / ((dn - c) * dy)) : T(0);
+  auto field = [&](int k, int i) -> S {
+    const ChCellT<S>& q = cells[k];
+    return i < 3 ? q.U[i] : i == 3 ? q.Ttr : i == 4 ? q.Trot : i == 5 ? S(q.Tvib) : q.Pi[i - 6];
+  };
+  if (t < 12) {
+    const S f = field(c, t);
+    P.F[t] = (T)f;
+    P.Sp[t] = (recon && up >= 0) ? (T)((field(up, t) - f) / ((up - c) * dy)) : T(0);
+    P.Sm[t] = (recon && dn >= 0) ? (T)((field(dn, t) - f) / ((dn - c) * dy)) : T(0);
+  } else if (t == 32) {
+    P.F[12] = P.Sp[12] = P.Sm[12] = T(0);   // padding field of the records
+    P.alpha = (T)cs.alpha; P.nu_ref = (T)cs.nu_ref; P.B = (T)cs.B; P.mu_p = (T)cs.mu_p;
+    P.Pr = (T)cs.Pr; P.gtr = (T)cs.gtr; P.gtv = (T)cs.gtv; P.grv = (T)cs.grv;
+    P.R = (T)gasR(sp); P.theta = (T)sp.theta_v; P.dt = (T)dt;
+    P.yc = (T)((c + 0.5) * dy);
   }
-  prm[c] = P;
 }
 
-// ---------------------------------------------------------------------------
-// per-particle collision with interpolated fields (working precision T)
-// ---------------------------------------------------------------------------
-template <typename T, typename S>
-__global__ void ch_collide(int ny, const ChCellT<S>* __restrict__ cells,
-                           const ChParams<T>* __restrict__ prm,
-                           const T* __restrict__ y, T* __restrict__ cx, T* __restrict__ cy,
-                           T* __restrict__ cz, T* __restrict__ er, int* __restrict__ lev,
-                           const uint32_t* __restrict__ pid, ChSumsT<S>* __restrict__ sums,
-                           const long long* __restrict__ dstep, const PhiloxRoundKeys rk,
-                           uint32_t* flags, unsigned long long* counters) {
-  const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (c >= ny) return;
+// METHOD 1: the plain FPM method (Sec. 2.C) with the cell values and the
+// per-cell constants rec
+template <typename T, typename S, int METHOD>
+__global__ void __launch_bounds__(kCB)
+ch_collide(int c0, int ny, double dy, int recon, double dt, const ChCellT<S>* __restrict__ cells,
+           const double* __restrict__ rec, const T* __restrict__ y, T* __restrict__ cx,
+           T* __restrict__ cy, T* __restrict__ cz, T* __restrict__ er, int* __restrict__ lev,
+           const uint32_t* __restrict__ pid, const long long* __restrict__ dstep,
+           const PhiloxRoundKeys rk, Species sp, uint32_t* flags, unsigned long long* counters) {
+  __shared__ ChParams<T> P;
+  const int c = c0 + blockIdx.y, lane = threadIdx.x & 31;
   const ChCellT<S>& cs = cells[c];
-  if (!cs.active) return;
-  const ChParams<T>& P = prm[c];
+  const long long off = cs.off, N = cs.N;
+  if (!cs.active || (long long)blockIdx.x * kCB >= N) return;   // uniform over the block
   const uint32_t step = (uint32_t)*dstep;
-  const T Uc0 = (T)cs.U[0], Uc1 = (T)cs.U[1], Uc2 = (T)cs.U[2];
-  T acc[10];
-  for (int i = 0; i < 10; ++i) acc[i] = T(0);
-  double accI = 0.0;
-  int maxI = 0;
   CollideTally tl = {0u, 0ull, 0ull, 0ull, 0ull};
   unsigned long long nfb = 0;
-  for (long long j = cs.off + lane; j < cs.off + cs.N; j += 32) {
-    // interpolated fields at the particle
-    const T dyv = y[j] - P.yc;
-    const bool above = dyv >= T(0);
-    T f[kNF];
+  if constexpr (METHOD == 0) {
+    ch_recon<T, S>(c, ny, dy, recon, dt, cells, P, sp);
+    __syncthreads();
+    for (long long i = (long long)blockIdx.x * kCB + threadIdx.x; i < N;
+         i += (long long)gridDim.x * kCB) {
+      const long long j = off + i;
+      // interpolated fields at the particle
+      const T dyv = y[j] - P.yc;
+      const bool above = dyv >= T(0);
+      T f[kNF];
 #pragma unroll
-    for (int i = 0; i < kNF; ++i) f[i] = P.F[i] + (above ? P.Sp[i] : P.Sm[i]) * dyv;
-    if (!(f[3] > T(0)) || !(f[4] > T(0)) || !(f[5] >= T(0))) {
+      for (int q = 0; q < kNF; ++q) f[q] = P.F[q] + (above ? P.Sp[q] : P.Sm[q]) * dyv;
+      if (!(f[3] > T(0)) || !(f[4] > T(0)) || !(f[5] >= T(0))) {
 #pragma unroll
-      for (int i = 0; i < kNF; ++i) f[i] = P.F[i];
-      ++nfb;
+        for (int q = 0; q < kNF; ++q) f[q] = P.F[q];
+        ++nfb;
+      }
+      T v0 = cx[j], v1 = cy[j], v2 = cz[j], en = er[j];
+      lev[j] = collide_particle_t<std::is_same<T, double>::value>(P, f, v0, v1, v2, en, lev[j],
+                                                                  pid[j], step, rk, tl);
+      cx[j] = v0; cy[j] = v1; cz[j] = v2; er[j] = en;
     }
-    T v0 = cx[j], v1 = cy[j], v2 = cz[j], en = er[j];
-    const int ln = collide_particle_t<std::is_same<T, double>::value>(P, f, v0, v1, v2, en, lev[j],
-                                                                      pid[j], step, rk, tl);
-    cx[j] = v0; cy[j] = v1; cz[j] = v2; er[j] = en;
-    lev[j] = ln;
-    maxI = max(maxI, ln);
-    const T d0 = v0 - Uc0, d1 = v1 - Uc1, d2 = v2 - Uc2;
-    acc[0] += d0; acc[1] += d1; acc[2] += d2;
-    acc[3] += d0 * d0; acc[4] += d1 * d1; acc[5] += d2 * d2;
-    acc[6] += d0 * d1; acc[7] += d0 * d2; acc[8] += d1 * d2;
-    acc[9] += en;
-    accI += (double)ln;
+  } else {
+    const double* r = rec + (size_t)c * kFpmRec;
+    const T U[3] = {(T)cs.U[0], (T)cs.U[1], (T)cs.U[2]};
+    const T Lp[6] = {(T)r[1], (T)r[2], (T)r[3], (T)r[4], (T)r[5], (T)r[6]};
+    const T a = (T)r[0], a_rot = (T)r[7], sqrt_a = (T)r[8], lu = (T)r[9], ld = (T)r[10];
+    for (long long i = (long long)blockIdx.x * kCB + threadIdx.x; i < N;
+         i += (long long)gridDim.x * kCB) {
+      const long long j = off + i;
+      T v0 = cx[j], v1 = cy[j], v2 = cz[j], en = er[j];
+      lev[j] = fpm_particle<T>(U, a, Lp, a_rot, sqrt_a, lu, ld, v0, v1, v2, en, lev[j], pid[j],
+                               step, rk, tl.fl);
+      cx[j] = v0; cy[j] = v1; cz[j] = v2; er[j] = en;
+    }
   }
-  S s[10];
-#pragma unroll
-  for (int i = 0; i < 10; ++i) s[i] = S(wsum(acc[i]));
-  const double sI = wsum(accI);
   const unsigned long long fix = wsum(tl.nfix), fb = wsum(nfb), ncl2 = wsum(tl.ncl),
                            pb = wsum(tl.npb), nz = wsum(tl.nnz);
-  const int mI = __reduce_max_sync(0xffffffffu, maxI);
   const uint32_t fla = __reduce_or_sync(0xffffffffu, tl.fl);
   if (lane != 0) return;
-  ChSumsT<S>& sm = sums[c];
-  for (int i = 0; i < 10; ++i) sm.v[i] = s[i];
-  sm.I = (unsigned long long)(long long)llrint(sI);
-  sm.net = 0;
-  sm.maxI = mI;
   if (fla) atomicOr(flags, fla);
   if (fix) atomicAdd(&counters[C_CHOL_FIX], fix);
   if (fb) atomicAdd(&counters[C_INTERP_FALLBACK], fb);
@@ -417,99 +498,231 @@ __global__ void ch_collide(int ny, const ChCellT<S>* __restrict__ cells,
   if (nz) atomicAdd(&counters[C_NU_ZERO], nz);
 }
 
-// the plain FPM method (Sec. 2.C) per particle with the cell values: one warp
-// per cell, per-cell sums for the conservation step as in ch_collide
-template <typename T>
-__global__ void ch_collide_fpm(int ny, const ChCellT<double>* __restrict__ cells,
-                               const double* __restrict__ rec, T* __restrict__ cx,
-                               T* __restrict__ cy, T* __restrict__ cz, T* __restrict__ er,
-                               int* __restrict__ lev, const uint32_t* __restrict__ pid,
-                               ChSumsT<double>* __restrict__ sums,
-                               const long long* __restrict__ dstep, const PhiloxRoundKeys rk,
-                               uint32_t* flags) {
-  const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (c >= ny) return;
-  const ChCellT<double>& cs = cells[c];
-  if (!cs.active) return;
-  const uint32_t step = (uint32_t)*dstep;
-  const double* r = rec + (size_t)c * kFpmRec;
-  const T U[3] = {(T)cs.U[0], (T)cs.U[1], (T)cs.U[2]};
-  const T Lp[6] = {(T)r[1], (T)r[2], (T)r[3], (T)r[4], (T)r[5], (T)r[6]};
-  const T a = (T)r[0], a_rot = (T)r[7], sqrt_a = (T)r[8], lu = (T)r[9], ld = (T)r[10];
-  T acc[10];
-  for (int i = 0; i < 10; ++i) acc[i] = T(0);
-  double accI = 0.0;
-  int maxI = 0;
-  uint32_t fl = 0;
-  for (long long j = cs.off + lane; j < cs.off + cs.N; j += 32) {
-    T v0 = cx[j], v1 = cy[j], v2 = cz[j], en = er[j];
-    const int ln = fpm_particle<T>(U, a, Lp, a_rot, sqrt_a, lu, ld, v0, v1, v2, en, lev[j],
-                                   pid[j], step, rk, fl);
-    cx[j] = v0; cy[j] = v1; cz[j] = v2; er[j] = en;
-    lev[j] = ln;
-    maxI = max(maxI, ln);
-    const T d0 = v0 - U[0], d1 = v1 - U[1], d2 = v2 - U[2];
-    acc[0] += d0; acc[1] += d1; acc[2] += d2;
-    acc[3] += d0 * d0; acc[4] += d1 * d1; acc[5] += d2 * d2;
-    acc[6] += d0 * d1; acc[7] += d0 * d2; acc[8] += d1 * d2;
-    acc[9] += en;
-    accI += (double)ln;
+// ---------------------------------------------------------------------------
+// conservation of Sec. 4.C, time averages, end of the step
+// ---------------------------------------------------------------------------
+constexpr int kFB = 256;         // threads per cell
+constexpr int kFW = kFB / 32;
+
+// Totals over the block of the ten sums a[] of every thread (FP64 kinds) into
+// tot[0..9] in shared memory: the warps by halving, their totals by ten lanes
+// of warp 0 (ten lanes of each of four warps for derivative numbers).
+__device__ __forceinline__ void block_ten(double* a, double (*red)[kFW][10], double* tot) {
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int at = halve_totals<10>(a);
+  if (at >= 0) red[0][wid][at] = a[0];
+  __syncthreads();
+  if (wid == 0 && lane < 10) {
+    double v = red[0][0][lane];
+    for (int w = 1; w < kFW; ++w) v += red[0][w][lane];
+    tot[lane] = v;
   }
-  double s[10];
+  __syncthreads();
+}
+template <typename V>
+__device__ __forceinline__ void block_ten(dual::Dual<V>* a, double (*red)[kFW][10],
+                                          dual::Dual<V>* tot) {
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int i = 0; i < 10; ++i) s[i] = (double)wsum(acc[i]);
-  const double sI = wsum(accI);
-  const int mI = __reduce_max_sync(0xffffffffu, maxI);
-  const uint32_t fla = __reduce_or_sync(0xffffffffu, fl);
-  if (lane != 0) return;
-  ChSumsT<double>& sm = sums[c];
-  for (int i = 0; i < 10; ++i) sm.v[i] = s[i];
-  sm.I = (unsigned long long)(long long)llrint(sI);
-  sm.net = 0;
-  sm.maxI = mI;
-  if (fla) atomicOr(flags, fla);
+  for (int k = 0; k <= kND; ++k) {
+    double b[10];
+#pragma unroll
+    for (int i = 0; i < 10; ++i) b[i] = k == 0 ? a[i].v : a[i].d[k == 0 ? 0 : k - 1];
+    const int at = halve_totals<10>(b);
+    if (at >= 0) red[k][wid][at] = b[0];
+  }
+  __syncthreads();
+  if (wid <= kND && lane < 10) {
+    double v = red[wid][0][lane];
+    for (int w = 1; w < kFW; ++w) v += red[wid][w][lane];
+    if (wid == 0) tot[lane].v = v;
+    else tot[lane].d[wid - 1] = v;
+  }
+  __syncthreads();
 }
 
-// time-average sums of the post-step state, one warp per cell (the state is
-// in cell order), each sum reduced across the warp in a fixed order and added
-// by one lane, so that runs are reproducible bit for bit (gradient form:
-// block 0 holds the sums, blocks 1..3 their derivatives)
+// The sums of an FP32 state keep the order and precision of one warp walking
+// the cell with its lanes 32 apart: the block stages the particles, warp 0 adds
+// them up.  FP64 states are summed by all threads.
+template <typename T>
+constexpr bool kOneWarpSums = std::is_same<T, float>::value || std::is_same<T, F3>::value;
+
 template <typename T, typename S>
-__global__ void ch_sample(int ny, const long long* __restrict__ off,
-                          const ChCellT<S>* __restrict__ cells, const T* __restrict__ cx,
-                          const T* __restrict__ cy, const T* __restrict__ cz,
-                          const T* __restrict__ er, const int* __restrict__ lev,
-                          double* __restrict__ acc, const double* __restrict__ wallmom) {
-  const int lane = threadIdx.x & 31;
-  const size_t blk = (size_t)ny * kNAcc + 2;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    acc[(size_t)ny * kNAcc] += 1.0;
-    acc[(size_t)ny * kNAcc + 1] += *wallmom;
+__global__ void __launch_bounds__(kFB)
+ch_finish(int ny, ChCellT<S>* __restrict__ cells, const T* __restrict__ cx,
+          const T* __restrict__ cy, const T* __restrict__ cz, const T* __restrict__ er,
+          int* __restrict__ lev, long long* dstep, Species sp, uint32_t k0, uint32_t k1,
+          uint32_t* flags, unsigned long long* counters, int sampling, double* __restrict__ acc,
+          double* wallmom) {
+  constexpr bool one = kOneWarpSums<T>;
+  __shared__ T stage[4][one ? kFB : 1];
+  __shared__ double red[std::is_same<S, double>::value ? 1 : 1 + kND][kFW][10];
+  __shared__ S ten[10];
+  __shared__ S pend[8];            // Un, Us, s, r
+  __shared__ S e_rot_new, etr_star, e_sum;
+  __shared__ long long levsum;
+  __shared__ int maxl;
+  const int c = blockIdx.x, t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  ChCellT<S>& cs = cells[c];
+  const uint32_t step = (uint32_t)dstep[0];
+  const long long N = cs.N, off = cs.off;
+  const bool active = cs.active;
+  if (t == 0) {
+    levsum = 0;
+    maxl = 0;
+    if (!active) {
+      for (int i = 0; i < 3; ++i) { pend[i] = cs.Un[i]; pend[3 + i] = cs.Us[i]; }
+      pend[6] = cs.s;
+      pend[7] = cs.r;
+    }
   }
-  for (int k = warp_global(); k < ny; k += warps_total()) {
-    const ChCellT<S>& cc = cells[k];
+  __syncthreads();
+  if (active) {                    // uniform over the block
+    const T U0 = (T)cs.U[0], U1 = (T)cs.U[1], U2 = (T)cs.U[2];
+    T a[10];
+#pragma unroll
+    for (int i = 0; i < 10; ++i) a[i] = T(0);
+    auto add = [&](const T& d0, const T& d1, const T& d2, const T& e) {
+      a[0] += d0; a[1] += d1; a[2] += d2;
+      a[3] += d0 * d0; a[4] += d1 * d1; a[5] += d2 * d2;
+      a[6] += d0 * d1; a[7] += d0 * d2; a[8] += d1 * d2;
+      a[9] += e;
+    };
+    long long sl = 0;
+    int ml = 0;
+    for (long long q = 0; q < N; q += kFB) {
+      const long long j = off + q + t;
+      const bool in = q + t < N;
+      if (in) {
+        const int l = lev[j];
+        sl += l;
+        ml = max(ml, l);
+      }
+      if constexpr (one) {
+        __syncthreads();
+        if (in) { stage[0][t] = cx[j]; stage[1][t] = cy[j]; stage[2][t] = cz[j]; stage[3][t] = er[j]; }
+        __syncthreads();
+        const int m = (int)(N - q < kFB ? N - q : kFB);
+        if (wid == 0)
+          for (int i = lane; i < m; i += 32)
+            add(stage[0][i] - U0, stage[1][i] - U1, stage[2][i] - U2, stage[3][i]);
+      } else if (in) {
+        add(cx[j] - U0, cy[j] - U1, cz[j] - U2, er[j]);
+      }
+    }
+    sl = wsum(sl);
+    ml = __reduce_max_sync(0xffffffffu, ml);
+    if (lane == 0) {
+      if (sl) atomicAdd((unsigned long long*)&levsum, (unsigned long long)sl);
+      atomicMax(&maxl, ml);
+    }
+    if constexpr (one) {
+      if (wid == 0) {
+#pragma unroll
+        for (int i = 0; i < 10; ++i) {
+          const S v = S(wsum(a[i]));
+          if (lane == 0) ten[i] = v;
+        }
+      }
+      __syncthreads();
+    } else {
+      block_ten(a, red, ten);
+    }
+    // the vibrational +-1 correction | what of the rescale does not need it
+    const double R = gasR(sp), Rth = R * sp.theta_v;
+    if (wid == 0) {
+      long long remaining = 0, draws = 0, net = 0;
+      if (lane == 0) {
+        const U4 w = philox4x32_10((uint32_t)c, step, CTAG_IDELTA, 0u, k0, k1);
+        const double u = uniform_open<double>(w.x);
+        remaining = (long long)floor((double)N * value(cs.e_vib_tgt) / Rth - (double)levsum + u);
+      }
+      remaining = __shfl_sync(0xffffffffu, remaining, 0);
+      level_correction(c, step, N, lev + off, remaining, draws, net, k0, k1);
+      if (lane == 0) {
+        if (remaining != 0) atomicOr(flags, (uint32_t)F_VIB_LOOP_CAP);
+        if (draws) atomicAdd(&counters[C_VIB_DRAWS], (unsigned long long)draws);
+        levsum += net;
+      }
+    } else if (t == 32) {
+      const double invN = d_rcp((double)N);
+      const S er_star = ten[9] * invN;
+      pend[7] = er_star > 0.0 ? c_div(cs.e_rot_tgt, er_star) : S(1.0);
+      e_rot_new = pend[7] * er_star;
+    } else if (t == 64) {
+      const double invN = d_rcp((double)N);
+      const S m0 = ten[0] * invN, m1 = ten[1] * invN, m2 = ten[2] * invN;
+      etr_star = 0.5 * (ten[3] * invN - m0 * m0 + ten[4] * invN - m1 * m1 + ten[5] * invN - m2 * m2);
+      pend[3] = cs.U[0] + m0; pend[4] = cs.U[1] + m1; pend[5] = cs.U[2] + m2;
+    } else if (t == 96) {
+      e_sum = 0.5 * (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]) + R * cs.Trot + Rth * cs.ebar;
+    }
+    __syncthreads();
+    if (t == 0) {
+      const double e_vib_new = Rth * (double)levsum * d_rcp((double)N);
+      const S rad = c_div(e_sum - e_rot_new - e_vib_new, etr_star);
+      const bool neg = !(etr_star > 0.0) || !(rad > 0.0);
+      if (neg) {
+        atomicOr(flags, (uint32_t)F_NEG_RADICAND);
+        atomicAdd(&counters[C_NEG_RADICAND], 1ull);
+      }
+      for (int i = 0; i < 3; ++i) {
+        pend[i] = cs.Un[i] = neg ? pend[3 + i] : cs.U[i];
+        cs.Us[i] = pend[3 + i];
+      }
+      pend[6] = cs.s = neg ? S(1.0) : sqrt(rad);
+      cs.r = pend[7];
+      cs.maxI = maxl + 1;
+    }
+    __syncthreads();
+  }
+  if (sampling) {
+    // time-average sums of the post-step state, reduced in a fixed order, so
+    // that runs are reproducible bit for bit (gradient form: block 0 of acc
+    // holds the sums, blocks 1..3 their derivatives)
     S q[10];
+#pragma unroll
     for (int i = 0; i < 10; ++i) q[i] = S(0.0);
     long long sl = 0;
-    const long long b = off[k], e = off[k + 1];
-    for (long long j = b + lane; j < e; j += 32) {
-      const S v0 = cc.Un[0] + cc.s * (S(cx[j]) - cc.Us[0]);
-      const S v1 = cc.Un[1] + cc.s * (S(cy[j]) - cc.Us[1]);
-      const S v2 = cc.Un[2] + cc.s * (S(cz[j]) - cc.Us[2]);
+    for (long long i = t; i < N; i += kFB) {
+      const long long j = off + i;
+      const S v0 = pend[0] + pend[6] * (S(cx[j]) - pend[3]);
+      const S v1 = pend[1] + pend[6] * (S(cy[j]) - pend[4]);
+      const S v2 = pend[2] + pend[6] * (S(cz[j]) - pend[5]);
       q[0] += v0; q[1] += v1; q[2] += v2;
       q[3] += v0 * v0; q[4] += v1 * v1; q[5] += v2 * v2;
       q[6] += v0 * v1; q[7] += v0 * v2; q[8] += v1 * v2;
-      q[9] += cc.r * S(er[j]);
-      sl += lev[j];
+      q[9] += pend[7] * S(er[j]);
+      if (!active) sl += lev[j];
     }
-    for (int i = 0; i < 10; ++i) q[i] = wsum(q[i]);
-    for (int o = 16; o > 0; o >>= 1) sl += __shfl_xor_sync(0xffffffffu, sl, o);
-    if (lane == 0) {
-      double* a = acc + (size_t)k * kNAcc;
-      a[0] += (double)(e - b);
-      for (int i = 0; i < 10; ++i) acc_add(&a[1 + i], blk, q[i]);
-      a[11] += (double)sl;
+    block_ten(q, red, ten);
+    if (!active) {
+      sl = wsum(sl);
+      if (lane == 0 && sl) atomicAdd((unsigned long long*)&levsum, (unsigned long long)sl);
+      __syncthreads();
+    }
+    double* a = acc + (size_t)c * kNAcc;
+    if (t < 10) {
+      acc_add(&a[1 + t], (size_t)ny * kNAcc + 2, ten[t]);
+    } else if (t == 32) {
+      a[0] += (double)N;
+      a[11] += (double)levsum;
+      if (c == 0) {
+        acc[(size_t)ny * kNAcc] += 1.0;
+        acc[(size_t)ny * kNAcc + 1] += *wallmom;
+      }
+    }
+    __syncthreads();   // the read of wallmom comes before the block's count below
+  }
+  // the last block to finish advances the step and clears the walls' momentum,
+  // after every block has read them
+  if (t == 0) {
+    __threadfence();
+    if (atomicAdd(reinterpret_cast<unsigned long long*>(dstep + 1), 1ull) ==
+        (unsigned long long)gridDim.x - 1) {
+      dstep[1] = 0;
+      dstep[0] += 1;
+      *wallmom = 0.0;
     }
   }
 }
@@ -648,6 +861,7 @@ __global__ void ch_from_host_layout(long long n, const double* __restrict__ in, 
 // ===========================================================================
 struct ChannelCtx {
   int ny, recon, passes, nblk;
+  bool placed;              // the one-pass sort (else radix passes)
   double L, dy, Tw, g, Fnum, area, dt;
   long long n;
   size_t es;
@@ -661,8 +875,6 @@ struct ChannelCtx {
   int* bh;
   long long* off;
   void* cells;              // ChCellT<S>
-  void* prm;                // ChParams<T>
-  void* sums;               // ChSumsT<S>
   int blocks;               // accumulator blocks: 1, or 4 in the gradient form
   double* acc;
   double* wallmom;
@@ -697,7 +909,6 @@ template <typename T, typename S>
 int ch_step_t(ChannelCtx* h, const ChEnv& env, ch_prof_fn prof) {
   cudaStream_t s = env.stream;
   ChCellT<S>* cells = (ChCellT<S>*)h->cells;
-  ChSumsT<S>* sums = (ChSumsT<S>*)h->sums;
   const S Tw = param<S>(h->Tw, 2);
   const S omega = param<S>(env.sp.omega, 1);
   const S zrot = param<S>(env.sp.Z_rot, 0);
@@ -706,76 +917,84 @@ int ch_step_t(ChannelCtx* h, const ChEnv& env, ch_prof_fn prof) {
   const int a = h->cur, b = a ^ 1;
   T* y = (T*)h->st[a][0]; T* cx = (T*)h->st[a][1]; T* cy = (T*)h->st[a][2];
   T* cz = (T*)h->st[a][3]; T* er = (T*)h->st[a][4];
+  T* y1 = (T*)h->st[b][0]; T* cx1 = (T*)h->st[b][1]; T* cy1 = (T*)h->st[b][2];
+  T* cz1 = (T*)h->st[b][3]; T* er1 = (T*)h->st[b][4];
   if (prof) prof(env.owner, 0, 1);
-  CHK(cudaMemsetAsync(h->wallmom, 0, sizeof(double), s));
-  ch_advect<T, S><<<nb, 256, 0, s>>>(n, h->ny, h->L, h->dy, Tw, h->g, h->dt, h->keycell, cells,
+  const int nba = std::max(1, (int)((n + kAB - 1) / kAB));
+  ch_advect<T, S><<<nba, kAB, 0, s>>>(n, h->ny, h->L, h->dy, Tw, h->g, h->dt, h->keycell, cells,
                                    y, cx, cy, cz, er, h->lv[a], h->pd[a], h->kbuf[0], h->ibuf[0],
                                    h->dstep, env.sp, env.k0, env.k1, h->wallmom, env.flags,
-                                   env.counters);
+                                   env.counters, h->placed ? h->bh : nullptr);
   CHK(cudaGetLastError());
-  int src = 0;
-  for (int p = 0; p < h->passes; ++p) {
-    rad_hist<<<h->nblk, kRB, 0, s>>>(h->kbuf[src], n, 8 * p, h->bh);
-    rad_scan<<<1, 256, 0, s>>>(h->bh, h->nblk);
-    rad_scatter<<<h->nblk, kRB, 0, s>>>(h->kbuf[src], h->ibuf[src], h->kbuf[src ^ 1],
-                                        h->ibuf[src ^ 1], n, 8 * p, h->bh);
-    CHK(cudaGetLastError());
-    src ^= 1;
+  if (h->placed) {
+    ch_place<T><<<nb, 256, 0, s>>>((int)n, h->ny, h->bh, h->kbuf[0], y, cx, cy, cz, er, h->lv[a],
+                                   h->pd[a], y1, cx1, cy1, cz1, er1, h->lv[b], h->pd[b],
+                                   h->keycell, h->off);
+  } else {
+    int src = 0;
+    for (int p = 0; p < h->passes; ++p) {
+      rad_hist<<<h->nblk, kRB, 0, s>>>(h->kbuf[src], n, 8 * p, h->bh);
+      rad_scan<<<1, 256, 0, s>>>(h->bh, h->nblk);
+      rad_scatter<<<h->nblk, kRB, 0, s>>>(h->kbuf[src], h->ibuf[src], h->kbuf[src ^ 1],
+                                          h->ibuf[src ^ 1], n, 8 * p, h->bh);
+      CHK(cudaGetLastError());
+      src ^= 1;
+    }
+    ch_gather<T><<<nb, 256, 0, s>>>(n, h->ibuf[src], y, cx, cy, cz, er, h->lv[a], h->pd[a], y1,
+                                    cx1, cy1, cz1, er1, h->lv[b], h->pd[b]);
+    CHK(cudaMemcpyAsync(h->keycell, h->kbuf[src], sizeof(int) * (n > 0 ? n : 1),
+                        cudaMemcpyDeviceToDevice, s));
+    ch_offsets<<<std::max(nb, (h->ny + 256) / 256), 256, 0, s>>>(n, h->ny, h->keycell, h->off);
   }
-  ch_gather<T><<<nb, 256, 0, s>>>(n, h->ibuf[src], y, cx, cy, cz, er, h->lv[a], h->pd[a],
-                                  (T*)h->st[b][0], (T*)h->st[b][1], (T*)h->st[b][2],
-                                  (T*)h->st[b][3], (T*)h->st[b][4], h->lv[b], h->pd[b]);
-  CHK(cudaMemcpyAsync(h->keycell, h->kbuf[src], sizeof(int) * (n > 0 ? n : 1),
-                      cudaMemcpyDeviceToDevice, s));
-  ch_offsets<<<std::max(nb, (h->ny + 256) / 256), 256, 0, s>>>(n, h->ny, h->keycell, h->off);
   CHK(cudaGetLastError());
   h->cur = b;
-  y = (T*)h->st[b][0]; cx = (T*)h->st[b][1]; cy = (T*)h->st[b][2]; cz = (T*)h->st[b][3];
-  er = (T*)h->st[b][4];
   if (prof) prof(env.owner, 0, 0);
   if (prof) prof(env.owner, 1, 1);
-  const int wb = (h->ny * 32 + 127) / 128;
-  const int cb = (h->ny + 127) / 128;
-  ch_moments<T, S><<<wb, 128, 0, s>>>(h->ny, 1, h->off, nullptr, cx, cy, cz, er, h->lv[b], cells,
-                                      env.sp, env.counters, nullptr, (T*)nullptr, nullptr);
-  if constexpr (std::is_same<S, double>::value) {
-    if (h->fpmrec) {
-      // the plain FPM method: cell values at every particle, no reconstruction
-      ch_coeffs_fpm<<<cb, 128, 0, s>>>(h->ny, h->Fnum, h->area * h->dy, nullptr, h->dt, cells,
-                                       h->fpmrec, env.sp, env.flags, env.counters);
-      CHK(cudaGetLastError());
-      if (prof) prof(env.owner, 1, 0);
-      if (prof) prof(env.owner, 0, 1);
-      ch_collide_fpm<T><<<wb, 128, 0, s>>>(h->ny, cells, h->fpmrec, cx, cy, cz, er, h->lv[b],
-                                           h->pd[b], sums, h->dstep,
-                                           env.rk, env.flags);
+  // one warp per block: the cells' chains spread over all SMs
+  const double vol = h->area * h->dy;
+  if (h->fpmrec) {
+    if constexpr (std::is_same<S, double>::value) {
+      ch_moments<T, S><<<h->ny, 32, 0, s>>>(h->ny, 1, h->off, nullptr, cx1, cy1, cz1, er1,
+                                            h->lv[b], cells, env.sp, env.counters, nullptr,
+                                            (T*)nullptr, nullptr);
+      ch_coeffs_fpm<<<h->ny, 32, 0, s>>>(h->ny, h->Fnum, vol, nullptr, h->dt, cells, h->fpmrec,
+                                         env.sp, env.flags, env.counters);
     }
+  } else {
+    ch_prepare<T, S><<<h->ny, 128, 0, s>>>(h->off, cx1, cy1, cz1, er1, h->lv[b], cells,
+                                          env.sp, h->Fnum, vol, h->dt, omega, zrot, env.flags,
+                                          env.counters);
   }
-  if (!h->fpmrec) {
-  ch_coeffs<S><<<cb, 128, 0, s>>>(h->ny, h->Fnum, h->area * h->dy, nullptr, h->dt, cells, env.sp,
-                                  omega, zrot, env.flags, env.counters);
-  ch_recon<T, S><<<cb, 128, 0, s>>>(h->ny, h->dy, h->recon, h->dt, cells, (ChParams<T>*)h->prm,
-                                    env.sp);
   CHK(cudaGetLastError());
   if (prof) prof(env.owner, 1, 0);
   if (prof) prof(env.owner, 0, 1);
-  ch_collide<T, S><<<wb, 128, 0, s>>>(h->ny, cells, (const ChParams<T>*)h->prm, y, cx, cy, cz,
-                                      er, h->lv[b], h->pd[b], sums, h->dstep,
-                                      env.rk, env.flags, env.counters);
+  // enough blocks per cell for a mean cell's particles, and for every SM
+  const long long mean = (n + h->ny - 1) / h->ny;
+  const dim3 grid((unsigned)std::max<long long>(1, std::min<long long>(1024, (mean + kCB - 1) / kCB)),
+                  (unsigned)h->ny);
+  if (h->fpmrec) {
+    if constexpr (std::is_same<S, double>::value)
+      for (int c0 = 0; c0 < h->ny; c0 += 65535) {
+        const dim3 g(grid.x, (unsigned)std::min(65535, h->ny - c0));
+        ch_collide<T, S, 1><<<g, kCB, 0, s>>>(c0, h->ny, h->dy, h->recon, h->dt, cells, h->fpmrec,
+                                              y1, cx1, cy1, cz1, er1, h->lv[b], h->pd[b],
+                                              h->dstep, env.rk, env.sp, env.flags, env.counters);
+      }
+  } else {
+    for (int c0 = 0; c0 < h->ny; c0 += 65535) {
+      const dim3 g(grid.x, (unsigned)std::min(65535, h->ny - c0));
+      ch_collide<T, S, 0><<<g, kCB, 0, s>>>(c0, h->ny, h->dy, h->recon, h->dt, cells, nullptr, y1,
+                                            cx1, cy1, cz1, er1, h->lv[b], h->pd[b], h->dstep,
+                                            env.rk, env.sp, env.flags, env.counters);
+    }
   }
   CHK(cudaGetLastError());
   if (prof) prof(env.owner, 0, 0);
   if (prof) prof(env.owner, 1, 1);
-  ch_levelfix<S><<<wb, 128, 0, s>>>(h->ny, 1, cells, sums, h->lv[b], h->dstep, env.sp, env.k0,
-                                    env.k1, env.flags, env.counters);
-  ch_update<S><<<cb, 128, 0, s>>>(h->ny, cells, sums, h->dstep, env.sp, env.flags, env.counters,
-                                  nullptr);
+  ch_finish<T, S><<<h->ny, kFB, 0, s>>>(h->ny, cells, cx1, cy1, cz1, er1, h->lv[b], h->dstep,
+                                        env.sp, env.k0, env.k1, env.flags, env.counters,
+                                        h->sampling, h->acc, h->wallmom);
   CHK(cudaGetLastError());
-  if (h->sampling) {
-    ch_sample<T, S><<<wb, 128, 0, s>>>(h->ny, h->off, cells, cx, cy, cz, er, h->lv[b], h->acc,
-                                       h->wallmom);
-    CHK(cudaGetLastError());
-  }
   if (prof) prof(env.owner, 1, 0);
   return USP_OK;
 }
@@ -783,7 +1002,8 @@ int ch_step_t(ChannelCtx* h, const ChEnv& env, ch_prof_fn prof) {
 }  // namespace
 
 int ch_kernels_per_step(const ChannelCtx* h) {
-  return 2 + 3 * h->passes + (h->fpmrec ? 7 : 8) + (h->sampling ? 1 : 0);
+  const int sort = h->placed ? 1 : 3 * h->passes + 2;
+  return 1 + sort + (h->fpmrec ? 2 : 1) + (h->ny + 65534) / 65535 + 1;
 }
 
 int ch_launch_step(ChannelCtx* h, const ChEnv& env, ch_prof_fn prof) {
@@ -812,7 +1032,6 @@ int ch_create(ChannelCtx** out, const ChEnv& env, const usp_channel* chp, double
   h->es = env.precision == USP_FP32 ? 4 : (g32 ? sizeof(F3) : (grad ? sizeof(D3) : 8));
   h->blocks = grad ? 1 + kND : 1;
   const size_t cell_bytes = grad ? sizeof(ChCellT<D3>) : sizeof(ChCellT<double>);
-  const size_t sums_bytes = grad ? sizeof(ChSumsT<D3>) : sizeof(ChSumsT<double>);
   const size_t acc_bytes = sizeof(double) * ((size_t)chp->ny * kNAcc + 2) * h->blocks;
   h->cur = 0;
   h->sampling = 0;
@@ -820,6 +1039,7 @@ int ch_create(ChannelCtx** out, const ChEnv& env, const usp_channel* chp, double
   while ((1 << bits) < h->ny) ++bits;
   h->passes = (bits + 7) / 8;
   h->nblk = (int)std::max<long long>(1, (n + kChunk - 1) / kChunk);
+  h->placed = h->ny <= kPlaceCells && n <= 256ll * kPlaceBlocks;
   const size_t nn = (size_t)std::max<long long>(n, 1);
   auto A = [&](size_t bytes) { return env.alloc(env.owner, bytes); };
   for (int k = 0; k < 2; ++k) {
@@ -830,24 +1050,18 @@ int ch_create(ChannelCtx** out, const ChEnv& env, const usp_channel* chp, double
     h->ibuf[k] = (int*)A(nn * 4);
   }
   h->keycell = (int*)A(nn * 4);
-  h->bh = (int*)A((size_t)h->nblk * 256 * 4);
+  h->bh = (int*)A(h->placed ? (nn + kAB - 1) / kAB * h->ny * 4 : (size_t)h->nblk * 256 * 4);
   h->off = (long long*)A(sizeof(long long) * (h->ny + 1));
   h->cells = A(cell_bytes * h->ny);
-  h->prm = A((env.precision == USP_FP32 ? sizeof(ChParams<float>)
-                                        : (g32 ? sizeof(ChParams<F3>)
-                                               : (grad ? sizeof(ChParams<D3>)
-                                                       : sizeof(ChParams<double>)))) *
-             h->ny);
-  h->sums = A(sums_bytes * h->ny);
   if (env.sp.method == 1) h->fpmrec = (double*)A(sizeof(double) * kFpmRec * (size_t)h->ny);
   h->acc = (double*)A(acc_bytes);
   h->wallmom = (double*)A(sizeof(double));
   h->macc = (double*)A(sizeof(double) * 21 * h->ny);
   h->mout = (double*)A(sizeof(double) * USP_NMOM * h->ny);
-  h->dstep = (long long*)A(sizeof(long long));
+  h->dstep = (long long*)A(2 * sizeof(long long));   // step, finished blocks
   h->prof = (double*)A(sizeof(double) * USP_NPROF * h->ny * h->blocks);
   h->grad = (double*)A(sizeof(double) * kND);
-  bool ok = h->keycell && h->bh && h->off && h->cells && h->prm && h->sums && h->acc &&
+  bool ok = h->keycell && h->bh && h->off && h->cells && h->acc &&
             h->prof && h->grad &&
             (env.sp.method != 1 || h->fpmrec) &&
             h->wallmom && h->macc && h->mout && h->dstep;
@@ -887,7 +1101,8 @@ int ch_create(ChannelCtx** out, const ChEnv& env, const usp_channel* chp, double
   cok = cok && cudaMemcpyAsync(h->pd[0], hp.data(), nn * 4, cudaMemcpyHostToDevice, s) == cudaSuccess;
   cok = cok && cudaMemcpyAsync(h->keycell, key.data(), nn * 4, cudaMemcpyHostToDevice, s) == cudaSuccess;
   cok = cok && cudaMemsetAsync(h->cells, 0, cell_bytes * h->ny, s) == cudaSuccess;
-  cok = cok && cudaMemsetAsync(h->sums, 0, sums_bytes * h->ny, s) == cudaSuccess;
+  cok = cok && cudaMemsetAsync(h->wallmom, 0, sizeof(double), s) == cudaSuccess;
+  cok = cok && cudaMemsetAsync(h->dstep, 0, 2 * sizeof(long long), s) == cudaSuccess;
   cok = cok && cudaMemsetAsync(h->acc, 0, acc_bytes, s) == cudaSuccess;
   cok = cok && cudaMemcpyAsync(h->dstep, &dstep0, sizeof(long long), cudaMemcpyHostToDevice, s) == cudaSuccess;
   if (n > 0) {

@@ -461,54 +461,17 @@ __device__ __forceinline__ double gasR(const Species& s) { return s.R; }
 // viscosity index omega and the rotational collision number Z_rot passed as
 // S so that derivatives with respect to them propagate).
 
-// e_vib(T) = R Theta / (exp(Theta/T) - 1) (Sec. 2.A)
-template <typename S>
-__device__ __forceinline__ S e_vib_T(const Species& s, const S& T) {
-  if (T <= 0.0) return S(0.0);
-  return gasR(s) * s.theta_v / expm1(s.theta_v / T);
-}
-// c_v,vib(T) = R (Theta/2T)^2 / sinh^2(Theta/2T): the derivative of e_vib.
-template <typename S>
-__device__ __forceinline__ S cv_vib_T(const Species& s, const S& T) {
-  if (T <= 0.0) return S(0.0);
-  const S h = 0.5 * s.theta_v / T;
-  const S sh = sinh(h);
-  return gasR(s) * (h * h) / (sh * sh);
-}
 // temperature whose e_vib is R Theta ebar
 template <typename S>
 __device__ __forceinline__ S T_vib_of_level(const Species& s, const S& ebar) {
   if (ebar <= 0.0) return S(0.0);
   return s.theta_v / log1p(1.0 / ebar);
 }
-// VSS viscosity and the factor tau_c = K mu / p (Sec. 4.A)
-template <typename S>
-__device__ __forceinline__ S mu_of_T_w(const Species& s, const S& T, const S& w) {
-  const double ca = s.c_alpha;
-  const S mu_ref = 5.0 * (ca + 1.0) * (ca + 2.0) * sqrt(s.m * kB * s.T_ref / kPi) /
-                   (4.0 * ca * (5.0 - 2.0 * w) * (7.0 - 2.0 * w) * s.d_ref * s.d_ref);
-  return mu_ref * pow(T / s.T_ref, w);
-}
+// the VSS factor tau_c = K mu / p (Sec. 4.A)
 template <typename S>
 __device__ __forceinline__ S tau_c_factor_w(const Species& s, const S& w) {
   const double ca = s.c_alpha;
   return ca * (5.0 - 2.0 * w) * (7.0 - 2.0 * w) / (5.0 * (ca + 1.0) * (ca + 2.0));
-}
-__device__ __forceinline__ double mu_of_T(const Species& s, double T) {
-  return mu_of_T_w<double>(s, T, s.omega);
-}
-__device__ __forceinline__ double tau_c_factor(const Species& s) {
-  return tau_c_factor_w<double>(s, s.omega);
-}
-// Eucken Pr (Sec. 4.B), xi_vib evaluated at the cell vibrational temperature
-template <typename S>
-__device__ __forceinline__ S prandtl_T(const Species& s, const S& Tv) {
-  S xi(0.0);
-  if (Tv > 0.0) {
-    const S x = s.theta_v / Tv;
-    xi = x / expm1(x);
-  }
-  return (14.0 + 2.0 * xi) / (19.0 + 2.0 * xi);
 }
 // Collision numbers: zmodel 0 the fixed ones, zmodel 1 Parker's Z_rot and
 // Millikan-White with the high-temperature term for Z_vib (Sec. 5.C).  xw is
@@ -598,80 +561,12 @@ struct CellCoeffsT {
   bool ok;
   bool tgt_clamped;   // a negative target was set to 0
 };
-
-template <typename S>
-__device__ inline CellCoeffsT<S> cell_coeffs_t(const Species& s, const S& omega, const S& zrot,
-                                               double n, double dt, const S& Ttr, const S& Trot,
-                                               const S& Tvib) {
-  CellCoeffsT<S> c;
-  const double R = gasR(s);
-  const double ctr = 1.5 * R, crot = R;
-  const S p = n * kB * Ttr;
-  // (T/T_ref)^omega, shared by the viscosity and the collision numbers
-  const S xw = exp(omega * log(Ttr / s.T_ref));
-  S mu_ref, tauf;
-  if constexpr (sizeof(S) == sizeof(double)) {   // plain forms: species constants
-    mu_ref = S(s.mu_ref0);
-    tauf = S(s.tauf0);
-  } else {                                        // derivative form: through omega
-    const double ca = s.c_alpha;
-    mu_ref = 5.0 * (ca + 1.0) * (ca + 2.0) * sqrt(s.m * kB * s.T_ref / kPi) /
-             (4.0 * ca * (5.0 - 2.0 * omega) * (7.0 - 2.0 * omega) * s.d_ref * s.d_ref);
-    tauf = tau_c_factor_w<S>(s, omega);
-  }
-  c.mu_p = mu_ref * xw / p;
-  const S tau_c = tauf * c.mu_p;
-  S zr, zv;
-  collision_numbers<S>(s, Ttr, xw, zrot, zr, zv);
-  const S tau_rot = zr * tau_c, tau_vib = zv * tau_c;
-  c.Pr = prandtl_T<S>(s, Tvib);
-  c.A = (2.0 * c.mu_p - c.Pr * dt) / (2.0 * c.mu_p + c.Pr * dt);
-  c.B = (2.0 * c.mu_p - dt) / (2.0 * c.mu_p + dt);
-  c.ok = c.A > -1.0 && c.A < 1.0;
-  c.alpha = c.ok ? cbrt(c.A) : S(0.0);
-  const S a2 = c.alpha * c.alpha;
-  c.nu_ref = (c.B - a2) / (1.0 - a2);
-  const S gr = dt / (dt + 2.0 * tau_rot);
-  const S gv = dt / (dt + 2.0 * tau_vib);
-  const S evT = e_vib_T<S>(s, Tvib);
-  // the value of the fixed point, then its derivatives: those of F at that
-  // value, over 1 - F'
-  const double xv = solve_cv_T1(R * s.theta_v, s.theta_v, R, (double)gr, (double)gv, (double)Ttr,
-                                (double)Trot, (double)Tvib, (double)evT,
-                                cv_vib_T<double>(s, (double)Tvib));
-  S x(xv);
-  if constexpr (sizeof(S) != sizeof(double)) {
-    const S iden = 1.0 / (ctr + gr * crot + gv * xv);
-    const S Tc = Ttr + (gr * crot * (Trot - Ttr) + gv * xv * (Tvib - Ttr)) * iden;
-    if (!(fabs(Tc - Tvib) <= 1e-9 * fmax(fabs(Tc), fabs(Tvib)))) {
-      const S F = (e_vib_T<S>(s, Tc) - evT) / (Tc - Tvib);
-      const double dF = -(double)gv * (cv_vib_T<double>(s, (double)Tc) - xv) * (double)iden;
-      const double k = 1.0 / (1.0 - dF);
-      for (int i = 0; i < 3; ++i) x.d[i] = F.d[i] * k;
-    } else {
-      const S F = cv_vib_T<S>(s, Tvib);
-      for (int i = 0; i < 3; ++i) x.d[i] = F.d[i];
-    }
-  }
-  const S idn = 1.0 / (ctr + gr * crot + gv * x);
-  c.g_tr_rot = 2.0 * gr * ctr * crot * idn;
-  c.g_tr_vib = 2.0 * gv * ctr * x * idn;
-  c.g_rot_vib = 2.0 * gr * gv * crot * x * idn;
-  c.e_rot_tgt = crot * Trot + c.g_tr_rot * (Ttr - Trot) - c.g_rot_vib * (Trot - Tvib);
-  c.e_vib_tgt = evT + c.g_tr_vib * (Ttr - Tvib) + c.g_rot_vib * (Trot - Tvib);
-  // far above tau_rot the exchange terms can overshoot below zero: such a
-  // target is 0 (the velocity rescale still conserves the cell's energy)
-  c.tgt_clamped = false;
-  if (c.e_rot_tgt < 0.0) { c.e_rot_tgt = S(0.0); c.tgt_clamped = true; }
-  if (c.e_vib_tgt < 0.0) { c.e_vib_tgt = S(0.0); c.tgt_clamped = true; }
-  return c;
-}
-
 typedef CellCoeffsT<double> CellCoeffs;
 
 // A cell's vibrational state from its mean level: L = Theta / T_vib = log(1 +
 // 1/ebar), so that exp(L) - 1 = 1/ebar and T_vib, e_vib = R Theta ebar, c_v,vib and
-// the Eucken fraction x / (exp x - 1) take one logarithm.
+// the Eucken fraction x / (exp x - 1) take one logarithm.  Levels carry no
+// derivative.
 struct VibState {
   double Tvib, ev, cv, xi;
 };
@@ -682,40 +577,97 @@ __device__ __forceinline__ VibState vib_state(const Species& s, double ebar) {
               : VibState{d_div(s.theta_v, L), s.R * s.theta_v * ebar,
                          s.R * (L * L) * (ebar * (1.0 + ebar)), L * ebar};
 }
+// Eucken Pr (Sec. 4.B) at the cell's vibrational temperature
+__device__ __forceinline__ double cell_prandtl(const VibState& v) {
+  return d_div(fma(2.0, v.xi, 14.0), fma(2.0, v.xi, 19.0));
+}
 
-// cell_coeffs_t for plain FP64 on the functions of usp_math.cuh, with the
-// cell's mean level in place of T_vib.  One thread's chain: 37 us with the
-// library's functions and the plain T_1 iteration (the cell update of one
-// cell), 9 us now.
-__device__ inline CellCoeffs cell_coeffs(const Species& s, double n, double dt, double Ttr,
-                                         double Trot, const VibState& v) {
-  CellCoeffs c;
-  const double R = s.R, ctr = 1.5 * R;
-  const double lt = d_log(Ttr * s.iT_ref);
-  const double xw = d_exp(s.omega * lt);
-  c.mu_p = s.mu_ref0 * xw * d_rcp(n * kB * Ttr);
-  const double tau_c = s.tauf0 * c.mu_p;
-  double zr, zv;
-  collision_numbers<double>(s, Ttr, xw, s.Z_rot, zr, zv);
-  c.Pr = d_div(fma(2.0, v.xi, 14.0), fma(2.0, v.xi, 19.0));
-  const double m2 = 2.0 * c.mu_p, pd = c.Pr * dt;
-  c.A = d_div(m2 - pd, m2 + pd);
-  c.B = d_div(m2 - dt, m2 + dt);
-  const double gr = d_div(dt, fma(2.0 * zr, tau_c, dt)), gv = d_div(dt, fma(2.0 * zv, tau_c, dt));
+// quotient and cube root by type (derivative numbers bring their own)
+__device__ __forceinline__ double c_div(double a, double b) { return d_div(a, b); }
+__device__ __forceinline__ double c_cbrt(double a) { return d_cbrt(a); }
+template <typename S>
+__device__ __forceinline__ S c_div(const S& a, const S& b) { return a / b; }
+template <typename S>
+__device__ __forceinline__ S c_cbrt(const S& a) { return cbrt(a); }
+
+// The coefficients in the parts that depend on one another: mu / p and xw = (T /
+// T_ref)^omega; A, B, alpha and nu (from mu / p and Pr); the gamma coefficients
+// and the targets (from mu / p and xw).  omega and zrot are the independent
+// variables of the derivative form.
+template <typename S>
+__device__ __forceinline__ void cell_mu_p(const Species& s, double n, const S& Ttr, const S& omega,
+                                          S& mu_p, S& xw) {
+  if constexpr (sizeof(S) == sizeof(double)) {   // plain forms: species constants
+    xw = d_exp(s.omega * d_log(Ttr * s.iT_ref));
+    mu_p = s.mu_ref0 * xw * d_rcp(n * kB * Ttr);
+  } else {                                        // derivative form: through omega
+    const double ca = s.c_alpha;
+    xw = exp(omega * log(Ttr / s.T_ref));
+    const S mu_ref = 5.0 * (ca + 1.0) * (ca + 2.0) * sqrt(s.m * kB * s.T_ref / kPi) /
+                     (4.0 * ca * (5.0 - 2.0 * omega) * (7.0 - 2.0 * omega) * s.d_ref * s.d_ref);
+    mu_p = mu_ref * xw / (n * kB * Ttr);
+  }
+}
+template <typename S>
+__device__ __forceinline__ void cell_alpha(CellCoeffsT<S>& c, double dt) {
+  const S m2 = 2.0 * c.mu_p, pd = c.Pr * dt;
+  c.A = c_div(m2 - pd, m2 + pd);
+  c.B = c_div(m2 - dt, m2 + dt);
   c.ok = c.A > -1.0 && c.A < 1.0;
-  c.alpha = c.ok ? d_cbrt(c.A) : 0.0;
-  const double a2 = c.alpha * c.alpha;
-  c.nu_ref = d_div(c.B - a2, 1.0 - a2);
-  const double x = solve_cv_T1(R * s.theta_v, s.theta_v, R, gr, gv, Ttr, Trot, v.Tvib, v.ev, v.cv);
-  const double idn = d_rcp(fma(gv, x, fma(gr, R, ctr)));
+  c.alpha = c.ok ? c_cbrt(c.A) : S(0.0);
+  const S a2 = c.alpha * c.alpha;
+  c.nu_ref = c_div(c.B - a2, 1.0 - a2);
+}
+template <typename S>
+__device__ __forceinline__ void cell_gammas(const Species& s, CellCoeffsT<S>& c, const S& omega,
+                                            const S& zrot, double dt, const S& Ttr, const S& Trot,
+                                            const VibState& v, const S& xw) {
+  const double R = s.R, ctr = 1.5 * R, th = s.theta_v;
+  S tauf(s.tauf0);
+  if constexpr (sizeof(S) != sizeof(double)) tauf = tau_c_factor_w<S>(s, omega);
+  const S tau_c = tauf * c.mu_p;
+  S zr, zv;
+  collision_numbers<S>(s, Ttr, xw, zrot, zr, zv);
+  const S gr = c_div(S(dt), dt + 2.0 * zr * tau_c), gv = c_div(S(dt), dt + 2.0 * zv * tau_c);
+  // the value of the fixed point, then its derivatives: those of F at that
+  // value, over 1 - F'
+  const double xv = solve_cv_T1(R * th, th, R, (double)gr, (double)gv, (double)Ttr, (double)Trot,
+                                v.Tvib, v.ev, v.cv);
+  S x(xv);
+  if constexpr (sizeof(S) != sizeof(double)) {
+    const S iden = 1.0 / (ctr + gr * R + gv * xv);
+    const S Tc = Ttr + (gr * R * (Trot - Ttr) + gv * xv * (v.Tvib - Ttr)) * iden;
+    const double d = (double)Tc - v.Tvib;
+    if (!(::fabs(d) <= 1e-9 * ::fmax(::fabs((double)Tc), ::fabs(v.Tvib))) && Tc > 0.0) {
+      // dF = (c_v,vib(T_check) - F) / (T_check - T_vib) dT_check
+      const double xx = th * d_rcp((double)Tc), iE = d_rcp(d_expm1(xx));
+      const double cvc = R * (xx * xx) * (iE * (1.0 + iE));
+      const double dF = -(double)gv * (cvc - xv) * (double)iden;
+      const double k = d_div(cvc - xv, d * (1.0 - dF));
+      for (int i = 0; i < 3; ++i) x.d[i] = Tc.d[i] * k;
+    }
+  }
+  const S idn = c_div(S(1.0), ctr + gr * R + gv * x);
   c.g_tr_rot = 2.0 * gr * ctr * R * idn;
   c.g_tr_vib = 2.0 * gv * ctr * x * idn;
   c.g_rot_vib = 2.0 * gr * gv * R * x * idn;
   c.e_rot_tgt = R * Trot + c.g_tr_rot * (Ttr - Trot) - c.g_rot_vib * (Trot - v.Tvib);
   c.e_vib_tgt = v.ev + c.g_tr_vib * (Ttr - v.Tvib) + c.g_rot_vib * (Trot - v.Tvib);
+  // far above tau_rot the exchange terms can overshoot below zero: such a
+  // target is 0 (the velocity rescale still conserves the cell's energy)
   c.tgt_clamped = false;
-  if (c.e_rot_tgt < 0.0) { c.e_rot_tgt = 0.0; c.tgt_clamped = true; }
-  if (c.e_vib_tgt < 0.0) { c.e_vib_tgt = 0.0; c.tgt_clamped = true; }
+  if (c.e_rot_tgt < 0.0) { c.e_rot_tgt = S(0.0); c.tgt_clamped = true; }
+  if (c.e_vib_tgt < 0.0) { c.e_vib_tgt = S(0.0); c.tgt_clamped = true; }
+}
+// all of them by one thread
+__device__ inline CellCoeffs cell_coeffs(const Species& s, double n, double dt, double Ttr,
+                                         double Trot, const VibState& v) {
+  CellCoeffs c;
+  double xw;
+  cell_mu_p<double>(s, n, Ttr, s.omega, c.mu_p, xw);
+  c.Pr = cell_prandtl(v);
+  cell_alpha<double>(c, dt);
+  cell_gammas<double>(s, c, s.omega, s.Z_rot, dt, Ttr, Trot, v, xw);
   return c;
 }
 

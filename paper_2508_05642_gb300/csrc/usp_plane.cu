@@ -1698,9 +1698,8 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
     ch_coeffs_fpm<<<tb, kBlk, 0, s>>>(ncell, h->Fnum, h->vol, h->afv, h->g.dt, h->cells,
                                       h->fpmrec, env.sp, env.flags, env.counters);
   else if (!fused)
-    ch_coeffs<double><<<tb, kBlk, 0, s>>>(ncell, h->Fnum, h->vol, h->afv, h->g.dt, h->cells,
-                                          env.sp, env.sp.omega, env.sp.Z_rot, env.flags,
-                                          env.counters);
+    ch_coeffs<<<tb, kBlk, 0, s>>>(ncell, h->Fnum, h->vol, h->afv, h->g.dt, h->cells, env.sp,
+                                  env.flags, env.counters);
   if (fpm || h->levels < 2)
     pl_params<T><<<(ncell + kStencilBlock<T> - 1) / kStencilBlock<T>, kStencilBlock<T>, 0, s>>>(
         h->g, gt, fpm ? 0 : h->recon, h->cells, (const T*)h->fT, h->usable_c,

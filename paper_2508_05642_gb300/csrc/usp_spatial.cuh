@@ -69,6 +69,33 @@ __device__ __forceinline__ dual::Dual<V> wsum(dual::Dual<V> v) {
   return v;
 }
 
+// The warp totals of a[0 .. N-1] on every lane (N 4 or 6): by halving, then
+// from the lanes that hold them.
+template <int N, typename V>
+__device__ __forceinline__ void all_totals(V* a) {
+  static_assert(N == 4 || N == 6, "places below");
+  halve_totals<N>(a);
+  const V mine = a[0];
+  constexpr int at[2][6] = {{0, 8, 16, 24, 0, 0}, {0, 4, 8, 16, 20, 24}};
+#pragma unroll
+  for (int i = 0; i < N; ++i) a[i] = __shfl_sync(0xffffffffu, mine, at[N == 6][i]);
+}
+template <int N, typename V>
+__device__ __forceinline__ void all_totals(dual::Dual<V>* a) {
+#pragma unroll
+  for (int k = 0; k <= kND; ++k) {
+    V b[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) b[i] = k == 0 ? a[i].v : a[i].d[k == 0 ? 0 : k - 1];
+    all_totals<N>(b);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      if (k == 0) a[i].v = b[i];
+      else a[i].d[k == 0 ? 0 : k - 1] = b[i];
+    }
+  }
+}
+
 // e_vib in the working precision
 template <typename T>
 __device__ __forceinline__ T evib_t(const T& Rth, const T& theta, const T& Tv) {
@@ -328,138 +355,51 @@ __device__ __forceinline__ void tally_flush(BlockTally& t, uint32_t* flags,
 __device__ __forceinline__ int warp_global() { return (blockIdx.x * blockDim.x + threadIdx.x) >> 5; }
 __device__ __forceinline__ int warps_total() { return (gridDim.x * blockDim.x) >> 5; }
 
-// vibrational +-1 correction (Sec. 4.C), one warp per cell; same acceptance
-// rule as the one-at-a-time loop (see the homogeneous path)
-template <typename S>
-__global__ void ch_levelfix(int ny, int cpw, const ChCellT<S>* __restrict__ cells,
-                            ChSumsT<S>* __restrict__ sums,
-                            int* __restrict__ lev, const long long* __restrict__ dstep, Species sp,
-                            uint32_t k0, uint32_t k1, uint32_t* flags,
-                            unsigned long long* counters) {
-  __shared__ BlockTally tal;
-  tally_init(tal);
+// The vibrational +-1 correction of Sec. 4.C for one cell of N particles by
+// one warp: `remaining` level changes are made, `draws` and `net` counted; same
+// acceptance rule as the one-at-a-time loop (see the homogeneous path)
+__device__ __forceinline__ void level_correction(long long c, uint32_t step, long long N,
+                                                 int* __restrict__ lv, long long& remaining,
+                                                 long long& draws, long long& net, uint32_t k0,
+                                                 uint32_t k1) {
   const int lane = threadIdx.x & 31;
-  const uint32_t step = (uint32_t)*dstep;
-  const double Rth = gasR(sp) * sp.theta_v;
-  for (long long c0 = (long long)warp_global() * cpw; c0 < ny;
-       c0 += (long long)warps_total() * cpw) {
-    const int ng = (int)(ny - c0 < cpw ? ny - c0 : cpw);
-    // I_Delta of Sec. 4.C for cell c0 + lane (FP64, one cell per lane)
-    long long myId = 0;
-    if (lane < ng) {
-      const long long c = c0 + lane;
-      const ChCellT<S>& cs = cells[c];
-      if (cs.active) {
-        const U4 w = philox4x32_10((uint32_t)c, step, CTAG_IDELTA, 0u, k0, k1);
-        const double u = uniform_open<double>(w.x);
-        myId = (long long)floor((double)cs.N * value(cs.e_vib_tgt) / Rth -
-                                (double)(long long)sums[c].I + u);
-      }
-    }
-    for (int g = 0; g < ng; ++g) {
-      const long long Id = __shfl_sync(0xffffffffu, myId, g);
-      const long long c = c0 + g;
-      const ChCellT<S>& cs = cells[c];
-      if (!cs.active) continue;
-      const long long N = cs.N;
-      long long remaining = Id, draws = 0, net = 0;
-      const long long cap = 64 * N;
-      int* lv = lev + cs.off;
-      while (remaining != 0 && draws < cap) {
-        const long long j = draws + lane;
-        const U4 w = philox4x32_10((uint32_t)c, step, CTAG_PICK, (uint32_t)(j >> 2), k0, k1);
-        const uint32_t word = (j & 3) == 0 ? w.x : (j & 3) == 1 ? w.y : (j & 3) == 2 ? w.z : w.w;
-        const long long k = (long long)(((unsigned long long)word * (unsigned long long)N) >> 32);
-        const bool valid = j < cap;
-        bool accept;
-        if (remaining > 0) {
-          accept = valid;
-        } else {
-          const int cur = valid ? __ldcg(&lv[k]) : 0;
-          const unsigned grp = __match_any_sync(0xffffffffu, valid ? k : -1ll);
-          accept = valid && __popc(grp & lane_lt()) < cur;
-        }
-        const unsigned am = __ballot_sync(0xffffffffu, accept);
-        const long long need = remaining > 0 ? remaining : -remaining;
-        const int nacc = __popc(am);
-        const int take = (int)(nacc < need ? nacc : need);
-        const bool eff = accept && __popc(am & lane_lt()) < take;
-        __syncwarp();
-        if (eff) atomicAdd(&lv[k], remaining > 0 ? 1 : -1);
-        __syncwarp();
-        long long used = 32;
-        if (take == need && take > 0) {
-          unsigned m = am;
-          for (int i = 1; i < take; ++i) m &= m - 1;
-          used = __ffs((int)m);
-        }
-        if (draws + used > cap) used = cap - draws;
-        draws += used;
-        if (remaining > 0) { remaining -= take; net += take; }
-        else { remaining += take; net -= take; }
-      }
-      if (lane == 0) {
-        if (remaining != 0) tally_or(tal, (uint32_t)F_VIB_LOOP_CAP);
-        tally_add(tal, C_VIB_DRAWS, (unsigned long long)draws);
-        sums[c].net = net;
-      }
-    }
-  }
-  tally_flush(tal, flags, counters);
-}
-
-// rescale factors of Sec. 4.C, kept pending for the next move; the step
-// counter advances after the last reader of this step
-template <typename S>
-__global__ void ch_update(int ny, ChCellT<S>* __restrict__ cells,
-                          const ChSumsT<S>* __restrict__ sums, long long* dstep, Species sp,
-                          uint32_t* flags, unsigned long long* counters,
-                          float* __restrict__ pend) {
-  __shared__ BlockTally tal;
-  tally_init(tal);
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ny; c += gridDim.x * blockDim.x) {
-    ChCellT<S>& cs = cells[c];
-    if (!cs.active) continue;
-    const double R = gasR(sp), Rth = R * sp.theta_v;
-    const ChSumsT<S>& sm = sums[c];
-    const double invN = 1.0 / (double)cs.N;
-    const double sumI = (double)((long long)sm.I + sm.net);
-    const S er_star = sm.v[9] * invN;
-    const S r = er_star > 0.0 ? cs.e_rot_tgt / er_star : S(1.0);
-    const S e_rot_new = r * er_star;
-    const double e_vib_new = Rth * sumI * invN;
-    const S m0 = sm.v[0] * invN, m1 = sm.v[1] * invN, m2 = sm.v[2] * invN;
-    const S etr_star = 0.5 * (sm.v[3] * invN - m0 * m0 + sm.v[4] * invN - m1 * m1 +
-                              sm.v[5] * invN - m2 * m2);
-    const S e_tr_n = 0.5 * (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]);
-    const S rad = (e_tr_n + R * cs.Trot + Rth * cs.ebar - e_rot_new - e_vib_new) / etr_star;
-    S Us[3] = {cs.U[0] + m0, cs.U[1] + m1, cs.U[2] + m2};
-    if (!(etr_star > 0.0) || !(rad > 0.0)) {
-      tally_or(tal, (uint32_t)F_NEG_RADICAND);
-      tally_add(tal, C_NEG_RADICAND, 1ull);
-      for (int i = 0; i < 3; ++i) { cs.Un[i] = Us[i]; cs.Us[i] = Us[i]; }
-      cs.s = S(1.0);
+  const long long cap = 64 * N;
+  while (remaining != 0 && draws < cap) {
+    const long long j = draws + lane;
+    const U4 w = philox4x32_10((uint32_t)c, step, CTAG_PICK, (uint32_t)(j >> 2), k0, k1);
+    const uint32_t word = (j & 3) == 0 ? w.x : (j & 3) == 1 ? w.y : (j & 3) == 2 ? w.z : w.w;
+    const long long k = (long long)(((unsigned long long)word * (unsigned long long)N) >> 32);
+    const bool valid = j < cap;
+    bool accept;
+    if (remaining > 0) {
+      accept = valid;
     } else {
-      for (int i = 0; i < 3; ++i) { cs.Un[i] = cs.U[i]; cs.Us[i] = Us[i]; }
-      cs.s = sqrt(rad);
+      const int cur = valid ? __ldcg(&lv[k]) : 0;
+      const unsigned grp = __match_any_sync(0xffffffffu, valid ? k : -1ll);
+      accept = valid && __popc(grp & lane_lt()) < cur;
     }
-    cs.r = r;
-    cs.maxI = sm.maxI + 1;
-    if (pend) {   // FP32 copy for the next move of an FP32 state
-      float* pc = pend + (size_t)c * 8;
-      for (int i = 0; i < 3; ++i) {
-        pc[i] = (float)value(cs.Un[i]);
-        pc[3 + i] = (float)value(cs.Us[i]);
-      }
-      pc[6] = (float)value(cs.s);
-      pc[7] = (float)value(cs.r);
+    const unsigned am = __ballot_sync(0xffffffffu, accept);
+    const long long need = remaining > 0 ? remaining : -remaining;
+    const int nacc = __popc(am);
+    const int take = (int)(nacc < need ? nacc : need);
+    const bool eff = accept && __popc(am & lane_lt()) < take;
+    __syncwarp();
+    if (eff) atomicAdd(&lv[k], remaining > 0 ? 1 : -1);
+    __syncwarp();
+    long long used = 32;
+    if (take == need && take > 0) {
+      unsigned m = am;
+      for (int i = 1; i < take; ++i) m &= m - 1;
+      used = __ffs((int)m);
     }
+    if (draws + used > cap) used = cap - draws;
+    draws += used;
+    if (remaining > 0) { remaining -= take; net += take; }
+    else { remaining += take; net -= take; }
   }
-  tally_flush(tal, flags, counters);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *dstep += 1;
 }
 
-// ch_levelfix and ch_update in one pass (FP64 cell records): the warp makes
+// Conservation of Sec. 4.C on the plane (FP64 cell records): the warp makes
 // the +-1 corrections of its 32 cells one after the other, lane k keeping
 // cell k's net change, then every lane computes its cell's rescale factors.
 // F32: the factors in FP32 arithmetic (the FP32 state's own precision) from
@@ -499,41 +439,7 @@ __global__ void ch_fix_update(int ncell, ChCellT<double>* __restrict__ cells,
       if (!cs.active) continue;
       const long long N = cs.N;
       long long remaining = Id, draws = 0, net = 0;
-      const long long cap = 64 * N;
-      int* lv = lev + cs.off;
-      while (remaining != 0 && draws < cap) {
-        const long long j = draws + lane;
-        const U4 w = philox4x32_10((uint32_t)c, step, CTAG_PICK, (uint32_t)(j >> 2), k0, k1);
-        const uint32_t word = (j & 3) == 0 ? w.x : (j & 3) == 1 ? w.y : (j & 3) == 2 ? w.z : w.w;
-        const long long k = (long long)(((unsigned long long)word * (unsigned long long)N) >> 32);
-        const bool valid = j < cap;
-        bool accept;
-        if (remaining > 0) {
-          accept = valid;
-        } else {
-          const int cur = valid ? __ldcg(&lv[k]) : 0;
-          const unsigned grp = __match_any_sync(0xffffffffu, valid ? k : -1ll);
-          accept = valid && __popc(grp & lane_lt()) < cur;
-        }
-        const unsigned am = __ballot_sync(0xffffffffu, accept);
-        const long long need = remaining > 0 ? remaining : -remaining;
-        const int nacc = __popc(am);
-        const int take = (int)(nacc < need ? nacc : need);
-        const bool eff = accept && __popc(am & lane_lt()) < take;
-        __syncwarp();
-        if (eff) atomicAdd(&lv[k], remaining > 0 ? 1 : -1);
-        __syncwarp();
-        long long used = 32;
-        if (take == need && take > 0) {
-          unsigned m = am;
-          for (int i = 1; i < take; ++i) m &= m - 1;
-          used = __ffs((int)m);
-        }
-        if (draws + used > cap) used = cap - draws;
-        draws += used;
-        if (remaining > 0) { remaining -= take; net += take; }
-        else { remaining += take; net -= take; }
-      }
+      level_correction(c, step, N, lev + cs.off, remaining, draws, net, k0, k1);
       if (lane == g) mynet = net;
       if (lane == 0) {
         if (remaining != 0) tally_or(tal, (uint32_t)F_VIB_LOOP_CAP);
@@ -603,20 +509,17 @@ __global__ void ch_fix_update(int ncell, ChCellT<double>* __restrict__ cells,
 // for the k-th cell; the FP64 per-cell arithmetic then runs one cell per lane,
 // so each FP64 warp instruction serves up to 32 cells on the narrow FP64 pipe.
 template <typename T, typename S>
-__global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
-                           const double* __restrict__ af, const T* __restrict__ cx,
-                           const T* __restrict__ cy, const T* __restrict__ cz,
-                           const T* __restrict__ er, const int* __restrict__ lev,
-                           ChCellT<S>* __restrict__ cells, Species sp,
-                           unsigned long long* counters, float* __restrict__ pend,
-                           T* __restrict__ fT, int* __restrict__ usable_c) {
-  __shared__ BlockTally tal;
-  tally_init(tal);
+__device__ __forceinline__ void
+moments_of_cells(long long first, long long stride, long long ny, int cpw,
+                 const long long* __restrict__ off, const double* __restrict__ af,
+                 const T* __restrict__ cx, const T* __restrict__ cy, const T* __restrict__ cz,
+                 const T* __restrict__ er, const int* __restrict__ lev,
+                 ChCellT<S>* __restrict__ cells, const Species& sp, float* __restrict__ pend,
+                 T* __restrict__ fT, int* __restrict__ usable_c, BlockTally& tal) {
   const int lane = threadIdx.x & 31;
   const double R = gasR(sp);
   constexpr bool f32 = sizeof(T) == 4;
-  for (long long c0 = (long long)warp_global() * cpw; c0 < ny;
-       c0 += (long long)warps_total() * cpw) {
+  for (long long c0 = first; c0 < ny; c0 += stride) {
     const int ng = (int)(ny - c0 < cpw ? ny - c0 : cpw);
     T k0 = T(0), k1 = T(0), k2 = T(0), ke = T(0), kq[6];
     long long kl = 0, kb = 0, kN = 0;
@@ -653,13 +556,10 @@ __global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
         a0 += cx[j]; a1 += cy[j]; a2 += cz[j]; ae += er[j]; al += lev[j];
       }
       T t0, t1, t2, te;
-      if constexpr (sizeof(T) <= 8) {
+      {
         T tot[4] = {a0, a1, a2, ae};
-        halve_totals<4>(tot);   // totals 0, 1, 2, 3 end on lanes 0, 8, 16, 24
-        t0 = __shfl_sync(0xffffffffu, tot[0], 0); t1 = __shfl_sync(0xffffffffu, tot[0], 8);
-        t2 = __shfl_sync(0xffffffffu, tot[0], 16); te = __shfl_sync(0xffffffffu, tot[0], 24);
-      } else {
-        t0 = wsum(a0); t1 = wsum(a1); t2 = wsum(a2); te = wsum(ae);
+        all_totals<4>(tot);
+        t0 = tot[0]; t1 = tot[1]; t2 = tot[2]; te = tot[3];
       }
       const long long sl = wsum(al);
       // the reference mean of the second pass (an FP32 state keeps FP32)
@@ -668,7 +568,7 @@ __global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
         const float fn = N > 0 ? (float)N : 1.0f;
         m0 = t0 / fn; m1 = t1 / fn; m2 = t2 / fn;
       } else {
-        const double inv = N > 0 ? 1.0 / (double)N : 0.0;
+        const double inv = N > 0 ? d_rcp((double)N) : 0.0;
         m0 = (T)(S(t0) * inv); m1 = (T)(S(t1) * inv); m2 = (T)(S(t2) * inv);
       }
       T p[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
@@ -683,14 +583,9 @@ __global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
         p[3] += C0 * C1; p[4] += C0 * C2; p[5] += C1 * C2;
       }
       T q[6];
-      if constexpr (sizeof(T) <= 8) {
-        halve_totals<6>(p);     // totals 0 .. 5 end on lanes 0, 4, 8, 16, 20, 24
-        constexpr int at[6] = {0, 4, 8, 16, 20, 24};
+      all_totals<6>(p);
 #pragma unroll
-        for (int i = 0; i < 6; ++i) q[i] = __shfl_sync(0xffffffffu, p[0], at[i]);
-      } else {
-        for (int i = 0; i < 6; ++i) q[i] = wsum(p[i]);
-      }
+      for (int i = 0; i < 6; ++i) q[i] = p[i];
       if (lane == g) {
         k0 = t0; k1 = t1; k2 = t2; ke = te; kl = sl; kb = b; kN = N;
         for (int i = 0; i < 6; ++i) kq[i] = q[i];
@@ -699,7 +594,7 @@ __global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
     if (lane >= ng) continue;
     const long long c = c0 + lane;
     const long long N = kN;
-    const double inv = N > 0 ? 1.0 / (double)N : 0.0;
+    const double inv = N > 0 ? d_rcp((double)N) : 0.0;
     const S s0 = S(k0), s1 = S(k1), s2 = S(k2), se = S(ke);
     S P[6];
     for (int i = 0; i < 6; ++i) P[i] = S(kq[i]) * inv;
@@ -726,10 +621,10 @@ __global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
       continue;
     }
     for (int i = 0; i < 6; ++i) cs.Pi[i] = P[i];
-    cs.Ttr = (P[0] + P[1] + P[2]) / (3.0 * R);
-    cs.Trot = se * inv / R;
+    cs.Ttr = (P[0] + P[1] + P[2]) * (sp.iR * (1.0 / 3.0));
+    cs.Trot = se * (inv * sp.iR);
     cs.ebar = (double)kl * inv;
-    cs.Tvib = T_vib_of_level<double>(sp, cs.ebar);
+    cs.Tvib = vib_state(sp, cs.ebar).Tvib;
     if (fT) {   // the 13 fields in the particle precision, for the stencils
       T* o = fT + (size_t)c * kNF;
       for (int i = 0; i < 3; ++i) o[i] = (T)cs.U[i];
@@ -737,42 +632,99 @@ __global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
       for (int i = 0; i < 6; ++i) o[6 + i] = (T)cs.Pi[i];
     }
   }
+}
+
+template <typename T, typename S>
+__global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
+                           const double* __restrict__ af, const T* __restrict__ cx,
+                           const T* __restrict__ cy, const T* __restrict__ cz,
+                           const T* __restrict__ er, const int* __restrict__ lev,
+                           ChCellT<S>* __restrict__ cells, Species sp,
+                           unsigned long long* counters, float* __restrict__ pend,
+                           T* __restrict__ fT, int* __restrict__ usable_c) {
+  __shared__ BlockTally tal;
+  tally_init(tal);
+  moments_of_cells<T, S>((long long)warp_global() * cpw, (long long)warps_total() * cpw, ny, cpw,
+                         off, af, cx, cy, cz, er, lev, cells,
+                         sp, pend, fT, usable_c, tal);
   tally_flush(tal, nullptr, counters);
 }
 
+// a cell's coefficients into its record
 template <typename S>
+__device__ __forceinline__ void put_coeffs(ChCellT<S>& cs, const CellCoeffsT<S>& k,
+                                           BlockTally& tal) {
+  if (!k.ok) {
+    tally_or(tal, (uint32_t)F_A_NONPOS);
+    cs.active = 0;
+    return;
+  }
+  cs.alpha = k.alpha; cs.nu_ref = k.nu_ref; cs.B = k.B; cs.mu_p = k.mu_p; cs.Pr = k.Pr;
+  cs.gtr = k.g_tr_rot; cs.gtv = k.g_tr_vib; cs.grv = k.g_rot_vib;
+  cs.e_rot_tgt = k.e_rot_tgt;
+  cs.e_vib_tgt = k.e_vib_tgt;
+  if (k.tgt_clamped) {
+    tally_or(tal, (uint32_t)F_TREL_CLAMP);
+    tally_add(tal, C_TREL_CLAMP, 1ull);
+  }
+}
+
+// coefficients of the plane's cells (FP64 form), one thread per cell
 __global__ void ch_coeffs(int ny, double F_num, double vol, const double* __restrict__ af,
-                          double dt, ChCellT<S>* __restrict__ cells, Species sp, S omega, S zrot,
+                          double dt, ChCellT<double>* __restrict__ cells, Species sp,
                           uint32_t* flags, unsigned long long* counters) {
   __shared__ BlockTally tal;
   tally_init(tal);
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ny; c += gridDim.x * blockDim.x) {
-    ChCellT<S>& cs = cells[c];
+    ChCellT<double>& cs = cells[c];
     if (!cs.active) continue;
-    const double v = af ? af[c] * vol : vol;   // fluid volume of a cut cell
+    const double v = af[c] * vol;   // fluid volume of a cut cell
     if (!(v > 0.0)) {
       cs.active = 0;
       continue;
     }
     cs.n = (double)cs.N * F_num / v;
-    CellCoeffsT<S> k;
-    if constexpr (std::is_same<S, double>::value)
-      k = cell_coeffs(sp, cs.n, dt, cs.Ttr, cs.Trot, vib_state(sp, cs.ebar));
-    else
-      k = cell_coeffs_t<S>(sp, omega, zrot, cs.n, dt, cs.Ttr, cs.Trot, S(cs.Tvib));
-    if (!k.ok) {
-      tally_or(tal, (uint32_t)F_A_NONPOS);
-      cs.active = 0;
-      continue;
+    put_coeffs<double>(cs, cell_coeffs(sp, cs.n, dt, cs.Ttr, cs.Trot, vib_state(sp, cs.ebar)),
+                       tal);
+  }
+  tally_flush(tal, flags, counters);
+}
+
+// moments and coefficients of the channel's cells, one block per cell: one warp
+// sums, then the parts of the coefficients that do not need one another run
+// on different warps, that is on different quarters of the SM
+template <typename T, typename S>
+__global__ void __launch_bounds__(128)
+ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T* __restrict__ cy,
+           const T* __restrict__ cz, const T* __restrict__ er, const int* __restrict__ lev,
+           ChCellT<S>* __restrict__ cells, Species sp, double F_num, double vol, double dt, S omega,
+           S zrot, uint32_t* flags, unsigned long long* counters) {
+  __shared__ BlockTally tal;
+  __shared__ CellCoeffsT<S> k;
+  __shared__ S xw;
+  __shared__ VibState vib;
+  tally_init(tal);
+  const int c = blockIdx.x, t = threadIdx.x;
+  ChCellT<S>& cs = cells[c];
+  if (t < 32)
+    moments_of_cells<T, S>(c, 1, c + 1, 1, off, nullptr, cx, cy, cz, er, lev, cells, sp, nullptr,
+                           (T*)nullptr, nullptr, tal);
+  __syncthreads();
+  if (cs.active && vol > 0.0) {        // uniform over the block
+    if (t == 0) {
+      cs.n = (double)cs.N * F_num / vol;
+      cell_mu_p<S>(sp, cs.n, cs.Ttr, omega, k.mu_p, xw);
+    } else if (t == 32) {
+      vib = vib_state(sp, cs.ebar);
+      k.Pr = S(cell_prandtl(vib));
     }
-    cs.alpha = k.alpha; cs.nu_ref = k.nu_ref; cs.B = k.B; cs.mu_p = k.mu_p; cs.Pr = k.Pr;
-    cs.gtr = k.g_tr_rot; cs.gtv = k.g_tr_vib; cs.grv = k.g_rot_vib;
-    cs.e_rot_tgt = k.e_rot_tgt;
-    cs.e_vib_tgt = k.e_vib_tgt;
-    if (k.tgt_clamped) {
-      tally_or(tal, (uint32_t)F_TREL_CLAMP);
-      tally_add(tal, C_TREL_CLAMP, 1ull);
-    }
+    __syncthreads();
+    if (t == 0) cell_alpha<S>(k, dt);
+    else if (t == 32) cell_gammas<S>(sp, k, omega, zrot, dt, cs.Ttr, cs.Trot, vib, xw);
+    __syncthreads();
+    if (t == 0) put_coeffs<S>(cs, k, tal);
+  } else if (t == 0 && cs.active) {
+    cs.active = 0;
   }
   tally_flush(tal, flags, counters);
 }
@@ -987,13 +939,6 @@ __device__ __forceinline__ int fpm_particle(const T* U, T a, const T* Lp, T a_ro
   const T root = root_sel<sizeof(T) == 8>(en) * a + sqrt_a * g3;
   en = a_rot + root * root;
   return gillespie<T>(l0, lam_up, lam_dn, id, step, rk, fl);
-}
-
-template <typename S>
-__device__ __forceinline__ void cell_fields(const ChCellT<S>& c, S* f) {
-  f[0] = c.U[0]; f[1] = c.U[1]; f[2] = c.U[2];
-  f[3] = c.Ttr; f[4] = c.Trot; f[5] = S(c.Tvib);
-  for (int i = 0; i < 6; ++i) f[6 + i] = c.Pi[i];
 }
 
 __global__ void ch_mom_out(int ny, const double* __restrict__ a, double* __restrict__ out,
