@@ -419,13 +419,12 @@ __device__ void ch_recon(int c, int ny, double dy, int recon, double dt,
     const ChCellT<S>& q = cells[k];
     return i < 3 ? q.U[i] : i == 3 ? q.Ttr : i == 4 ? q.Trot : i == 5 ? S(q.Tvib) : q.Pi[i - 6];
   };
-  if (t < 12) {
+  if (t < kNF) {
     const S f = field(c, t);
     P.F[t] = (T)f;
     P.Sp[t] = (recon && up >= 0) ? (T)((field(up, t) - f) / ((up - c) * dy)) : T(0);
     P.Sm[t] = (recon && dn >= 0) ? (T)((field(dn, t) - f) / ((dn - c) * dy)) : T(0);
   } else if (t == 32) {
-    P.F[12] = P.Sp[12] = P.Sm[12] = T(0);   // padding field of the records
     P.alpha = (T)cs.alpha; P.nu_ref = (T)cs.nu_ref; P.B = (T)cs.B; P.mu_p = (T)cs.mu_p;
     P.Pr = (T)cs.Pr; P.gtr = (T)cs.gtr; P.gtv = (T)cs.gtv; P.grv = (T)cs.grv;
     P.R = (T)gasR(sp); P.theta = (T)sp.theta_v; P.dt = (T)dt;

@@ -48,7 +48,8 @@ constexpr uint32_t CTAG_INFLOW = 0x80000004u;
 constexpr int kInflowTries = 64;
 constexpr int kBlk = 256;
 constexpr int kNSurf = USP_NSURF;   // cylinder surface bins of the polar angle
-constexpr int kParamBlock = 32;   // cells per block of the stencil pass
+constexpr int kParamBlock = 32;   // cells per block of the stencil passes
+constexpr int kPF = 16;           // threads per cell there: one per field
 
 // Device-resident counts of the current step.
 struct PlCount {
@@ -97,6 +98,7 @@ struct PlTree {
   const int* lvl;
   const int* lii;
   const int* ljj;
+  const int* nb;   // per cell its eight neighbouring squares (pg_neighbours)
 };
 
 struct PlInflow {
@@ -108,12 +110,11 @@ struct PlInflow {
   double RT, U, T;    // freestream R T, x velocity, temperature
 };
 
-// Per-cell parameters of the particle kernel, working precision T.
+// Per-cell parameters of the particle kernel, working precision T; the field
+// arrays come first, in multiples of 16 bytes, so that the particle pass reads
+// them as 16-byte vectors.
 template <typename T>
-struct PlParams {
-  T alpha, nu_ref, B, mu_p, Pr, gtr, gtv, grv;
-  T R, theta, dt;
-  T xc, yc;
+struct alignas(16) PlParams {
   T F[kNF];
   // the bilinear polynomial of each quadrant (sx, sy = 0 below / 1 at or
   // above the centroid): f = F + gx[sx] dx + gy[sy] dy + gxy[2 sy + sx] dx dy
@@ -124,6 +125,9 @@ struct PlParams {
     // alpha^2) L, the rotational square-form constants and the level rates
     struct { T as, Lp[6], a_rot, sqrt_a, lam_up, lam_dn; } fpm;
   };
+  T alpha, nu_ref, B, mu_p, Pr, gtr, gtv, grv;
+  T R, theta, dt;
+  T xc, yc;
   int active, pad;
 };
 
@@ -745,112 +749,86 @@ __global__ void pl_gather(PlCount* __restrict__ cnt, int ncell, long long* __res
 // the centroid the x and y neighbour used (that side's if usable, else the
 // opposite one, else none) and the quadrant's diagonal when usable
 // ---------------------------------------------------------------------------
-// cells per block of the uniform grid's stencil pass (its static shared
-// memory stays under 48 KB)
+// Both stencil passes give a cell kPF threads, thread q < kNF field q: loads
+// and stores of a cell's fields are consecutive, and a thread holds one
+// value per neighbour (one thread per cell kept up to 65 in local memory and
+// built the record in shared memory: 71 us on the 600 x 400 grid, 245 us for
+// the 422,730 cells of the refined one).  The scalars, converted from FP64 or
+// formed in it, are written by one warp for the block's cells together.
 template <typename T>
-constexpr int kStencilBlock = sizeof(T) == 4 ? 64 : 32;
+__device__ __forceinline__ void pl_scalars(PlParams<T>& P, const ChCellT<double>& cs,
+                                           const PlGeomT<T>& gt, const Species& sp, double xc,
+                                           double yc) {
+  P.active = cs.active;
+  P.pad = 0;
+  P.alpha = (T)cs.alpha; P.nu_ref = (T)cs.nu_ref; P.B = (T)cs.B; P.mu_p = (T)cs.mu_p;
+  P.Pr = (T)cs.Pr; P.gtr = (T)cs.gtr; P.gtv = (T)cs.gtv; P.grv = (T)cs.grv;
+  P.R = (T)gasR(sp); P.theta = gt.theta; P.dt = gt.dt;
+  P.xc = (T)xc;
+  P.yc = (T)yc;
+}
 
 template <typename T>
-__global__ void __launch_bounds__(kStencilBlock<T>)
+__global__ void __launch_bounds__(kParamBlock * kPF)
 pl_params(PlGeom g, PlGeomT<T> gt, int recon, const ChCellT<double>* __restrict__ cells,
           const T* __restrict__ fT, const int* __restrict__ usable_c,
           PlParams<T>* __restrict__ prm, Species sp, const double* __restrict__ fpm) {
-  // a thread builds its cell's record in shared memory; the block then copies
-  // its records out as consecutive 8-byte words (coalesced), where one thread
-  // storing a ~0.5 KB record would scatter every store.  The fields and
-  // usable flags of the block's cells and their neighbours (three runs of
-  // kSpan consecutive cells: the rows below, at and above) are staged first,
-  // with coalesced loads.
-  constexpr int kB = kStencilBlock<T>;
-  constexpr int kSpan = kB + 2;
-  __shared__ PlParams<T> buf[kB];
-  __shared__ T sf[3][kSpan][kNF];
-  __shared__ int su[3][kSpan];
-  const int c0 = blockIdx.x * kB;
-  const int c = c0 + threadIdx.x;
-  const int nb = min(kB, g.ncell - c0);
-  // cell of run r (row offset r - 1), place m: c0 - 1 + (r - 1) nx + m
-  for (int e = threadIdx.x; e < 3 * kSpan * kNF; e += kB) {
-    const int r = e / (kSpan * kNF), m = (e / kNF) % kSpan, k = e % kNF;
-    const int cc = c0 - 1 + (r - 1) * g.nx + m;
-    sf[r][m][k] = cc >= 0 && cc < g.ncell ? fT[(size_t)cc * kNF + k] : T(0);
+  const int c0 = blockIdx.x * kParamBlock;
+  if (threadIdx.x < kParamBlock && c0 + (int)threadIdx.x < g.ncell) {
+    const int c = c0 + threadIdx.x;
+    pl_scalars<T>(prm[c], cells[c], gt, sp, g.x0 + (c % g.nx + 0.5) * g.dx,
+                  g.y0 + (c / g.nx + 0.5) * g.dy);
   }
-  for (int e = threadIdx.x; e < 3 * kSpan; e += kB) {
-    const int r = e / kSpan, m = e % kSpan;
-    const int cc = c0 - 1 + (r - 1) * g.nx + m;
-    su[r][m] = cc >= 0 && cc < g.ncell ? usable_c[cc] : 0;
+  const int c = c0 + threadIdx.x / kPF, q = threadIdx.x % kPF;
+  if (c >= g.ncell || q >= kNF) return;
+  const int i = c % g.nx, j = c / g.nx;
+  PlParams<T>& P = prm[c];
+  const T f = fT[(size_t)c * kNF + q];
+  P.F[q] = f;
+  if (fpm) {
+    // the plain FPM method: cell values, its per-cell constants
+    P.gx[0][q] = P.gx[1][q] = P.gy[0][q] = P.gy[1][q] = T(0);
+    static_assert(sizeof(P.fpm) == kFpmRec * sizeof(T), "the record's order");
+    if (q < kFpmRec) (&P.fpm.as)[q] = (T)fpm[(size_t)c * kFpmRec + q];
+    return;
   }
-  __syncthreads();
-  if (c < g.ncell) {
-    const ChCellT<double>& cs = cells[c];
-    PlParams<T>& P = buf[threadIdx.x];
-    P.active = cs.active;
-    P.pad = 0;
-    P.alpha = (T)cs.alpha; P.nu_ref = (T)cs.nu_ref; P.B = (T)cs.B; P.mu_p = (T)cs.mu_p;
-    P.Pr = (T)cs.Pr; P.gtr = (T)cs.gtr; P.gtv = (T)cs.gtv; P.grv = (T)cs.grv;
-    P.R = (T)gasR(sp); P.theta = gt.theta; P.dt = gt.dt;
-    const int i = c % g.nx, j = c / g.nx;
-    P.xc = (T)(g.x0 + (i + 0.5) * g.dx);
-    P.yc = (T)(g.y0 + (j + 0.5) * g.dy);
-    // neighbour (i + di, j + dj): run dj + 1, place threadIdx.x + 1 + di
-    const int m0 = threadIdx.x + 1;
-    const T* f = sf[1][m0];
-    for (int k = 0; k < kNF; ++k) P.F[k] = f[k];
-    if (fpm) {
-      // the plain FPM method: cell values, its per-cell constants
-      for (int k = 0; k < kNF; ++k) { P.gx[0][k] = P.gx[1][k] = P.gy[0][k] = P.gy[1][k] = T(0); }
-      const double* r = fpm + (size_t)c * kFpmRec;
-      P.fpm.as = (T)r[0];
-      for (int k = 0; k < 6; ++k) P.fpm.Lp[k] = (T)r[1 + k];
-      P.fpm.a_rot = (T)r[7]; P.fpm.sqrt_a = (T)r[8];
-      P.fpm.lam_up = (T)r[9]; P.fpm.lam_dn = (T)r[10];
-    } else {
-      auto usable = [&](int di, int dj) {
-        const int ii = i + di, jj = j + dj;
-        return recon && ii >= 0 && ii < g.nx && jj >= 0 && jj < g.ny && su[dj + 1][m0 + di];
-      };
-      auto field = [&](int di, int dj) { return sf[dj + 1][m0 + di]; };
-      // slopes in the working precision from the cell values, times 1/offset
-      int ox[2], oy[2];   // the x and y neighbour of each side (offset; 0: none)
-      for (int sd = 0; sd < 2; ++sd) {
-        const int sg = sd ? 1 : -1;
-        ox[sd] = usable(sg, 0) ? sg : (usable(-sg, 0) ? -sg : 0);
-        oy[sd] = usable(0, sg) ? sg : (usable(0, -sg) ? -sg : 0);
-        if (ox[sd] != 0) {
-          const T* fn = field(ox[sd], 0);
-          const T ih = ox[sd] > 0 ? gt.idx : -gt.idx;
-          for (int k = 0; k < kNF; ++k) P.gx[sd][k] = (fn[k] - f[k]) * ih;
-        } else {
-          for (int k = 0; k < kNF; ++k) P.gx[sd][k] = T(0);
-        }
-        if (oy[sd] != 0) {
-          const T* fn = field(0, oy[sd]);
-          const T ih = oy[sd] > 0 ? gt.idy : -gt.idy;
-          for (int k = 0; k < kNF; ++k) P.gy[sd][k] = (fn[k] - f[k]) * ih;
-        } else {
-          for (int k = 0; k < kNF; ++k) P.gy[sd][k] = T(0);
-        }
-      }
-      for (int q = 0; q < 4; ++q) {
-        const int sx = q & 1, sy = q >> 1;
-        if (ox[sx] != 0 && oy[sy] != 0 && usable(ox[sx], oy[sy])) {
-          const T* fd = field(ox[sx], oy[sy]);
-          const T* fx = field(ox[sx], 0);
-          const T* fy = field(0, oy[sy]);
-          const T ih = ((ox[sx] > 0) == (oy[sy] > 0) ? T(1) : T(-1)) * gt.idx * gt.idy;
-          for (int k = 0; k < kNF; ++k) P.gxy[q][k] = (fd[k] - fx[k] - fy[k] + f[k]) * ih;
-        } else {
-          for (int k = 0; k < kNF; ++k) P.gxy[q][k] = T(0);
-        }
-      }
-    }
+  // the flags and values of the 3 x 3 cells, loaded together (a square outside
+  // the domain reads its own cell and counts as not usable)
+  bool us[9];
+  T fn[9];
+#pragma unroll
+  for (int m = 0; m < 9; ++m) {
+    const int di = m % 3 - 1, dj = m / 3 - 1, ii = i + di, jj = j + dj;
+    const bool in = recon && ii >= 0 && ii < g.nx && jj >= 0 && jj < g.ny;
+    const int cc = in ? jj * g.nx + ii : c;
+    us[m] = in && usable_c[cc];
+    fn[m] = fT[(size_t)cc * kNF + q];
   }
-  __syncthreads();
-  static_assert(sizeof(PlParams<T>) % 8 == 0, "records copied as 8-byte words");
-  const int words = nb * (int)(sizeof(PlParams<T>) / 8);
-  const unsigned long long* src = reinterpret_cast<const unsigned long long*>(buf);
-  unsigned long long* dst = reinterpret_cast<unsigned long long*>(prm + c0);
-  for (int w = threadIdx.x; w < words; w += kB) dst[w] = src[w];
+  // slopes in the working precision from the cell values, times 1/offset: the
+  // x and y neighbour of each side (offset; 0: none)
+  int ox[2], oy[2];
+  T fx[2], fy[2];
+#pragma unroll
+  for (int sd = 0; sd < 2; ++sd) {
+    const int hi = sd ? 1 : -1;
+    ox[sd] = us[4 + hi] ? hi : (us[4 - hi] ? -hi : 0);
+    oy[sd] = us[4 + 3 * hi] ? hi : (us[4 - 3 * hi] ? -hi : 0);
+    fx[sd] = ox[sd] > 0 ? fn[5] : fn[3];
+    fy[sd] = oy[sd] > 0 ? fn[7] : fn[1];
+    P.gx[sd][q] = ox[sd] != 0 ? (fx[sd] - f) * (ox[sd] > 0 ? gt.idx : -gt.idx) : T(0);
+    P.gy[sd][q] = oy[sd] != 0 ? (fy[sd] - f) * (oy[sd] > 0 ? gt.idy : -gt.idy) : T(0);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int sx = k & 1, sy = k >> 1;
+    const bool px = ox[sx] > 0, py = oy[sy] > 0;
+    const bool ud = py ? (px ? us[8] : us[6]) : (px ? us[2] : us[0]);
+    const T fd = py ? (px ? fn[8] : fn[6]) : (px ? fn[2] : fn[0]);
+    T v = T(0);
+    if (ox[sx] != 0 && oy[sy] != 0 && ud)
+      v = (fd - fx[sx] - fy[sy] + f) * ((px == py ? T(1) : T(-1)) * gt.idx * gt.idy);
+    P.gxy[k][q] = v;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -863,128 +841,121 @@ pl_params(PlGeom g, PlGeomT<T> gt, int recon, const ChCellT<double>* __restrict_
 // (whole, two particles or more).  One launch per level, coarsest first, so that
 // a coarser neighbour's record is complete when a finer cell reads it.
 // ---------------------------------------------------------------------------
-// The cell holding the centre of the level-L square (I, J) (integer
-// coordinates at level L, inside the domain): the point location of that
-// centre in integer form.  A centre never lies on the edge of a cell of level
-// L or coarser; where it is the common corner of finer cells, any of them
-// stands for "finer" (here the one the >= rule of the point location takes).
-__device__ __forceinline__ int leaf_at(const PlGeom& g, const PlTree* __restrict__ tr, int L, int I,
-                                       int J) {
-  const int c = (J >> (L - 1)) * g.nx + (I >> (L - 1));
-  if (tr->l2_first[4 * c] < 0) return tr->l1_first[c];
-  const int k = L == 1 ? 3 : ((((J >> (L - 2)) & 1) << 1) | ((I >> (L - 2)) & 1));
-  const int l = tr->l2_first[4 * c + k];
-  if (!tr->l2_ref[4 * c + k]) return l;
-  return L <= 2 ? l + 3 : l + (((J & 1) << 1) | (I & 1));
-}
+// What fills the eight squares of a cell's own size around it does not change,
+// so it is tabulated at creation (pg_neighbours): per cell and square the
+// kind (two low bits) and a cell: the one of that size, the first of the four
+// finer cells (consecutive in the cell numbering), or the coarser cell.
+enum : int { kNbNone = 0, kNbSame = 1, kNbFiner = 2, kNbCoarser = 3 };
 
+// Per-level constants of the refined stencils, formed once on the host.
 template <typename T>
-__device__ bool pl_region(const PlGeom& g, const PlTree* __restrict__ tr,
-                          const PlParams<T>* __restrict__ prm,
-                          const T* __restrict__ fT, const int* __restrict__ usable_c,
-                          const long long* __restrict__ off, int lvl, int ii, int jj, int di,
-                          int dj, double h, double k, T* val) {
-  const int I = ii + di, J = jj + dj;
-  if (I < 0 || J < 0 || I >= (g.nx << (lvl - 1)) || J >= (g.ny << (lvl - 1))) return false;
-  const int l = leaf_at(g, tr, lvl, I, J);
-  const int ll = tr->lvl[l];
-  if (ll == lvl) {
-    if (!usable_c[l]) return false;
-    for (int f = 0; f < kNF; ++f) val[f] = fT[(size_t)l * kNF + f];
-    return true;
+struct PlLevel {
+  int level;
+  double h, k;        // cell size
+  T ih, ik;           // (T)(1 / h), (T)(1 / k)
+};
+
+// value of field f over the square `nb` at offset (di, dj) of the cell (ii, jj);
+// false: not usable
+template <typename T>
+__device__ __forceinline__ bool
+pl_region(const PlGeom& g, int nb, const PlParams<T>* __restrict__ prm, const T* __restrict__ fT,
+          const int* __restrict__ usable_c, const long long* __restrict__ off,
+          const PlLevel<T>& lv, int ii, int jj, int di, int dj, int f, T& val) {
+  const int l = nb >> 2, kind = nb & 3;
+  if (kind == kNbSame) {
+    val = fT[(size_t)l * kNF + f];
+    return usable_c[l];
   }
-  if (ll > lvl) {
-    int q[4];
-    long long nq[4], ns = 0;
+  if (kind == kNbNone) return false;
+  if (kind == kNbFiner) {
+    T sum = T(0);
+    bool ok = true;
+    const long long n0 = off[l];
+    long long at = n0;
+#pragma unroll
     for (int a = 0; a < 4; ++a) {
-      q[a] = leaf_at(g, tr, lvl + 1, 2 * I + (a & 1), 2 * J + (a >> 1));
-      if (tr->lvl[q[a]] != lvl + 1 || !usable_c[q[a]]) return false;
-      nq[a] = off[q[a] + 1] - off[q[a]];
-      ns += nq[a];
+      const long long nx = off[l + a + 1];
+      ok = ok && usable_c[l + a];
+      sum += (T)(nx - at) * fT[(size_t)(l + a) * kNF + f];
+      at = nx;
     }
-    for (int f = 0; f < kNF; ++f) {
-      T sum = T(0);
-      for (int a = 0; a < 4; ++a) sum += (T)nq[a] * fT[(size_t)q[a] * kNF + f];
-      val[f] = sum / (T)ns;
-    }
-    return true;
+    val = sum / (T)(at - n0);
+    return ok;
   }
   if (!usable_c[l]) return false;
   const PlParams<T>& C = prm[l];
-  const double cx = rn_add(g.x0, rn_mul((double)I + 0.5, h));
-  const double cy = rn_add(g.y0, rn_mul((double)J + 0.5, k));
+  const double cx = rn_add(g.x0, rn_mul((double)(ii + di) + 0.5, lv.h));
+  const double cy = rn_add(g.y0, rn_mul((double)(jj + dj) + 0.5, lv.k));
   const T ex = (T)cx - C.xc, ey = (T)cy - C.yc;
   const int sx = ex >= T(0) ? 1 : 0, sy = ey >= T(0) ? 1 : 0;
-  for (int f = 0; f < kNF; ++f)
-    val[f] = C.F[f] + C.gx[sx][f] * ex + C.gy[sy][f] * ey + C.gxy[2 * sy + sx][f] * ex * ey;
+  val = C.F[f] + C.gx[sx][f] * ex + C.gy[sy][f] * ey + C.gxy[2 * sy + sx][f] * ex * ey;
   return true;
 }
 
-// blocks: the kParamBlock-cell blocks holding cells of this level
+// blocks: the kParamBlock-cell blocks holding cells of this level (the
+// records of the other levels belong to the other launches)
 template <typename T>
-__global__ void pl_params_amr(PlGeom g, const PlTree* __restrict__ tr, int recon, int level,
-                              const int* __restrict__ blocks,
-                              const ChCellT<double>* __restrict__ cells, const T* __restrict__ fT,
-                              const int* __restrict__ usable_c, const long long* __restrict__ off,
-                              PlParams<T>* __restrict__ prm, Species sp) {
-  __shared__ PlParams<T> buf[kParamBlock];
+__global__ void __launch_bounds__(kParamBlock * kPF)
+pl_params_amr(PlGeom g, PlGeomT<T> gt, const PlTree* __restrict__ tr, int recon, PlLevel<T> lv,
+              const int* __restrict__ blocks, const ChCellT<double>* __restrict__ cells,
+              const T* __restrict__ fT, const int* __restrict__ usable_c,
+              const long long* __restrict__ off, PlParams<T>* __restrict__ prm, Species sp) {
   const int c0 = blocks[blockIdx.x] * kParamBlock;
-  const int c = c0 + threadIdx.x;
-  const int nb = min(kParamBlock, g.ncell - c0);
-  if (c < g.ncell && tr->lvl[c] == level) {
-    const ChCellT<double>& cs = cells[c];
-    PlParams<T>& P = buf[threadIdx.x];
-    P.active = cs.active;
-    P.pad = 0;
-    P.alpha = (T)cs.alpha; P.nu_ref = (T)cs.nu_ref; P.B = (T)cs.B; P.mu_p = (T)cs.mu_p;
-    P.Pr = (T)cs.Pr; P.gtr = (T)cs.gtr; P.gtv = (T)cs.gtv; P.grv = (T)cs.grv;
-    P.R = (T)gasR(sp); P.theta = (T)sp.theta_v; P.dt = (T)g.dt;
-    const double sc = (double)(1 << (level - 1));
-    const double h = g.dx / sc, k = g.dy / sc;
-    const int ii = tr->lii[c], jj = tr->ljj[c];
-    P.xc = (T)rn_add(g.x0, rn_mul((double)ii + 0.5, h));
-    P.yc = (T)rn_add(g.y0, rn_mul((double)jj + 0.5, k));
-    const T* f = fT + (size_t)c * kNF;
-    for (int q = 0; q < kNF; ++q) P.F[q] = f[q];
-    const T ih = (T)(1.0 / h), ik = (T)(1.0 / k);
-    T PX[2][kNF], PY[2][kNF], PD[kNF];
-    int ox[2] = {0, 0}, oy[2] = {0, 0};
-    for (int sd = 0; sd < 2; ++sd) {
-      const int sg = sd ? 1 : -1;
-      if (recon) {
-        if (pl_region<T>(g, tr, prm, fT, usable_c, off, level, ii, jj, sg, 0, h, k, PX[sd]))
-          ox[sd] = sg;
-        else if (pl_region<T>(g, tr, prm, fT, usable_c, off, level, ii, jj, -sg, 0, h, k, PX[sd]))
-          ox[sd] = -sg;
-        if (pl_region<T>(g, tr, prm, fT, usable_c, off, level, ii, jj, 0, sg, h, k, PY[sd]))
-          oy[sd] = sg;
-        else if (pl_region<T>(g, tr, prm, fT, usable_c, off, level, ii, jj, 0, -sg, h, k, PY[sd]))
-          oy[sd] = -sg;
-      }
-      const T sx = ox[sd] > 0 ? ih : -ih, sy = oy[sd] > 0 ? ik : -ik;
-      for (int q = 0; q < kNF; ++q) {
-        P.gx[sd][q] = ox[sd] ? (PX[sd][q] - f[q]) * sx : T(0);
-        P.gy[sd][q] = oy[sd] ? (PY[sd][q] - f[q]) * sy : T(0);
-      }
-    }
-    for (int q = 0; q < 4; ++q) {
-      const int sx = q & 1, sy = q >> 1;
-      const bool d = ox[sx] && oy[sy] &&
-                     pl_region<T>(g, tr, prm, fT, usable_c, off, level, ii, jj, ox[sx], oy[sy], h,
-                                  k, PD);
-      const T s = (ox[sx] * oy[sy] > 0 ? T(1) : T(-1)) * ih * ik;
-      for (int m = 0; m < kNF; ++m)
-        P.gxy[q][m] = d ? (PD[m] - PX[sx][m] - PY[sy][m] + f[m]) * s : T(0);
-    }
+  if (threadIdx.x < kParamBlock) {
+    const int c = c0 + threadIdx.x;
+    if (c < g.ncell && tr->lvl[c] == lv.level)
+      pl_scalars<T>(prm[c], cells[c], gt, sp,
+                    rn_add(g.x0, rn_mul((double)tr->lii[c] + 0.5, lv.h)),
+                    rn_add(g.y0, rn_mul((double)tr->ljj[c] + 0.5, lv.k)));
   }
-  __syncthreads();
-  // copy out the records of this level only (the others belong to the other
-  // launches)
-  constexpr int kW = (int)(sizeof(PlParams<T>) / 8);
-  const unsigned long long* src = reinterpret_cast<const unsigned long long*>(buf);
-  unsigned long long* dst = reinterpret_cast<unsigned long long*>(prm + c0);
-  for (int w = threadIdx.x; w < nb * kW; w += kParamBlock)
-    if (tr->lvl[c0 + w / kW] == level) dst[w] = src[w];
+  const int c = c0 + threadIdx.x / kPF, q = threadIdx.x % kPF;
+  if (c >= g.ncell || q >= kNF || tr->lvl[c] != lv.level) return;
+  PlParams<T>& P = prm[c];
+  const int ii = tr->lii[c], jj = tr->ljj[c];
+  const int4* nb4 = reinterpret_cast<const int4*>(tr->nb + (size_t)c * 8);
+  const int4 na = nb4[0], nc = nb4[1];
+  const T f = fT[(size_t)c * kNF + q];
+  P.F[q] = f;
+  // the values and flags of the eight squares, (-1,-1) (0,-1) (1,-1) (-1,0)
+  // (1,0) (-1,1) (0,1) (1,1)
+  const int nb[8] = {na.x, na.y, na.z, na.w, nc.x, nc.y, nc.z, nc.w};
+  bool us[8];
+  T fn[8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    const int k = m < 4 ? m : m + 1, di = k % 3 - 1, dj = k / 3 - 1;
+    fn[m] = T(0);
+    us[m] = recon && pl_region<T>(g, nb[m], prm, fT, usable_c, off, lv, ii, jj, di, dj, q, fn[m]);
+  }
+  int ox[2], oy[2];
+  T fx[2], fy[2];
+#pragma unroll
+  for (int sd = 0; sd < 2; ++sd) {
+    const int hi = sd ? 1 : -1;
+    const bool xh = sd ? us[4] : us[3], xl = sd ? us[3] : us[4];
+    const bool yh = sd ? us[6] : us[1], yl = sd ? us[1] : us[6];
+    ox[sd] = xh ? hi : (xl ? -hi : 0);
+    oy[sd] = yh ? hi : (yl ? -hi : 0);
+    fx[sd] = ox[sd] > 0 ? fn[4] : fn[3];
+    fy[sd] = oy[sd] > 0 ? fn[6] : fn[1];
+    const T sx = ox[sd] > 0 ? lv.ih : -lv.ih, sy = oy[sd] > 0 ? lv.ik : -lv.ik;
+    P.gx[sd][q] = ox[sd] ? (fx[sd] - f) * sx : T(0);
+    P.gy[sd][q] = oy[sd] ? (fy[sd] - f) * sy : T(0);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int sx = k & 1, sy = k >> 1;
+    const bool px = ox[sx] > 0, py = oy[sy] > 0;
+    const bool ud = py ? (px ? us[7] : us[5]) : (px ? us[2] : us[0]);
+    const T fd = py ? (px ? fn[7] : fn[5]) : (px ? fn[2] : fn[0]);
+    T v = T(0);
+    if (ox[sx] && oy[sy] && ud) {
+      const T s = (px == py ? T(1) : T(-1)) * lv.ih * lv.ik;
+      v = (fd - fx[sx] - fy[sy] + f) * s;
+    }
+    P.gxy[k][q] = v;
+  }
 }
 
 // Asynchronous global -> shared copies of 4, 8 or 16 bytes (cp.async): the
@@ -1496,7 +1467,7 @@ struct PlaneCtx {
   PlCount* cnt;
   ChCellT<double>* cells;
   float* pend;              // FP32 copy of the pending rescale (Un, Us, s, r) per cell
-  void* fT;                 // cell fields in the particle precision (ncell x 13)
+  void* fT;                 // cell fields in the particle precision (ncell x kNF)
   int* usable_c;            // reconstruction-neighbour flag per cell
   void* prm;                // PlParams<T>
   ChSumsT<double>* sums;
@@ -1624,6 +1595,48 @@ int pg_leaf(const usp_plane* p, const PlGrid& G, double x, double y) {
   return l + 2 * (vy >= 1.0 ? 1 : 0) + (vx >= 1.0 ? 1 : 0);
 }
 
+// The neighbouring squares of every cell, as the stencil pass reads them (the
+// cell holding the square's centre decides; on a balanced grid a finer one
+// means that four consecutive cells of the next level fill the square, else
+// the square holds cells finer still and is never usable).
+void pg_neighbours(const usp_plane* p, const PlGrid& G, std::vector<int>& nb) {
+  const int nx = p->nx, ny = p->ny;
+  // the cell at the centre of the level-L square (I, J)
+  auto leaf_at = [&](int L, int I, int J) {
+    const int c = (J >> (L - 1)) * nx + (I >> (L - 1));
+    if (G.l2_first[(size_t)4 * c] < 0) return G.l1_first[c];
+    const int k = L == 1 ? 3 : ((((J >> (L - 2)) & 1) << 1) | ((I >> (L - 2)) & 1));
+    const int l = G.l2_first[(size_t)4 * c + k];
+    if (!G.l2_ref[(size_t)4 * c + k]) return l;
+    return L <= 2 ? l + 3 : l + (((J & 1) << 1) | (I & 1));
+  };
+  nb.assign((size_t)8 * G.nleaf, kNbNone);
+  for (int c = 0; c < G.nleaf; ++c) {
+    const int L = G.lvl[c];
+    for (int m = 0; m < 8; ++m) {
+      const int k = m < 4 ? m : m + 1;
+      const int I = G.lii[c] + k % 3 - 1, J = G.ljj[c] + k / 3 - 1;
+      if (I < 0 || J < 0 || I >= (nx << (L - 1)) || J >= (ny << (L - 1))) continue;
+      const int l = leaf_at(L, I, J);
+      int v = kNbNone;
+      if (G.lvl[l] == L) {
+        v = (l << 2) | kNbSame;
+      } else if (G.lvl[l] < L) {
+        v = (l << 2) | kNbCoarser;
+      } else {
+        int q[4];
+        bool all = true;
+        for (int a = 0; a < 4; ++a) {
+          q[a] = leaf_at(L + 1, 2 * I + (a & 1), 2 * J + (a >> 1));
+          all = all && G.lvl[q[a]] == L + 1 && q[a] == q[0] + a;
+        }
+        if (all) v = (q[0] << 2) | kNbFiner;
+      }
+      nb[(size_t)8 * c + m] = v;
+    }
+  }
+}
+
 // sizes and refinement parameters of a plane; 0 or USP_EINVAL
 int pg_check(const usp_plane* p) {
   if (!p || p->nx <= 0 || p->ny <= 0 || (long long)p->nx * p->ny >= (1 << 24) ||
@@ -1701,15 +1714,18 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
     ch_coeffs<<<tb, kBlk, 0, s>>>(ncell, h->Fnum, h->vol, h->afv, h->g.dt, h->cells, env.sp,
                                   env.flags, env.counters);
   if (fpm || h->levels < 2)
-    pl_params<T><<<(ncell + kStencilBlock<T> - 1) / kStencilBlock<T>, kStencilBlock<T>, 0, s>>>(
+    pl_params<T><<<(ncell + kParamBlock - 1) / kParamBlock, kParamBlock * kPF, 0, s>>>(
         h->g, gt, fpm ? 0 : h->recon, h->cells, (const T*)h->fT, h->usable_c,
         (PlParams<T>*)h->prm, env.sp, h->fpmrec);
   else
     for (int L = 1; L <= h->levels; ++L)
-      if (h->nblk_lv[L] > 0)
-        pl_params_amr<T><<<h->nblk_lv[L], kParamBlock, 0, s>>>(
-            h->g, h->tree, h->recon, L, h->blk_lv + h->blk_off[L], h->cells, (const T*)h->fT,
-            h->usable_c, h->off, (PlParams<T>*)h->prm, env.sp);
+      if (h->nblk_lv[L] > 0) {
+        const double sc = (double)(1 << (L - 1)), lh = h->g.dx / sc, lk = h->g.dy / sc;
+        pl_params_amr<T><<<h->nblk_lv[L], kParamBlock * kPF, 0, s>>>(
+            h->g, gt, h->tree, h->recon, PlLevel<T>{L, lh, lk, (T)(1.0 / lh), (T)(1.0 / lk)},
+            h->blk_lv + h->blk_off[L], h->cells, (const T*)h->fT, h->usable_c, h->off,
+            (PlParams<T>*)h->prm, env.sp);
+      }
   CHK(cudaGetLastError());
   if (prof) prof(env.owner, 1, 0);
   if (prof) prof(env.owner, 0, 1);
@@ -1879,6 +1895,7 @@ int pl_create(PlaneCtx** out, const ChEnv& env, const usp_plane* pp, double dt,
     t.lvl = (const int*)A(sizeof(int) * ncell);
     t.lii = (const int*)A(sizeof(int) * ncell);
     t.ljj = (const int*)A(sizeof(int) * ncell);
+    t.nb = (const int*)A(sizeof(int) * 8 * (size_t)ncell);
     h->tree = (PlTree*)A(sizeof(PlTree));
   }
   // per level the stencil blocks (kParamBlock consecutive cells) holding its cells
@@ -1914,7 +1931,7 @@ int pl_create(PlaneCtx** out, const ChEnv& env, const usp_plane* pp, double dt,
   bool ok = h->keycell && h->bh && h->tot && h->face_off && h->off && h->af && h->afv && h->cnt &&
             (env.sp.method != 1 || h->fpmrec) &&
             (G.levels < 2 || (h->htree.l1_first && h->htree.l2_first && h->htree.l2_ref &&
-                               h->htree.lvl && h->htree.lii && h->htree.ljj && h->blk_lv &&
+                               h->htree.lvl && h->htree.lii && h->htree.ljj && h->htree.nb && h->blk_lv &&
                                h->tree)) &&
             h->cells && h->pend && h->fT && h->usable_c && h->prm && h->sums && h->acc && h->macc && h->mout && h->dstep;
   for (int k = 0; k < 2; ++k) {
@@ -1970,6 +1987,8 @@ int pl_create(PlaneCtx** out, const ChEnv& env, const usp_plane* pp, double dt,
   cok = cok && cudaMemcpyAsync(h->af, area_frac, sizeof(double) * ncell, cudaMemcpyHostToDevice,
                                s) == cudaSuccess;
   std::vector<double> afv;
+  std::vector<int> nbs;
+  if (G.levels >= 2) pg_neighbours(pp, G, nbs);
   if (G.levels >= 2) {
     // the grid tables and the volume factor af / 4^(level-1) of every cell
     afv.resize(ncell);
@@ -1989,6 +2008,7 @@ int pl_create(PlaneCtx** out, const ChEnv& env, const usp_plane* pp, double dt,
     cok = cok && up(t.lvl, G.lvl.data(), sizeof(int) * ncell);
     cok = cok && up(t.lii, G.lii.data(), sizeof(int) * ncell);
     cok = cok && up(t.ljj, G.ljj.data(), sizeof(int) * ncell);
+    cok = cok && up(t.nb, nbs.data(), sizeof(int) * nbs.size());
     cok = cok && up(h->tree, &h->htree, sizeof(PlTree));
     if (!blk.empty()) cok = cok && up(h->blk_lv, blk.data(), sizeof(int) * blk.size());
   }

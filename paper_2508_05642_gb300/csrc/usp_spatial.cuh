@@ -17,7 +17,7 @@ namespace {
 
 using namespace usp;
 
-constexpr int kNF = 13;            // U(3), T_tr, T_rot, T_vib, Pi(6)
+constexpr int kNF = 12;            // U(3), T_tr, T_rot, T_vib, Pi(6)
 constexpr int kRB = 256;           // radix block
 constexpr int kRPT = 16;           // keys per thread per radix block
 constexpr int kChunk = kRB * kRPT;
@@ -625,7 +625,7 @@ moments_of_cells(long long first, long long stride, long long ny, int cpw,
     cs.Trot = se * (inv * sp.iR);
     cs.ebar = (double)kl * inv;
     cs.Tvib = vib_state(sp, cs.ebar).Tvib;
-    if (fT) {   // the 13 fields in the particle precision, for the stencils
+    if (fT) {   // the fields in the particle precision, for the stencils
       T* o = fT + (size_t)c * kNF;
       for (int i = 0; i < 3; ++i) o[i] = (T)cs.U[i];
       o[3] = (T)cs.Ttr; o[4] = (T)cs.Trot; o[5] = (T)cs.Tvib;
@@ -836,7 +836,7 @@ ch_moments_coeffs_f32(int ncell, const long long* __restrict__ off,
     cs.Trot = Trot;
     cs.ebar = ebar;
     cs.Tvib = Tvib;
-    float* o = fT + (size_t)c * kNF;   // the 13 fields for the stencils
+    float* o = fT + (size_t)c * kNF;   // the fields for the stencils
     o[0] = U0; o[1] = U1; o[2] = U2;
     o[3] = Ttr; o[4] = Trot; o[5] = Tvib;
     for (int i = 0; i < 6; ++i) o[6 + i] = P[i];
