@@ -960,6 +960,54 @@ __host__ __device__ inline void guide_part(const float* T, uint8_t* __restrict__
   }
 }
 
+// The tables of cell c with parameters p_nb, p_b and levels up to maxI, by the
+// kJT threads of a block.
+// The rows are built in shared memory (one word of padding each: the threads
+// build one row each, entry by entry), copied out coalesced, and the
+// guides read them there.
+typedef float JumpRows[2][kJR][kJK + 1];
+template <typename F>
+__device__ __forceinline__ void build_tables(int c, F p_nb, F p_b, int maxI, JumpRows& rs,
+                                             float* __restrict__ tab_nb,
+                                             float* __restrict__ tab_b,
+                                             uint8_t* __restrict__ gd_nb,
+                                             uint8_t* __restrict__ gd_b) {
+  const int j = threadIdx.x;
+  const int rows = min(kJR, maxI + 1);
+  F pb = p_b;
+  if (pb > F(0.5) && pb < F(1)) pb = rn_sub(F(1), pb);
+  if (j < kJR) {
+    if (nb_row_used(j, rows, p_nb)) nb_row(j + 1, p_nb, rs[0][j]);
+  } else if (j < 2 * kJR) {
+    const int n = j - kJR;
+    if (b_row_used(n, rows, p_b)) b_row(n, pb, rs[1][n]);
+  }
+  __syncthreads();
+  for (int e = j; e < 2 * kJR * kJK; e += kJT) {
+    const int t = e / (kJR * kJK), row = (e / kJK) % kJR, k = e % kJK;
+    if (t == 0 ? nb_row_used(row, rows, p_nb) : b_row_used(row, rows, p_b))
+      (t == 0 ? tab_nb : tab_b)[((size_t)c * kJR + row) * kJK + k] = rs[t][row][k];
+  }
+  static_assert(2 * kJR * kGP == kJT, "one guide part per thread");
+  const int row = j / kGP, q = j % kGP;      // 2 kJR rows, kGP parts each
+  if (row < kJR) {
+    uint8_t* g = gd_nb + ((size_t)c * kJR + row) * kGB;
+    if (nb_row_used(row, rows, p_nb))
+      guide_part(rs[0][row], g, q, -1);
+    else if (row < rows)
+      guide_fill(g, q, 0x80u);              // p_NB >= 1: no jump up
+  } else {
+    const int n = row - kJR;
+    uint8_t* g = gd_b + ((size_t)c * kJR + n) * kGB;
+    if (b_row_used(n, rows, p_b))
+      guide_part(rs[1][n], g, q, p_b > F(0.5) ? n : -1);
+    else if (n < rows)
+      // n = 0 or p_B <= 0: no jump down; p_B = 1: n; p_B > 1: the general
+      // path, which flags the clamp
+      guide_fill(g, q, n >= 1 && p_b >= F(1) ? (p_b > F(1) ? 0x7fu : 0x80u | (uint32_t)n) : 0x80u);
+  }
+}
+
 template <typename F>
 __global__ void __launch_bounds__(kJT)
 jumptable_kernel(int c0, int c1, const CollideParams<F>* __restrict__ prm,
@@ -967,48 +1015,11 @@ jumptable_kernel(int c0, int c1, const CollideParams<F>* __restrict__ prm,
                  float* __restrict__ tab_b, uint8_t* __restrict__ gd_nb,
                  uint8_t* __restrict__ gd_b) {
   const int c = c0 + blockIdx.x;
-  const int j = threadIdx.x;
   if (c >= c1) return;                       // uniform over the block
   const CollideParams<F>& P = prm[c];
   if (!P.active) return;                     // uniform over the block
-  // the rows are built in shared memory (one word of padding each: the threads
-  // build one row each, entry by entry), copied out coalesced, and the
-  // guides read them there
-  __shared__ float rs[2][kJR][kJK + 1];
-  const int rows = min(kJR, cells[c].maxI + 1);
-  F pb = P.p_b;
-  if (pb > F(0.5) && pb < F(1)) pb = rn_sub(F(1), pb);
-  if (j < kJR) {
-    if (nb_row_used(j, rows, P.p_nb)) nb_row(j + 1, P.p_nb, rs[0][j]);
-  } else if (j < 2 * kJR) {
-    const int n = j - kJR;
-    if (b_row_used(n, rows, P.p_b)) b_row(n, pb, rs[1][n]);
-  }
-  __syncthreads();
-  for (int e = j; e < 2 * kJR * kJK; e += kJT) {
-    const int t = e / (kJR * kJK), row = (e / kJK) % kJR, k = e % kJK;
-    if (t == 0 ? nb_row_used(row, rows, P.p_nb) : b_row_used(row, rows, P.p_b))
-      (t == 0 ? tab_nb : tab_b)[((size_t)c * kJR + row) * kJK + k] = rs[t][row][k];
-  }
-  static_assert(2 * kJR * kGP == kJT, "one guide part per thread");
-  const int row = j / kGP, q = j % kGP;      // 2 kJR rows, kGP parts each
-  if (row < kJR) {
-    uint8_t* g = gd_nb + ((size_t)c * kJR + row) * kGB;
-    if (nb_row_used(row, rows, P.p_nb))
-      guide_part(rs[0][row], g, q, -1);
-    else if (row < rows)
-      guide_fill(g, q, 0x80u);              // p_NB >= 1: no jump up
-  } else {
-    const int n = row - kJR;
-    uint8_t* g = gd_b + ((size_t)c * kJR + n) * kGB;
-    const F p = P.p_b;
-    if (b_row_used(n, rows, p))
-      guide_part(rs[1][n], g, q, p > F(0.5) ? n : -1);
-    else if (n < rows)
-      // n = 0 or p_B <= 0: no jump down; p_B = 1: n; p_B > 1: the general
-      // path, which flags the clamp
-      guide_fill(g, q, n >= 1 && p >= F(1) ? (p > F(1) ? 0x7fu : 0x80u | (uint32_t)n) : 0x80u);
-  }
+  __shared__ JumpRows rs;
+  build_tables<F>(c, P.p_nb, P.p_b, cells[c].maxI, rs, tab_nb, tab_b, gd_nb, gd_b);
 }
 
 // ---------------------------------------------------------------------------
@@ -1150,16 +1161,12 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 // acceptance of draw j is decided exactly as in the one-at-a-time loop: a
 // decrement on particle k is accepted iff fewer than lev[k] earlier accepted
 // decrements in the round hit k.  The net level change goes to sums[c].net.
-__global__ void __launch_bounds__(128, 8)
-levelfix_kernel(Species sp, int c0, int c1, const CellState* __restrict__ cells,
-                                CellSums* __restrict__ sums, int* __restrict__ lev,
-                                uint32_t* flags, unsigned long long* counters, uint32_t k0,
-                                uint32_t k1) {
+// Returns the net change (every lane).
+__device__ __forceinline__ long long
+level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long sumI,
+               int* __restrict__ lev, uint32_t* flags, unsigned long long* counters, uint32_t k0,
+               uint32_t k1) {
   const int lane = threadIdx.x & 31;
-  const int c = c0 + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (c >= c1) return;
-  const CellState& cs = cells[c];
-  if (!cs.active) return;
   const double Rth = gasR(sp) * sp.theta_v;
   const long long N = cs.N;
   const unsigned int step = cs.step;
@@ -1167,7 +1174,7 @@ levelfix_kernel(Species sp, int c0, int c1, const CellState* __restrict__ cells,
   if (lane == 0) {
     const U4 w = philox4x32_10((uint32_t)c, step, CTAG_IDELTA, 0u, k0, k1);
     const double u = uniform_open<double>(w.x);
-    Id = (long long)floor((double)N * cs.e_vib_tgt / Rth - (double)(long long)sums[c].I + u);
+    Id = (long long)floor((double)N * cs.e_vib_tgt / Rth - (double)(long long)sumI + u);
   }
   Id = __shfl_sync(0xffffffffu, Id, 0);
   long long remaining = Id, draws = 0;
@@ -1259,10 +1266,24 @@ levelfix_kernel(Species sp, int c0, int c1, const CellState* __restrict__ cells,
       }
     }
   }
-  if (lane != 0) return;
-  if (remaining != 0) atomicOr(flags, (uint32_t)F_VIB_LOOP_CAP);
-  if (draws) atomicAdd(&counters[C_VIB_DRAWS], (unsigned long long)draws);
-  sums[c].net = net;
+  if (lane == 0) {
+    if (remaining != 0) atomicOr(flags, (uint32_t)F_VIB_LOOP_CAP);
+    if (draws) atomicAdd(&counters[C_VIB_DRAWS], (unsigned long long)draws);
+  }
+  return net;
+}
+
+__global__ void __launch_bounds__(128, 8)
+levelfix_kernel(Species sp, int c0, int c1, const CellState* __restrict__ cells,
+                CellSums* __restrict__ sums, int* __restrict__ lev, uint32_t* flags,
+                unsigned long long* counters, uint32_t k0, uint32_t k1) {
+  const int lane = threadIdx.x & 31;
+  const int c = c0 + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (c >= c1) return;
+  const CellState& cs = cells[c];
+  if (!cs.active) return;
+  const long long net = level_fix_cell(sp, c, cs, sums[c].I, lev, flags, counters, k0, k1);
+  if (lane == 0) sums[c].net = net;
 }
 
 // Rotational and velocity rescale factors of Sec. 4.C, the moments of the
@@ -1329,6 +1350,152 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
   CellSums z;
   memset(&z, 0, sizeof(z));
   sums[c] = z;
+}
+
+// ---------------------------------------------------------------------------
+// The per-cell passes of a step in one kernel, for contexts of at most
+// kFewCells cells and the USP-FPM method: one block per cell.  A cell's update is some 400
+// FP64 operations in a row, 64 cycles each (usp_math.cuh); here its
+// independent parts run on different warps, which sit on different quarters
+// of the SM, the level correction runs beside the sums' part, and the jump
+// tables follow in the same block.  With more cells than SMs one thread per
+// cell (cellupdate_kernel) is the better split: its instructions serve 32
+// cells.  One cell of 20,000 particles, FP32: the three kernels took 54 us a
+// step at first (37 the update with the library's functions).
+// ---------------------------------------------------------------------------
+constexpr int kFewCells = 152;
+
+template <typename T>
+__global__ void __launch_bounds__(kJT)
+few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
+                 CollideParams<T>* __restrict__ prm, CellSums* __restrict__ sums,
+                 int* __restrict__ lev, uint32_t* flags, unsigned long long* counters, uint32_t k0,
+                 uint32_t k1, float* __restrict__ tab_nb, float* __restrict__ tab_b,
+                 uint8_t* __restrict__ gd_nb, uint8_t* __restrict__ gd_b) {
+  __shared__ JumpRows rs;
+  __shared__ CellState cs;
+  __shared__ CellSums S;
+  __shared__ CellCoeffs K;
+  __shared__ DriftDiff dd;
+  __shared__ VibState vib;
+  __shared__ CollideParams<T> P;
+  __shared__ double xw, invN, er_star, e_rot_new, etr_star, e_n, m[3], Ps[6];
+  __shared__ int clamps;
+  const int c = c0 + blockIdx.x, t = threadIdx.x, w = t >> 5;
+  if (!cells[c].active) return;                                   // uniform over the block
+  for (int i = t; i < (int)(sizeof(CellState) / 4); i += kJT)
+    reinterpret_cast<uint32_t*>(&cs)[i] = reinterpret_cast<const uint32_t*>(&cells[c])[i];
+  for (int i = t; i < (int)(sizeof(CellSums) / 4); i += kJT)
+    reinterpret_cast<uint32_t*>(&S)[i] = reinterpret_cast<const uint32_t*>(&sums[c])[i];
+  __syncthreads();
+  const double R = sp.R, Rth = R * sp.theta_v;
+  const bool lead = (t & 31) == 0;
+  // the +-1 correction | the sums' part of cellupdate_kernel
+  if (w == 0) {
+    const long long net = level_fix_cell(sp, c, cs, S.I, lev, flags, counters, k0, k1);
+    if (lead) S.net = net;
+  } else if (t == 32) {
+    const double in = d_rcp((double)cs.N);
+    er_star = S.v[9] * in;
+    cs.r = er_star > 0.0 ? d_div(cs.e_rot_tgt, er_star) : 1.0;
+    e_rot_new = cs.r * er_star;
+    invN = in;
+  } else if (t == 64) {
+    const double in = d_rcp((double)cs.N);
+    const double m0 = S.v[0] * in, m1 = S.v[1] * in, m2 = S.v[2] * in;
+    m[0] = m0; m[1] = m1; m[2] = m2;
+    Ps[0] = S.v[3] * in - m0 * m0;
+    Ps[1] = S.v[4] * in - m1 * m1;
+    Ps[2] = S.v[5] * in - m2 * m2;
+    Ps[3] = S.v[6] * in - m0 * m1;
+    Ps[4] = S.v[7] * in - m0 * m2;
+    Ps[5] = S.v[8] * in - m1 * m2;
+    etr_star = 0.5 * (Ps[0] + Ps[1] + Ps[2]);
+  } else if (t == 96) {
+    e_n = 0.5 * (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]) + R * cs.Trot + Rth * cs.ebar;
+  }
+  __syncthreads();
+  // temperatures, viscosity, relaxation times | the vibrational state
+  const double sumI = (double)((long long)S.I + S.net);
+  if (t == 0) {
+    const double rad = d_div(e_n - e_rot_new - Rth * sumI * invN, etr_star);
+    double Un[3] = {cs.U[0], cs.U[1], cs.U[2]}, sc = 1.0;
+    const double Us[3] = {cs.U[0] + m[0], cs.U[1] + m[1], cs.U[2] + m[2]};
+    if (!(etr_star > 0.0) || !(rad > 0.0)) {
+      atomicOr(flags, (uint32_t)F_NEG_RADICAND);
+      atomicAdd(&counters[C_NEG_RADICAND], 1ull);
+      for (int i = 0; i < 3; ++i) Un[i] = Us[i];
+    } else {
+      sc = d_sqrt(rad);
+    }
+    for (int i = 0; i < 3; ++i) { cs.U[i] = Un[i]; cs.Us[i] = Us[i]; }
+    for (int i = 0; i < 6; ++i) cs.Pi[i] = sc * sc * Ps[i];
+    cs.Ttr = (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]) * (sp.iR * (1.0 / 3.0));
+    cs.Trot = e_rot_new * sp.iR;
+    cs.s = sc;
+    cs.step += 1;
+    cs.maxI = S.maxI + 1;
+    cell_mu_p<double>(sp, cs.ndens, cs.Ttr, sp.omega, K.mu_p, xw);
+  } else if (t == 32) {
+    cs.ebar = sumI * invN;
+    vib = vib_state(sp, cs.ebar);
+    K.Pr = cell_prandtl(vib);
+  }
+  __syncthreads();
+  // A, B, alpha | the gamma coefficients and targets
+  if (t == 0) {
+    cell_alpha<double>(K, cs.dt);
+  } else if (t == 32) {
+    cell_gammas<double>(sp, K, sp.omega, sp.Z_rot, cs.dt, cs.Ttr, cs.Trot, vib, xw);
+  }
+  __syncthreads();
+  if (!K.ok) {                                                    // uniform over the block
+    if (t == 0) {
+      atomicOr(flags, (uint32_t)F_A_NONPOS);
+      cs.active = 0;
+    }
+  } else if (t == 0) {
+    cs.e_rot_tgt = K.e_rot_tgt;
+    cs.e_vib_tgt = K.e_vib_tgt;
+    dd = drift_diffusion(sp, K, cs.dt, cs.Pi, cs.Ttr, cs.Trot, vib);
+    clamps = (K.tgt_clamped ? 1 : 0) + (dd.clamped ? 1 : 0);
+    if (clamps) {
+      atomicOr(flags, (uint32_t)F_TREL_CLAMP);
+      atomicAdd(&counters[C_TREL_CLAMP], (unsigned long long)clamps);
+    }
+    if (dd.fixed) atomicAdd(&counters[C_CHOL_FIX], 1ull);
+    if (dd.nu_zero) atomicAdd(&counters[C_NU_ZERO], 1ull);
+    if (dd.failed) atomicOr(flags, (uint32_t)F_CHOL_FAIL_AFTER_FIX);
+  }
+  __syncthreads();
+  // the particle pass's record, its parts on four warps
+  if (t == 0) {
+    P.step = cs.step; P.pid0 = cs.pid0; P.off = cs.off; P.count = (int)cs.N;
+    P.active = cs.active; P.method = sp.method; P.pad_ = 0;
+    for (int i = 0; i < 3; ++i) { P.U[i] = (T)cs.U[i]; P.Us[i] = (T)cs.Us[i]; }
+  } else if (K.ok && t == 32) {
+    const double a = dd.alpha, sq = sqrt_fast(1.0 - a * a);
+    P.as = (T)(a * cs.s);
+    for (int i = 0; i < 6; ++i) P.Lp[i] = (T)(sq * dd.L[i]);
+  } else if (K.ok && t == 64) {
+    const double a = dd.alpha, arot = R * dd.Trot_rel * (1.0 - a * a) / 2.0;
+    P.ar = (T)(a * sqrt_fast(cs.r));
+    P.a_rot = (T)arot;
+    P.sqrt_a = (T)sqrt_fast(arot);
+  } else if (K.ok && t == 96) {
+    const double oma2 = 1.0 - dd.alpha * dd.alpha, eb = dd.evib_rel * sp.iRtheta;
+    P.p_nb = (T)d_rcp(1.0 + eb * oma2);
+    P.p_b = (T)((1.0 + eb) * oma2);
+  }
+  __syncthreads();
+  for (int i = t; i < (int)(sizeof(CellState) / 4); i += kJT)
+    reinterpret_cast<uint32_t*>(&cells[c])[i] = reinterpret_cast<const uint32_t*>(&cs)[i];
+  for (int i = t; i < (int)(sizeof(CollideParams<T>) / 4); i += kJT)
+    reinterpret_cast<uint32_t*>(&prm[c])[i] = reinterpret_cast<const uint32_t*>(&P)[i];
+  for (int i = t; i < (int)(sizeof(CellSums) / 4); i += kJT)
+    reinterpret_cast<uint32_t*>(&sums[c])[i] = 0u;
+  if (tab_nb && K.ok)
+    build_tables<T>(c, P.p_nb, P.p_b, cs.maxI, rs, tab_nb, tab_b, gd_nb, gd_b);
 }
 
 // ---------------------------------------------------------------------------
@@ -1794,7 +1961,11 @@ int make_tiles(usp_ctx* c, int tile, Tile** out, int* nout, std::vector<int>& fi
 int build_tiles(usp_ctx* c, int tile) {
   int rc = make_tiles(c, tile, &c->tiles, &c->ntiles, c->h_tfirst);
   if (rc) return rc;
-  rc = make_tiles(c, std::min(tile, kWT), &c->wtiles, &c->nwtiles, c->h_wfirst);
+  // An FP64 state of few particles is cut into tiles of one particle per lane,
+  // so that its warps cover every quarter of every SM, each with half an FP64
+  // lane per clock (an FP32 state keeps its tiles: its sums are FP32 per warp)
+  const bool fine = c->precision == USP_FP64 && c->nparticles <= 152ll * 4 * 32 * 4;
+  rc = make_tiles(c, std::min(tile, fine ? 32 : kWT), &c->wtiles, &c->nwtiles, c->h_wfirst);
   if (rc) return rc;
   c->tile = tile;
   return USP_OK;
@@ -1916,6 +2087,7 @@ int launch_collide(usp_ctx* c, int warp_tiles, int minb, int grid, void* cx, voi
 }
 
 bool has_tables(const usp_ctx* c) { return c->tab_nb && c->sp.method == 0; }
+bool few_cells(const usp_ctx* c) { return c->ncell <= kFewCells && c->sp.method == 0; }
 
 // jump tables for the coming step
 template <typename T>
@@ -1949,6 +2121,14 @@ int launch_step(usp_ctx* c, const CellRange& r) {
   if ((rc = prof_end(c, e1))) return rc;
   if ((rc = prof_begin(c, 1, &e1))) return rc;
   const int n = r.c1 - r.c0;
+  if (few_cells(c)) {
+    const bool tab = has_tables(c);
+    few_cells_kernel<T><<<n, kJT, 0, c->stream>>>(
+        c->sp, r.c0, c->cells, (CollideParams<T>*)c->prm, c->sums, c->lev, c->flags, c->counters,
+        key0(c), key1(c), tab ? c->tab_nb : nullptr, c->tab_b, c->gd_nb, c->gd_b);
+    CK(cudaGetLastError());
+    return prof_end(c, e1);
+  }
   const int warps_per_block = 4;
   const int blocks = (n + warps_per_block - 1) / warps_per_block;
   levelfix_kernel<<<blocks, 32 * warps_per_block, 0, c->stream>>>(
@@ -1965,7 +2145,7 @@ int launch_step(usp_ctx* c, const CellRange& r) {
 int kernels_per_step(const usp_ctx* c) {
   if (c->kind == 1) return ch_kernels_per_step(c->ch);
   if (c->kind == 2) return pl_kernels_per_step(c->pl);
-  return has_tables(c) ? 4 : 3;
+  return few_cells(c) ? 2 : has_tables(c) ? 4 : 3;
 }
 
 int step_once(usp_ctx* c) {
@@ -1973,6 +2153,14 @@ int step_once(usp_ctx* c) {
   if (c->kind == 2) return pl_launch_step(c->pl, make_env(c), c->profiling ? prof_cb : nullptr);
   return c->precision == USP_FP32 ? launch_step<float>(c, all_cells(c))
                                   : launch_step<double>(c, all_cells(c));
+}
+
+// Blocks of the FP32 moments passes: the particle pass's grid, for warp tiles
+// no more than would hold one tile per warp.  A block's tiles of a cell are one
+// FP32 partial sum, so this is part of the result.
+int moments_grid(const usp_ctx* c) {
+  return c->warp_tiles ? std::max(1, std::min(c->grid_collide, (c->nwtiles + kWarps - 1) / kWarps))
+                       : c->grid_collide;
 }
 
 // moments of the cells of r (pending rescale applied) into mout
@@ -1995,7 +2183,7 @@ int compute_moments(usp_ctx* c, double* levsum, const CellRange& r) {
   } else {
   if (r.t1 > r.t0) {
     for (int pass = 0; pass < 2; ++pass) {
-      moments_kernel<T><<<c->grid_collide, kBlock, 0, c->stream>>>(
+      moments_kernel<T><<<moments_grid(c), kBlock, 0, c->stream>>>(
           pass, c->tiles + r.t0, r.t1 - r.t0, c->cells, (const T*)c->cx, (const T*)c->cy,
           (const T*)c->cz, (const T*)c->er, c->lev, c->macc);
       CK(cudaGetLastError());
@@ -2495,7 +2683,7 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
   if (rc) return fail(rc);
   {
     // persistent grid per design and register-budget variant: as many
-    // resident blocks as the SMs hold (warp-tiled: no more warps than tiles)
+    // resident blocks as the SMs hold, no more than tiles
     const bool f32 = c->precision == USP_FP32;
     for (int wt = 0; wt < 2; ++wt) {
       const size_t smem = f32 ? collide_smem<float>(wt) : collide_smem<double>(wt);
@@ -2507,7 +2695,8 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
                 cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, smem) != cudaSuccess)
           return fail(USP_ECUDA);
-        const int units = wt ? (c->nwtiles + kWarps - 1) / kWarps : c->ntiles;
+        // (few tiles go one to a block, on all SMs, before a block gets a second)
+        const int units = wt ? c->nwtiles : c->ntiles;
         c->grid_by_minb[wt][mb] = std::max(1, std::min(units, sm_count() * std::max(1, per_sm)));
       }
     }
