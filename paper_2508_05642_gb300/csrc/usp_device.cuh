@@ -921,14 +921,15 @@ __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const 
 // round-to-nearest one in the working precision, so the outcome is a fixed
 // function of (I, lam_up, lam_dn, the draws) up to the logarithm.
 constexpr int kGillespieCap = 4096;
+// the level, or its complement where the cap was met; k0, k1: the key
 template <typename T>
-__device__ __forceinline__ int gillespie(int I, T lu, T ld, uint32_t pid, uint32_t step,
-                                         const PhiloxRoundKeys& rk, uint32_t& fl) {
+__device__ __noinline__ int gillespie_exact(int I, T lu, T ld, uint32_t pid, uint32_t step,
+                                            uint32_t k0, uint32_t k1) {
   T t = T(0);
   U4 w = {0u, 0u, 0u, 0u};
 #pragma unroll 1
   for (int ev = 0; ev < kGillespieCap; ++ev) {
-    if ((ev & 1) == 0) w = philox4x32_10(pid, step, PTAG_GILLESPIE, (uint32_t)(ev >> 1), rk);
+    if ((ev & 1) == 0) w = philox4x32_10(pid, step, PTAG_GILLESPIE, (uint32_t)(ev >> 1), k0, k1);
     const T u1 = uniform_open<T>((ev & 1) ? w.z : w.x);
     const T u2 = uniform_open<T>((ev & 1) ? w.w : w.y);
     const T up = rn_mul(lu, rn_i2f(I + 1, T(0))), dn = rn_mul(ld, rn_i2f(I, T(0)));
@@ -938,8 +939,58 @@ __device__ __forceinline__ int gillespie(int I, T lu, T ld, uint32_t pid, uint32
     if (t > T(1)) return I;
     I += (u2 < rn_div(up, rate)) ? 1 : -1;
   }
-  fl |= F_SAMPLER_CAP;
-  return I;
+  return ~I;
+}
+
+// The same outcome from FP32 estimates.  What the method decides -- is the
+// step over, does the level rise -- is almost always clear of rounding: the
+// time is summed with the hardware's logarithm and reciprocal together with
+// a bound on its error (a relative 1e-6 of each waiting time, and an absolute
+// error of 1e-6 of each logarithm, over the rate), the branch is compared
+// without its division, and a particle for which either falls within its
+// bound (about one in 10^5), or whose rates are no ordinary numbers, or that makes 64
+// transitions, goes through gillespie_exact from the start.  A particle makes
+// a few transitions a step and a warp waits for its busiest one, so their
+// cost was the pass: a logarithm, two divisions and half a Philox block
+// each (FP64 form: some 60 FP64 operations, none now).
+__device__ __forceinline__ float uniform_estimate(uint32_t x, float) {
+  return uniform_open<float>(x);
+}
+__device__ __forceinline__ float uniform_estimate(uint32_t x, double) {
+  return fmaf((float)x, 0x1p-32f, 0x1p-33f);
+}
+template <typename T>
+__device__ __forceinline__ int gillespie(int I, T lu, T ld, uint32_t pid, uint32_t step,
+                                         const PhiloxRoundKeys& rk, uint32_t& fl) {
+  const float fu = (float)lu, fd = (float)ld;
+  float t = 0.0f, err = 1e-6f;
+  int J = I;
+  U4 w = {0u, 0u, 0u, 0u};
+#pragma unroll 1
+  for (int ev = 0; ev < 64; ++ev) {
+    if ((ev & 1) == 0) w = philox4x32_10(pid, step, PTAG_GILLESPIE, (uint32_t)(ev >> 1), rk);
+    const float u1 = uniform_estimate((ev & 1) ? w.z : w.x, T(0));
+    const float u2 = uniform_estimate((ev & 1) ? w.w : w.y, T(0));
+    const float up = rn_mul(fu, (float)(J + 1)), rate = rn_add(up, rn_mul(fd, (float)J));
+    if (!(rate > 1e-30f && rate < 1e30f)) break;
+    float l2, inv;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l2) : "f"(u1));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(rate));
+    const float x = -0.693147180559945f * l2 * inv;
+    t += x;
+    err = fmaf(1e-6f, x + inv, err);
+    if (!(fabsf(t - 1.0f) > err)) break;
+    if (t > 1.0f) return J;
+    const float d = fmaf(u2, rate, -up);
+    if (!(fabsf(d) > 2e-6f * rate)) break;
+    J += d < 0.0f ? 1 : -1;
+  }
+  J = gillespie_exact<T>(I, lu, ld, pid, step, rk.k0[0], rk.k1[0]);
+  if (J < 0) {
+    fl |= F_SAMPLER_CAP;
+    J = ~J;
+  }
+  return J;
 }
 
 struct DriftDiff {
