@@ -307,8 +307,7 @@ __global__ void __launch_bounds__(kBlk, 3) pl_advect(PlGeom g, PlGeomT<T> gt,
                           T* __restrict__ x, T* __restrict__ y, T* __restrict__ cx,
                           T* __restrict__ cy, T* __restrict__ cz, T* __restrict__ er,
                           int* __restrict__ lev, const uint32_t* __restrict__ pid,
-                          int* keyout, int* __restrict__ idxout,
-                          const long long* __restrict__ dstep, Species sp, uint32_t k0,
+                          int* keyout, const long long* __restrict__ dstep, Species sp, uint32_t k0,
                           uint32_t k1, uint32_t* flags, unsigned long long* counters,
                           double* surf) {
   __shared__ BlockTally tal;
@@ -343,9 +342,9 @@ __global__ void __launch_bounds__(kBlk, 3) pl_advect(PlGeom g, PlGeomT<T> gt,
                                    hits, fl, surf);
     nhit += hits;
     nout += keep ? 0 : 1;
-    x[j] = px; y[j] = py; cx[j] = vx; cy[j] = vy; cz[j] = vz; er[j] = e; lev[j] = l;
+    x[j] = px; y[j] = py; cx[j] = vx; cy[j] = vy; cz[j] = vz; er[j] = e;
+    if (hits) lev[j] = l;   // only a wall event changes it
     keyout[j] = keep ? plane_cell<T, AMR>(g, gt, tr, px, py) : g.ncell;
-    idxout[j] = (int)j;
   }
   fl = __reduce_or_sync(0xffffffffu, fl);
   nhit = wsum(nhit);
@@ -486,7 +485,7 @@ __global__ void __launch_bounds__(kBlk, 3) pl_inject(PlGeom g, PlGeomT<T> gt,
                           const int* __restrict__ face_off, T* __restrict__ x, T* __restrict__ y,
                           T* __restrict__ cx, T* __restrict__ cy, T* __restrict__ cz,
                           T* __restrict__ er, int* __restrict__ lev, uint32_t* __restrict__ pid,
-                          int* __restrict__ keyout, int* __restrict__ idxout,
+                          int* __restrict__ keyout,
                           const long long* __restrict__ dstep, Species sp, uint32_t k0,
                           uint32_t k1, uint32_t* flags, unsigned long long* counters,
                           double* surf) {
@@ -544,7 +543,6 @@ __global__ void __launch_bounds__(kBlk, 3) pl_inject(PlGeom g, PlGeomT<T> gt,
     const long long j = n + m;
     x[j] = X; y[j] = Y; cx[j] = VX; cy[j] = VY; cz[j] = VZ; er[j] = E; lev[j] = L; pid[j] = id;
     keyout[j] = keep ? plane_cell<T, AMR>(g, gt, tr, X, Y) : g.ncell;
-    idxout[j] = (int)j;
   }
   fl = __reduce_or_sync(0xffffffffu, fl);
   nhit = wsum(nhit);
@@ -625,6 +623,7 @@ __global__ void pl_scan_digits(int* __restrict__ bh, int nblk, const PlCount* __
   if (t == 0) tot[d] = carry;
 }
 
+// iin null: the indices of the first pass, 0, 1, 2, ...
 __global__ void pl_scatter(const int* __restrict__ kin, const int* __restrict__ iin,
                            int* __restrict__ kout, int* __restrict__ iout,
                            const PlCount* __restrict__ cnt, int shift, const int* __restrict__ bh,
@@ -671,7 +670,7 @@ __global__ void pl_scatter(const int* __restrict__ kin, const int* __restrict__ 
     for (int d = t; d < kNB; d += kRB) cntw[q][d] = 0;
   auto load = [&](int r, int& k_, int& i_) {
     const long long i = b + (long long)r * kRB + t;
-    if (r < kRPT && i < n) { k_ = kin[i]; i_ = iin[i]; }
+    if (r < kRPT && i < n) { k_ = kin[i]; i_ = iin ? iin[i] : (int)i; }
   };
   int k0 = 0, i0 = 0, k1 = 0, i1 = 0;
   load(0, k0, i0);
@@ -1663,19 +1662,19 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
   const PlGeomT<T> gt = geom_t<T>(h->g, env.sp);
   (amr ? pl_advect<T, true> : pl_advect<T, false>)<<<h->grid_p, kBlk, 0, s>>>(
       h->g, gt, h->tree, h->cnt, h->keycell, h->cells, h->pend, x, y, cx, cy, cz, er, h->lv[a], h->pd[a],
-      h->kbuf[0], h->ibuf[0], h->dstep, env.sp, env.k0, env.k1, env.flags, env.counters, surf);
+      h->kbuf[0], h->dstep, env.sp, env.k0, env.k1, env.flags, env.counters, surf);
   pl_inflow<<<1, 1024, 0, s>>>(h->inf, h->cnt, h->face_off, h->cap, h->dstep, env.k0, env.k1,
                                env.flags, env.counters);
   if (h->inf.nfaces > 0)
     (amr ? pl_inject<T, true> : pl_inject<T, false>)<<<h->grid_inj, kBlk, 0, s>>>(
         h->g, gt, h->tree, h->inf, h->cnt, h->face_off, x, y, cx, cy, cz, er, h->lv[a], h->pd[a], h->kbuf[0],
-        h->ibuf[0], h->dstep, env.sp, env.k0, env.k1, env.flags, env.counters, surf);
+        h->dstep, env.sp, env.k0, env.k1, env.flags, env.counters, surf);
   CHK(cudaGetLastError());
   int src = 0;
   for (int p = 0; p < h->passes; ++p) {
     pl_hist<<<h->nblk, kRB, 0, s>>>(h->kbuf[src], h->cnt, kDig * p, h->bh, h->nblk);
     pl_scan_digits<<<kNB, kRB, 0, s>>>(h->bh, h->nblk, h->cnt, h->tot);
-    pl_scatter<<<h->nblk, kRB, 0, s>>>(h->kbuf[src], h->ibuf[src], h->kbuf[src ^ 1],
+    pl_scatter<<<h->nblk, kRB, 0, s>>>(h->kbuf[src], p ? h->ibuf[src] : nullptr, h->kbuf[src ^ 1],
                                        h->ibuf[src ^ 1], h->cnt, kDig * p, h->bh, h->tot, h->nblk);
     CHK(cudaGetLastError());
     src ^= 1;
