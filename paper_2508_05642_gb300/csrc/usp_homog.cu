@@ -1508,9 +1508,9 @@ constexpr int kMomAcc = 20;
 
 // Per-particle arithmetic in the state precision T; partial sums stay in T
 // within a thread (a few particles) and a warp, then combine in FP64.
-template <typename T>
+template <typename T, int pass>
 __global__ void __launch_bounds__(kBlock)
-moments_kernel(int pass, const Tile* __restrict__ tiles, int ntiles,
+moments_kernel(const Tile* __restrict__ tiles, int ntiles,
                const CellState* __restrict__ cells, const T* __restrict__ cx,
                const T* __restrict__ cy, const T* __restrict__ cz, const T* __restrict__ er,
                const int* __restrict__ lev, double* __restrict__ acc_out) {
@@ -1523,9 +1523,9 @@ moments_kernel(int pass, const Tile* __restrict__ tiles, int ntiles,
   const int G = gridDim.x;
   const int t_begin = (int)(((long long)ntiles * blockIdx.x) / G);
   const int t_end = (int)(((long long)ntiles * (blockIdx.x + 1)) / G);
-  const int na = pass == 0 ? 5 : 15;
-  T a[15];
-  for (int i = 0; i < 15; ++i) a[i] = T(0);
+  constexpr int na = pass == 0 ? 5 : 15;
+  T a[na];
+  for (int i = 0; i < na; ++i) a[i] = T(0);
   for (int t = t_begin; t < t_end; ++t) {
     const Tile tl = tiles[t];
     const CellState& cs = cells[tl.cell];
@@ -1551,13 +1551,27 @@ moments_kernel(int pass, const Tile* __restrict__ tiles, int ntiles,
     const T S0 = cp[3], S1 = cp[4], S2 = cp[5];
     const T sc = cp[6], rc = cp[7];
     const T mean0 = cp[8], mean1 = cp[9], mean2 = cp[10];
-    for (int k = threadIdx.x; k < tl.count; k += kBlock) {
-      const long long e = base + k;
-      const T c0 = U0 + sc * (cx[e] - S0);
-      const T c1 = U1 + sc * (cy[e] - S1);
-      const T c2 = U2 + sc * (cz[e] - S2);
-      const T ep = rc * er[e];
-      const T li = (T)lev[e];
+    // a thread's particles of the tile (six at most) are loaded together and
+    // then added in order, so that their latencies overlap
+    constexpr int kPer = kTileMax / kBlock;
+    T vx[kPer], vy[kPer], vz[kPer], ve[kPer];
+    int vl[kPer];
+#pragma unroll
+    for (int m = 0; m < kPer; ++m) {
+      const int k = threadIdx.x + m * kBlock;
+      if (k < tl.count) {
+        const long long e = base + k;
+        vx[m] = cx[e]; vy[m] = cy[e]; vz[m] = cz[e]; ve[m] = er[e]; vl[m] = lev[e];
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < kPer; ++m) {
+      if ((int)threadIdx.x + m * kBlock >= tl.count) break;
+      const T c0 = U0 + sc * (vx[m] - S0);
+      const T c1 = U1 + sc * (vy[m] - S1);
+      const T c2 = U2 + sc * (vz[m] - S2);
+      const T ep = rc * ve[m];
+      const T li = (T)vl[m];
       if (pass == 0) {
         a[0] += c0; a[1] += c1; a[2] += c2; a[3] += ep; a[4] += li;
       } else {
@@ -1572,20 +1586,16 @@ moments_kernel(int pass, const Tile* __restrict__ tiles, int ntiles,
     }
     const bool last = t + 1 >= t_end || tiles[t + 1].cell != tl.cell;
     if (last) {
-      // warp totals; lane i < na converts total i (one conversion per warp)
-      T mine = T(0);
-      for (int i = 0; i < na; ++i) {
-        const T sm = warp_sum(a[i]);
-        mine = lane == i ? sm : mine;
-      }
-      if (lane < na) red[wid][lane] = (double)mine;
+      // warp totals, each converted by the lane that holds it
+      const int at = halve_totals<na>(a);
+      if (at >= 0) red[wid][at] = (double)a[0];
       __syncthreads();
       if (threadIdx.x < na) {
         double sm = 0.0;
         for (int w = 0; w < kBlock / 32; ++w) sm += red[w][threadIdx.x];
         atomicAdd(&acc_out[(size_t)tl.cell * kMomAcc + (pass == 0 ? 0 : 5) + threadIdx.x], sm);
       }
-      for (int i = 0; i < 15; ++i) a[i] = T(0);
+      for (int i = 0; i < na; ++i) a[i] = T(0);
     }
   }
 }
@@ -2182,12 +2192,14 @@ int compute_moments(usp_ctx* c, double* levsum, const CellRange& r) {
     return USP_OK;
   } else {
   if (r.t1 > r.t0) {
-    for (int pass = 0; pass < 2; ++pass) {
-      moments_kernel<T><<<moments_grid(c), kBlock, 0, c->stream>>>(
-          pass, c->tiles + r.t0, r.t1 - r.t0, c->cells, (const T*)c->cx, (const T*)c->cy,
-          (const T*)c->cz, (const T*)c->er, c->lev, c->macc);
-      CK(cudaGetLastError());
-    }
+    const int grid = moments_grid(c);
+    const T* x = (const T*)c->cx; const T* y = (const T*)c->cy; const T* z = (const T*)c->cz;
+    moments_kernel<T, 0><<<grid, kBlock, 0, c->stream>>>(
+        c->tiles + r.t0, r.t1 - r.t0, c->cells, x, y, z, (const T*)c->er, c->lev, c->macc);
+    CK(cudaGetLastError());
+    moments_kernel<T, 1><<<grid, kBlock, 0, c->stream>>>(
+        c->tiles + r.t0, r.t1 - r.t0, c->cells, x, y, z, (const T*)c->er, c->lev, c->macc);
+    CK(cudaGetLastError());
     c->launches += 2;
   }
   assemble_moments<<<(r.c1 - r.c0 + 127) / 128, 128, 0, c->stream>>>(
