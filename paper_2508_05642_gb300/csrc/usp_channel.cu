@@ -112,6 +112,8 @@ template <typename T>
 struct ChParams {
   T alpha, nu_ref, B, mu_p, Pr, gtr, gtv, grv;
   T R, theta, dt, yc;
+  T iRth;                       // FP64 form: 1 / (R theta)
+  std::conditional_t<std::is_same<T, double>::value, AlphaParts<T>, int> ap;
   T F[kNF], Sm[kNF], Sp[kNF];   // cell values; slopes used below / above the centroid
   int active, pad;
 };
@@ -429,6 +431,10 @@ __device__ void ch_recon(int c, int ny, double dy, int recon, double dt,
     P.Pr = (T)cs.Pr; P.gtr = (T)cs.gtr; P.gtv = (T)cs.gtv; P.grv = (T)cs.grv;
     P.R = (T)gasR(sp); P.theta = (T)sp.theta_v; P.dt = (T)dt;
     P.yc = (T)((c + 0.5) * dy);
+    if constexpr (std::is_same<T, double>::value) {
+      P.iRth = sp.iRtheta;
+      P.ap = alpha_parts(P.alpha, P.R);
+    }
   }
 }
 

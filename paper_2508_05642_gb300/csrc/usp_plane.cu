@@ -128,6 +128,8 @@ struct alignas(16) PlParams {
   T alpha, nu_ref, B, mu_p, Pr, gtr, gtv, grv;
   T R, theta, dt;
   T xc, yc;
+  T iRth;               // 1 / (R theta)
+  AlphaParts<T> ap;
   int active, pad;
 };
 
@@ -765,6 +767,8 @@ __device__ __forceinline__ void pl_scalars(PlParams<T>& P, const ChCellT<double>
   P.R = (T)gasR(sp); P.theta = gt.theta; P.dt = gt.dt;
   P.xc = (T)xc;
   P.yc = (T)yc;
+  P.iRth = rcp_fast(P.R * P.theta);
+  P.ap = alpha_parts(P.alpha, P.R);
 }
 
 template <typename T>
