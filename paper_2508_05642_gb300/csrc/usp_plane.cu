@@ -1368,6 +1368,93 @@ __global__ void pl_mom_out(int ncell, const long long* __restrict__ off,
   }
 }
 
+// The cells' moments of a step in the FP64 form, in the same two parts: kCL
+// lanes per cell sum d = c - c_first, d d, eps and I into rec (kNAcc doubles per
+// cell), then one thread per cell forms the fields.  (A warp per cell spent
+// 70 FP64 instructions on a cell of 20 particles, most of them in reductions
+// and in the mean that the whole warp divided out: 173 us for 0.77 million
+// particles in 38,400 cells.)
+__global__ void __launch_bounds__(kBlk)
+pl_cell_sums(int ncell, const long long* __restrict__ off, const double* __restrict__ cx,
+             const double* __restrict__ cy, const double* __restrict__ cz,
+             const double* __restrict__ er, const int* __restrict__ lev,
+             double* __restrict__ rec) {
+  const int q = threadIdx.x & (kCL - 1);
+  const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kCL;
+  const long long b = c < ncell ? off[c] : 0, e = c < ncell ? off[c + 1] : 0;
+  double a[kNAcc];
+#pragma unroll
+  for (int i = 0; i < kNAcc; ++i) a[i] = 0.0;
+  double r0 = 0.0, r1 = 0.0, r2 = 0.0;
+  if (b < e) { r0 = cx[b]; r1 = cy[b]; r2 = cz[b]; }
+  long long sl = 0;
+#pragma unroll 2
+  for (long long j = b + q; j < e; j += kCL) {
+    const double d0 = cx[j] - r0, d1 = cy[j] - r1, d2 = cz[j] - r2;
+    a[0] += d0; a[1] += d1; a[2] += d2;
+    a[3] = fma(d0, d0, a[3]); a[4] = fma(d1, d1, a[4]); a[5] = fma(d2, d2, a[5]);
+    a[6] = fma(d0, d1, a[6]); a[7] = fma(d0, d2, a[7]); a[8] = fma(d1, d2, a[8]);
+    a[9] += er[j];
+    sl += lev[j];
+  }
+  if (sl != 0) a[10] = (double)sl;
+  cl_totals<kNAcc>(a);
+  if (c < ncell) {
+#pragma unroll
+    for (int i = 0; i < kNAcc / 4; ++i) rec[(size_t)c * kNAcc + q * (kNAcc / 4) + i] = a[i];
+  }
+}
+
+__global__ void __launch_bounds__(kBlk)
+pl_cell_fields(int ncell, const long long* __restrict__ off, const double* __restrict__ af,
+               const double* __restrict__ cx, const double* __restrict__ cy,
+               const double* __restrict__ cz, const double* __restrict__ rec,
+               ChCellT<double>* __restrict__ cells, Species sp, unsigned long long* counters,
+               double* __restrict__ fT, int* __restrict__ usable_c) {
+  __shared__ BlockTally tal;
+  tally_init(tal);
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < ncell) {
+    const long long b = off[c], N = off[c + 1] - b;
+    ChCellT<double>& cs = cells[c];
+    cs.off = b;
+    cs.N = N;
+    cs.active = N >= 2;
+    // a neighbour for the reconstruction of Sec. 3.B: two or more particles
+    // and not cut by a body
+    cs.usable = N >= 2 && af[c] >= 1.0;
+    usable_c[c] = cs.usable;
+    const double* S = rec + (size_t)c * kNAcc;
+    const double inv = N > 0 ? d_rcp((double)N) : 0.0;
+    const double m0 = S[0] * inv, m1 = S[1] * inv, m2 = S[2] * inv;
+    const double U[3] = {N > 0 ? cx[b] + m0 : 0.0, N > 0 ? cy[b] + m1 : 0.0,
+                         N > 0 ? cz[b] + m2 : 0.0};
+    for (int i = 0; i < 3; ++i) {   // identity pending rescale until the cell is updated
+      cs.U[i] = U[i];
+      cs.Un[i] = 0.0;
+      cs.Us[i] = 0.0;
+    }
+    cs.s = 1.0;
+    cs.r = 1.0;
+    if (!cs.active) {
+      tally_add(tal, C_SKIPPED_CELLS, 1ull);
+    } else {
+      const double P[6] = {fma(S[3], inv, -(m0 * m0)), fma(S[4], inv, -(m1 * m1)),
+                           fma(S[5], inv, -(m2 * m2)), fma(S[6], inv, -(m0 * m1)),
+                           fma(S[7], inv, -(m0 * m2)), fma(S[8], inv, -(m1 * m2))};
+      cs.Ttr = (P[0] + P[1] + P[2]) * (sp.iR * (1.0 / 3.0));
+      cs.Trot = S[9] * (inv * sp.iR);
+      cs.ebar = S[10] * inv;
+      cs.Tvib = vib_state(sp, cs.ebar).Tvib;
+      double* o = fT + (size_t)c * kNF;
+      for (int i = 0; i < 3; ++i) o[i] = U[i];
+      o[3] = cs.Ttr; o[4] = cs.Trot; o[5] = cs.Tvib;
+      for (int i = 0; i < 6; ++i) cs.Pi[i] = o[6 + i] = P[i];
+    }
+  }
+  tally_flush(tal, nullptr, counters);
+}
+
 // on-demand moments of a state in any order (before the first step): pass 0
 // raw sums, pass 1 central
 template <typename T>
@@ -1706,10 +1793,16 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
         ncell, h->off, h->af, h->afv, (float)(h->Fnum / h->vol), h->g.dt, (const float*)cx,
         (const float*)cy, (const float*)cz, (const float*)er, h->lv[b], h->cells, env.sp,
         env.flags, env.counters, pend, (float*)h->fT, h->usable_c);
-  else
+  else if constexpr (sizeof(T) == 8) {
+    pl_cell_sums<<<cell_grid(h), kBlk, 0, s>>>(ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc);
+    pl_cell_fields<<<(ncell + kBlk - 1) / kBlk, kBlk, 0, s>>>(
+        ncell, h->off, h->af, cx, cy, cz, h->macc, h->cells, env.sp, env.counters, (T*)h->fT,
+        h->usable_c);
+  } else {
     ch_moments<T, double><<<wb, kBlk, 0, s>>>(ncell, 32, h->off, h->af, cx, cy, cz, er, h->lv[b],
                                               h->cells, env.sp, env.counters, pend, (T*)h->fT,
                                               h->usable_c);
+  }
   if (fpm)
     ch_coeffs_fpm<<<tb, kBlk, 0, s>>>(ncell, h->Fnum, h->vol, h->afv, h->g.dt, h->cells,
                                       h->fpmrec, env.sp, env.flags, env.counters);
@@ -1768,7 +1861,8 @@ int pl_kernels_per_step(const PlaneCtx* h) {
     params = 0;
     for (int L = 1; L <= h->levels; ++L) params += h->nblk_lv[L] > 0 ? 1 : 0;
   }
-  const int cellpass = h->es == sizeof(float) && !h->fpmrec ? 1 : 2;
+  // FP32 USP-FPM: one pass; FP64: sums, fields, coefficients; else moments, coefficients
+  const int cellpass = h->es == sizeof(double) ? 3 : h->fpmrec ? 2 : 1;
   return 2 + (h->inf.nfaces > 0 ? 1 : 0) + 3 * h->passes + 1 + cellpass + params + 1 + 1 +
          (h->sampling ? 2 : 0);
 }
