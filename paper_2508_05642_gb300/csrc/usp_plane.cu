@@ -207,9 +207,12 @@ __device__ bool plane_fly(const PlGeom& g, const PlGeomT<T>& gt, uint32_t pid, u
       const T a = vx * vx + vy * vy;
       const T b = dx * vx + dy * vy;
       const T c = dx * dx + dy * dy - gt.cr * gt.cr;
+      // a particle that by te is neither past its closest approach nor inside
+      // the circle by a margin far above rounding does not hit it: no root
+      const bool far = b + a * te < T(0) && c + te * (T(2) * b + a * te) > gt.margin * gt.cr;
       if (c > T(0) && b < T(0) && a > T(0)) {
         const T disc = b * b - a * c;
-        if (disc >= T(0)) {
+        if (!far && disc >= T(0)) {
           const T t = (-b - sqrt(disc)) / a;
           if (t >= T(0) && t <= te) { te = t; ev = 0; }
         }
@@ -220,17 +223,12 @@ __device__ bool plane_fly(const PlGeom& g, const PlGeomT<T>& gt, uint32_t pid, u
         ev = 0;
       }
     }
-    // a side's time is formed only when the side may be met by te: in FP32
-    // a particle whose straight move stops short of the side by more than a
-    // margin far above rounding cannot reach it (the FP64 form always forms
-    // the time)
+    // a side's time is formed only when the side may be met by te: a
+    // particle whose straight move stops short of the side by more than a
+    // margin far above rounding cannot reach it
     auto may = [&](T pos, T v, T side, bool lower) {
-      if constexpr (sizeof(T) == 4) {
-        const T end = pos + v * te;
-        return lower ? end <= side + gt.margin : end >= side - gt.margin;
-      } else {
-        return true;
-      }
+      const T end = pos + v * te;
+      return lower ? end <= side + gt.margin : end >= side - gt.margin;
     };
     if (vx < T(0) && may(x, vx, gt.x0, true)) {
       const T t = (gt.x0 - x) / vx;
