@@ -704,16 +704,17 @@ __device__ __forceinline__ bool chol3(const T* M, T* L) {
 }
 
 // the same for a per-cell matrix, by reciprocal square roots (usp_math.cuh)
+constexpr double kLeastPivot = 0x1p-1000;   // the reciprocal root needs a normal number
 __device__ __forceinline__ bool chol3_cell(const double* M, double* L) {
-  if (!(M[0] > 0.0)) return false;
+  if (!(M[0] > kLeastPivot)) return false;
   const double r0 = d_rsqrt(M[0]);
   const double l10 = M[3] * r0, l20 = M[4] * r0;
   const double d1 = M[1] - l10 * l10;
-  if (!(d1 > 0.0)) return false;
+  if (!(d1 > kLeastPivot)) return false;
   const double r1 = d_rsqrt(d1);
   const double l21 = (M[5] - l20 * l10) * r1;
   const double d2 = M[2] - l20 * l20 - l21 * l21;
-  if (!(d2 > 0.0)) return false;
+  if (!(d2 > kLeastPivot)) return false;
   L[0] = M[0] * r0; L[1] = l10; L[2] = d1 * r1; L[3] = l20; L[4] = l21; L[5] = d_sqrt(d2);
   return true;
 }

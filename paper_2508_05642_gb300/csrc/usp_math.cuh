@@ -19,18 +19,23 @@ constexpr double kLn2Hi = 0x1.62e42fefa2p-1;        // 40 bits: times an exponen
 constexpr double kLn2Lo = 0x1.9ef35793c7673p-41;    // ln 2 - kLn2Hi
 constexpr double kLog2e = 0x1.71547652b82fep+0;
 
+// zero, denormal, infinite or not a number (integer work, beside the FP64 pipe)
+__device__ __forceinline__ bool d_ends(double b) {
+  return ((unsigned)__double2hiint(b) & 0x7ff00000u) - 0x00100000u >= 0x7fe00000u;
+}
 // 1 / b: hardware seed (about 2^-20), then y (1 + e + e^2), e = 1 - b y, whose
-// remainder is e^3
+// remainder is e^3; the seed itself where b has no such e (0 of an infinity, an
+// infinity of 0)
 __device__ __forceinline__ double d_rcp(double b) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
   const double e = fma(-b, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  return d_ends(b) ? y : fma(y, fma(e, e, e), y);
 }
 // a / b with the residual of the quotient added (Markstein)
 __device__ __forceinline__ double d_div(double a, double b) {
   const double y = d_rcp(b), q = a * y;
-  return fma(fma(-b, q, a), y, q);
+  return d_ends(b) || d_ends(a) ? q : fma(fma(-b, q, a), y, q);
 }
 // 1 / sqrt(x): the seed times (1 - e)^(-1/2) to second order, e = 1 - x y^2
 __device__ __forceinline__ double d_rsqrt(double x) {
