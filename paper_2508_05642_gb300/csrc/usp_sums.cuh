@@ -90,6 +90,12 @@ __device__ __forceinline__ RawMoments raw_moments(const double* a, double n, con
     r.qr[k] = a[kRE + k] * inv - m[k] * r.eps;
     r.ql[k] = a[kRL + k] * inv - m[k] * r.lev;
   }
+  // a single particle has no spread and no variance is negative: what the
+  // differences above leave of either is rounding
+  for (int i = 0; i < 6; ++i)
+    if (n == 1.0 || (i < 3 && r.P[i] < 0.0)) r.P[i] = 0.0;
+  if (n == 1.0)
+    for (int k = 0; k < 3; ++k) r.qt[k] = r.qr[k] = r.ql[k] = 0.0;
   return r;
 }
 

@@ -1,0 +1,263 @@
+"""GPU tests of the size-dependent paths of the library at the sizes where they
+change: one-pass moments, the tables of the FP64 draws and jumps, the channel's
+one-pass sort, the per-cell passes of few cells in one kernel, the host-buffer
+step's copies, the plane's sums over the sorted state and FP32 estimates of
+Gillespie's method.  Each is compared with the oracle or with plain sums.
+
+Tolerances: a sum of n FP64 terms in any order is within n 2^-53 of the sum of
+the terms' magnitudes (n below 10^6 here: 1.2e-10 of it, 1e-12 for the cells of
+at most 5,000); values that pass through a step's arithmetic take the
+bars of the parity tests (1e-9 of the scale after a few steps)."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2508_05642_gb300 import inputs as I
+from paper_2508_05642_gb300 import usp
+
+pytestmark = pytest.mark.gpu
+
+
+def _moments(sp, off, c, e, lev):
+    """USP_NMOM fields by plain two-pass sums, and each field's sum of
+    magnitudes over n (the scale of its rounding)."""
+    R = 1.380649e-23 / sp["m"]
+    m = np.zeros((usp.USP_NMOM, len(off) - 1))
+    s = np.zeros_like(m)
+    for i in range(len(off) - 1):
+        b, f = off[i], off[i + 1]
+        n = f - b
+        if n == 0:
+            continue
+        v, er, l = c[:, b:f], e[b:f], lev[b:f].astype(float)
+        U = v.mean(axis=1)
+        C = v - U[:, None]
+        q = 0.5 * (C * C).sum(axis=0)
+        rows = {1: v[0], 2: v[1], 3: v[2], 5: er / R}
+        for k, (a, d) in enumerate(((0, 0), (1, 1), (2, 2), (0, 1), (0, 2), (1, 2))):
+            rows[7 + k] = C[a] * C[d]
+        for k in range(3):
+            rows[13 + k], rows[16 + k], rows[19 + k] = q * C[k], C[k] * er, C[k] * l * R * sp["theta_v"]
+        m[0, i] = n
+        s[0, i] = n
+        for k, t in rows.items():
+            m[k, i], s[k, i] = t.mean(), np.abs(t).mean() + np.sqrt((t * t).mean())
+        m[4, i] = m[7:10, i].sum() / (3 * R)
+        s[4, i] = m[4, i]
+        eb = l.mean()
+        m[6, i] = sp["theta_v"] / np.log1p(1 / eb) if eb > 0 else 0.0
+        s[6, i] = m[6, i]
+    return m, s
+
+
+def _near(got, ref, bar):
+    bad = np.argwhere(~(np.abs(got - ref) <= bar))
+    assert len(bad) == 0, [(tuple(int(v) for v in i), float(got[tuple(i)]), float(ref[tuple(i)]),
+                            float(bar[tuple(i)])) for i in bad[:8]] + [len(bad)]
+
+
+SIZES = [0, 1, 2, 3, 31, 32, 33, 63, 64, 65, 127, 511, 512, 513, 1025, 4999, 0]
+
+
+@pytest.mark.parametrize("ncell", [1, 17, 300, 1100])
+def test_one_pass_moments_at_odd_cell_sizes(ncell):
+    torch = pytest.importorskip("torch")
+    sp = I.n2_vhs_relaxation_species()
+    rng = np.random.default_rng(ncell)
+    sizes = [5000] if ncell == 1 else (SIZES * (ncell // len(SIZES) + 1))[:ncell]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    n = int(off[-1])
+    c = 2900.0 * np.array([[1.0], [-0.2], [0.0]]) + 250.0 * rng.standard_normal((3, n))
+    e = rng.exponential(6e4, n)
+    lev = rng.poisson(0.3, n).astype(np.int32)
+    ref, scale = _moments(sp, off, c, e, lev)
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    dc, de, dl, do = [d(a) for a in c], d(e), d(lev), d(off)
+    out = torch.full((usp.USP_NMOM, ncell), np.nan, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    usp.usp_moments_noalloc(sp, ncell, do.data_ptr(), *[a.data_ptr() for a in dc], de.data_ptr(),
+                            dl.data_ptr(), out.data_ptr(),
+                            torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    # third moments about a shifted reference lose a little: 16 times the bar
+    bar = 1e-12 * scale * 16 + 1e-300
+    _near(out.cpu().numpy(), ref, bar)
+    ctx = usp.usp_init_homogeneous(sp, off, np.full(ncell, 1e23), np.full(ncell, 1e-10), *c, e,
+                                   lev, precision=usp.USP_FP64)
+    _near(usp.usp_moments(ctx), ref, bar)
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("sizes,T_vib", [
+    ([70000], 20000.0),                 # tabled draws and jumps, levels past the table's rows
+    ([65536], 1500.0),
+    ([65535], 9000.0),                  # one short of the draw tables
+    ([511] * 3, 3000.0),                # too small for jump tables
+    ([2, 40000, 600, 31000], 12000.0),
+    ([300] * 160, 4000.0),              # more cells than the one-kernel passes take
+    ([2000] * 156, 20000.0),            # levels corrected by hundreds of decrements
+])
+def test_fp64_forms_by_size_match_oracle(sizes, T_vib):
+    spd = I.n2_vhs_relaxation_species()
+    sp = O.species(**spd)
+    rng = np.random.default_rng(len(sizes) + sizes[0])
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    p = I.equilibrium_particles(rng, int(off[-1]), spd["m"], spd["theta_v"], T_tr=15000.0,
+                                T_rot=800.0, T_vib=T_vib)
+    nd = np.full(len(sizes), 1e23)
+    dto = np.full(len(sizes), 0.5 * O.tau_c(sp, 1e23, 15000.0))
+    st = O.State.from_arrays(p.cx, p.cy, p.cz, p.erot, p.lev)
+    O.homog_step(sp, 0, 11, 0, 4, off, nd, dto, st)
+    ctx = usp.usp_init_homogeneous(spd, off, nd, dto, p.cx, p.cy, p.cz, p.erot, p.lev,
+                                   precision=usp.USP_FP64, seed=11)
+    usp.usp_step(ctx, 3)
+    buf = usp.usp_save(ctx)             # the FP64 tables are not in a checkpoint
+    usp.usp_step(ctx, 1)
+    one = usp.usp_get_particles(ctx)
+    usp.usp_load(ctx, buf)
+    usp.usp_step(ctx, 1)
+    for got in (one, usp.usp_get_particles(ctx)):
+        assert np.array_equal(got[4], st.lev)
+        for a, b in zip(got[:4], (st.cx, st.cy, st.cz, st.erot)):
+            assert np.max(np.abs(a - b)) <= 1e-9 * np.max(np.abs(b))
+    fl, _ = usp.usp_status(ctx)
+    assert fl & usp.ERROR_FLAGS == 0
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("ny,ppc", [(1, 70), (3, 1), (256, 20), (257, 20), (64, 512), (65, 505)])
+@pytest.mark.parametrize("precision", [usp.USP_FP64, usp.USP_FP32])
+def test_channel_sorts_match_oracle(ny, ppc, precision):
+    """The one-pass sort ends at 256 cells and at 32,768 particles."""
+    w = I.channel_poiseuille(ny=ny, ppc=ppc, steps=0)
+    sp, ch = O.species(**w.species), O.channel(**w.channel)
+    form = 1 if precision == usp.USP_FP32 else 0
+    p = w.particles.astype_f32_exact() if form else w.particles
+    y = w.y.astype(np.float32).astype(np.float64) if form else w.y
+    dt = w.dt_over_tau_c * O.tau_c(sp, w.n, w.channel["T_wall"])
+    st = O.ChannelState.from_arrays(y, p.cx, p.cy, p.cz, p.erot, p.lev)
+    ctx = usp.usp_init_channel(w.species, w.channel, dt, y, p.cx, p.cy, p.cz, p.erot, p.lev,
+                               precision=precision, seed=w.seed)
+    steps = 1 if form else 5            # FP32 positions part from the oracle's at cell faces
+    acc = np.zeros(ny * O.NACC + 2)
+    usp.usp_channel_sample(ctx, True)
+    O.channel_step(sp, form, w.seed, 0, steps, ch, dt, st, acc)
+    usp.usp_step(ctx, steps)
+    gy, gx, gv, gz, ge, gl, gp = usp.usp_channel_get_particles(ctx)
+    if form == 0:
+        assert np.array_equal(gp, st.pid) and np.array_equal(gl, st.lev)
+        assert np.max(np.abs(gx - st.cx)) < 1e-8 * 300.0
+        np.testing.assert_allclose(usp.usp_channel_read(ctx), acc, rtol=1e-9, atol=1e-6)
+    else:
+        assert np.mean(gp == st.pid) > 0.999
+        a = usp.usp_channel_read(ctx)
+        assert a[0:ny * O.NACC:O.NACC].sum() == len(gp)
+    assert usp.usp_status(ctx)[0] & usp.ERROR_FLAGS == 0
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("kind", ["pinned", "pageable", "in place", "crossed"])
+def test_host_step_returns_the_stepped_state(kind):
+    """The state comes down while later cells go up only where the buffers
+    allow it; every arrangement gives the same state."""
+    torch = pytest.importorskip("torch")
+    w = I.batched_instances(seed=5, n_inst=40, nmin=1, nmax=9000, steps=0)
+    p = w.particles.astype_f32_exact()
+    n = p.n
+    dt = np.array([0.5 * usp.usp_tau_c(w.species, w.ndens[i], w.T_nominal[i, 0])
+                   for i in range(w.n_cells)])
+    ctx = usp.usp_init_homogeneous(w.species, w.offsets, w.ndens, dt, p.cx, p.cy, p.cz, p.erot,
+                                   p.lev, precision=usp.USP_FP32, seed=3)
+    mk = (lambda m, t: torch.empty(m, dtype=t, pin_memory=True).numpy()) if kind != "pageable" \
+        else (lambda m, t: torch.empty(m, dtype=t).numpy())
+    src = [mk(n, torch.float32) for _ in range(4)] + [mk(n, torch.int32)]
+    for a, b in zip(src, (p.cx, p.cy, p.cz, p.erot, p.lev)):
+        a[:] = b
+    mom = np.zeros((usp.USP_NMOM, w.n_cells))
+    if kind == "in place":
+        out = src
+    elif kind == "crossed":
+        # the outputs overlap the inputs, shifted: they may come down only
+        # after every cell is up
+        big = mk(2 * n + 64, torch.float32)
+        src[0], out0 = big[:n], big[33:n + 33]
+        src[0][:] = p.cx
+        out = [out0] + [mk(n, torch.float32) for _ in range(3)] + [mk(n, torch.int32)]
+    else:
+        out = [mk(n, torch.float32) for _ in range(4)] + [mk(n, torch.int32)]
+    usp.usp_step_host(ctx, *src, 2, mom, out=out)
+    got = [a.copy() for a in out]
+    ref = usp.usp_get_particles(ctx)        # the state the call left on the device
+    for a, b in zip(got[:4], ref[:4]):
+        assert np.array_equal(a, b.astype(np.float32))
+    assert np.array_equal(got[4], ref[4])
+    # and it is the state that the device path steps to
+    ctx2 = usp.usp_init_homogeneous(w.species, w.offsets, w.ndens, dt, p.cx, p.cy, p.cz, p.erot,
+                                    p.lev, precision=usp.USP_FP32, seed=3)
+    usp.usp_step(ctx2, 2)
+    two = usp.usp_get_particles(ctx2)
+    assert np.mean(two[4] != ref[4]) < 1e-3
+    assert np.max(np.abs(two[0] - ref[0])) < 1e-4 * np.max(np.abs(ref[0]))
+    ctx.destroy()
+    ctx2.destroy()
+
+
+@pytest.mark.parametrize("precision", [usp.USP_FP64, usp.USP_FP32])
+@pytest.mark.parametrize("refined", [False, True])
+def test_plane_sums_are_the_particles(precision, refined):
+    """Moments and time averages over the sorted state against sums of the
+    particles that the context returns (cells with no, one and many
+    particles)."""
+    kw = dict(amr_levels=3, amr_r2=0.24, amr_r3=0.16) if refined else {}
+    w = I.cylinder_flow(nx=32, ny=24, ppc=5.0, **kw)
+    p = w.particles
+    dt = w.dt_over_tau_c * usp.usp_tau_c(w.species, w.plane["n_inf"], w.plane["T_inf"])
+    ctx = usp.usp_init_plane(w.species, w.plane, dt, w.area_frac, w.x, w.y, p.cx, p.cy, p.cz,
+                             p.erot, p.lev, w.capacity, precision=precision, seed=4)
+    before = usp.usp_moments(ctx)           # a state that no step has sorted
+    usp.usp_step(ctx, 5)
+    usp.usp_sample(ctx, True)
+    usp.usp_step(ctx, 1)
+    x, y, cx, cy, cz, er, lev, pid = usp.usp_plane_get_particles(ctx)
+    mom = usp.usp_moments(ctx)
+    acc = usp.usp_sample_read(ctx)
+    nc = ctx.n_cells
+    assert before[0].sum() == len(w.x) and mom[0].sum() == len(x)
+    assert (mom[0] == 0).any() and (mom[0] == 1).any()
+    off = np.concatenate([[0], np.cumsum(mom[0].astype(np.int64))])
+    c = np.stack([cx, cy, cz])
+    ref, scale = _moments(w.species, off, c, er, lev)
+    _near(mom, ref, 16e-12 * scale + 1e-300)
+    a = acc[:nc * 12].reshape(nc, 12)
+    seg = lambda t: np.add.reduceat(np.append(t, 0.0), off[:-1]) * (mom[0] > 0)
+    terms = [np.ones(len(x)), cx, cy, cz, cx * cx, cy * cy, cz * cz, cx * cy, cx * cz, cy * cz, er,
+             lev.astype(float)]
+    for k, t in enumerate(terms):
+        _near(a[:, k], seg(t), 1e-12 * seg(np.abs(t)) + 1e-9 * (k > 0))
+    assert acc[nc * 12] == 1.0
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("precision", [usp.USP_FP64, usp.USP_FP32])
+@pytest.mark.parametrize("T", [300.0, 4000.0, 20000.0])
+def test_gillespie_levels_match_oracle(precision, T):
+    """The levels of the first-order method, from cold cells (rates near
+    zero) to ones where a particle makes many transitions a step."""
+    spd = I.n2_vhs_relaxation_species()
+    sp = O.species(**spd)
+    n = 60000
+    rng = np.random.default_rng(int(T))
+    p = I.equilibrium_particles(rng, n, spd["m"], spd["theta_v"], T_tr=T, T_rot=T, T_vib=0.7 * T)
+    form = 1 if precision == usp.USP_FP32 else 0
+    p = p.astype_f32_exact() if form else p
+    off, nd = np.array([0, n], dtype=np.int64), np.array([1e23])
+    dt = np.array([1.5 * O.tau_c(sp, 1e23, T)])
+    st = O.State.from_arrays(p.cx, p.cy, p.cz, p.erot, p.lev)
+    O.homog_step_fpm(sp, form, 7, 0, 1, off, nd, dt, st)
+    ctx = usp.usp_init_homogeneous(spd, off, nd, dt, p.cx, p.cy, p.cz, p.erot, p.lev,
+                                   precision=precision, seed=7, method=usp.USP_METHOD_FPM)
+    usp.usp_step(ctx, 1)
+    lev = usp.usp_get_particles(ctx)[4]
+    # FP32 rates differ from the oracle's in the last bit: a few decisions turn
+    assert np.sum(lev != st.lev) <= (0 if form == 0 else 20)
+    ctx.destroy()
