@@ -108,12 +108,18 @@ namespace {
 constexpr int kPlaceCells = 256, kPlaceBlocks = 128;
 constexpr int kAB = 128;   // threads per block of the move
 
+// forms whose collision takes reciprocals in place of groups of divisions
+template <typename T>
+constexpr bool kFastForm = std::is_same<T, double>::value || std::is_same<T, D3>::value;
+
 template <typename T>
 struct ChParams {
   T alpha, nu_ref, B, mu_p, Pr, gtr, gtv, grv;
-  T R, theta, dt, yc;
-  T iRth;                       // FP64 form: 1 / (R theta)
-  std::conditional_t<std::is_same<T, double>::value, AlphaParts<T>, int> ap;
+  // the derivative form differentiates by none of these
+  using C = std::conditional_t<std::is_same<T, D3>::value, double, T>;
+  C R, theta, dt, yc;
+  C iRth;                       // kFastForm: 1 / (R theta)
+  std::conditional_t<kFastForm<T>, AlphaParts<T>, int> ap;
   T F[kNF], Sm[kNF], Sp[kNF];   // cell values; slopes used below / above the centroid
   int active, pad;
 };
@@ -429,9 +435,10 @@ __device__ void ch_recon(int c, int ny, double dy, int recon, double dt,
   } else if (t == 32) {
     P.alpha = (T)cs.alpha; P.nu_ref = (T)cs.nu_ref; P.B = (T)cs.B; P.mu_p = (T)cs.mu_p;
     P.Pr = (T)cs.Pr; P.gtr = (T)cs.gtr; P.gtv = (T)cs.gtv; P.grv = (T)cs.grv;
-    P.R = (T)gasR(sp); P.theta = (T)sp.theta_v; P.dt = (T)dt;
-    P.yc = (T)((c + 0.5) * dy);
-    if constexpr (std::is_same<T, double>::value) {
+    using C = typename ChParams<T>::C;
+    P.R = (C)gasR(sp); P.theta = (C)sp.theta_v; P.dt = (C)dt;
+    P.yc = (C)((c + 0.5) * dy);
+    if constexpr (kFastForm<T>) {
       P.iRth = sp.iRtheta;
       P.ap = alpha_parts(P.alpha, P.R);
     }
@@ -466,15 +473,18 @@ ch_collide(int c0, int ny, double dy, int recon, double dt, const ChCellT<S>* __
       const bool above = dyv >= T(0);
       T f[kNF];
 #pragma unroll
-      for (int q = 0; q < kNF; ++q) f[q] = P.F[q] + (above ? P.Sp[q] : P.Sm[q]) * dyv;
+      for (int q = 0; q < kNF; ++q) {
+        if constexpr (kFastForm<T>) f[q] = madd(P.F[q], above ? P.Sp[q] : P.Sm[q], dyv);
+        else f[q] = P.F[q] + (above ? P.Sp[q] : P.Sm[q]) * dyv;
+      }
       if (!(f[3] > T(0)) || !(f[4] > T(0)) || !(f[5] >= T(0))) {
 #pragma unroll
         for (int q = 0; q < kNF; ++q) f[q] = P.F[q];
         ++nfb;
       }
       T v0 = cx[j], v1 = cy[j], v2 = cz[j], en = er[j];
-      lev[j] = collide_particle_t<std::is_same<T, double>::value>(P, f, v0, v1, v2, en, lev[j],
-                                                                  pid[j], step, rk, tl);
+      lev[j] = collide_particle_t<kFastForm<T>>(P, f, v0, v1, v2, en, lev[j], pid[j], step, rk,
+                                                tl);
       cx[j] = v0; cy[j] = v1; cz[j] = v2; er[j] = en;
     }
   } else {

@@ -189,6 +189,22 @@ __device__ inline Dual<V> sqrt(const Dual<V>& a) {
   const V s = vsqrt(a.v);
   return chain(a, s, s > V(0) ? vdiv(V(0.5), s) : V(0));
 }
+__device__ inline Dual<double> rcp(const Dual<double>& a) {
+  const double r = d_rcp(a.v);
+  return chain(a, r, -(r * r));
+}
+__device__ inline Dual<double> rsqrt(const Dual<double>& a) {
+  const double r = d_rsqrt(a.v);
+  return chain(a, r, -0.5 * r * (r * r));
+}
+// f + a b
+__device__ inline Dual<double> madd(const Dual<double>& f, const Dual<double>& a,
+                                    const Dual<double>& b) {
+  Dual<double> r;
+  r.v = fma(a.v, b.v, f.v);
+  for (int i = 0; i < kND; ++i) r.d[i] = fma(a.d[i], b.v, fma(a.v, b.d[i], f.d[i]));
+  return r;
+}
 template <typename V>
 __device__ inline Dual<V> log(const Dual<V>& a) { return chain(a, vlog(a.v), vdiv(V(1), a.v)); }
 template <typename V>

@@ -215,6 +215,47 @@ __device__ __forceinline__ void relax_fast(const P_& P, double ioR, const double
   if (evr < 0.0) { evr = 0.0; cl = true; }
 }
 
+// The derivative form: the same with one reciprocal or reciprocal root per group
+// of divisions (a derivative number's division takes 17 FP64 operations, its
+// product 7).
+template <typename T>
+__device__ __forceinline__ AlphaParts<T> alpha_parts(const T& alpha, double R) {
+  const T o = 1.0 - alpha * alpha;
+  return {o, sqrt(o), rcp(o * R)};
+}
+template <typename T>
+__device__ __forceinline__ bool chol3_fast(const T* M, T* L) {
+  if (!(M[0] > kLeastPivot)) return false;
+  const T r0 = rsqrt(M[0]);
+  const T l10 = M[3] * r0, l20 = M[4] * r0;
+  const T d1 = M[1] - l10 * l10;
+  if (!(d1 > kLeastPivot)) return false;
+  const T r1 = rsqrt(d1);
+  const T l21 = (M[5] - l20 * l10) * r1;
+  const T d2 = M[2] - l20 * l20 - l21 * l21;
+  if (!(d2 > kLeastPivot)) return false;
+  L[0] = M[0] * r0; L[1] = l10; L[2] = d1 * r1; L[3] = l20; L[4] = l21; L[5] = sqrt(d2);
+  return true;
+}
+template <typename P_, typename T>
+__device__ __forceinline__ void relax_fast(const P_& P, const T& ioR, const T* f, T& ttr, T& trot,
+                                           T& evr, bool& cl) {
+  const T x = P.gtr * (f[3] - f[4]), y = P.gtv * (f[3] - f[5]), z = P.grv * (f[4] - f[5]);
+  ttr = f[3] - (x + y) * (ioR * (2.0 / 3.0));
+  trot = f[4] + (x - z) * ioR;
+  const T ev = f[5] > 0.0 ? P.R * P.theta * rcp(expm1(P.theta * rcp(f[5]))) : T(0);
+  evr = ev + (y + z) * (ioR * P.R);
+  cl = false;
+  if (ttr < 0.0) { ttr = T(0); cl = true; }
+  if (trot < 0.0) { trot = T(0); cl = true; }
+  if (evr < 0.0) { evr = T(0); cl = true; }
+}
+template <typename T>
+__device__ __forceinline__ T rcp_fast(const T& x) { return rcp(x); }
+// f + a b
+__device__ __forceinline__ float madd(float f, float a, float b) { return f + a * b; }
+__device__ __forceinline__ double madd(double f, double a, double b) { return f + a * b; }
+
 // the square roots and reciprocals of the collision: FP32 as the form always
 // took them, FP64 on usp_math.cuh
 template <bool kFast, typename T>
@@ -246,7 +287,6 @@ template <bool kFast = false, typename T, typename P_>
 __device__ __forceinline__ int collide_particle_t(const P_& P, const T* f, T& vx, T& vy, T& vz,
                                                   T& e, int I, uint32_t id, uint32_t step,
                                                   const PhiloxRoundKeys& rk, CollideTally& t) {
-  static_assert(!kFast || sizeof(T) == 4 || sizeof(T) == 8, "float or double");
   T alpha = P.alpha, nu = P.nu_ref, ttr, trot, evr;
   bool cl;
   std::conditional_t<kFast, AlphaParts<T>, int> ap_;
