@@ -519,49 +519,6 @@ ch_collide(int c0, int ny, double dy, int recon, double dt, const ChCellT<S>* __
 constexpr int kFB = 256;         // threads per cell
 constexpr int kFW = kFB / 32;
 
-// Totals over the block of the ten sums a[] of every thread (FP64 kinds) into
-// tot[0..9] in shared memory: the warps by halving, their totals by ten lanes
-// of warp 0 (ten lanes of each of four warps for derivative numbers).
-__device__ __forceinline__ void block_ten(double* a, double (*red)[kFW][10], double* tot) {
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int at = halve_totals<10>(a);
-  if (at >= 0) red[0][wid][at] = a[0];
-  __syncthreads();
-  if (wid == 0 && lane < 10) {
-    double v = red[0][0][lane];
-    for (int w = 1; w < kFW; ++w) v += red[0][w][lane];
-    tot[lane] = v;
-  }
-  __syncthreads();
-}
-template <typename V>
-__device__ __forceinline__ void block_ten(dual::Dual<V>* a, double (*red)[kFW][10],
-                                          dual::Dual<V>* tot) {
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k <= kND; ++k) {
-    double b[10];
-#pragma unroll
-    for (int i = 0; i < 10; ++i) b[i] = k == 0 ? a[i].v : a[i].d[k == 0 ? 0 : k - 1];
-    const int at = halve_totals<10>(b);
-    if (at >= 0) red[k][wid][at] = b[0];
-  }
-  __syncthreads();
-  if (wid <= kND && lane < 10) {
-    double v = red[wid][0][lane];
-    for (int w = 1; w < kFW; ++w) v += red[wid][w][lane];
-    if (wid == 0) tot[lane].v = v;
-    else tot[lane].d[wid - 1] = v;
-  }
-  __syncthreads();
-}
-
-// The sums of an FP32 state keep the order and precision of one warp walking
-// the cell with its lanes 32 apart: the block stages the particles, warp 0 adds
-// them up.  FP64 states are summed by all threads.
-template <typename T>
-constexpr bool kOneWarpSums = std::is_same<T, float>::value || std::is_same<T, F3>::value;
-
 template <typename T, typename S>
 __global__ void __launch_bounds__(kFB)
 ch_finish(int ny, ChCellT<S>* __restrict__ cells, const T* __restrict__ cx,
@@ -569,7 +526,11 @@ ch_finish(int ny, ChCellT<S>* __restrict__ cells, const T* __restrict__ cx,
           int* __restrict__ lev, long long* dstep, Species sp, uint32_t k0, uint32_t k1,
           uint32_t* flags, unsigned long long* counters, int sampling, double* __restrict__ acc,
           double* wallmom) {
-  constexpr bool one = kOneWarpSums<T>;
+  constexpr bool one = kOneWarpSums<T>;   // the block stages the particles, warp 0 adds them up
+  using Q = typename dual::Lanes<S>::type;
+  constexpr int nl = dual::Lanes<S>::n;
+  using dual::lane_part;
+  using dual::put_part;
   __shared__ T stage[4][one ? kFB : 1];
   __shared__ double red[std::is_same<S, double>::value ? 1 : 1 + kND][kFW][10];
   __shared__ S ten[10];
@@ -641,7 +602,7 @@ ch_finish(int ny, ChCellT<S>* __restrict__ cells, const T* __restrict__ cx,
       }
       __syncthreads();
     } else {
-      block_ten(a, red, ten);
+      block_totals<10, kFW>(a, red, ten);
     }
     // the vibrational +-1 correction | what of the rescale does not need it
     const double R = gasR(sp), Rth = R * sp.theta_v;
@@ -659,67 +620,108 @@ ch_finish(int ny, ChCellT<S>* __restrict__ cells, const T* __restrict__ cx,
         if (draws) atomicAdd(&counters[C_VIB_DRAWS], (unsigned long long)draws);
         levsum += net;
       }
-    } else if (t == 32) {
+    } else if (t >= 32 && t < 32 + nl) {
+      const int i = t - 32;
+      const Q er_star = lane_part(ten[9], i) * d_rcp((double)N);
+      const Q r = er_star > 0.0 ? c_div(lane_part(cs.e_rot_tgt, i), er_star) : Q(1.0);
+      put_part(pend[7], r, i);
+      put_part(e_rot_new, r * er_star, i);
+    } else if (t >= 64 && t < 64 + nl) {
+      const int i = t - 64;
       const double invN = d_rcp((double)N);
-      const S er_star = ten[9] * invN;
-      pend[7] = er_star > 0.0 ? c_div(cs.e_rot_tgt, er_star) : S(1.0);
-      e_rot_new = pend[7] * er_star;
-    } else if (t == 64) {
-      const double invN = d_rcp((double)N);
-      const S m0 = ten[0] * invN, m1 = ten[1] * invN, m2 = ten[2] * invN;
-      etr_star = 0.5 * (ten[3] * invN - m0 * m0 + ten[4] * invN - m1 * m1 + ten[5] * invN - m2 * m2);
-      pend[3] = cs.U[0] + m0; pend[4] = cs.U[1] + m1; pend[5] = cs.U[2] + m2;
-    } else if (t == 96) {
-      e_sum = 0.5 * (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]) + R * cs.Trot + Rth * cs.ebar;
+      const Q m0 = lane_part(ten[0], i) * invN, m1 = lane_part(ten[1], i) * invN,
+              m2 = lane_part(ten[2], i) * invN;
+      put_part(etr_star,
+               0.5 * (lane_part(ten[3], i) * invN - m0 * m0 + lane_part(ten[4], i) * invN -
+                      m1 * m1 + lane_part(ten[5], i) * invN - m2 * m2), i);
+      put_part(pend[3], lane_part(cs.U[0], i) + m0, i);
+      put_part(pend[4], lane_part(cs.U[1], i) + m1, i);
+      put_part(pend[5], lane_part(cs.U[2], i) + m2, i);
+    } else if (t >= 96 && t < 96 + nl) {
+      const int i = t - 96;
+      put_part(e_sum,
+               0.5 * (lane_part(cs.Pi[0], i) + lane_part(cs.Pi[1], i) + lane_part(cs.Pi[2], i)) +
+                   R * lane_part(cs.Trot, i) + Rth * cs.ebar, i);
     }
     __syncthreads();
-    if (t == 0) {
+    if (t < nl) {
       const double e_vib_new = Rth * (double)levsum * d_rcp((double)N);
-      const S rad = c_div(e_sum - e_rot_new - e_vib_new, etr_star);
-      const bool neg = !(etr_star > 0.0) || !(rad > 0.0);
-      if (neg) {
+      const Q etr = lane_part(etr_star, t);
+      const Q rad = c_div(lane_part(e_sum, t) - lane_part(e_rot_new, t) - e_vib_new, etr);
+      const bool neg = !(etr > 0.0) || !(rad > 0.0);
+      if (neg && t == 0) {
         atomicOr(flags, (uint32_t)F_NEG_RADICAND);
         atomicAdd(&counters[C_NEG_RADICAND], 1ull);
       }
-      for (int i = 0; i < 3; ++i) {
-        pend[i] = cs.Un[i] = neg ? pend[3 + i] : cs.U[i];
-        cs.Us[i] = pend[3 + i];
-      }
-      pend[6] = cs.s = neg ? S(1.0) : sqrt(rad);
+      put_part(pend[6], neg ? Q(1.0) : sqrt(rad), t);
+      for (int i = 0; i < 3; ++i)
+        put_part(pend[i], neg ? lane_part(pend[3 + i], t) : lane_part(cs.U[i], t), t);
+    }
+    __syncthreads();
+    if (t < 3) {
+      cs.Un[t] = pend[t];
+      cs.Us[t] = pend[3 + t];
+    } else if (t == 32) {
+      cs.s = pend[6];
       cs.r = pend[7];
       cs.maxI = maxl + 1;
     }
-    __syncthreads();
   }
   if (sampling) {
     // time-average sums of the post-step state, reduced in a fixed order, so
     // that runs are reproducible bit for bit (gradient form: block 0 of acc
     // holds the sums, blocks 1..3 their derivatives)
-    S q[10];
-#pragma unroll
-    for (int i = 0; i < 10; ++i) q[i] = S(0.0);
-    long long sl = 0;
-    for (long long i = t; i < N; i += kFB) {
-      const long long j = off + i;
-      const S v0 = pend[0] + pend[6] * (S(cx[j]) - pend[3]);
-      const S v1 = pend[1] + pend[6] * (S(cy[j]) - pend[4]);
-      const S v2 = pend[2] + pend[6] * (S(cz[j]) - pend[5]);
-      q[0] += v0; q[1] += v1; q[2] += v2;
-      q[3] += v0 * v0; q[4] += v1 * v1; q[5] += v2 * v2;
-      q[6] += v0 * v1; q[7] += v0 * v2; q[8] += v1 * v2;
-      q[9] += pend[7] * S(er[j]);
-      if (!active) sl += lev[j];
-    }
-    block_ten(q, red, ten);
-    if (!active) {
-      sl = wsum(sl);
-      if (lane == 0 && sl) atomicAdd((unsigned long long*)&levsum, (unsigned long long)sl);
-      __syncthreads();
-    }
     double* a = acc + (size_t)c * kNAcc;
-    if (t < 10) {
-      acc_add(&a[1 + t], (size_t)ny * kNAcc + 2, ten[t]);
-    } else if (t == 32) {
+    const size_t blk = (size_t)ny * kNAcc + 2;
+    if (!one && active) {
+      // FP64 kinds: v = t + s d with d the particle's velocity about U, t = Un -
+      // s (Us - U), so the sums follow from those above (the pass over the
+      // particles was a third of the kernel in the derivative form)
+      if (t < 10 * nl) {
+        const int i = t / nl, k = t % nl;
+        const Q s = lane_part(pend[6], k), D = lane_part(ten[i], k);
+        auto shift = [&](int q) {
+          return lane_part(pend[q], k) - s * (lane_part(pend[3 + q], k) - lane_part(cs.U[q], k));
+        };
+        Q r;
+        if (i < 3) {
+          r = shift(i) * (double)N + s * D;
+        } else if (i < 9) {
+          const int x = i < 6 ? i - 3 : i < 8 ? 0 : 1, y = i < 6 ? i - 3 : i == 6 ? 1 : 2;
+          const Q tx = shift(x), ty = shift(y);
+          r = tx * ty * (double)N + s * (tx * lane_part(ten[y], k) + ty * lane_part(ten[x], k)) +
+              s * s * D;
+        } else {
+          r = lane_part(pend[7], k) * D;
+        }
+        if (k == 0) a[1 + i] += value(r);
+        if constexpr (nl > 1) a[(k + 1) * blk + 1 + i] += r.d[0];
+      }
+    } else {
+      S q[10];
+#pragma unroll
+      for (int i = 0; i < 10; ++i) q[i] = S(0.0);
+      long long sl = 0;
+      for (long long i = t; i < N; i += kFB) {
+        const long long j = off + i;
+        const S v0 = pend[0] + pend[6] * (S(cx[j]) - pend[3]);
+        const S v1 = pend[1] + pend[6] * (S(cy[j]) - pend[4]);
+        const S v2 = pend[2] + pend[6] * (S(cz[j]) - pend[5]);
+        q[0] += v0; q[1] += v1; q[2] += v2;
+        q[3] += v0 * v0; q[4] += v1 * v1; q[5] += v2 * v2;
+        q[6] += v0 * v1; q[7] += v0 * v2; q[8] += v1 * v2;
+        q[9] += pend[7] * S(er[j]);
+        if (!active) sl += lev[j];
+      }
+      block_totals<10, kFW>(q, red, ten);
+      if (!active) {
+        sl = wsum(sl);
+        if (lane == 0 && sl) atomicAdd((unsigned long long*)&levsum, (unsigned long long)sl);
+        __syncthreads();
+      }
+      if (t < 10) acc_add(&a[1 + t], blk, ten[t]);
+    }
+    if (t == 32) {
       a[0] += (double)N;
       a[11] += (double)levsum;
       if (c == 0) {

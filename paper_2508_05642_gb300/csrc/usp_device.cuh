@@ -644,7 +644,7 @@ __device__ __forceinline__ void cell_gammas(const Species& s, CellCoeffsT<S>& c,
       const double cvc = R * (xx * xx) * (iE * (1.0 + iE));
       const double dF = -(double)gv * (cvc - xv) * (double)iden;
       const double k = d_div(cvc - xv, d * (1.0 - dF));
-      for (int i = 0; i < 3; ++i) x.d[i] = Tc.d[i] * k;
+      for (int i = 0; i < (int)(sizeof(S) / sizeof(double)) - 1; ++i) x.d[i] = Tc.d[i] * k;
     }
   }
   const S idn = c_div(S(1.0), ctr + gr * R + gv * x);

@@ -61,48 +61,50 @@ __device__ inline double vpow(double x, double y) { return ::pow(x, y); }
 // a / b, and the quotients d_i / b of the derivatives
 __device__ inline float vdiv(float a, float b) { return a / b; }
 __device__ inline double vdiv(double a, double b) { return d_div(a, b); }
-__device__ inline void vdiv3(float* d, float b) { for (int i = 0; i < kND; ++i) d[i] = d[i] / b; }
-__device__ inline void vdiv3(double* d, double b) {
+template <int N>
+__device__ inline void vdivn(float (&d)[N], float b) { for (int i = 0; i < N; ++i) d[i] = d[i] / b; }
+template <int N>
+__device__ inline void vdivn(double (&d)[N], double b) {
   const double y = d_rcp(b);
-  for (int i = 0; i < kND; ++i) d[i] *= y;
+  for (int i = 0; i < N; ++i) d[i] *= y;
 }
 
-template <typename V>
+template <typename V, int N = kND>
 struct Dual {
   V v;
-  V d[kND];
-  __host__ __device__ Dual() : v(V(0)) { d[0] = d[1] = d[2] = V(0); }
-  __host__ __device__ Dual(double x) : v(V(x)) { d[0] = d[1] = d[2] = V(0); }
+  V d[N];
+  __host__ __device__ Dual() : v(V(0)) { for (int i = 0; i < N; ++i) d[i] = V(0); }
+  __host__ __device__ Dual(double x) : v(V(x)) { for (int i = 0; i < N; ++i) d[i] = V(0); }
   __host__ __device__ Dual(double x, double d0, double d1, double d2) : v(V(x)) {
     d[0] = V(d0); d[1] = V(d1); d[2] = V(d2);
   }
   // between precisions (FP32 particle values <-> FP64 cell values)
   template <typename U>
-  __host__ __device__ explicit Dual(const Dual<U>& o) : v(V(o.v)) {
-    for (int i = 0; i < kND; ++i) d[i] = V(o.d[i]);
+  __host__ __device__ explicit Dual(const Dual<U, N>& o) : v(V(o.v)) {
+    for (int i = 0; i < N; ++i) d[i] = V(o.d[i]);
   }
   __host__ __device__ explicit operator double() const { return (double)v; }
   __host__ __device__ explicit operator float() const { return (float)v; }
   __host__ __device__ explicit operator int() const { return (int)v; }
   __host__ __device__ Dual& operator+=(const Dual& b) {
     v += b.v;
-    for (int i = 0; i < kND; ++i) d[i] += b.d[i];
+    for (int i = 0; i < N; ++i) d[i] += b.d[i];
     return *this;
   }
   __host__ __device__ Dual& operator-=(const Dual& b) {
     v -= b.v;
-    for (int i = 0; i < kND; ++i) d[i] -= b.d[i];
+    for (int i = 0; i < N; ++i) d[i] -= b.d[i];
     return *this;
   }
   __host__ __device__ Dual& operator*=(const Dual& b) {
-    for (int i = 0; i < kND; ++i) d[i] = d[i] * b.v + v * b.d[i];
+    for (int i = 0; i < N; ++i) d[i] = d[i] * b.v + v * b.d[i];
     v *= b.v;
     return *this;
   }
   __device__ Dual& operator/=(const Dual& b) {
     const V q = vdiv(v, b.v);
-    for (int i = 0; i < kND; ++i) d[i] = d[i] - q * b.d[i];
-    vdiv3(d, b.v);
+    for (int i = 0; i < N; ++i) d[i] = d[i] - q * b.d[i];
+    vdivn(d, b.v);
     v = q;
     return *this;
   }
@@ -111,62 +113,89 @@ struct Dual {
 using D3 = Dual<double>;
 using F3 = Dual<float>;
 
-template <typename V>
-__host__ __device__ inline Dual<V> operator+(Dual<V> a, const Dual<V>& b) { return a += b; }
-template <typename V>
-__host__ __device__ inline Dual<V> operator-(Dual<V> a, const Dual<V>& b) { return a -= b; }
-template <typename V>
-__host__ __device__ inline Dual<V> operator*(Dual<V> a, const Dual<V>& b) { return a *= b; }
-template <typename V>
-__device__ inline Dual<V> operator/(Dual<V> a, const Dual<V>& b) { return a /= b; }
-template <typename V>
-__host__ __device__ inline Dual<V> operator+(Dual<V> a, double b) { a.v += V(b); return a; }
-template <typename V>
-__host__ __device__ inline Dual<V> operator+(double b, Dual<V> a) { a.v += V(b); return a; }
-template <typename V>
-__host__ __device__ inline Dual<V> operator-(Dual<V> a, double b) { a.v -= V(b); return a; }
-template <typename V>
-__host__ __device__ inline Dual<V> operator-(double b, const Dual<V>& a) {
-  Dual<V> r;
-  r.v = V(b) - a.v;
-  for (int i = 0; i < kND; ++i) r.d[i] = -a.d[i];
+// A cell's chains of FP64 operations run on one thread, and a warp's FP64
+// instruction takes 64 cycles whatever the number of its lanes that work.  In the
+// derivative form lane i of three carries the value and derivative i: three
+// operations for a product in place of seven.  Lanes<S>::type is that number
+// (S itself in the plain forms, one lane), lane_part and put_part convert.
+template <typename S>
+struct Lanes {
+  using type = S;
+  static constexpr int n = 1;
+};
+template <>
+struct Lanes<D3> {
+  using type = Dual<double, 1>;
+  static constexpr int n = kND;
+};
+__device__ inline double lane_part(double x, int) { return x; }
+__device__ inline Dual<double, 1> lane_part(const D3& x, int i) {
+  Dual<double, 1> r(x.v);
+  r.d[0] = x.d[i];
   return r;
 }
-template <typename V>
-__host__ __device__ inline Dual<V> operator*(Dual<V> a, double b) {
+__device__ inline void put_part(double& x, double y, int) { x = y; }
+__device__ inline void put_part(D3& x, const Dual<double, 1>& y, int i) {
+  if (i == 0) x.v = y.v;
+  x.d[i] = y.d[0];
+}
+
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator+(Dual<V, N> a, const Dual<V, N>& b) { return a += b; }
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator-(Dual<V, N> a, const Dual<V, N>& b) { return a -= b; }
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator*(Dual<V, N> a, const Dual<V, N>& b) { return a *= b; }
+template <typename V, int N>
+__device__ inline Dual<V, N> operator/(Dual<V, N> a, const Dual<V, N>& b) { return a /= b; }
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator+(Dual<V, N> a, double b) { a.v += V(b); return a; }
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator+(double b, Dual<V, N> a) { a.v += V(b); return a; }
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator-(Dual<V, N> a, double b) { a.v -= V(b); return a; }
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator-(double b, const Dual<V, N>& a) {
+  Dual<V, N> r;
+  r.v = V(b) - a.v;
+  for (int i = 0; i < N; ++i) r.d[i] = -a.d[i];
+  return r;
+}
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator*(Dual<V, N> a, double b) {
   const V c = V(b);
   a.v *= c;
-  for (int i = 0; i < kND; ++i) a.d[i] *= c;
+  for (int i = 0; i < N; ++i) a.d[i] *= c;
   return a;
 }
-template <typename V>
-__host__ __device__ inline Dual<V> operator*(double b, Dual<V> a) { return a * b; }
-template <typename V>
-__device__ inline Dual<V> operator/(Dual<V> a, double b) {
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator*(double b, Dual<V, N> a) { return a * b; }
+template <typename V, int N>
+__device__ inline Dual<V, N> operator/(Dual<V, N> a, double b) {
   const V c = V(b);
   a.v = vdiv(a.v, c);
-  vdiv3(a.d, c);
+  vdivn(a.d, c);
   return a;
 }
-template <typename V>
-__device__ inline Dual<V> operator/(double b, const Dual<V>& a) { return Dual<V>(b) / a; }
-template <typename V>
-__host__ __device__ inline Dual<V> operator-(const Dual<V>& a) {
-  Dual<V> r;
+template <typename V, int N>
+__device__ inline Dual<V, N> operator/(double b, const Dual<V, N>& a) { return Dual<V, N>(b) / a; }
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> operator-(const Dual<V, N>& a) {
+  Dual<V, N> r;
   r.v = -a.v;
-  for (int i = 0; i < kND; ++i) r.d[i] = -a.d[i];
+  for (int i = 0; i < N; ++i) r.d[i] = -a.d[i];
   return r;
 }
 
 #define USP_DUAL_CMP(op)                                                                       \
-  template <typename V>                                                                        \
-  __host__ __device__ inline bool operator op(const Dual<V>& a, const Dual<V>& b) {            \
+  template <typename V, int N>                                                                        \
+  __host__ __device__ inline bool operator op(const Dual<V, N>& a, const Dual<V, N>& b) {            \
     return a.v op b.v;                                                                         \
   }                                                                                            \
-  template <typename V>                                                                        \
-  __host__ __device__ inline bool operator op(const Dual<V>& a, double b) { return a.v op b; } \
-  template <typename V>                                                                        \
-  __host__ __device__ inline bool operator op(double a, const Dual<V>& b) { return a op b.v; }
+  template <typename V, int N>                                                                        \
+  __host__ __device__ inline bool operator op(const Dual<V, N>& a, double b) { return a.v op b; } \
+  template <typename V, int N>                                                                        \
+  __host__ __device__ inline bool operator op(double a, const Dual<V, N>& b) { return a op b.v; }
 USP_DUAL_CMP(<)
 USP_DUAL_CMP(>)
 USP_DUAL_CMP(<=)
@@ -176,94 +205,97 @@ USP_DUAL_CMP(!=)
 #undef USP_DUAL_CMP
 
 // f(a) with f'(a) = df
-template <typename V>
-__host__ __device__ inline Dual<V> chain(const Dual<V>& a, V fv, V df) {
-  Dual<V> r;
+template <typename V, int N>
+__host__ __device__ inline Dual<V, N> chain(const Dual<V, N>& a, V fv, V df) {
+  Dual<V, N> r;
   r.v = fv;
-  for (int i = 0; i < kND; ++i) r.d[i] = df * a.d[i];
+  for (int i = 0; i < N; ++i) r.d[i] = df * a.d[i];
   return r;
 }
 
-template <typename V>
-__device__ inline Dual<V> sqrt(const Dual<V>& a) {
+template <typename V, int N>
+__device__ inline Dual<V, N> sqrt(const Dual<V, N>& a) {
   const V s = vsqrt(a.v);
   return chain(a, s, s > V(0) ? vdiv(V(0.5), s) : V(0));
 }
-__device__ inline Dual<double> rcp(const Dual<double>& a) {
+template <int N>
+__device__ inline Dual<double, N> rcp(const Dual<double, N>& a) {
   const double r = d_rcp(a.v);
   return chain(a, r, -(r * r));
 }
-__device__ inline Dual<double> rsqrt(const Dual<double>& a) {
+template <int N>
+__device__ inline Dual<double, N> rsqrt(const Dual<double, N>& a) {
   const double r = d_rsqrt(a.v);
   return chain(a, r, -0.5 * r * (r * r));
 }
 // f + a b
-__device__ inline Dual<double> madd(const Dual<double>& f, const Dual<double>& a,
-                                    const Dual<double>& b) {
-  Dual<double> r;
+template <int N>
+__device__ inline Dual<double, N> madd(const Dual<double, N>& f, const Dual<double, N>& a,
+                                       const Dual<double, N>& b) {
+  Dual<double, N> r;
   r.v = fma(a.v, b.v, f.v);
-  for (int i = 0; i < kND; ++i) r.d[i] = fma(a.d[i], b.v, fma(a.v, b.d[i], f.d[i]));
+  for (int i = 0; i < N; ++i) r.d[i] = fma(a.d[i], b.v, fma(a.v, b.d[i], f.d[i]));
   return r;
 }
-template <typename V>
-__device__ inline Dual<V> log(const Dual<V>& a) { return chain(a, vlog(a.v), vdiv(V(1), a.v)); }
-template <typename V>
-__device__ inline Dual<V> log1p(const Dual<V>& a) {
+template <typename V, int N>
+__device__ inline Dual<V, N> log(const Dual<V, N>& a) { return chain(a, vlog(a.v), vdiv(V(1), a.v)); }
+template <typename V, int N>
+__device__ inline Dual<V, N> log1p(const Dual<V, N>& a) {
   return chain(a, vlog1p(a.v), V(1) / (V(1) + a.v));
 }
-template <typename V>
-__device__ inline Dual<V> exp(const Dual<V>& a) {
+template <typename V, int N>
+__device__ inline Dual<V, N> exp(const Dual<V, N>& a) {
   const V e = vexp(a.v);
   return chain(a, e, e);
 }
-template <typename V>
-__device__ inline Dual<V> expm1(const Dual<V>& a) {
+template <typename V, int N>
+__device__ inline Dual<V, N> expm1(const Dual<V, N>& a) {
   V df;
   const V e = vexpm1(a.v, df);
   return chain(a, e, df);
 }
-template <typename V>
-__device__ inline Dual<V> sinh(const Dual<V>& a) { return chain(a, vsinh(a.v), vcosh(a.v)); }
-template <typename V>
-__device__ inline Dual<V> cos(const Dual<V>& a) { return chain(a, vcos(a.v), -vsin(a.v)); }
-template <typename V>
-__device__ inline Dual<V> acos(const Dual<V>& a) {
+template <typename V, int N>
+__device__ inline Dual<V, N> sinh(const Dual<V, N>& a) { return chain(a, vsinh(a.v), vcosh(a.v)); }
+template <typename V, int N>
+__device__ inline Dual<V, N> cos(const Dual<V, N>& a) { return chain(a, vcos(a.v), -vsin(a.v)); }
+template <typename V, int N>
+__device__ inline Dual<V, N> acos(const Dual<V, N>& a) {
   const V den = vsqrt(V(1) - a.v * a.v);
   return chain(a, vacos(a.v), den > V(0) ? V(-1) / den : V(0));
 }
-template <typename V>
-__device__ inline Dual<V> cbrt(const Dual<V>& a) {
+template <typename V, int N>
+__device__ inline Dual<V, N> cbrt(const Dual<V, N>& a) {
   const V c = vcbrt(a.v);
   return chain(a, c, c != V(0) ? vdiv(c, V(3) * a.v) : V(0));
 }
-template <typename V>
-__device__ inline Dual<V> fabs(const Dual<V>& a) { return a.v < V(0) ? -a : a; }
-template <typename V>
-__device__ inline Dual<V> fmin(const Dual<V>& a, const Dual<V>& b) { return b.v < a.v ? b : a; }
-template <typename V>
-__device__ inline Dual<V> fmax(const Dual<V>& a, const Dual<V>& b) { return b.v > a.v ? b : a; }
+template <typename V, int N>
+__device__ inline Dual<V, N> fabs(const Dual<V, N>& a) { return a.v < V(0) ? -a : a; }
+template <typename V, int N>
+__device__ inline Dual<V, N> fmin(const Dual<V, N>& a, const Dual<V, N>& b) { return b.v < a.v ? b : a; }
+template <typename V, int N>
+__device__ inline Dual<V, N> fmax(const Dual<V, N>& a, const Dual<V, N>& b) { return b.v > a.v ? b : a; }
 // a^b with a > 0 (both carrying derivatives)
-template <typename V>
-__device__ inline Dual<V> pow(const Dual<V>& a, const Dual<V>& b) {
+template <typename V, int N>
+__device__ inline Dual<V, N> pow(const Dual<V, N>& a, const Dual<V, N>& b) {
   const V p = vpow(a.v, b.v);
-  Dual<V> r;
+  Dual<V, N> r;
   r.v = p;
   const V la = vlog(a.v);
-  for (int i = 0; i < kND; ++i) r.d[i] = p * (b.d[i] * la + b.v * a.d[i] / a.v);
+  for (int i = 0; i < N; ++i) r.d[i] = p * (b.d[i] * la + b.v * a.d[i] / a.v);
   return r;
 }
-template <typename V>
-__device__ inline Dual<V> pow(const Dual<V>& a, double b) {
+template <typename V, int N>
+__device__ inline Dual<V, N> pow(const Dual<V, N>& a, double b) {
   const V p = vpow(a.v, V(b));
   return chain(a, p, V(b) * vpow(a.v, V(b - 1.0)));
 }
-template <typename V>
-__device__ inline Dual<V> pow(double a, const Dual<V>& b) {
+template <typename V, int N>
+__device__ inline Dual<V, N> pow(double a, const Dual<V, N>& b) {
   const V p = vpow(V(a), b.v);
   return chain(b, p, p * vlog(V(a)));
 }
-template <typename V>
-__device__ inline V value(const Dual<V>& a) { return a.v; }
+template <typename V, int N>
+__device__ inline V value(const Dual<V, N>& a) { return a.v; }
 
 }  // namespace dual
 
@@ -276,8 +308,8 @@ __device__ inline float value(float a) { return a; }
 
 // A quantity held at its value in the gradient form: its derivative is
 // dropped (the identity in the plain forms).
-template <typename V>
-__device__ inline dual::Dual<V> held(const dual::Dual<V>& a) { return dual::Dual<V>(a.v); }
+template <typename V, int N>
+__device__ inline dual::Dual<V, N> held(const dual::Dual<V, N>& a) { return dual::Dual<V, N>(a.v); }
 __device__ inline double held(double a) { return a; }
 __device__ inline float held(float a) { return a; }
 

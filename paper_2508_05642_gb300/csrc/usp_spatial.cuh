@@ -759,15 +759,127 @@ __global__ void ch_coeffs(int ny, double F_num, double vol, const double* __rest
   tally_flush(tal, flags, counters);
 }
 
-// moments and coefficients of the channel's cells, one block per cell: one warp
-// sums, then the parts of the coefficients that do not need one another run
-// on different warps, that is on different quarters of the SM
+// Totals over a block of W warps of the M sums a[] of every thread (FP64 kinds)
+// into tot[0 .. M-1] in shared memory: the warps by halving, their totals by M
+// lanes of warp 0 (M lanes of each of four warps for derivative numbers).
+template <int M, int W>
+__device__ __forceinline__ void block_totals(double* a, double (*red)[W][M], double* tot) {
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int at = halve_totals<M>(a);
+  if (at >= 0) red[0][wid][at] = a[0];
+  __syncthreads();
+  if (wid == 0 && lane < M) {
+    double v = red[0][0][lane];
+    for (int w = 1; w < W; ++w) v += red[0][w][lane];
+    tot[lane] = v;
+  }
+  __syncthreads();
+}
+template <int M, int W>
+__device__ __forceinline__ void block_totals(D3* a, double (*red)[W][M], D3* tot) {
+  static_assert(W > kND, "a warp per component");
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k <= kND; ++k) {
+    double b[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) b[i] = k == 0 ? a[i].v : a[i].d[k == 0 ? 0 : k - 1];
+    const int at = halve_totals<M>(b);
+    if (at >= 0) red[k][wid][at] = b[0];
+  }
+  __syncthreads();
+  if (wid <= kND && lane < M) {
+    double v = red[wid][0][lane];
+    for (int w = 1; w < W; ++w) v += red[wid][w][lane];
+    if (wid == 0) tot[lane].v = v;
+    else tot[lane].d[wid - 1] = v;
+  }
+  __syncthreads();
+}
+
+// The sums of an FP32 state keep the order and precision of one warp walking
+// the cell with its lanes 32 apart.  FP64 states are summed by all threads of a
+// block: one warp uses one of the four FP64 pipes of its SM, and in the
+// derivative form its 7 passes over 200 particles were half of ch_prepare.
+template <typename T>
+constexpr bool kOneWarpSums = std::is_same<T, float>::value || std::is_same<T, F3>::value;
+
+// Moments of cell c by the block of kPB threads, with the record's fields that
+// moments_of_cells sets (T_vib apart).
+constexpr int kPB = 128;
+template <typename T>
+__device__ void block_moments(int c, const long long* __restrict__ off, const T* __restrict__ cx,
+                              const T* __restrict__ cy, const T* __restrict__ cz,
+                              const T* __restrict__ er, const int* __restrict__ lev,
+                              ChCellT<T>* __restrict__ cells, const Species& sp, BlockTally& tal) {
+  constexpr int K = sizeof(T) / sizeof(double);   // value and derivatives
+  __shared__ double red4[K][kPB / 32][4], red6[K][kPB / 32][6];
+  __shared__ T tot[4], cen[6];
+  __shared__ unsigned long long levels;
+  const int t = threadIdx.x;
+  const long long b = off[c], e = off[c + 1], N = e - b;
+  if (t == 0) levels = 0;
+  T a[4] = {T(0), T(0), T(0), T(0)};
+  long long al = 0;
+  for (long long j = b + t; j < e; j += kPB) {
+    a[0] += cx[j]; a[1] += cy[j]; a[2] += cz[j]; a[3] += er[j];
+    al += lev[j];
+  }
+  block_totals<4, kPB / 32>(a, red4, tot);
+  al = wsum(al);
+  if ((t & 31) == 0 && al) atomicAdd(&levels, (unsigned long long)al);
+  const double inv = N > 0 ? d_rcp((double)N) : 0.0;
+  const T m0 = tot[0] * inv, m1 = tot[1] * inv, m2 = tot[2] * inv;
+  T p[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+  for (long long j = b + t; j < e; j += kPB) {
+    const T C0 = cx[j] - m0, C1 = cy[j] - m1, C2 = cz[j] - m2;
+    p[0] = madd(p[0], C0, C0); p[1] = madd(p[1], C1, C1); p[2] = madd(p[2], C2, C2);
+    p[3] = madd(p[3], C0, C1); p[4] = madd(p[4], C0, C2); p[5] = madd(p[5], C1, C2);
+  }
+  block_totals<6, kPB / 32>(p, red6, cen);
+  ChCellT<T>& cs = cells[c];
+  // the components of the fields, one per thread
+  const double* f4 = reinterpret_cast<const double*>(tot);
+  const double* f6 = reinterpret_cast<const double*>(cen);
+  if (t < 3 * K) {
+    reinterpret_cast<double*>(cs.U)[t] = f4[t] * inv;
+  } else if (t >= 32 && t < 32 + 6 * K) {
+    if (N >= 2) reinterpret_cast<double*>(cs.Pi)[t - 32] = f6[t - 32] * inv;
+  } else if (t >= 64 && t < 64 + K) {
+    const int k = t - 64;
+    if (N >= 2)
+      reinterpret_cast<double*>(&cs.Ttr)[k] =
+          (f6[k] + f6[K + k] + f6[2 * K + k]) * (inv * (sp.iR * (1.0 / 3.0)));
+  } else if (t >= 96 && t < 96 + K) {
+    if (N >= 2) reinterpret_cast<double*>(&cs.Trot)[t - 96] = f4[3 * K + t - 96] * (inv * sp.iR);
+  } else if (t == 31) {
+    cs.off = b;
+    cs.N = N;
+    cs.active = cs.usable = N >= 2;
+    // identity pending rescale until the cell is updated
+    for (int i = 0; i < 3; ++i) { cs.Un[i] = T(0.0); cs.Us[i] = T(0.0); }
+    cs.s = T(1.0);
+    cs.r = T(1.0);
+    if (N >= 2) cs.ebar = (double)(long long)levels * inv;
+    else tally_add(tal, C_SKIPPED_CELLS, 1ull);
+  }
+}
+
+// moments and coefficients of the channel's cells, one block per cell: the
+// sums, then the parts of the coefficients that do not need one another on
+// different warps, that is on different quarters of the SM (64 cells of 200
+// particles in the derivative form: PREP_US us; one warp's sums and whole
+// derivative numbers on one thread 52 us)
 template <typename T, typename S>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kPB)
 ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T* __restrict__ cy,
            const T* __restrict__ cz, const T* __restrict__ er, const int* __restrict__ lev,
            ChCellT<S>* __restrict__ cells, Species sp, double F_num, double vol, double dt, S omega,
            S zrot, uint32_t* flags, unsigned long long* counters) {
+  using Q = typename dual::Lanes<S>::type;
+  constexpr int nl = dual::Lanes<S>::n;
+  using dual::lane_part;
+  using dual::put_part;
   __shared__ BlockTally tal;
   __shared__ CellCoeffsT<S> k;
   __shared__ S xw;
@@ -775,21 +887,47 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
   tally_init(tal);
   const int c = blockIdx.x, t = threadIdx.x;
   ChCellT<S>& cs = cells[c];
-  if (t < 32)
+  if constexpr (!kOneWarpSums<T>)
+    block_moments(c, off, cx, cy, cz, er, lev, cells, sp, tal);
+  else if (t < 32)
     moments_of_cells<T, S>(c, 1, c + 1, 1, off, nullptr, cx, cy, cz, er, lev, cells, sp, nullptr,
                            (T*)nullptr, nullptr, tal);
   __syncthreads();
   if (cs.active && vol > 0.0) {        // uniform over the block
-    if (t == 0) {
-      cs.n = (double)cs.N * F_num / vol;
-      cell_mu_p<S>(sp, cs.n, cs.Ttr, omega, k.mu_p, xw);
+    if (t < nl) {
+      const double n = (double)cs.N * F_num / vol;
+      Q mu, x;
+      cell_mu_p<Q>(sp, n, lane_part(cs.Ttr, t), lane_part(omega, t), mu, x);
+      put_part(k.mu_p, mu, t);
+      put_part(xw, x, t);
+      if (t == 0) cs.n = n;
     } else if (t == 32) {
       vib = vib_state(sp, cs.ebar);
       k.Pr = S(cell_prandtl(vib));
+      if (!kOneWarpSums<T>) cs.Tvib = vib.Tvib;
     }
     __syncthreads();
-    if (t == 0) cell_alpha<S>(k, dt);
-    else if (t == 32) cell_gammas<S>(sp, k, omega, zrot, dt, cs.Ttr, cs.Trot, vib, xw);
+    CellCoeffsT<Q> q;
+    if (t < nl) {
+      q.mu_p = lane_part(k.mu_p, t);
+      q.Pr = lane_part(k.Pr, t);
+      cell_alpha<Q>(q, dt);
+      put_part(k.B, q.B, t);
+      put_part(k.alpha, q.alpha, t);
+      put_part(k.nu_ref, q.nu_ref, t);
+      if (t == 0) k.ok = q.ok;
+    } else if (t >= 32 && t < 32 + nl) {
+      const int i = t - 32;
+      q.mu_p = lane_part(k.mu_p, i);
+      cell_gammas<Q>(sp, q, lane_part(omega, i), lane_part(zrot, i), dt, lane_part(cs.Ttr, i),
+                     lane_part(cs.Trot, i), vib, lane_part(xw, i));
+      put_part(k.g_tr_rot, q.g_tr_rot, i);
+      put_part(k.g_tr_vib, q.g_tr_vib, i);
+      put_part(k.g_rot_vib, q.g_rot_vib, i);
+      put_part(k.e_rot_tgt, q.e_rot_tgt, i);
+      put_part(k.e_vib_tgt, q.e_vib_tgt, i);
+      if (i == 0) k.tgt_clamped = q.tgt_clamped;
+    }
     __syncthreads();
     if (t == 0) put_coeffs<S>(cs, k, tal);
   } else if (t == 0 && cs.active) {
