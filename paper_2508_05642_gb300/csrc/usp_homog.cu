@@ -83,7 +83,7 @@ struct CellSums {
   unsigned long long I;      // sum of levels after the collision
   long long net;             // net change of the level sum by the +-1 correction
   int maxI;                  // largest level after the collision
-  int pad_;
+  int top;                   // FP64 form: largest level after the correction
 };
 
 struct Tile {
@@ -1161,11 +1161,13 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 // acceptance of draw j is decided exactly as in the one-at-a-time loop: a
 // decrement on particle k is accepted iff fewer than lev[k] earlier accepted
 // decrements in the round hit k.  The net level change goes to sums[c].net.
-// Returns the net change (every lane).
+// Returns the net change (every lane).  kTop: raises top to the largest level that
+// an increment reaches (a particle can be picked more than once).
+template <bool kTop>
 __device__ __forceinline__ long long
 level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long sumI,
                int* __restrict__ lev, uint32_t* flags, unsigned long long* counters, uint32_t k0,
-               uint32_t k1) {
+               uint32_t k1, int& top) {
   const int lane = threadIdx.x & 31;
   const double Rth = gasR(sp) * sp.theta_v;
   const long long N = cs.N;
@@ -1231,7 +1233,11 @@ level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long
       const int order = __popc(am & lanemask_lt());
       const bool eff = accept && order < take;
       __syncwarp();
-      if (eff) atomicAdd(&lv[k], down ? -1 : 1);
+      if (kTop && !down) {
+        if (eff) top = max(top, atomicAdd(&lv[k], 1) + 1);
+      } else if (eff) {
+        atomicAdd(&lv[k], down ? -1 : 1);
+      }
       __syncwarp();
       long long used = 32;
       if (take == need && take > 0) {
@@ -1270,9 +1276,11 @@ level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long
     if (remaining != 0) atomicOr(flags, (uint32_t)F_VIB_LOOP_CAP);
     if (draws) atomicAdd(&counters[C_VIB_DRAWS], (unsigned long long)draws);
   }
+  if (kTop) top = __reduce_max_sync(0xffffffffu, top);
   return net;
 }
 
+template <bool kTop>
 __global__ void __launch_bounds__(128, 8)
 levelfix_kernel(Species sp, int c0, int c1, const CellState* __restrict__ cells,
                 CellSums* __restrict__ sums, int* __restrict__ lev, uint32_t* flags,
@@ -1282,8 +1290,13 @@ levelfix_kernel(Species sp, int c0, int c1, const CellState* __restrict__ cells,
   if (c >= c1) return;
   const CellState& cs = cells[c];
   if (!cs.active) return;
-  const long long net = level_fix_cell(sp, c, cs, sums[c].I, lev, flags, counters, k0, k1);
-  if (lane == 0) sums[c].net = net;
+  int top = sums[c].maxI;
+  const long long net =
+      level_fix_cell<kTop>(sp, c, cs, sums[c].I, lev, flags, counters, k0, k1, top);
+  if (lane == 0) {
+    sums[c].net = net;
+    if (kTop) sums[c].top = top;
+  }
 }
 
 // Rotational and velocity rescale factors of Sec. 4.C, the moments of the
@@ -1342,7 +1355,7 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
   cs.s = s;
   cs.r = r;
   cs.step += 1;
-  cs.maxI = S.maxI + 1;   // the +-1 correction can raise the largest level by one
+  cs.maxI = sizeof(T) == 8 ? S.top : S.maxI + 1;
   CollideParams<T> P;
   write_params<T>(sp, cs, P, flags, counters);
   cells[c] = cs;
@@ -1392,8 +1405,13 @@ few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
   const bool lead = (t & 31) == 0;
   // the +-1 correction | the sums' part of cellupdate_kernel
   if (w == 0) {
-    const long long net = level_fix_cell(sp, c, cs, S.I, lev, flags, counters, k0, k1);
-    if (lead) S.net = net;
+    int top = S.maxI;
+    const long long net =
+        level_fix_cell<sizeof(T) == 8>(sp, c, cs, S.I, lev, flags, counters, k0, k1, top);
+    if (lead) {
+      S.net = net;
+      S.top = top;
+    }
   } else if (t == 32) {
     const double in = d_rcp((double)cs.N);
     er_star = S.v[9] * in;
@@ -1434,7 +1452,7 @@ few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
     cs.Trot = e_rot_new * sp.iR;
     cs.s = sc;
     cs.step += 1;
-    cs.maxI = S.maxI + 1;
+    cs.maxI = sizeof(T) == 8 ? S.top : S.maxI + 1;
     cell_mu_p<double>(sp, cs.ndens, cs.Ttr, sp.omega, K.mu_p, xw);
   } else if (t == 32) {
     cs.ebar = sumI * invN;
@@ -2141,7 +2159,7 @@ int launch_step(usp_ctx* c, const CellRange& r) {
   }
   const int warps_per_block = 4;
   const int blocks = (n + warps_per_block - 1) / warps_per_block;
-  levelfix_kernel<<<blocks, 32 * warps_per_block, 0, c->stream>>>(
+  levelfix_kernel<sizeof(T) == 8><<<blocks, 32 * warps_per_block, 0, c->stream>>>(
       c->sp, r.c0, r.c1, c->cells, c->sums, c->lev, c->flags, c->counters, key0(c), key1(c));
   CK(cudaGetLastError());
   // one warp per block: the cells' FP64 work spreads over all SMs' FP64 pipes
