@@ -1265,7 +1265,7 @@ pl_sample(int ncell, const long long* __restrict__ off, const double* __restrict
 // which so carry less rounding than with one FP64 operation per term.  Cells
 // whose values have no such E (infinities, NaN, or a component's largest value
 // outside 2^-27 .. 2^53 and not 0) take the FP64 sums.  8.5 million particles in 422,730 cells:
-// FP64 274 us, this 147 us.
+// FP64 274 us, this SAMPLE_US us.
 constexpr int kFold = 32;   // particles per fold, kFold / kCL per lane
 // 1.5 2^k
 __device__ __forceinline__ float split_point(int k) {
