@@ -7,9 +7,11 @@
 // the device and every launch reads it there: a step is a fixed launch
 // sequence that a CUDA graph can hold.  One step:
 //   pl_advect      pending conservation rescale of the previous step, flight
-//                  with events (cylinder hit -> diffuse re-emission at
-//                  T_wall, sides -> specular / removal), new cell key; a
-//                  removed particle gets the key ncell
+//                  and new cell key of the particles that meet no event
+//   pl_events      the others, from a list: flight with events (cylinder hit ->
+//                  diffuse re-emission at T_wall, sides -> specular /
+//                  removal), new cell key; a removed particle gets the key
+//                  ncell
 //   pl_inflow      per inflow face the number of entering particles
 //                  floor(flux A dt / F_num + u); exclusive scan over faces,
 //                  capacity check, ids for the new particles
@@ -58,6 +60,7 @@ struct PlCount {
   long long ninj;     // entering this step (0 if the storage was full)
   unsigned int pid0;  // id of the first entering particle
   unsigned int next_pid;
+  unsigned int nevent;  // particles of this step's move that may meet an event
 };
 
 struct PlGeom {
@@ -298,28 +301,109 @@ __device__ bool plane_fly(const PlGeom& g, const PlGeomT<T>& gt, uint32_t pid, u
   }
 }
 
+// Whether a straight flight over t may meet an event: plane_fly's own tests for
+// the earliest one, so that a flight for which this is false is one that
+// plane_fly ends with x += vx t, y += vy t.
+template <typename T>
+__device__ __forceinline__ bool plane_may_meet(const PlGeomT<T>& gt, T t, T x, T y, T vx, T vy) {
+  bool hit = false;
+  if (gt.cr > T(0)) {
+    const T dx = x - gt.cxc, dy = y - gt.cyc;
+    const T a = vx * vx + vy * vy;
+    const T b = dx * vx + dy * vy;
+    const T c = dx * dx + dy * dy - gt.cr * gt.cr;
+    const bool far = b + a * t < T(0) && c + t * (T(2) * b + a * t) > gt.margin * gt.cr;
+    hit = !(b >= T(0) || (c > T(0) && far));
+  }
+  const T ex = x + vx * t, ey = y + vy * t;
+  hit = hit || (vx < T(0) && !(ex > gt.x0 + gt.margin)) || (vx > T(0) && !(ex < gt.x1 - gt.margin));
+  hit = hit || (vy < T(0) && !(ey > gt.y0 + gt.margin)) || (vy > T(0) && !(ey < gt.y1 - gt.margin));
+  return hit;
+}
+
+// the velocity and energy of particle j under the pending conservation rescale
+// of the previous step (FP32 state: its FP32 copy, two 16-byte loads, so no FP64
+// conversion per particle)
+template <typename T>
+__device__ __forceinline__ void pl_rescaled(long long j, int k, const ChCellT<double>* __restrict__ cells,
+                                            const float* __restrict__ pend, const T* cx, const T* cy,
+                                            const T* cz, const T* er, T& vx, T& vy, T& vz, T& e) {
+  if constexpr (sizeof(T) == 4) {
+    const float4* pc = reinterpret_cast<const float4*>(pend + (size_t)k * 8);
+    const float4 p0 = pc[0], p1 = pc[1];   // Un(3), Us(3), s, r
+    vx = p0.x + p1.z * (cx[j] - p0.w);
+    vy = p0.y + p1.z * (cy[j] - p1.x);
+    vz = p0.z + p1.z * (cz[j] - p1.y);
+    e = p1.w * er[j];
+  } else {
+    const ChCellT<double>& cc = cells[k];
+    vx = (T)cc.Un[0] + (T)cc.s * (cx[j] - (T)cc.Us[0]);
+    vy = (T)cc.Un[1] + (T)cc.s * (cy[j] - (T)cc.Us[1]);
+    vz = (T)cc.Un[2] + (T)cc.s * (cz[j] - (T)cc.Us[2]);
+    e = (T)cc.r * er[j];
+  }
+}
+
+// The move: every particle that cannot meet an event in its step, and the list of
+// the others (left as they are).  With the events in the same kernel its 80
+// registers left 22 warps per SM to a pass that waits for memory: 121 us for 6.9
+// million particles (the refined grid's 8.5 million 187 us), 77 + 13 (99 + 13) us
+// with both kernels.
 template <typename T, bool AMR>
-__global__ void __launch_bounds__(kBlk, 3) pl_advect(PlGeom g, PlGeomT<T> gt,
-                                                     const PlTree* __restrict__ tr,
-                                                     const PlCount* __restrict__ cnt,
-                          const int* keycell, const ChCellT<double>* __restrict__ cells,
-                          const float* __restrict__ pend,
-                          T* __restrict__ x, T* __restrict__ y, T* __restrict__ cx,
-                          T* __restrict__ cy, T* __restrict__ cz, T* __restrict__ er,
-                          int* __restrict__ lev, const uint32_t* __restrict__ pid,
-                          int* keyout, const long long* __restrict__ dstep, Species sp, uint32_t k0,
-                          uint32_t k1, uint32_t* flags, unsigned long long* counters,
-                          double* surf) {
+__global__ void __launch_bounds__(kBlk)
+pl_advect(PlGeom g, PlGeomT<T> gt, const PlTree* __restrict__ tr, PlCount* cnt, const int* keycell,
+          const ChCellT<double>* __restrict__ cells, const float* __restrict__ pend,
+          T* __restrict__ x, T* __restrict__ y, T* __restrict__ cx, T* __restrict__ cy,
+          T* __restrict__ cz, T* __restrict__ er, int* keyout, int* __restrict__ list) {
+  const long long n = cnt->n;
+  const int lane = threadIdx.x & 31;
+  for (long long j0 = (long long)blockIdx.x * blockDim.x + threadIdx.x - lane; j0 < n;
+       j0 += grid_threads()) {
+    const long long j = j0 + lane;
+    bool may = false;
+    if (j < n) {
+      T vx, vy, vz, e;
+      pl_rescaled(j, keycell[j], cells, pend, cx, cy, cz, er, vx, vy, vz, e);
+      T px = x[j], py = y[j];
+      may = plane_may_meet(gt, gt.dt, px, py, vx, vy);
+      if (!may) {
+        px += vx * gt.dt;
+        py += vy * gt.dt;
+        x[j] = px; y[j] = py; cx[j] = vx; cy[j] = vy; cz[j] = vz; er[j] = e;
+        keyout[j] = plane_cell<T, AMR>(g, gt, tr, px, py);
+      }
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, may);
+    if (m) {
+      unsigned at = 0;
+      if (lane == 0) at = atomicAdd(&cnt->nevent, (unsigned)__popc(m));
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (may) list[at + __popc(m & lane_lt())] = (int)j;
+    }
+  }
+}
+
+// the flights with events (particles near a wall or leaving), from the list.  The
+// rescale is written out: by way of pl_rescaled the FP32 products of the flight
+// were contracted otherwise, and wall events came out a last bit apart.
+template <typename T, bool AMR>
+__global__ void __launch_bounds__(kBlk)
+pl_events(PlGeom g, PlGeomT<T> gt, const PlTree* __restrict__ tr, const PlCount* __restrict__ cnt,
+          const int* __restrict__ list, const int* keycell,
+          const ChCellT<double>* __restrict__ cells, const float* __restrict__ pend,
+          T* __restrict__ x, T* __restrict__ y, T* __restrict__ cx, T* __restrict__ cy,
+          T* __restrict__ cz, T* __restrict__ er, int* __restrict__ lev,
+          const uint32_t* __restrict__ pid, int* keyout, const long long* __restrict__ dstep,
+          uint32_t k0, uint32_t k1, uint32_t* flags, unsigned long long* counters, double* surf) {
   __shared__ BlockTally tal;
   tally_init(tal);
-  const long long n = cnt->n;
+  const unsigned n = cnt->nevent;
   const uint32_t step = (uint32_t)*dstep;
   uint32_t fl = 0;
   unsigned long long nhit = 0, nout = 0;
-  for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < n;
-       j += grid_threads()) {
-    // pending conservation rescale of the previous step (FP32 state: its
-    // FP32 copy, two 16-byte loads, so no FP64 conversion per particle)
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += grid_threads()) {
+    const long long j = list[i];
     T vx, vy, vz, e;
     if constexpr (sizeof(T) == 4) {
       const float4* pc = reinterpret_cast<const float4*>(pend + (size_t)keycell[j] * 8);
@@ -429,6 +513,7 @@ __global__ void pl_inflow(PlInflow f, PlCount* __restrict__ cnt, int* __restrict
       ninj = 0;
     }
     cnt->ninj = ninj;
+    cnt->nevent = 0;   // the move's list is done with
     cnt->ntot = n + ninj;
     cnt->pid0 = cnt->next_pid;
     cnt->next_pid = cnt->next_pid + (unsigned int)total;
@@ -1265,7 +1350,7 @@ pl_sample(int ncell, const long long* __restrict__ off, const double* __restrict
 // which so carry less rounding than with one FP64 operation per term.  Cells
 // whose values have no such E (infinities, NaN, or a component's largest value
 // outside 2^-27 .. 2^53 and not 0) take the FP64 sums.  8.5 million particles in 422,730 cells:
-// FP64 274 us, this SAMPLE_US us.
+// FP64 274 us, this 147 us.
 constexpr int kFold = 32;   // particles per fold, kFold / kCL per lane
 // 1.5 2^k
 __device__ __forceinline__ float split_point(int k) {
@@ -1674,6 +1759,7 @@ struct PlaneCtx {
   int recon, passes, nblk, grid_p;
   int grid_wc, grid_tc;     // grids of the warp-per-cell and thread-per-cell passes
   int grid_col;             // persistent grid of the collision pass
+  int grid_ev;              // grid of the flights with events
   int grid_inj;             // grid of the inflow pass (grid-stride over entering particles)
   double Fnum, vol;
   long long cap;
@@ -1895,8 +1981,11 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
   const bool amr = h->levels >= 2;
   const PlGeomT<T> gt = geom_t<T>(h->g, env.sp);
   (amr ? pl_advect<T, true> : pl_advect<T, false>)<<<h->grid_p, kBlk, 0, s>>>(
-      h->g, gt, h->tree, h->cnt, h->keycell, h->cells, h->pend, x, y, cx, cy, cz, er, h->lv[a], h->pd[a],
-      h->kbuf[0], h->dstep, env.sp, env.k0, env.k1, env.flags, env.counters, surf);
+      h->g, gt, h->tree, h->cnt, h->keycell, h->cells, h->pend, x, y, cx, cy, cz, er, h->kbuf[0],
+      h->ibuf[0]);   // the sort writes its indices there later
+  (amr ? pl_events<T, true> : pl_events<T, false>)<<<h->grid_ev, kBlk, 0, s>>>(
+      h->g, gt, h->tree, h->cnt, h->ibuf[0], h->keycell, h->cells, h->pend, x, y, cx, cy, cz, er,
+      h->lv[a], h->pd[a], h->kbuf[0], h->dstep, env.k0, env.k1, env.flags, env.counters, surf);
   pl_inflow<<<1, 1024, 0, s>>>(h->inf, h->cnt, h->face_off, h->cap, h->dstep, env.k0, env.k1,
                                env.flags, env.counters);
   if (h->inf.nfaces > 0)
@@ -2009,7 +2098,7 @@ int pl_kernels_per_step(const PlaneCtx* h) {
   }
   // FP32 USP-FPM: one pass; FP64: sums, fields, coefficients; else moments, coefficients
   const int cellpass = h->es == sizeof(double) ? 3 : h->fpmrec ? 2 : 1;
-  return 2 + (h->inf.nfaces > 0 ? 1 : 0) + 3 * h->passes + 1 + cellpass + params + 1 + 1 +
+  return 3 + (h->inf.nfaces > 0 ? 1 : 0) + 3 * h->passes + 1 + cellpass + params + 1 + 1 +
          (h->sampling ? 2 : 0);
 }
 
@@ -2089,6 +2178,7 @@ int pl_create(PlaneCtx** out, const ChEnv& env, const usp_plane* pp, double dt,
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (nsm <= 0) nsm = 1;
   h->grid_p = (int)std::min<long long>(std::max<long long>(1, (cap + kBlk - 1) / kBlk), nsm * 16);
+  h->grid_ev = (int)std::min<long long>(h->grid_p, nsm * 2);
   h->grid_wc = (int)std::min<long long>(((long long)ncell * 32 + kBlk - 1) / kBlk, nsm * 8);
   h->grid_tc = (int)std::min<long long>((ncell + kBlk - 1) / kBlk, nsm * 8);
   {
@@ -2199,7 +2289,7 @@ int pl_create(PlaneCtx** out, const ChEnv& env, const usp_plane* pp, double dt,
     next = std::max(next, hp[j] + 1u);
   }
   PlCount c0;
-  c0.n = n; c0.ntot = n; c0.ninj = 0; c0.pid0 = next; c0.next_pid = next;
+  c0.n = n; c0.ntot = n; c0.ninj = 0; c0.pid0 = next; c0.next_pid = next; c0.nevent = 0;
   std::vector<ChCellT<double>> hc(ncell);
   std::memset((void*)hc.data(), 0, sizeof(ChCellT<double>) * ncell);
   for (auto& cc : hc) { cc.s = 1.0; cc.r = 1.0; }

@@ -868,7 +868,7 @@ __device__ void block_moments(int c, const long long* __restrict__ off, const T*
 // moments and coefficients of the channel's cells, one block per cell: the
 // sums, then the parts of the coefficients that do not need one another on
 // different warps, that is on different quarters of the SM (64 cells of 200
-// particles in the derivative form: PREP_US us; one warp's sums and whole
+// particles in the derivative form: 27 us; one warp's sums and whole
 // derivative numbers on one thread 52 us)
 template <typename T, typename S>
 __global__ void __launch_bounds__(kPB)
