@@ -592,21 +592,18 @@ __device__ __forceinline__ S c_cbrt(const S& a) { return cbrt(a); }
 
 // The coefficients in the parts that depend on one another: mu / p and xw = (T /
 // T_ref)^omega; A, B, alpha and nu (from mu / p and Pr); the gamma coefficients
-// and the targets (from mu / p and xw).  omega and zrot are the independent
-// variables of the derivative form.
+// and the targets (from mu / p, xw and tauf = tau_c / (mu / p)).
+__device__ __forceinline__ void cell_mu_p(const Species& s, double n, double Ttr, double& mu_p,
+                                          double& xw) {
+  xw = d_exp(s.omega * d_log(Ttr * s.iT_ref));
+  mu_p = s.mu_ref0 * xw * d_rcp(n * kB * Ttr);
+}
+// mu at T_ref through omega (derivative form)
 template <typename S>
-__device__ __forceinline__ void cell_mu_p(const Species& s, double n, const S& Ttr, const S& omega,
-                                          S& mu_p, S& xw) {
-  if constexpr (sizeof(S) == sizeof(double)) {   // plain forms: species constants
-    xw = d_exp(s.omega * d_log(Ttr * s.iT_ref));
-    mu_p = s.mu_ref0 * xw * d_rcp(n * kB * Ttr);
-  } else {                                        // derivative form: through omega
-    const double ca = s.c_alpha;
-    xw = exp(omega * log(Ttr / s.T_ref));
-    const S mu_ref = 5.0 * (ca + 1.0) * (ca + 2.0) * sqrt(s.m * kB * s.T_ref / kPi) /
-                     (4.0 * ca * (5.0 - 2.0 * omega) * (7.0 - 2.0 * omega) * s.d_ref * s.d_ref);
-    mu_p = mu_ref * xw / (n * kB * Ttr);
-  }
+__device__ __forceinline__ S mu_ref_w(const Species& s, const S& omega) {
+  const double ca = s.c_alpha;
+  return 5.0 * (ca + 1.0) * (ca + 2.0) * sqrt(s.m * kB * s.T_ref / kPi) /
+         (4.0 * ca * (5.0 - 2.0 * omega) * (7.0 - 2.0 * omega) * s.d_ref * s.d_ref);
 }
 template <typename S>
 __device__ __forceinline__ void cell_alpha(CellCoeffsT<S>& c, double dt) {
@@ -619,12 +616,10 @@ __device__ __forceinline__ void cell_alpha(CellCoeffsT<S>& c, double dt) {
   c.nu_ref = c_div(c.B - a2, 1.0 - a2);
 }
 template <typename S>
-__device__ __forceinline__ void cell_gammas(const Species& s, CellCoeffsT<S>& c, const S& omega,
+__device__ __forceinline__ void cell_gammas(const Species& s, CellCoeffsT<S>& c, const S& tauf,
                                             const S& zrot, double dt, const S& Ttr, const S& Trot,
                                             const VibState& v, const S& xw) {
   const double R = s.R, ctr = 1.5 * R, th = s.theta_v;
-  S tauf(s.tauf0);
-  if constexpr (sizeof(S) != sizeof(double)) tauf = tau_c_factor_w<S>(s, omega);
   const S tau_c = tauf * c.mu_p;
   S zr, zv;
   collision_numbers<S>(s, Ttr, xw, zrot, zr, zv);
@@ -664,10 +659,10 @@ __device__ inline CellCoeffs cell_coeffs(const Species& s, double n, double dt, 
                                          double Trot, const VibState& v) {
   CellCoeffs c;
   double xw;
-  cell_mu_p<double>(s, n, Ttr, s.omega, c.mu_p, xw);
+  cell_mu_p(s, n, Ttr, c.mu_p, xw);
   c.Pr = cell_prandtl(v);
   cell_alpha<double>(c, dt);
-  cell_gammas<double>(s, c, s.omega, s.Z_rot, dt, Ttr, Trot, v, xw);
+  cell_gammas<double>(s, c, s.tauf0, s.Z_rot, dt, Ttr, Trot, v, xw);
   return c;
 }
 

@@ -1475,7 +1475,7 @@ few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
     cs.s = sc;
     cs.step += 1;
     cs.maxI = sizeof(T) == 8 ? S.top : S.maxI + 1;
-    cell_mu_p<double>(sp, cs.ndens, cs.Ttr, sp.omega, K.mu_p, xw);
+    cell_mu_p(sp, cs.ndens, cs.Ttr, K.mu_p, xw);
   } else if (t == 32) {
     cs.ebar = sumI * invN;
     vib = vib_state(sp, cs.ebar);
@@ -1486,7 +1486,7 @@ few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
   if (t == 0) {
     cell_alpha<double>(K, cs.dt);
   } else if (t == 32) {
-    cell_gammas<double>(sp, K, sp.omega, sp.Z_rot, cs.dt, cs.Ttr, cs.Trot, vib, xw);
+    cell_gammas<double>(sp, K, sp.tauf0, sp.Z_rot, cs.dt, cs.Ttr, cs.Trot, vib, xw);
   }
   __syncthreads();
   if (!K.ok) {                                                    // uniform over the block

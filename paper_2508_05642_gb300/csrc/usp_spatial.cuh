@@ -923,7 +923,7 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
   using dual::put_part;
   __shared__ BlockTally tal;
   __shared__ CellCoeffsT<S> k;
-  __shared__ S xw;
+  __shared__ S xw, mu_ref, tauf, ip;   // (T / T_ref)^omega, mu(T_ref), tau_c p / mu, 1 / p
   __shared__ VibState vib;
   tally_init(tal);
   const int c = blockIdx.x, t = threadIdx.x;
@@ -936,21 +936,37 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
   __syncthreads();
   if (cs.active && vol > 0.0) {        // uniform over the block
     if (t < nl) {
-      const double n = (double)cs.N * F_num / vol;
-      Q mu, x;
-      cell_mu_p<Q>(sp, n, lane_part(cs.Ttr, t), lane_part(omega, t), mu, x);
-      put_part(k.mu_p, mu, t);
-      put_part(xw, x, t);
-      if (t == 0) cs.n = n;
+      const Q T = lane_part(cs.Ttr, t);
+      if constexpr (nl > 1)
+        put_part(xw, exp(lane_part(omega, t) * log(T * sp.iT_ref)), t);
+      else
+        xw = d_exp(sp.omega * d_log(T * sp.iT_ref));
     } else if (t == 32) {
       vib = vib_state(sp, cs.ebar);
       k.Pr = S(cell_prandtl(vib));
       if (!kOneWarpSums<T>) cs.Tvib = vib.Tvib;
+    } else if (t >= 64 && t < 64 + nl) {
+      if constexpr (nl > 1) put_part(mu_ref, mu_ref_w<Q>(sp, lane_part(omega, t - 64)), t - 64);
+      else mu_ref = sp.mu_ref0;
+    } else if (t >= 96 && t < 96 + nl) {
+      const int i = t - 96;
+      const double n = (double)cs.N * F_num / vol;
+      const Q p = n * kB * lane_part(cs.Ttr, i);
+      if constexpr (nl > 1) {
+        put_part(ip, rcp(p), i);
+        put_part(tauf, tau_c_factor_w<Q>(sp, lane_part(omega, i)), i);
+      } else {
+        ip = d_rcp(p);
+        tauf = sp.tauf0;
+      }
+      if (i == 0) cs.n = n;
     }
     __syncthreads();
     CellCoeffsT<Q> q;
+    const int i = t & 31;
+    if (t < 64 && i < nl) q.mu_p = lane_part(mu_ref, i) * lane_part(xw, i) * lane_part(ip, i);
     if (t < nl) {
-      q.mu_p = lane_part(k.mu_p, t);
+      put_part(k.mu_p, q.mu_p, t);
       q.Pr = lane_part(k.Pr, t);
       cell_alpha<Q>(q, dt);
       put_part(k.B, q.B, t);
@@ -958,9 +974,7 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
       put_part(k.nu_ref, q.nu_ref, t);
       if (t == 0) k.ok = q.ok;
     } else if (t >= 32 && t < 32 + nl) {
-      const int i = t - 32;
-      q.mu_p = lane_part(k.mu_p, i);
-      cell_gammas<Q>(sp, q, lane_part(omega, i), lane_part(zrot, i), dt, lane_part(cs.Ttr, i),
+      cell_gammas<Q>(sp, q, lane_part(tauf, i), lane_part(zrot, i), dt, lane_part(cs.Ttr, i),
                      lane_part(cs.Trot, i), vib, lane_part(xw, i));
       put_part(k.g_tr_rot, q.g_tr_rot, i);
       put_part(k.g_tr_vib, q.g_tr_vib, i);
