@@ -51,7 +51,7 @@ constexpr int kInflowTries = 64;
 constexpr int kBlk = 256;
 constexpr int kNSurf = USP_NSURF;   // cylinder surface bins of the polar angle
 constexpr int kParamBlock = 32;   // cells per block of the stencil passes
-constexpr int kPF = 16;           // threads per cell there: one per field
+constexpr int kPF = 4;            // threads per cell there: one per four fields
 
 // Device-resident counts of the current step.
 struct PlCount {
@@ -833,12 +833,26 @@ __global__ void pl_gather(PlCount* __restrict__ cnt, int ncell, long long* __res
 // the centroid the x and y neighbour used (that side's if usable, else the
 // opposite one, else none) and the quadrant's diagonal when usable
 // ---------------------------------------------------------------------------
-// Both stencil passes give a cell kPF threads, thread q < kNF field q: loads
-// and stores of a cell's fields are consecutive, and a thread holds one
-// value per neighbour (one thread per cell kept up to 65 in local memory and
-// built the record in shared memory: 71 us on the 600 x 400 grid, 245 us for
-// the 422,730 cells of the refined one).  The scalars, converted from FP64 or
-// formed in it, are written by one warp for the block's cells together.
+// Both stencil passes give a cell kPF threads, the first three four fields each:
+// 16-byte loads of the 3 x 3 values and 16-byte stores of the record.  The pass is
+// bound by the sectors and cache lines that its requests touch: with a field per
+// thread (16 threads a cell) a request covered two cells' 48 bytes (240,000 cells:
+// 52 us, 47 us so; 422,730 refined cells, three launches: 171 us, 111 us).
+// The scalars are one warp's work (FP64 conversions cost the pipe as much for one
+// lane as for 32).
+template <typename T>
+struct alignas(16) V4 {
+  T v[4];
+};
+template <typename T>
+__device__ __forceinline__ V4<T> load4(const T* p) {
+  return *reinterpret_cast<const V4<T>*>(p);
+}
+template <typename T>
+__device__ __forceinline__ void store4(T* p, const V4<T>& a) {
+  *reinterpret_cast<V4<T>*>(p) = a;
+}
+
 template <typename T>
 __device__ __forceinline__ void pl_scalars(PlParams<T>& P, const ChCellT<double>& cs,
                                            const PlGeomT<T>& gt, const Species& sp, double xc,
@@ -865,35 +879,38 @@ pl_params(PlGeom g, PlGeomT<T> gt, int recon, const ChCellT<double>* __restrict_
     pl_scalars<T>(prm[c], cells[c], gt, sp, g.x0 + (c % g.nx + 0.5) * g.dx,
                   g.y0 + (c / g.nx + 0.5) * g.dy);
   }
-  const int c = c0 + threadIdx.x / kPF, q = threadIdx.x % kPF;
+  const int c = c0 + threadIdx.x / kPF, q = threadIdx.x % kPF * 4;   // fields q .. q + 3
   if (c >= g.ncell || q >= kNF) return;
   const int i = c % g.nx, j = c / g.nx;
   PlParams<T>& P = prm[c];
-  const T f = fT[(size_t)c * kNF + q];
-  P.F[q] = f;
+  const V4<T> f = load4(fT + (size_t)c * kNF + q);
+  store4(&P.F[q], f);
   if (fpm) {
     // the plain FPM method: cell values, its per-cell constants
-    P.gx[0][q] = P.gx[1][q] = P.gy[0][q] = P.gy[1][q] = T(0);
+    const V4<T> z = {{T(0), T(0), T(0), T(0)}};
+    store4(&P.gx[0][q], z); store4(&P.gx[1][q], z);
+    store4(&P.gy[0][q], z); store4(&P.gy[1][q], z);
     static_assert(sizeof(P.fpm) == kFpmRec * sizeof(T), "the record's order");
-    if (q < kFpmRec) (&P.fpm.as)[q] = (T)fpm[(size_t)c * kFpmRec + q];
+    for (int n = q; n < q + 4 && n < kFpmRec; ++n)
+      (&P.fpm.as)[n] = (T)fpm[(size_t)c * kFpmRec + n];
     return;
   }
   // the flags and values of the 3 x 3 cells, loaded together (a square outside
   // the domain reads its own cell and counts as not usable)
   bool us[9];
-  T fn[9];
+  V4<T> fn[9];
 #pragma unroll
   for (int m = 0; m < 9; ++m) {
     const int di = m % 3 - 1, dj = m / 3 - 1, ii = i + di, jj = j + dj;
     const bool in = recon && ii >= 0 && ii < g.nx && jj >= 0 && jj < g.ny;
     const int cc = in ? jj * g.nx + ii : c;
     us[m] = in && usable_c[cc];
-    fn[m] = fT[(size_t)cc * kNF + q];
+    fn[m] = load4(fT + (size_t)cc * kNF + q);
   }
   // slopes in the working precision from the cell values, times 1/offset: the
   // x and y neighbour of each side (offset; 0: none)
   int ox[2], oy[2];
-  T fx[2], fy[2];
+  V4<T> fx[2], fy[2];
 #pragma unroll
   for (int sd = 0; sd < 2; ++sd) {
     const int hi = sd ? 1 : -1;
@@ -901,19 +918,28 @@ pl_params(PlGeom g, PlGeomT<T> gt, int recon, const ChCellT<double>* __restrict_
     oy[sd] = us[4 + 3 * hi] ? hi : (us[4 - 3 * hi] ? -hi : 0);
     fx[sd] = ox[sd] > 0 ? fn[5] : fn[3];
     fy[sd] = oy[sd] > 0 ? fn[7] : fn[1];
-    P.gx[sd][q] = ox[sd] != 0 ? (fx[sd] - f) * (ox[sd] > 0 ? gt.idx : -gt.idx) : T(0);
-    P.gy[sd][q] = oy[sd] != 0 ? (fy[sd] - f) * (oy[sd] > 0 ? gt.idy : -gt.idy) : T(0);
+    V4<T> gx, gy;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      gx.v[n] = ox[sd] != 0 ? (fx[sd].v[n] - f.v[n]) * (ox[sd] > 0 ? gt.idx : -gt.idx) : T(0);
+      gy.v[n] = oy[sd] != 0 ? (fy[sd].v[n] - f.v[n]) * (oy[sd] > 0 ? gt.idy : -gt.idy) : T(0);
+    }
+    store4(&P.gx[sd][q], gx);
+    store4(&P.gy[sd][q], gy);
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int sx = k & 1, sy = k >> 1;
     const bool px = ox[sx] > 0, py = oy[sy] > 0;
     const bool ud = py ? (px ? us[8] : us[6]) : (px ? us[2] : us[0]);
-    const T fd = py ? (px ? fn[8] : fn[6]) : (px ? fn[2] : fn[0]);
-    T v = T(0);
+    const V4<T> fd = py ? (px ? fn[8] : fn[6]) : (px ? fn[2] : fn[0]);
+    V4<T> v = {{T(0), T(0), T(0), T(0)}};
     if (ox[sx] != 0 && oy[sy] != 0 && ud)
-      v = (fd - fx[sx] - fy[sy] + f) * ((px == py ? T(1) : T(-1)) * gt.idx * gt.idy);
-    P.gxy[k][q] = v;
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+        v.v[n] = (fd.v[n] - fx[sx].v[n] - fy[sy].v[n] + f.v[n]) *
+                 ((px == py ? T(1) : T(-1)) * gt.idx * gt.idy);
+    store4(&P.gxy[k][q], v);
   }
 }
 
@@ -947,15 +973,15 @@ template <typename T>
 __device__ __forceinline__ bool
 pl_region(const PlGeom& g, int nb, const PlParams<T>* __restrict__ prm, const T* __restrict__ fT,
           const int* __restrict__ usable_c, const long long* __restrict__ off,
-          const PlLevel<T>& lv, int ii, int jj, int di, int dj, int f, T& val) {
+          const PlLevel<T>& lv, int ii, int jj, int di, int dj, int f, V4<T>& val) {
   const int l = nb >> 2, kind = nb & 3;
   if (kind == kNbSame) {
-    val = fT[(size_t)l * kNF + f];
+    val = load4(fT + (size_t)l * kNF + f);
     return usable_c[l];
   }
   if (kind == kNbNone) return false;
   if (kind == kNbFiner) {
-    T sum = T(0);
+    V4<T> sum = {{T(0), T(0), T(0), T(0)}};
     bool ok = true;
     const long long n0 = off[l];
     long long at = n0;
@@ -963,10 +989,13 @@ pl_region(const PlGeom& g, int nb, const PlParams<T>* __restrict__ prm, const T*
     for (int a = 0; a < 4; ++a) {
       const long long nx = off[l + a + 1];
       ok = ok && usable_c[l + a];
-      sum += (T)(nx - at) * fT[(size_t)(l + a) * kNF + f];
+      const V4<T> w = load4(fT + (size_t)(l + a) * kNF + f);
+#pragma unroll
+      for (int n = 0; n < 4; ++n) sum.v[n] += (T)(nx - at) * w.v[n];
       at = nx;
     }
-    val = sum / (T)(at - n0);
+#pragma unroll
+    for (int n = 0; n < 4; ++n) val.v[n] = sum.v[n] / (T)(at - n0);
     return ok;
   }
   if (!usable_c[l]) return false;
@@ -975,7 +1004,11 @@ pl_region(const PlGeom& g, int nb, const PlParams<T>* __restrict__ prm, const T*
   const double cy = rn_add(g.y0, rn_mul((double)(jj + dj) + 0.5, lv.k));
   const T ex = (T)cx - C.xc, ey = (T)cy - C.yc;
   const int sx = ex >= T(0) ? 1 : 0, sy = ey >= T(0) ? 1 : 0;
-  val = C.F[f] + C.gx[sx][f] * ex + C.gy[sy][f] * ey + C.gxy[2 * sy + sx][f] * ex * ey;
+  const V4<T> F = load4(&C.F[f]), gx = load4(&C.gx[sx][f]), gy = load4(&C.gy[sy][f]),
+              gxy = load4(&C.gxy[2 * sy + sx][f]);
+#pragma unroll
+  for (int n = 0; n < 4; ++n)
+    val.v[n] = F.v[n] + gx.v[n] * ex + gy.v[n] * ey + gxy.v[n] * ex * ey;
   return true;
 }
 
@@ -995,27 +1028,27 @@ pl_params_amr(PlGeom g, PlGeomT<T> gt, const PlTree* __restrict__ tr, int recon,
                     rn_add(g.x0, rn_mul((double)tr->lii[c] + 0.5, lv.h)),
                     rn_add(g.y0, rn_mul((double)tr->ljj[c] + 0.5, lv.k)));
   }
-  const int c = c0 + threadIdx.x / kPF, q = threadIdx.x % kPF;
+  const int c = c0 + threadIdx.x / kPF, q = threadIdx.x % kPF * 4;   // fields q .. q + 3
   if (c >= g.ncell || q >= kNF || tr->lvl[c] != lv.level) return;
   PlParams<T>& P = prm[c];
   const int ii = tr->lii[c], jj = tr->ljj[c];
   const int4* nb4 = reinterpret_cast<const int4*>(tr->nb + (size_t)c * 8);
   const int4 na = nb4[0], nc = nb4[1];
-  const T f = fT[(size_t)c * kNF + q];
-  P.F[q] = f;
+  const V4<T> f = load4(fT + (size_t)c * kNF + q);
+  store4(&P.F[q], f);
   // the values and flags of the eight squares, (-1,-1) (0,-1) (1,-1) (-1,0)
   // (1,0) (-1,1) (0,1) (1,1)
   const int nb[8] = {na.x, na.y, na.z, na.w, nc.x, nc.y, nc.z, nc.w};
   bool us[8];
-  T fn[8];
+  V4<T> fn[8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
     const int k = m < 4 ? m : m + 1, di = k % 3 - 1, dj = k / 3 - 1;
-    fn[m] = T(0);
+    fn[m] = V4<T>{{T(0), T(0), T(0), T(0)}};
     us[m] = recon && pl_region<T>(g, nb[m], prm, fT, usable_c, off, lv, ii, jj, di, dj, q, fn[m]);
   }
   int ox[2], oy[2];
-  T fx[2], fy[2];
+  V4<T> fx[2], fy[2];
 #pragma unroll
   for (int sd = 0; sd < 2; ++sd) {
     const int hi = sd ? 1 : -1;
@@ -1026,21 +1059,29 @@ pl_params_amr(PlGeom g, PlGeomT<T> gt, const PlTree* __restrict__ tr, int recon,
     fx[sd] = ox[sd] > 0 ? fn[4] : fn[3];
     fy[sd] = oy[sd] > 0 ? fn[6] : fn[1];
     const T sx = ox[sd] > 0 ? lv.ih : -lv.ih, sy = oy[sd] > 0 ? lv.ik : -lv.ik;
-    P.gx[sd][q] = ox[sd] ? (fx[sd] - f) * sx : T(0);
-    P.gy[sd][q] = oy[sd] ? (fy[sd] - f) * sy : T(0);
+    V4<T> gx, gy;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      gx.v[n] = ox[sd] ? (fx[sd].v[n] - f.v[n]) * sx : T(0);
+      gy.v[n] = oy[sd] ? (fy[sd].v[n] - f.v[n]) * sy : T(0);
+    }
+    store4(&P.gx[sd][q], gx);
+    store4(&P.gy[sd][q], gy);
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int sx = k & 1, sy = k >> 1;
     const bool px = ox[sx] > 0, py = oy[sy] > 0;
     const bool ud = py ? (px ? us[7] : us[5]) : (px ? us[2] : us[0]);
-    const T fd = py ? (px ? fn[7] : fn[5]) : (px ? fn[2] : fn[0]);
-    T v = T(0);
+    const V4<T> fd = py ? (px ? fn[7] : fn[5]) : (px ? fn[2] : fn[0]);
+    V4<T> v = {{T(0), T(0), T(0), T(0)}};
     if (ox[sx] && oy[sy] && ud) {
       const T s = (px == py ? T(1) : T(-1)) * lv.ih * lv.ik;
-      v = (fd - fx[sx] - fy[sy] + f) * s;
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+        v.v[n] = (fd.v[n] - fx[sx].v[n] - fy[sy].v[n] + f.v[n]) * s;
     }
-    P.gxy[k][q] = v;
+    store4(&P.gxy[k][q], v);
   }
 }
 
