@@ -930,9 +930,28 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
   ChCellT<S>& cs = cells[c];
   if constexpr (!kOneWarpSums<T>)
     block_moments(c, off, cx, cy, cz, er, lev, cells, sp, tal);
-  else if (t < 32)
-    moments_of_cells<T, S>(c, 1, c + 1, 1, off, nullptr, cx, cy, cz, er, lev, cells, sp, nullptr,
-                           (T*)nullptr, nullptr, tal);
+  else {
+    // a small cell's particles come in by all threads; the warp's two passes then
+    // read shared memory (64 cells of 200 FP32 particles: 12.8 us, 13.4 us with
+    // the warp's own loads)
+    constexpr int kStage = 256;
+    __shared__ T st[4][kStage];
+    __shared__ int sl[kStage];
+    const long long b = off[c], n = off[c + 1] - b;
+    if (n <= kStage) {
+      for (int i = t; i < n; i += kPB) {
+        st[0][i] = cx[b + i]; st[1][i] = cy[b + i]; st[2][i] = cz[b + i]; st[3][i] = er[b + i];
+        sl[i] = lev[b + i];
+      }
+      __syncthreads();
+      if (t < 32)
+        moments_of_cells<T, S>(c, 1, c + 1, 1, off, nullptr, st[0] - b, st[1] - b, st[2] - b,
+                               st[3] - b, sl - b, cells, sp, nullptr, (T*)nullptr, nullptr, tal);
+    } else if (t < 32) {
+      moments_of_cells<T, S>(c, 1, c + 1, 1, off, nullptr, cx, cy, cz, er, lev, cells, sp, nullptr,
+                             (T*)nullptr, nullptr, tal);
+    }
+  }
   __syncthreads();
   if (cs.active && vol > 0.0) {        // uniform over the block
     if (t < nl) {
