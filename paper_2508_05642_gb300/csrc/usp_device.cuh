@@ -97,27 +97,6 @@ inline PhiloxRoundKeys philox_round_keys(uint32_t k0, uint32_t k1) {
   }
   return rk;
 }
-// Two blocks whose counters differ only in word 2, rounds interleaved so the
-// two independent multiply chains overlap.
-__device__ __forceinline__ void philox4x32_10_pair(uint32_t c0, uint32_t c1, uint32_t c2a,
-                                                   uint32_t c2b, uint32_t c3,
-                                                   const PhiloxRoundKeys& rk, U4& a, U4& b) {
-  uint32_t a0 = c0, a1 = c1, a2 = c2a, a3 = c3;
-  uint32_t b0 = c0, b1 = c1, b2 = c2b, b3 = c3;
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint64_t pa0 = (uint64_t)0xD2511F53u * a0, pa1 = (uint64_t)0xCD9E8D57u * a2;
-    const uint64_t pb0 = (uint64_t)0xD2511F53u * b0, pb1 = (uint64_t)0xCD9E8D57u * b2;
-    const uint32_t na0 = (uint32_t)(pa1 >> 32) ^ a1 ^ rk.k0[r];
-    const uint32_t na2 = (uint32_t)(pa0 >> 32) ^ a3 ^ rk.k1[r];
-    const uint32_t nb0 = (uint32_t)(pb1 >> 32) ^ b1 ^ rk.k0[r];
-    const uint32_t nb2 = (uint32_t)(pb0 >> 32) ^ b3 ^ rk.k1[r];
-    a0 = na0; a1 = (uint32_t)pa1; a2 = na2; a3 = (uint32_t)pa0;
-    b0 = nb0; b1 = (uint32_t)pb1; b2 = nb2; b3 = (uint32_t)pb0;
-  }
-  a = U4{a0, a1, a2, a3};
-  b = U4{b0, b1, b2, b3};
-}
 __device__ __forceinline__ U4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                                             const PhiloxRoundKeys& rk) {
 #pragma unroll
@@ -682,23 +661,8 @@ __device__ __forceinline__ void relax_temps(const Species& s, const CellCoeffs& 
   if (evr < 0.0) { evr = 0.0; clamped = true; }
 }
 
-// Cholesky factor (l00, l10, l11, l20, l21, l22) of (xx, yy, zz, xy, xz, yz).
-template <typename T>
-__device__ __forceinline__ bool chol3(const T* M, T* L) {
-  if (!(M[0] > T(0))) return false;
-  const T l00 = sqrt(M[0]);
-  const T l10 = M[3] / l00, l20 = M[4] / l00;
-  const T d1 = M[1] - l10 * l10;
-  if (!(d1 > T(0))) return false;
-  const T l11 = sqrt(d1);
-  const T l21 = (M[5] - l20 * l10) / l11;
-  const T d2 = M[2] - l20 * l20 - l21 * l21;
-  if (!(d2 > T(0))) return false;
-  L[0] = l00; L[1] = l10; L[2] = l11; L[3] = l20; L[4] = l21; L[5] = sqrt(d2);
-  return true;
-}
-
-// the same for a per-cell matrix, by reciprocal square roots (usp_math.cuh)
+// Cholesky factor (l00, l10, l11, l20, l21, l22) of a cell's (xx, yy, zz, xy, xz,
+// yz), by reciprocal square roots (usp_math.cuh)
 constexpr double kLeastPivot = 0x1p-1000;   // the reciprocal root needs a normal number
 __device__ __forceinline__ bool chol3_cell(const double* M, double* L) {
   if (!(M[0] > kLeastPivot)) return false;

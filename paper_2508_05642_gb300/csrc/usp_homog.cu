@@ -27,6 +27,7 @@
 //                    (Sec. 3.A) in FP64.
 //   jumptable_kernel the per-cell inversion tables of the
 //                    vibrational jump samplers for the next step.
+//   few_cells_kernel the three in one launch, for at most one cell per SM.
 // The rescale is never written back as a separate pass: it rides along with
 // the next collide pass, or with usp_moments / usp_get_particles.
 #include <cuda_runtime.h>
@@ -202,7 +203,6 @@ __device__ void b_row(int n, F p, float* T) {
 // inversion's, bit for bit.
 constexpr int kGBits = 8;             // guide bins per row: 2^kGBits
 constexpr int kGB = 1 << kGBits;      // guide bytes per row
-constexpr int kGS = 23 - kGBits;      // 23-bit uniform index -> bin: >> kGS
 
 // the guide byte of the word x's bin in the guide g of a row
 __device__ __forceinline__ unsigned guide_byte(const uint8_t* __restrict__ g, uint32_t x) {
@@ -359,41 +359,6 @@ __global__ void draw_tables_kernel(double* __restrict__ radius,
     sincospi(2.0 * ((2.0 * (double)a + 1.0) * 1.9073486328125e-06), &s, &c);
     direction[a] = make_double2(c, s);
   }
-}
-
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Block reduction of the tile sums and one FP64 atomic per sum.  Partial sums
-// stay in T inside a thread and a warp; warps combine in FP64.
-template <typename T>
-__device__ __forceinline__ void flush_sums(const T* acc, int accI, int maxI, CellSums* dst) {
-  __shared__ double red[kBlock / 32][11];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < 10; ++i) {
-    const T s = warp_sum(acc[i]);
-    if (lane == 0) red[wid][i] = (double)s;
-  }
-  const int sI = warp_sum(accI);
-  if (lane == 0) red[wid][10] = (double)sI;
-  const int mI = __reduce_max_sync(0xffffffffu, maxI);
-  if (lane == 0 && mI > 0) atomicMax(&dst->maxI, mI);
-  __syncthreads();
-  if (threadIdx.x < 11) {
-    double t = 0.0;
-#pragma unroll
-    for (int w = 0; w < kBlock / 32; ++w) t += red[w][threadIdx.x];
-    if (threadIdx.x < 10)
-      atomicAdd(&dst->v[threadIdx.x], t);
-    else
-      atomicAdd(&dst->I, (unsigned long long)(long long)t);
-  }
-  __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
@@ -1396,7 +1361,7 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
 // tables follow in the same block.  With more cells than SMs one thread per
 // cell (cellupdate_kernel) is the better split: its instructions serve 32
 // cells.  One cell of 20,000 particles, FP32: the three kernels took 54 us a
-// step at first (37 the update with the library's functions).
+// step at first (37 the update with the library's functions), 26 us so.
 // ---------------------------------------------------------------------------
 constexpr int kFewCells = 152;
 
