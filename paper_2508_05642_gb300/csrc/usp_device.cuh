@@ -661,6 +661,22 @@ __device__ __forceinline__ void relax_temps(const Species& s, const CellCoeffs& 
   if (evr < 0.0) { evr = 0.0; clamped = true; }
 }
 
+// Cholesky factor (l00, l10, l11, l20, l21, l22) of (xx, yy, zz, xy, xz, yz).
+template <typename T>
+__device__ __forceinline__ bool chol3(const T* M, T* L) {
+  if (!(M[0] > T(0))) return false;
+  const T l00 = sqrt(M[0]);
+  const T l10 = M[3] / l00, l20 = M[4] / l00;
+  const T d1 = M[1] - l10 * l10;
+  if (!(d1 > T(0))) return false;
+  const T l11 = sqrt(d1);
+  const T l21 = (M[5] - l20 * l10) / l11;
+  const T d2 = M[2] - l20 * l20 - l21 * l21;
+  if (!(d2 > T(0))) return false;
+  L[0] = l00; L[1] = l10; L[2] = l11; L[3] = l20; L[4] = l21; L[5] = sqrt(d2);
+  return true;
+}
+
 // Cholesky factor (l00, l10, l11, l20, l21, l22) of a cell's (xx, yy, zz, xy, xz,
 // yz), by reciprocal square roots (usp_math.cuh)
 constexpr double kLeastPivot = 0x1p-1000;   // the reciprocal root needs a normal number
@@ -812,24 +828,29 @@ struct FpmCell {
   bool ok, fixed, nu_zero, failed, clamped;
 };
 
+// (Library functions and divisions: the positivity fix below leaves a factor
+// within 1e-6 of singular, where the last bit of what goes in comes out as 1e-10
+// of L and turns roundings of an FP32 state.)
 __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const double* Pi,
-                                   double Ttr, double Trot, const VibState& v) {
+                                   double Ttr, double Trot, double Tvib) {
   FpmCell o;
   o.fixed = o.nu_zero = o.failed = o.clamped = false;
   const double R = gasR(s);
   const double p = n * kB * Ttr;
-  const double xw = d_exp(s.omega * d_log(Ttr * s.iT_ref));
-  const double mu_p = s.mu_ref0 * xw * d_rcp(p);
-  const double tau_c = s.tauf0 * mu_p;
+  const double xw = exp(s.omega * log(Ttr / s.T_ref));
+  const double mu = s.mu_ref0 * xw;
+  const double tau_c = s.tauf0 * mu / p;
   double zr, zv;
   collision_numbers<double>(s, Ttr, xw, s.Z_rot, zr, zv);
-  // nu = 1 - 3 / (2 Pr), Pr = (14 + 2 xi) / (19 + 2 xi)
-  const double nu0 = 1.0 - d_div(1.5 * fma(2.0, v.xi, 19.0), fma(2.0, v.xi, 14.0));
-  const double tau = 2.0 * mu_p * (1.0 - nu0), itau = d_rcp(tau);
+  const double x = Tvib > 0.0 ? s.theta_v / Tvib : 0.0, xi = Tvib > 0.0 ? x / expm1(x) : 0.0;
+  const double Pr = (14.0 + 2.0 * xi) / (19.0 + 2.0 * xi);
+  const double nu0 = 1.0 - 3.0 / (2.0 * Pr);
+  const double tau = 2.0 * mu * (1.0 - nu0) / p;
   o.ok = tau > 0.0;
-  o.alpha = o.ok ? d_exp(-dt * itau) : 0.0;
-  const double grot = d_div(tau, 2.0 * zr * tau_c), gvib = d_div(tau, 2.0 * zv * tau_c);
-  const double ev = v.ev, evt = R * s.theta_v * d_rcp(d_expm1(s.theta_v * d_rcp(Ttr)));
+  o.alpha = o.ok ? exp(-dt / tau) : 0.0;
+  const double grot = tau / (2.0 * zr * tau_c), gvib = tau / (2.0 * zv * tau_c);
+  auto e_vib = [&](double T) { return T > 0.0 ? R * s.theta_v / expm1(s.theta_v / T) : 0.0; };
+  const double ev = e_vib(Tvib), evt = e_vib(Ttr);
   double etr = 1.5 * R * Ttr + grot * (R * Trot - R * Ttr) + gvib * (ev - evt);
   double erot = R * Trot + grot * (R * Ttr - R * Trot);
   double evib = ev + gvib * (evt - ev);
@@ -837,10 +858,10 @@ __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const 
   if (erot < 0.0) { erot = 0.0; o.clamped = true; }
   if (evib < 0.0) { evib = 0.0; o.clamped = true; }
   const double RT = R * Ttr, RTrel = etr / 1.5;
-  o.Trot_rel = erot * s.iR;
-  const double ebar = evib * s.iRtheta;
-  o.lam_up = 2.0 * dt * ebar * itau;
-  o.lam_dn = 2.0 * dt * (1.0 + ebar) * itau;
+  o.Trot_rel = erot / R;
+  const double ebar = evib / (R * s.theta_v);
+  o.lam_up = 2.0 * dt * ebar / tau;
+  o.lam_dn = 2.0 * dt * (1.0 + ebar) / tau;
   const double a2 = o.alpha * o.alpha;
   o.e_rot_tgt = erot + (R * Trot - erot) * a2;
   o.e_vib_tgt = evib + (ev - evib) * a2;
@@ -854,7 +875,7 @@ __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const 
     M[5] = nu_ * Pi[5];
   };
   fill(nu);
-  if (chol3_cell(M, o.L)) return o;
+  if (chol3(M, o.L)) return o;
   o.fixed = true;
   double lmin, lmax;
   sym3_minmax(Pi, lmin, lmax);
@@ -865,7 +886,7 @@ __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const 
   }
   nu = nu * (1.0 - 1e-6);
   fill(nu);
-  if (chol3_cell(M, o.L)) return o;
+  if (chol3(M, o.L)) return o;
   o.nu_zero = true;
   const double sq = RTrel > 0.0 ? sqrt(RTrel) : 0.0;
   o.failed = !(RTrel > 0.0);

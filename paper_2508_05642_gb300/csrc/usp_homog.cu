@@ -1025,11 +1025,11 @@ __device__ void write_params(const Species& sp, CellState& cs, CollideParams<T>&
   P.method = sp.method;
   P.pad_ = 0;
   if (!cs.active) return;
-  const VibState vib = vib_state(sp, cs.ebar);
   if (sp.method == 1) {
     // the plain FPM method (Sec. 2.C): Gorji's velocity update and the
     // Milstein square form with alpha = exp(-dt/tau), Gillespie levels
-    const FpmCell f = fpm_cell(sp, cs.ndens, cs.dt, cs.Pi, cs.Ttr, cs.Trot, vib);
+    const FpmCell f = fpm_cell(sp, cs.ndens, cs.dt, cs.Pi, cs.Ttr, cs.Trot,
+                               T_vib_of_level(sp, cs.ebar));
     if (!f.ok) {
       atomicOr(flags, (uint32_t)F_A_NONPOS);
       cs.active = 0;
@@ -1056,6 +1056,7 @@ __device__ void write_params(const Species& sp, CellState& cs, CollideParams<T>&
     P.p_b = (T)f.lam_dn;
     return;
   }
+  const VibState vib = vib_state(sp, cs.ebar);
   const CellCoeffs c = cell_coeffs(sp, cs.ndens, cs.dt, cs.Ttr, cs.Trot, vib);
   if (!c.ok) {
     atomicOr(flags, (uint32_t)F_A_NONPOS);

@@ -618,7 +618,7 @@ __global__ void ch_fix_update(int ncell, ChCellT<double>* __restrict__ cells,
 // cell are warp-wide FP32 (or working-precision) reductions, kept by lane k
 // for the k-th cell; the FP64 per-cell arithmetic then runs one cell per lane,
 // so each FP64 warp instruction serves up to 32 cells on the narrow FP64 pipe.
-template <typename T, typename S>
+template <typename T, typename S, bool kFpm = false>
 __device__ __forceinline__ void
 moments_of_cells(long long first, long long stride, long long ny, int cpw,
                  const long long* __restrict__ off, const double* __restrict__ af,
@@ -731,10 +731,16 @@ moments_of_cells(long long first, long long stride, long long ny, int cpw,
       continue;
     }
     for (int i = 0; i < 6; ++i) cs.Pi[i] = P[i];
-    cs.Ttr = (P[0] + P[1] + P[2]) * (sp.iR * (1.0 / 3.0));
-    cs.Trot = se * (inv * sp.iR);
     cs.ebar = (double)kl * inv;
-    cs.Tvib = vib_state(sp, cs.ebar).Tvib;
+    if constexpr (kFpm) {   // for fpm_cell: divisions and the library's log1p
+      cs.Ttr = (P[0] + P[1] + P[2]) / (3.0 * R);
+      cs.Trot = se * inv / R;
+      cs.Tvib = T_vib_of_level<double>(sp, cs.ebar);
+    } else {
+      cs.Ttr = (P[0] + P[1] + P[2]) * (sp.iR * (1.0 / 3.0));
+      cs.Trot = se * (inv * sp.iR);
+      cs.Tvib = vib_state(sp, cs.ebar).Tvib;
+    }
     if (fT) {   // the fields in the particle precision, for the stencils
       T* o = fT + (size_t)c * kNF;
       for (int i = 0; i < 3; ++i) o[i] = (T)cs.U[i];
@@ -754,7 +760,7 @@ __global__ void ch_moments(int ny, int cpw, const long long* __restrict__ off,
                            T* __restrict__ fT, int* __restrict__ usable_c) {
   __shared__ BlockTally tal;
   tally_init(tal);
-  moments_of_cells<T, S>((long long)warp_global() * cpw, (long long)warps_total() * cpw, ny, cpw,
+  moments_of_cells<T, S, true>((long long)warp_global() * cpw, (long long)warps_total() * cpw, ny, cpw,
                          off, af, cx, cy, cz, er, lev, cells,
                          sp, pend, fT, usable_c, tal);
   tally_flush(tal, nullptr, counters);
@@ -1172,7 +1178,7 @@ __global__ void ch_coeffs_fpm(int ncell, double F_num, double vol, const double*
       continue;
     }
     cs.n = (double)cs.N * F_num / v;
-    const FpmCell f = fpm_cell(sp, cs.n, dt, cs.Pi, cs.Ttr, cs.Trot, vib_state(sp, cs.ebar));
+    const FpmCell f = fpm_cell(sp, cs.n, dt, cs.Pi, cs.Ttr, cs.Trot, cs.Tvib);
     if (!f.ok) {
       tally_or(tal, (uint32_t)F_A_NONPOS);
       cs.active = 0;
