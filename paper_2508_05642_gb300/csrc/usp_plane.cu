@@ -1347,23 +1347,45 @@ __device__ __forceinline__ void cl_totals(double* a) {
   }
 }
 
+// Small grids (kWideCells cells or fewer) take a warp per cell in these passes:
+// there a cell of some hundred particles, which four lanes walk alone, lasts
+// longer than all the others (80 x 59 cells, largest 381 particles: the moments'
+// sums 123 us by four lanes, 28 us by warps; 38,400 cells of 20 take 116 us
+// either way).  The totals of a[0 .. M-1] over the CL lanes, stored in out.
+constexpr int kWideCells = 32768;
+template <int CL, int M>
+__device__ __forceinline__ void cl_store(double* a, bool cell, double* __restrict__ out) {
+  if constexpr (CL == kCL) {
+    cl_totals<M>(a);
+    const int q = threadIdx.x & (kCL - 1);
+    if (cell)
+#pragma unroll
+      for (int i = 0; i < M / 4; ++i) out[q * (M / 4) + i] = a[i];
+  } else {
+    static_assert(CL == 32, "a warp");
+    const int at = halve_totals<M>(a);
+    if (cell && at >= 0) out[at] = a[0];
+  }
+}
+
 // Time averages of the post-step state, first part: kCL lanes per cell over
 // the sorted particles, sums of c*, c* c*, eps* and I into rec (kNAcc doubles per
 // cell: 3 sums of c, 6 of cc, eps, I, 0).  Bound by the FP64 pipe (10 operations
 // per particle).
+template <int CL>
 __global__ void __launch_bounds__(kBlk)
 pl_sample(int ncell, const long long* __restrict__ off, const double* __restrict__ cx,
           const double* __restrict__ cy, const double* __restrict__ cz, const double* __restrict__ er,
           const int* __restrict__ lev, double* __restrict__ rec) {
-  const int q = threadIdx.x & (kCL - 1);
-  const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kCL;
+  const int q = threadIdx.x & (CL - 1);
+  const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / CL;
   const long long b = c < ncell ? off[c] : 0, e = c < ncell ? off[c + 1] : 0;
   double a[kNAcc];
 #pragma unroll
   for (int i = 0; i < kNAcc; ++i) a[i] = 0.0;
   int sl = 0;   // a lane's share of a cell's levels stays far below 2^31
 #pragma unroll 4
-  for (long long j = b + q; j < e; j += kCL) {
+  for (long long j = b + q; j < e; j += CL) {
     const double v0 = cx[j], v1 = cy[j], v2 = cz[j];
     a[0] += v0; a[1] += v1; a[2] += v2;
     a[3] = fma(v0, v0, a[3]); a[4] = fma(v1, v1, a[4]); a[5] = fma(v2, v2, a[5]);
@@ -1372,11 +1394,7 @@ pl_sample(int ncell, const long long* __restrict__ off, const double* __restrict
     sl += lev[j];
   }
   if (sl != 0) a[10] = (double)sl;
-  cl_totals<kNAcc>(a);
-  if (c < ncell) {
-#pragma unroll
-    for (int i = 0; i < kNAcc / 4; ++i) rec[(size_t)c * kNAcc + q * (kNAcc / 4) + i] = a[i];
-  }
+  cl_store<CL, kNAcc>(a, c < ncell, rec + (size_t)c * kNAcc);
 }
 
 // The same sums of an FP32 state.  The FP64 pipe has 1/64 of the FP32 rate,
@@ -1581,13 +1599,13 @@ __device__ __forceinline__ void cl_reference(long long b, long long n, const T* 
   }
 }
 
-template <typename T>
+template <typename T, int CL>
 __global__ void __launch_bounds__(kBlk)
 pl_mom_sums(int ncell, const long long* __restrict__ off, const T* __restrict__ cx,
             const T* __restrict__ cy, const T* __restrict__ cz, const T* __restrict__ er,
             const int* __restrict__ lev, double* __restrict__ rec) {
-  const int q = threadIdx.x & (kCL - 1);
-  const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kCL;
+  const int q = threadIdx.x & (CL - 1);
+  const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / CL;
   const long long b = c < ncell ? off[c] : 0, e = c < ncell ? off[c + 1] : 0;
   float wf[3];
   cl_reference<T>(b, e - b, cx, cy, cz, wf);
@@ -1597,14 +1615,10 @@ pl_mom_sums(int ncell, const long long* __restrict__ off, const T* __restrict__ 
 #pragma unroll
   for (int i = 0; i < kRawN; ++i) a[i] = 0.0;
 #pragma unroll 2
-  for (long long j = b + q; j < e; j += kCL)
+  for (long long j = b + q; j < e; j += CL)
     raw_add(a, aI, wide(cx[j]) - w0, wide(cy[j]) - w1, wide(cz[j]) - w2, wide(er[j]), lev[j]);
   if (aI != 0) a[kRI] = (double)aI;
-  cl_totals<kRawN>(a);
-  if (c < ncell) {
-#pragma unroll
-    for (int i = 0; i < kRawN / 4; ++i) rec[(size_t)c * kRawN + q * (kRawN / 4) + i] = a[i];
-  }
+  cl_store<CL, kRawN>(a, c < ncell, rec + (size_t)c * kRawN);
 }
 
 template <typename T>
@@ -1644,13 +1658,14 @@ __global__ void pl_mom_out(int ncell, const long long* __restrict__ off,
 // 70 FP64 instructions on a cell of 20 particles, most of them in reductions
 // and in the mean that the whole warp divided out: 173 us for 0.77 million
 // particles in 38,400 cells.)
+template <int CL>
 __global__ void __launch_bounds__(kBlk)
 pl_cell_sums(int ncell, const long long* __restrict__ off, const double* __restrict__ cx,
              const double* __restrict__ cy, const double* __restrict__ cz,
              const double* __restrict__ er, const int* __restrict__ lev,
              double* __restrict__ rec) {
-  const int q = threadIdx.x & (kCL - 1);
-  const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kCL;
+  const int q = threadIdx.x & (CL - 1);
+  const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / CL;
   const long long b = c < ncell ? off[c] : 0, e = c < ncell ? off[c + 1] : 0;
   double a[kNAcc];
 #pragma unroll
@@ -1659,7 +1674,7 @@ pl_cell_sums(int ncell, const long long* __restrict__ off, const double* __restr
   if (b < e) { r0 = cx[b]; r1 = cy[b]; r2 = cz[b]; }
   long long sl = 0;
 #pragma unroll 2
-  for (long long j = b + q; j < e; j += kCL) {
+  for (long long j = b + q; j < e; j += CL) {
     const double d0 = cx[j] - r0, d1 = cy[j] - r1, d2 = cz[j] - r2;
     a[0] += d0; a[1] += d1; a[2] += d2;
     a[3] = fma(d0, d0, a[3]); a[4] = fma(d1, d1, a[4]); a[5] = fma(d2, d2, a[5]);
@@ -1668,11 +1683,7 @@ pl_cell_sums(int ncell, const long long* __restrict__ off, const double* __restr
     sl += lev[j];
   }
   if (sl != 0) a[10] = (double)sl;
-  cl_totals<kNAcc>(a);
-  if (c < ncell) {
-#pragma unroll
-    for (int i = 0; i < kNAcc / 4; ++i) rec[(size_t)c * kNAcc + q * (kNAcc / 4) + i] = a[i];
-  }
+  cl_store<CL, kNAcc>(a, c < ncell, rec + (size_t)c * kNAcc);
 }
 
 __global__ void __launch_bounds__(kBlk)
@@ -1842,10 +1853,12 @@ struct PlaneCtx {
 
 namespace {
 
-// grid of the passes with kCL lanes per cell
-int cell_grid(const PlaneCtx* h) {
-  return (int)(((long long)h->g.ncell * kCL + kBlk - 1) / kBlk);
+// grid of the passes with cl lanes per cell
+int cell_grid(const PlaneCtx* h, int cl = kCL) {
+  return (int)(((long long)h->g.ncell * cl + kBlk - 1) / kBlk);
 }
+// whether the FP64 sums by cell take a warp per cell
+bool wide_cells(const PlaneCtx* h) { return h->g.ncell <= kWideCells; }
 
 #define CHK(x)                                 \
   do {                                         \
@@ -2068,7 +2081,9 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
         (const float*)cy, (const float*)cz, (const float*)er, h->lv[b], h->cells, env.sp,
         env.flags, env.counters, pend, (float*)h->fT, h->usable_c);
   else if constexpr (sizeof(T) == 8) {
-    pl_cell_sums<<<cell_grid(h), kBlk, 0, s>>>(ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc);
+    const int cl = wide_cells(h) ? 32 : kCL;
+    (cl == 32 ? pl_cell_sums<32> : pl_cell_sums<kCL>)<<<cell_grid(h, cl), kBlk, 0, s>>>(
+        ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc);
     pl_cell_fields<<<(ncell + kBlk - 1) / kBlk, kBlk, 0, s>>>(
         ncell, h->off, h->af, cx, cy, cz, h->macc, h->cells, env.sp, env.counters, (T*)h->fT,
         h->usable_c);
@@ -2118,10 +2133,13 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
                                               env.k0, env.k1, env.flags, env.counters, nullptr);
   CHK(cudaGetLastError());
   if (h->sampling) {
-    if constexpr (sizeof(T) == 4)
+    if constexpr (sizeof(T) == 4) {
       pl_sample_f32<<<cell_grid(h), kBlk, 0, s>>>(ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc);
-    else
-      pl_sample<<<cell_grid(h), kBlk, 0, s>>>(ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc);
+    } else {
+      const int cl = wide_cells(h) ? 32 : kCL;
+      (cl == 32 ? pl_sample<32> : pl_sample<kCL>)<<<cell_grid(h, cl), kBlk, 0, s>>>(
+          ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc);
+    }
     pl_sample_add<<<(ncell + kBlk - 1) / kBlk, kBlk, 0, s>>>(ncell, h->off, h->cells, h->macc,
                                                              h->acc);
     CHK(cudaGetLastError());
@@ -2441,8 +2459,9 @@ int pl_moments(PlaneCtx* h, const ChEnv& env, double* out, int out_is_device) {
       using T = decltype(t);
       const T* cx = (const T*)h->st[b][2]; const T* cy = (const T*)h->st[b][3];
       const T* cz = (const T*)h->st[b][4]; const T* er = (const T*)h->st[b][5];
-      pl_mom_sums<T><<<cell_grid(h), kBlk, 0, s>>>(ncell, h->off, cx, cy, cz, er, h->lv[b],
-                                                   h->macc);
+      const int cl = wide_cells(h) ? 32 : kCL;
+      (cl == 32 ? pl_mom_sums<T, 32> : pl_mom_sums<T, kCL>)<<<cell_grid(h, cl), kBlk, 0, s>>>(
+          ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc);
       pl_mom_out<T><<<(ncell + kBlk - 1) / kBlk, kBlk, 0, s>>>(ncell, h->off, h->cells, cx, cy, cz,
                                                                h->macc, h->mout, env.sp);
     };

@@ -261,3 +261,29 @@ def test_gillespie_levels_match_oracle(precision, T):
     # FP32 rates differ from the oracle's in the last bit: a few decisions turn
     assert np.sum(lev != st.lev) <= (0 if form == 0 else 20)
     ctx.destroy()
+
+
+@pytest.mark.parametrize("precision", [usp.USP_FP64, usp.USP_FP32])
+@pytest.mark.parametrize("nx", [181, 182])          # 32,761 and 33,124 cells
+def test_plane_sums_on_both_sides_of_the_warp_per_cell_rule(precision, nx):
+    w = I.cylinder_flow(nx=nx, ny=nx, ppc=3.0)
+    p = w.particles
+    dt = w.dt_over_tau_c * usp.usp_tau_c(w.species, w.plane["n_inf"], w.plane["T_inf"])
+    ctx = usp.usp_init_plane(w.species, w.plane, dt, w.area_frac, w.x, w.y, p.cx, p.cy, p.cz,
+                             p.erot, p.lev, w.capacity, precision=precision, seed=4)
+    assert (ctx.n_cells <= 32768) == (nx == 181)
+    usp.usp_sample(ctx, True)
+    usp.usp_step(ctx, 2)
+    cx, cy, cz, er, lev = usp.usp_plane_get_particles(ctx)[2:7]
+    mom = usp.usp_moments(ctx)
+    off = np.concatenate([[0], np.cumsum(mom[0].astype(np.int64))])
+    pick = np.linspace(0, ctx.n_cells - 1, 900).astype(int)
+    ref, scale = [], []
+    c = np.stack([cx, cy, cz])
+    for i in pick:
+        k = slice(off[i], off[i + 1])
+        r, s = _moments(w.species, np.array([0, off[i + 1] - off[i]]), c[:, k], er[k], lev[k])
+        ref.append(r[:, 0])
+        scale.append(s[:, 0])
+    _near(mom[:, pick], np.array(ref).T, 16e-12 * np.array(scale).T + 1e-300)
+    ctx.destroy()
