@@ -473,10 +473,7 @@ ch_collide(int c0, int ny, double dy, int recon, double dt, const ChCellT<S>* __
       const bool above = dyv >= T(0);
       T f[kNF];
 #pragma unroll
-      for (int q = 0; q < kNF; ++q) {
-        if constexpr (kFastForm<T>) f[q] = madd(P.F[q], above ? P.Sp[q] : P.Sm[q], dyv);
-        else f[q] = P.F[q] + (above ? P.Sp[q] : P.Sm[q]) * dyv;
-      }
+      for (int q = 0; q < kNF; ++q) f[q] = madd(P.F[q], above ? P.Sp[q] : P.Sm[q], dyv);
       if (!(f[3] > T(0)) || !(f[4] > T(0)) || !(f[5] >= T(0))) {
 #pragma unroll
         for (int q = 0; q < kNF; ++q) f[q] = P.F[q];

@@ -228,7 +228,15 @@ __device__ inline Dual<double, N> rsqrt(const Dual<double, N>& a) {
   const double r = d_rsqrt(a.v);
   return chain(a, r, -0.5 * r * (r * r));
 }
-// f + a b
+// f + a b (FP32: the value by one fused operation whatever is compiled around it, so
+// that the form's values do not depend on it)
+__device__ inline Dual<float> madd(const Dual<float>& f, const Dual<float>& a,
+                                   const Dual<float>& b) {
+  Dual<float> r;
+  r.v = __fmaf_rn(a.v, b.v, f.v);
+  for (int i = 0; i < kND; ++i) r.d[i] = f.d[i] + (a.d[i] * b.v + a.v * b.d[i]);
+  return r;
+}
 template <int N>
 __device__ inline Dual<double, N> madd(const Dual<double, N>& f, const Dual<double, N>& a,
                                        const Dual<double, N>& b) {
