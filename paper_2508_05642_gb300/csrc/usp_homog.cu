@@ -2370,6 +2370,7 @@ int step_host_chunked(usp_ctx* c, const void* hx, const void* hy, const void* hz
     CK(cudaStreamWaitEvent(c->copy_stream, c->up_ev[0], 0));
     CK(cudaStreamWaitEvent(c->aux_stream, c->up_ev[0], 0));
     int cb = 0;
+    cudaEvent_t uploaded = c->up_ev[0];   // the last run's upload
     for (int k = 0; k < K; ++k) {
       const int ca = cb;
       const long long target = n * (k + 1) / K;
@@ -2380,6 +2381,7 @@ int step_host_chunked(usp_ctx* c, const void* hx, const void* hy, const void* hz
         CK(cudaMemcpyAsync(dst[f] + b * sz[f], src[f] + b * sz[f], (e - b) * sz[f],
                            cudaMemcpyHostToDevice, c->copy_stream));
       CK(cudaEventRecord(c->up_ev[k + 1], c->copy_stream));
+      uploaded = c->up_ev[k + 1];
       c->stream = (k & 1) ? c->aux_stream : main;
       CK(cudaStreamWaitEvent(c->stream, c->up_ev[k + 1], 0));
       const CellRange r = cell_range(c, ca, cb);
@@ -2408,6 +2410,9 @@ int step_host_chunked(usp_ctx* c, const void* hx, const void* hy, const void* hz
       }
     }
     if (out && !early) {
+      // the outputs may overlap the inputs: none is written before the last run
+      // has been read (uploads from pinned memory are still queued here)
+      CK(cudaStreamWaitEvent(c->down_stream, uploaded, 0));
       cb = 0;
       for (int k = 0; k < K; ++k) {
         const int ca = cb;

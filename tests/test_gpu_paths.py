@@ -287,3 +287,44 @@ def test_plane_sums_on_both_sides_of_the_warp_per_cell_rule(precision, nx):
         scale.append(s[:, 0])
     _near(mom[:, pick], np.array(ref).T, 16e-12 * np.array(scale).T + 1e-300)
     ctx.destroy()
+
+
+@pytest.mark.parametrize("precision", [usp.USP_FP64, usp.USP_FP32])
+@pytest.mark.parametrize("ncell", [40, 400])        # one compute kernel a run, or three
+def test_host_step_reads_every_input_before_it_writes_an_overlapping_output(precision, ncell):
+    """Pinned outputs half a state away from the inputs they overlap, within one
+    field and across two: what a first run of cells sends down lies where the later
+    runs still come from."""
+    torch = pytest.importorskip("torch")
+    spd = I.n2_vhs_relaxation_species()
+    sizes = np.random.default_rng(ncell).integers(1, 2 * (3_000_000 // ncell), ncell)
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    n = int(off[-1])
+    p = I.equilibrium_particles(np.random.default_rng(1), n, spd["m"], spd["theta_v"],
+                                T_tr=15000.0, T_rot=800.0, T_vib=2500.0)
+    p = p.astype_f32_exact()
+    nd = np.full(ncell, 1e23)
+    dt = np.full(ncell, 0.5 * usp.usp_tau_c(spd, 1e23, 15000.0))
+    new = lambda: usp.usp_init_homogeneous(spd, off, nd, dt, p.cx, p.cy, p.cz, p.erot, p.lev,
+                                           precision=precision, seed=3)
+    ft = torch.float32 if precision == usp.USP_FP32 else torch.float64
+    mk = lambda m, t: torch.empty(m, dtype=t, pin_memory=True).numpy()
+    ctx = new()
+    usp.usp_step(ctx, 1)
+    ref = usp.usp_get_particles(ctx)
+    ctx.destroy()
+    h = n // 2
+    # x comes down into x half a state on; y into the half of z's input
+    bx, bz = mk(n + h, ft), mk(n + h, ft)
+    src = [bx[:n], mk(n, ft), bz[:n], mk(n, ft), mk(n, torch.int32)]
+    out = [bx[h:], bz[h:], mk(n, ft), mk(n, ft), mk(n, torch.int32)]
+    for a, b in zip(src, (p.cx, p.cy, p.cz, p.erot, p.lev)):
+        a[:] = b
+    mom = np.zeros((usp.USP_NMOM, ncell))
+    ctx = new()
+    usp.usp_step_host(ctx, *src, 1, mom, out=out)
+    # the sums are atomic, so that two runs part by roundings
+    assert np.mean(out[4] != ref[4]) < 1e-5
+    for a, b in zip(out[:4], ref[:4]):
+        assert np.max(np.abs(a - b)) < 1e-4 * np.max(np.abs(b))
+    ctx.destroy()
