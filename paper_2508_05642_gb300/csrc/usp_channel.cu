@@ -149,17 +149,17 @@ __device__ void wall_emit(const Species& sp, uint32_t pid, uint32_t step, int hi
   const double u2 = (double)value(uniform_open<T>(w.z));
   const double u3 = (double)value(uniform_open<T>(w.w));
   const double u4 = (double)value(uniform_open<T>(v.x));
-  const S vn = sqrt(-2.0 * R * Tw * d_log(u0));
+  const S vn = sqrt(-2.0 * R * Tw * log(u0));
   vy = into_pos ? vn : -vn;
   double sn, cn;
-  const double rad = sqrt_fast(-2.0 * d_log(u1));
+  const double rad = sqrt_fast(-2.0 * log(u1));
   sincospi(2.0 * u2, &sn, &cn);
   const double g1 = rad * cn, g2 = rad * sn;
   const S s = sqrt(R * Tw);
   vx = s * g1;
   vz = s * g2;
-  e = -R * Tw * d_log(u3);
-  l = (int)floor(-d_log(u4) * value(Tw) / sp.theta_v);
+  e = -R * Tw * log(u3);
+  l = (int)floor(-log(u4) * value(Tw) / sp.theta_v);
 }
 
 template <typename T, typename S>

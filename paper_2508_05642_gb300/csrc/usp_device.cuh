@@ -129,29 +129,13 @@ template <> __device__ __forceinline__ float uniform_open<float>(uint32_t x) {
 
 // Square root in the FP32 particle arithmetic: the hardware approximation
 // (relative error about 2^-23), not the correctly rounded square root's longer
-// sequence; the double form keeps sqrt.
+// sequence; the double form is the square root (usp_math.cuh).
 __device__ __forceinline__ float sqrt_fast(float x) {
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// FP64: the hardware reciprocal square root (about 2^-20), one Goldschmidt
-// step for the root and its half reciprocal together and Markstein's residual
-// correction (P. Markstein, "IA-64 and Elementary Functions", 2000), five
-// multiply-adds in all; the library function outside exponents +-900, which
-// also answers zero, negative values, infinities and NaN.
-__device__ __forceinline__ double sqrt_fast(double x) {
-  const int hi = __double2hiint(x);
-  if ((unsigned)(hi - (123 << 20)) > (unsigned)(1800 << 20)) return sqrt(x);
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double g = x * y;
-  double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));   // y / 2
-  const double r = fma(-g, h, 0.5);
-  g = fma(g, r, g);
-  h = fma(h, r, h);
-  return fma(fma(-g, g, x), h, g);
-}
+__device__ __forceinline__ double sqrt_fast(double x) { return d_sqrt(x); }
 
 // Box-Muller pair: G_a = sqrt(-2 ln u_a) cos(2 pi u_b), G_b = ... sin(2 pi u_b).
 // The float version takes -2 ln u = -2 ln 2 log2 u with the hardware base-2
@@ -513,7 +497,7 @@ __device__ __forceinline__ double solve_cv_T1(double Rtheta, double theta, doubl
   for (int it = 0; it < 50; ++it) {
     const double iden = d_rcp(fma(gv, x, D));
     const double Tc = fma(fma(gv * x, dT, a0), iden, Ttr), d = Tc - Tvib;
-    const double xx = theta * d_rcp(Tc), iE = d_rcp(d_expm1(xx));
+    const double xx = theta * d_rcp(Tc), iE = d_rcp(expm1(xx));
     const bool cold = !(Tc > 0.0);
     const double ec = cold ? 0.0 : Rtheta * iE, cvc = cold ? 0.0 : R * (xx * xx) * (iE * (1.0 + iE));
     const bool near = fabs(d) <= 1e-9 * fmax(fabs(Tc), fabs(Tvib));
@@ -563,18 +547,15 @@ __device__ __forceinline__ double cell_prandtl(const VibState& v) {
 
 // quotient and cube root by type (derivative numbers bring their own)
 __device__ __forceinline__ double c_div(double a, double b) { return d_div(a, b); }
-__device__ __forceinline__ double c_cbrt(double a) { return d_cbrt(a); }
 template <typename S>
 __device__ __forceinline__ S c_div(const S& a, const S& b) { return a / b; }
-template <typename S>
-__device__ __forceinline__ S c_cbrt(const S& a) { return cbrt(a); }
 
 // The coefficients in the parts that depend on one another: mu / p and xw = (T /
 // T_ref)^omega; A, B, alpha and nu (from mu / p and Pr); the gamma coefficients
 // and the targets (from mu / p, xw and tauf = tau_c / (mu / p)).
 __device__ __forceinline__ void cell_mu_p(const Species& s, double n, double Ttr, double& mu_p,
                                           double& xw) {
-  xw = d_exp(s.omega * d_log(Ttr * s.iT_ref));
+  xw = exp(s.omega * log(Ttr * s.iT_ref));
   mu_p = s.mu_ref0 * xw * d_rcp(n * kB * Ttr);
 }
 // mu at T_ref through omega (derivative form)
@@ -590,7 +571,7 @@ __device__ __forceinline__ void cell_alpha(CellCoeffsT<S>& c, double dt) {
   c.A = c_div(m2 - pd, m2 + pd);
   c.B = c_div(m2 - dt, m2 + dt);
   c.ok = c.A > -1.0 && c.A < 1.0;
-  c.alpha = c.ok ? c_cbrt(c.A) : S(0.0);
+  c.alpha = c.ok ? cbrt(c.A) : S(0.0);
   const S a2 = c.alpha * c.alpha;
   c.nu_ref = c_div(c.B - a2, 1.0 - a2);
 }
@@ -614,7 +595,7 @@ __device__ __forceinline__ void cell_gammas(const Species& s, CellCoeffsT<S>& c,
     const double d = (double)Tc - v.Tvib;
     if (!(::fabs(d) <= 1e-9 * ::fmax(::fabs((double)Tc), ::fabs(v.Tvib))) && Tc > 0.0) {
       // dF = (c_v,vib(T_check) - F) / (T_check - T_vib) dT_check
-      const double xx = th * d_rcp((double)Tc), iE = d_rcp(d_expm1(xx));
+      const double xx = th * d_rcp((double)Tc), iE = d_rcp(expm1(xx));
       const double cvc = R * (xx * xx) * (iE * (1.0 + iE));
       const double dF = -(double)gv * (cvc - xv) * (double)iden;
       const double k = d_div(cvc - xv, d * (1.0 - dF));

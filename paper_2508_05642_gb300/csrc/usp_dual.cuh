@@ -32,15 +32,15 @@ constexpr int kND = 3;
 __device__ inline float vsqrt(float x) { return sqrtf(x); }
 __device__ inline double vsqrt(double x) { return sqrt_fast(x); }
 __device__ inline float vlog(float x) { return logf(x); }
-__device__ inline double vlog(double x) { return d_log(x); }
+__device__ inline double vlog(double x) { return ::log(x); }
 __device__ inline float vlog1p(float x) { return log1pf(x); }
 __device__ inline double vlog1p(double x) { return ::log1p(x); }
 __device__ inline float vexp(float x) { return expf(x); }
-__device__ inline double vexp(double x) { return d_exp(x); }
+__device__ inline double vexp(double x) { return ::exp(x); }
 // exp(x) - 1 and its derivative
 __device__ inline float vexpm1(float x, float& df) { df = expf(x); return expm1f(x); }
 __device__ inline double vexpm1(double x, double& df) {
-  const double e = d_expm1(x);
+  const double e = ::expm1(x);
   df = e + 1.0;
   return e;
 }
@@ -55,7 +55,7 @@ __device__ inline double vsin(double x) { return ::sin(x); }
 __device__ inline float vacos(float x) { return acosf(x); }
 __device__ inline double vacos(double x) { return ::acos(x); }
 __device__ inline float vcbrt(float x) { return cbrtf(x); }
-__device__ inline double vcbrt(double x) { return d_cbrt(x); }
+__device__ inline double vcbrt(double x) { return ::cbrt(x); }
 __device__ inline float vpow(float x, float y) { return powf(x, y); }
 __device__ inline double vpow(double x, double y) { return ::pow(x, y); }
 // a / b, and the quotients d_i / b of the derivatives

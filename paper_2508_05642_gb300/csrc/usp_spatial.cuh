@@ -207,7 +207,7 @@ __device__ __forceinline__ void relax_fast(const P_& P, double ioR, const double
   ttr = f[3] - (x + y) * (ioR * (2.0 / 3.0));
   trot = f[4] + (x - z) * ioR;
   const double ev =
-      f[5] > 0.0 ? P.R * P.theta * d_rcp(d_expm1(P.theta * d_rcp(f[5]))) : 0.0;
+      f[5] > 0.0 ? P.R * P.theta * d_rcp(expm1(P.theta * d_rcp(f[5]))) : 0.0;
   evr = ev + (y + z) * (ioR * P.R);
   cl = false;
   if (ttr < 0.0) { ttr = 0.0; cl = true; }
@@ -965,7 +965,7 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
       if constexpr (nl > 1)
         put_part(xw, exp(lane_part(omega, t) * log(T * sp.iT_ref)), t);
       else
-        xw = d_exp(sp.omega * d_log(T * sp.iT_ref));
+        xw = exp(sp.omega * log(T * sp.iT_ref));
     } else if (t == 32) {
       vib = vib_state(sp, cs.ebar);
       k.Pr = S(cell_prandtl(vib));
