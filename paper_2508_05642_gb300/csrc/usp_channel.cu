@@ -118,7 +118,6 @@ struct ChParams {
   // the derivative form differentiates by none of these
   using C = std::conditional_t<std::is_same<T, D3>::value, double, T>;
   C R, theta, dt, yc;
-  C iRth;                       // kFastForm: 1 / (R theta)
   std::conditional_t<kFastForm<T>, AlphaParts<T>, int> ap;
   T F[kNF], Sm[kNF], Sp[kNF];   // cell values; slopes used below / above the centroid
   int active, pad;
@@ -149,17 +148,17 @@ __device__ void wall_emit(const Species& sp, uint32_t pid, uint32_t step, int hi
   const double u2 = (double)value(uniform_open<T>(w.z));
   const double u3 = (double)value(uniform_open<T>(w.w));
   const double u4 = (double)value(uniform_open<T>(v.x));
-  const S vn = sqrt(-2.0 * R * Tw * log(u0));
+  const S vn = sqrt(-2.0 * R * Tw * d_log(u0));
   vy = into_pos ? vn : -vn;
   double sn, cn;
-  const double rad = sqrt_fast(-2.0 * log(u1));
+  const double rad = sqrt_fast(-2.0 * d_log(u1));
   sincospi(2.0 * u2, &sn, &cn);
   const double g1 = rad * cn, g2 = rad * sn;
   const S s = sqrt(R * Tw);
   vx = s * g1;
   vz = s * g2;
-  e = -R * Tw * log(u3);
-  l = (int)floor(-log(u4) * value(Tw) / sp.theta_v);
+  e = -R * Tw * d_log(u3);
+  l = (int)floor(-d_log(u4) * value(Tw) / sp.theta_v);
 }
 
 template <typename T, typename S>
@@ -438,11 +437,17 @@ __device__ void ch_recon(int c, int ny, double dy, int recon, double dt,
     using C = typename ChParams<T>::C;
     P.R = (C)gasR(sp); P.theta = (C)sp.theta_v; P.dt = (C)dt;
     P.yc = (C)((c + 0.5) * dy);
-    if constexpr (kFastForm<T>) {
-      P.iRth = sp.iRtheta;
-      P.ap = alpha_parts(P.alpha, P.R);
-    }
   }
+  if constexpr (kFastForm<T>)
+    if (t >= 64 && t < 70) {   // a factor each
+      const T alpha = (T)cs.alpha, oma2 = 1.0 - alpha * alpha;
+      const int i = t - 64;
+      P.ap.g[i] = alpha_factor<T>(i, oma2, (T)cs.gtr, (T)cs.gtv, (T)cs.grv, gasR(sp), sp.theta_v);
+      if (i == 0) {
+        P.ap.oma2 = oma2;
+        P.ap.sq = root_sel<true>(oma2);
+      }
+    }
 }
 
 // METHOD 1: the plain FPM method (Sec. 2.C) with the cell values and the

@@ -49,7 +49,8 @@ struct Species {
   // derived on the host: T_ref^omega, pi d_ref^2 / sigma_vib, R = k_B / m,
   // and the VSS mu_ref and tau_c / (mu / p) at this omega
   double Tref_w, zv_ht, R, mu_ref0, tauf0;
-  double iT_ref, iR, iRtheta;   // 1 / T_ref, 1 / R, 1 / (R Theta_v)
+  // divisors of the cell's fields and coefficients, and their reciprocals
+  double R3, Rtheta, iT_ref, iR, iR3, iRtheta;   // 3 R, R Theta_v
   int method;   // 0 USP-FPM (Sec. 3, 4), 1 the plain FPM method (Sec. 2.C)
 };
 
@@ -555,8 +556,8 @@ __device__ __forceinline__ S c_div(const S& a, const S& b) { return a / b; }
 // and the targets (from mu / p, xw and tauf = tau_c / (mu / p)).
 __device__ __forceinline__ void cell_mu_p(const Species& s, double n, double Ttr, double& mu_p,
                                           double& xw) {
-  xw = exp(s.omega * log(Ttr * s.iT_ref));
-  mu_p = s.mu_ref0 * xw * d_rcp(n * kB * Ttr);
+  xw = exp(s.omega * d_log(d_div_by(Ttr, s.T_ref, s.iT_ref)));
+  mu_p = d_div(s.mu_ref0 * xw, n * kB * Ttr);
 }
 // mu at T_ref through omega (derivative form)
 template <typename S>
@@ -632,10 +633,10 @@ __device__ __forceinline__ void relax_temps(const Species& s, const CellCoeffs& 
                                             double Ttr, double Trot, double Tvib, double ev,
                                             double& ttr, double& trot, double& evr,
                                             bool& clamped) {
-  const double io = d_rcp(1.0 - alpha * alpha), ioR = io * s.iR;
-  ttr = Ttr - (c.g_tr_rot * (Ttr - Trot) + c.g_tr_vib * (Ttr - Tvib)) * (ioR * (2.0 / 3.0));
-  trot = Trot + (c.g_tr_rot * (Ttr - Trot) - c.g_rot_vib * (Trot - Tvib)) * ioR;
-  evr = ev + (c.g_tr_vib * (Ttr - Tvib) + c.g_rot_vib * (Trot - Tvib)) * io;
+  const double R = s.R, oma2 = 1.0 - alpha * alpha;
+  ttr = Ttr - d_div(c.g_tr_rot * (Ttr - Trot) + c.g_tr_vib * (Ttr - Tvib), oma2 * 1.5 * R);
+  trot = Trot + d_div(c.g_tr_rot * (Ttr - Trot) - c.g_rot_vib * (Trot - Tvib), oma2 * R);
+  evr = ev + d_div(c.g_tr_vib * (Ttr - Tvib) + c.g_rot_vib * (Trot - Tvib), oma2);
   clamped = false;
   if (ttr < 0.0) { ttr = 0.0; clamped = true; }
   if (trot < 0.0) { trot = 0.0; clamped = true; }
@@ -658,20 +659,18 @@ __device__ __forceinline__ bool chol3(const T* M, T* L) {
   return true;
 }
 
-// Cholesky factor (l00, l10, l11, l20, l21, l22) of a cell's (xx, yy, zz, xy, xz,
-// yz), by reciprocal square roots (usp_math.cuh)
-constexpr double kLeastPivot = 0x1p-1000;   // the reciprocal root needs a normal number
+// the same on usp_math.cuh, both quotients of a pivot with its one reciprocal
 __device__ __forceinline__ bool chol3_cell(const double* M, double* L) {
-  if (!(M[0] > kLeastPivot)) return false;
-  const double r0 = d_rsqrt(M[0]);
-  const double l10 = M[3] * r0, l20 = M[4] * r0;
+  if (!d_pos(M[0])) return false;
+  double r0, r1;
+  const double l00 = d_sqrt(M[0], r0);
+  const double l10 = d_div_by(M[3], l00, r0), l20 = d_div_by(M[4], l00, r0);
   const double d1 = M[1] - l10 * l10;
-  if (!(d1 > kLeastPivot)) return false;
-  const double r1 = d_rsqrt(d1);
-  const double l21 = (M[5] - l20 * l10) * r1;
+  if (!d_pos(d1)) return false;
+  const double l11 = d_sqrt(d1, r1), l21 = d_div_by(M[5] - l20 * l10, l11, r1);
   const double d2 = M[2] - l20 * l20 - l21 * l21;
-  if (!(d2 > kLeastPivot)) return false;
-  L[0] = M[0] * r0; L[1] = l10; L[2] = d1 * r1; L[3] = l20; L[4] = l21; L[5] = d_sqrt(d2);
+  if (!d_pos(d2)) return false;
+  L[0] = l00; L[1] = l10; L[2] = l11; L[3] = l20; L[4] = l21; L[5] = d_sqrt(d2);
   return true;
 }
 

@@ -28,11 +28,11 @@ constexpr int kND = 3;
 
 // elementary functions of the value type: FP32 the library's, FP64 those of
 // usp_math.cuh (a derivative number's division took four divisions by the
-// same value, 38 FP64 operations of a particle's lane; now 17)
+// same value, 38 FP64 operations of a particle's lane; now 23)
 __device__ inline float vsqrt(float x) { return sqrtf(x); }
 __device__ inline double vsqrt(double x) { return sqrt_fast(x); }
 __device__ inline float vlog(float x) { return logf(x); }
-__device__ inline double vlog(double x) { return ::log(x); }
+__device__ inline double vlog(double x) { return d_log(x); }
 __device__ inline float vlog1p(float x) { return log1pf(x); }
 __device__ inline double vlog1p(double x) { return ::log1p(x); }
 __device__ inline float vexp(float x) { return expf(x); }
@@ -58,16 +58,14 @@ __device__ inline float vcbrt(float x) { return cbrtf(x); }
 __device__ inline double vcbrt(double x) { return ::cbrt(x); }
 __device__ inline float vpow(float x, float y) { return powf(x, y); }
 __device__ inline double vpow(double x, double y) { return ::pow(x, y); }
-// a / b, and the quotients d_i / b of the derivatives
+// a / b, and the same for y = 1 / b known (FP64: the value's and the derivatives'
+// quotients share it)
 __device__ inline float vdiv(float a, float b) { return a / b; }
 __device__ inline double vdiv(double a, double b) { return d_div(a, b); }
-template <int N>
-__device__ inline void vdivn(float (&d)[N], float b) { for (int i = 0; i < N; ++i) d[i] = d[i] / b; }
-template <int N>
-__device__ inline void vdivn(double (&d)[N], double b) {
-  const double y = d_rcp(b);
-  for (int i = 0; i < N; ++i) d[i] *= y;
-}
+__device__ inline float vrcp(float) { return 0.0f; }
+__device__ inline double vrcp(double b) { return d_rcp(b); }
+__device__ inline float vdiv_by(float a, float b, float) { return a / b; }
+__device__ inline double vdiv_by(double a, double b, double y) { return d_div_by(a, b, y); }
 
 template <typename V, int N = kND>
 struct Dual {
@@ -101,12 +99,15 @@ struct Dual {
     v *= b.v;
     return *this;
   }
-  __device__ Dual& operator/=(const Dual& b) {
-    const V q = vdiv(v, b.v);
-    for (int i = 0; i < N; ++i) d[i] = d[i] - q * b.d[i];
-    vdivn(d, b.v);
+  // y = 1 / b.v
+  __device__ Dual& div_by(const Dual& b, V y) {
+    const V q = vdiv_by(v, b.v, y);
+    for (int i = 0; i < N; ++i) d[i] = vdiv_by(d[i] - q * b.d[i], b.v, y);
     v = q;
     return *this;
+  }
+  __device__ Dual& operator/=(const Dual& b) {
+    return div_by(b, vrcp(b.v));
   }
 };
 
@@ -172,9 +173,9 @@ template <typename V, int N>
 __host__ __device__ inline Dual<V, N> operator*(double b, Dual<V, N> a) { return a * b; }
 template <typename V, int N>
 __device__ inline Dual<V, N> operator/(Dual<V, N> a, double b) {
-  const V c = V(b);
-  a.v = vdiv(a.v, c);
-  vdivn(a.d, c);
+  const V c = V(b), y = vrcp(c);
+  a.v = vdiv_by(a.v, c, y);
+  for (int i = 0; i < N; ++i) a.d[i] = vdiv_by(a.d[i], c, y);
   return a;
 }
 template <typename V, int N>
@@ -217,16 +218,6 @@ template <typename V, int N>
 __device__ inline Dual<V, N> sqrt(const Dual<V, N>& a) {
   const V s = vsqrt(a.v);
   return chain(a, s, s > V(0) ? vdiv(V(0.5), s) : V(0));
-}
-template <int N>
-__device__ inline Dual<double, N> rcp(const Dual<double, N>& a) {
-  const double r = d_rcp(a.v);
-  return chain(a, r, -(r * r));
-}
-template <int N>
-__device__ inline Dual<double, N> rsqrt(const Dual<double, N>& a) {
-  const double r = d_rsqrt(a.v);
-  return chain(a, r, -0.5 * r * (r * r));
 }
 // f + a b (FP32: the value by one fused operation whatever is compiled around it, so
 // that the form's values do not depend on it)

@@ -1087,7 +1087,7 @@ __device__ void write_params(const Species& sp, CellState& cs, CollideParams<T>&
   const double arot = R * dd.Trot_rel * oma2 / 2.0;
   P.a_rot = (T)arot;
   P.sqrt_a = (T)sqrt_fast(arot);
-  const double eb = dd.evib_rel * sp.iRtheta;
+  const double eb = d_div_by(dd.evib_rel, sp.Rtheta, sp.iRtheta);
   P.p_nb = (T)d_rcp(1.0 + eb * oma2);
   P.p_b = (T)((1.0 + eb) * oma2);
 }
@@ -1337,8 +1337,8 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
   }
   for (int i = 0; i < 3; ++i) { cs.U[i] = Un[i]; cs.Us[i] = Us[i]; }
   for (int i = 0; i < 6; ++i) cs.Pi[i] = s * s * Ps[i];
-  cs.Ttr = (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]) * (sp.iR * (1.0 / 3.0));
-  cs.Trot = e_rot_new * sp.iR;
+  cs.Ttr = d_div_by(cs.Pi[0] + cs.Pi[1] + cs.Pi[2], sp.R3, sp.iR3);
+  cs.Trot = d_div_by(e_rot_new, R, sp.iR);
   cs.ebar = sumI * invN;
   cs.s = s;
   cs.r = r;
@@ -1436,8 +1436,8 @@ few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
     }
     for (int i = 0; i < 3; ++i) { cs.U[i] = Un[i]; cs.Us[i] = Us[i]; }
     for (int i = 0; i < 6; ++i) cs.Pi[i] = sc * sc * Ps[i];
-    cs.Ttr = (cs.Pi[0] + cs.Pi[1] + cs.Pi[2]) * (sp.iR * (1.0 / 3.0));
-    cs.Trot = e_rot_new * sp.iR;
+    cs.Ttr = d_div_by(cs.Pi[0] + cs.Pi[1] + cs.Pi[2], sp.R3, sp.iR3);
+    cs.Trot = d_div_by(e_rot_new, R, sp.iR);
     cs.s = sc;
     cs.step += 1;
     cs.maxI = sizeof(T) == 8 ? S.top : S.maxI + 1;
@@ -1489,7 +1489,7 @@ few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
     P.a_rot = (T)arot;
     P.sqrt_a = (T)sqrt_fast(arot);
   } else if (K.ok && t == 96) {
-    const double oma2 = 1.0 - dd.alpha * dd.alpha, eb = dd.evib_rel * sp.iRtheta;
+    const double oma2 = 1.0 - dd.alpha * dd.alpha, eb = d_div_by(dd.evib_rel, sp.Rtheta, sp.iRtheta);
     P.p_nb = (T)d_rcp(1.0 + eb * oma2);
     P.p_b = (T)((1.0 + eb) * oma2);
   }
@@ -1869,9 +1869,12 @@ Species to_dev(const usp_species* s) {
   d.Tref_w = std::pow(s->T_ref, s->omega);
   d.zv_ht = s->sigma_vib > 0 ? kPi * s->d_ref * s->d_ref / s->sigma_vib : 0.0;
   d.R = kB / s->m;
+  d.R3 = 3.0 * d.R;
+  d.Rtheta = d.R * s->theta_v;
   d.iT_ref = 1.0 / s->T_ref;
   d.iR = 1.0 / d.R;
-  d.iRtheta = 1.0 / (d.R * s->theta_v);
+  d.iR3 = 1.0 / d.R3;
+  d.iRtheta = 1.0 / d.Rtheta;
   const double ca = s->c_alpha, w = s->omega;
   d.mu_ref0 = 5.0 * (ca + 1.0) * (ca + 2.0) * std::sqrt(s->m * kB * s->T_ref / kPi) /
               (4.0 * ca * (5.0 - 2.0 * w) * (7.0 - 2.0 * w) * s->d_ref * s->d_ref);

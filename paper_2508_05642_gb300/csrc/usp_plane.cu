@@ -131,7 +131,7 @@ struct alignas(16) PlParams {
   T alpha, nu_ref, B, mu_p, Pr, gtr, gtv, grv;
   T R, theta, dt;
   T xc, yc;
-  T iRth;               // 1 / (R theta)
+  T iRth;               // 1 / (R theta) (FP32 form)
   AlphaParts<T> ap;
   int active, pad;
 };
@@ -865,7 +865,7 @@ __device__ __forceinline__ void pl_scalars(PlParams<T>& P, const ChCellT<double>
   P.xc = (T)xc;
   P.yc = (T)yc;
   P.iRth = rcp_fast(P.R * P.theta);
-  P.ap = alpha_parts(P.alpha, P.R);
+  P.ap = alpha_parts(P, P.alpha);
 }
 
 template <typename T>
@@ -1723,8 +1723,8 @@ pl_cell_fields(int ncell, const long long* __restrict__ off, const double* __res
       const double P[6] = {fma(S[3], inv, -(m0 * m0)), fma(S[4], inv, -(m1 * m1)),
                            fma(S[5], inv, -(m2 * m2)), fma(S[6], inv, -(m0 * m1)),
                            fma(S[7], inv, -(m0 * m2)), fma(S[8], inv, -(m1 * m2))};
-      cs.Ttr = (P[0] + P[1] + P[2]) * (sp.iR * (1.0 / 3.0));
-      cs.Trot = S[9] * (inv * sp.iR);
+      cs.Ttr = d_div_by(P[0] + P[1] + P[2], sp.R3, sp.iR3);
+      cs.Trot = d_div_by(S[9] * inv, sp.R, sp.iR);
       cs.ebar = S[10] * inv;
       cs.Tvib = vib_state(sp, cs.ebar).Tvib;
       double* o = fT + (size_t)c * kNF;

@@ -162,26 +162,32 @@ __device__ __forceinline__ bool chol3_fast(const float* M, float* L) {
   return true;
 }
 
-// What of the collision depends on alpha alone: 1 - alpha^2, its root, and
-// 1 / ((1 - alpha^2) R).  A cell's particles share its alpha unless the
-// positivity fix changes it, so the stencil passes write these beside it
-// (28 of some 700 instructions of an FP32 particle, 20 of 210 FP64 operations).
+// What of the collision depends on alpha alone: 1 - alpha^2, its root, and what the
+// relaxation temperatures need.  A cell's particles share its alpha
+// unless the positivity fix changes it, so the stencil passes write these beside it
+// (28 of some 700 instructions of an FP32 particle).  FP32: 1 / ((1 - alpha^2) R).
+// FP64 and derivative numbers: the factors of the differences of temperatures, gamma_tr-rot
+// and gamma_tr-vib over (1 - alpha^2) 3/2 R, gamma_tr-rot and gamma_rot-vib over (1 -
+// alpha^2) R, gamma_tr-vib and gamma_rot-vib over (1 - alpha^2) R theta.
 template <typename T>
 struct AlphaParts {
-  T oma2, sq, ioR;
+  T oma2, sq, g[6];
 };
-__device__ __forceinline__ AlphaParts<float> alpha_parts(float alpha, float R) {
+template <>
+struct AlphaParts<float> {
+  float oma2, sq, ioR;
+};
+template <typename P_>
+__device__ __forceinline__ AlphaParts<float> alpha_parts(const P_& P, float alpha) {
   const float o = fmaf(-alpha, alpha, 1.f);
-  return {o, sqrtf(o), __frcp_rn(o * R)};
-}
-__device__ __forceinline__ AlphaParts<double> alpha_parts(double alpha, double R) {
-  const double o = fma(-alpha, alpha, 1.0);
-  return {o, sqrt_fast(o), d_rcp(o * R)};
+  return {o, sqrtf(o), __frcp_rn(o * P.R)};
 }
 
 template <typename P_>
-__device__ __forceinline__ void relax_fast(const P_& P, float ioR, const float* f, float& ttr,
-                                           float& trot, float& evr, bool& cl) {
+__device__ __forceinline__ void relax_fast(const P_& P, const AlphaParts<float>& ap,
+                                           const float* f, float& ttr, float& trot, float& evr,
+                                           bool& cl) {
+  const float ioR = ap.ioR;
   ttr = f[3] - (P.gtr * (f[3] - f[4]) + P.gtv * (f[3] - f[5])) * ioR * (2.f / 3.f);
   trot = f[4] + (P.gtr * (f[3] - f[4]) - P.grv * (f[4] - f[5])) * ioR;
   const float ev = f[5] > 0.f ? P.R * P.theta * __frcp_rn(expm1f(P.theta * __frcp_rn(f[5])))
@@ -193,78 +199,93 @@ __device__ __forceinline__ void relax_fast(const P_& P, float ioR, const float* 
   if (evr < 0.f) { evr = 0.f; cl = true; }
 }
 
-// FP64: the same on the functions of usp_math.cuh.  The library's divisions,
-// square roots and expm1 were two thirds of the FP64 operations of a particle
-// (0.77 million particles on 240 x 160 cells: the plane's FP64 collision pass
-// 1.47 ms).
+// FP64 and the derivative form, on the functions of usp_math.cuh: as many roundings as
+// relax_t and chol3_t have, but a product of a cell's factor where those divide, and
+// the vibrational energy in units of R theta.  The library's divisions, square roots and
+// expm1 were two thirds of the FP64 operations of a particle (0.77 million particles
+// on 240 x 160 cells: the plane's FP64 collision pass 1.47 ms).
+__device__ __forceinline__ float rcp_fast(float x) { return __frcp_rn(x); }   // as the form always took them
+__device__ __forceinline__ double rcp_fast(double x) { return d_rcp(x); }
+template <typename T>
+__device__ __forceinline__ T rcp_fast(const T& x) { return 1.0 / x; }
+__device__ __forceinline__ double div_by(double a, double b, double y) { return d_div_by(a, b, y); }
+template <int N>
+__device__ __forceinline__ dual::Dual<double, N> div_by(dual::Dual<double, N> a,
+                                                        const dual::Dual<double, N>& b, double y) {
+  return a.div_by(b, y);
+}
+template <bool kFast, typename T>
+__device__ __forceinline__ T root_sel(const T& x) {
+  if constexpr (kFast && sizeof(T) == 8) return d_sqrt(x);
+  else return sqrt(x);
+}
+// factor i of the six
+template <typename T>
+__device__ __forceinline__ T alpha_factor(int i, const T& oma2, const T& gtr, const T& gtv,
+                                          const T& grv, double R, double theta) {
+  const T num = i == 0 || i == 2 ? gtr : i == 1 || i == 4 ? gtv : grv;
+  const T den = i < 2 ? oma2 * 1.5 * R : oma2 * (i < 4 ? R : R * theta);
+  return c_div(num, den);
+}
+template <typename P_, typename T>
+__device__ __forceinline__ AlphaParts<T> alpha_parts(const P_& P, const T& alpha) {
+  AlphaParts<T> a;
+  a.oma2 = 1.0 - alpha * alpha;
+  a.sq = root_sel<true>(a.oma2);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) a.g[i] = alpha_factor<T>(i, a.oma2, P.gtr, P.gtv, P.grv, P.R, P.theta);
+  return a;
+}
 __device__ __forceinline__ bool chol3_fast(const double* M, double* L) {
   return chol3_cell(M, L);
 }
-template <typename P_>
-__device__ __forceinline__ void relax_fast(const P_& P, double ioR, const double* f, double& ttr,
-                                           double& trot, double& evr, bool& cl) {
-  const double x = P.gtr * (f[3] - f[4]), y = P.gtv * (f[3] - f[5]), z = P.grv * (f[4] - f[5]);
-  ttr = f[3] - (x + y) * (ioR * (2.0 / 3.0));
-  trot = f[4] + (x - z) * ioR;
-  const double ev =
-      f[5] > 0.0 ? P.R * P.theta * d_rcp(expm1(P.theta * d_rcp(f[5]))) : 0.0;
-  evr = ev + (y + z) * (ioR * P.R);
-  cl = false;
-  if (ttr < 0.0) { ttr = 0.0; cl = true; }
-  if (trot < 0.0) { trot = 0.0; cl = true; }
-  if (evr < 0.0) { evr = 0.0; cl = true; }
-}
-
-// The derivative form: the same with one reciprocal or reciprocal root per group
-// of divisions (a derivative number's division takes 17 FP64 operations, its
-// product 7).
 template <typename T>
-__device__ __forceinline__ AlphaParts<T> alpha_parts(const T& alpha, double R) {
-  const T o = 1.0 - alpha * alpha;
-  return {o, sqrt(o), rcp(o * R)};
-}
-template <typename T>
-__device__ __forceinline__ bool chol3_fast(const T* M, T* L) {
-  if (!(M[0] > kLeastPivot)) return false;
-  const T r0 = rsqrt(M[0]);
-  const T l10 = M[3] * r0, l20 = M[4] * r0;
-  const T d1 = M[1] - l10 * l10;
-  if (!(d1 > kLeastPivot)) return false;
-  const T r1 = rsqrt(d1);
-  const T l21 = (M[5] - l20 * l10) * r1;
-  const T d2 = M[2] - l20 * l20 - l21 * l21;
-  if (!(d2 > kLeastPivot)) return false;
-  L[0] = M[0] * r0; L[1] = l10; L[2] = d1 * r1; L[3] = l20; L[4] = l21; L[5] = sqrt(d2);
-  return true;
-}
-template <typename P_, typename T>
-__device__ __forceinline__ void relax_fast(const P_& P, const T& ioR, const T* f, T& ttr, T& trot,
-                                           T& evr, bool& cl) {
-  const T x = P.gtr * (f[3] - f[4]), y = P.gtv * (f[3] - f[5]), z = P.grv * (f[4] - f[5]);
-  ttr = f[3] - (x + y) * (ioR * (2.0 / 3.0));
-  trot = f[4] + (x - z) * ioR;
-  const T ev = f[5] > 0.0 ? P.R * P.theta * rcp(expm1(P.theta * rcp(f[5]))) : T(0);
-  evr = ev + (y + z) * (ioR * P.R);
-  cl = false;
-  if (ttr < 0.0) { ttr = T(0); cl = true; }
-  if (trot < 0.0) { trot = T(0); cl = true; }
-  if (evr < 0.0) { evr = T(0); cl = true; }
-}
-template <typename T>
-__device__ __forceinline__ T rcp_fast(const T& x) { return rcp(x); }
+__device__ __forceinline__ bool chol3_fast(const T* M, T* L) { return chol3_t(M, L); }
 // f + a b
 __device__ __forceinline__ float madd(float f, float a, float b) { return f + a * b; }
-__device__ __forceinline__ double madd(double f, double a, double b) { return f + a * b; }
-
-// the square roots and reciprocals of the collision: FP32 as the form always
-// took them, FP64 on usp_math.cuh
-template <bool kFast, typename T>
-__device__ __forceinline__ T root_sel(const T& x) {
-  if constexpr (kFast && sizeof(T) == 8) return sqrt_fast(x);
-  else return sqrt(x);
+__device__ __forceinline__ double madd(double f, double a, double b) { return fma(a, b, f); }
+// e_vib(T_vib) / (R theta)
+template <typename T>
+__device__ __forceinline__ T evib_fast(double theta, const T& Tv) {
+  return d_pos(value(Tv)) ? rcp_fast(T(expm1(c_div(T(theta), Tv)))) : T(0);
 }
-__device__ __forceinline__ float rcp_fast(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double rcp_fast(double x) { return d_rcp(x); }
+template <typename T>
+__device__ __forceinline__ bool clamp_temps(T& ttr, T& trot, T& evr) {
+  bool cl = false;
+  if (d_neg(value(ttr))) { ttr = T(0); cl = true; }
+  if (d_neg(value(trot))) { trot = T(0); cl = true; }
+  if (d_neg(value(evr))) { evr = T(0); cl = true; }
+  return cl;
+}
+template <typename T>
+__device__ __forceinline__ void relax_fast(const AlphaParts<T>& ap, const T* f, const T& ev, T& ttr,
+                                           T& trot, T& evr, bool& cl) {
+  const T tr = f[4] - f[3], tv = f[5] - f[3], rv = f[5] - f[4];
+  ttr = madd(madd(f[3], ap.g[1], tv), ap.g[0], tr);
+  trot = madd(madd(f[4], ap.g[3], rv), ap.g[2], -tr);
+  evr = madd(madd(ev, ap.g[5], -rv), ap.g[4], -tv);
+  cl = clamp_temps(ttr, trot, evr);
+}
+// the same after the positivity fix changed a particle's alpha, by quotients (the fix
+// is rare: a call)
+template <typename T>
+struct RelaxFixed {
+  T oma2, sq, ttr, trot, evr;
+  bool cl;
+};
+template <typename T>
+static __device__ __noinline__ RelaxFixed<T> relax_fixed(T alpha, T gtr, T gtv, T grv, double R,
+                                                         double theta, T Ttr, T Trot, T Tvib, T ev) {
+  RelaxFixed<T> r;
+  r.oma2 = 1.0 - alpha * alpha;
+  r.sq = root_sel<true>(r.oma2);
+  const T x = gtr * (Ttr - Trot), y = gtv * (Ttr - Tvib), z = grv * (Trot - Tvib);
+  r.ttr = Ttr - c_div(x + y, r.oma2 * 1.5 * R);
+  r.trot = Trot + c_div(x - z, r.oma2 * R);
+  r.evr = ev + c_div(y + z, r.oma2 * (R * theta));
+  r.cl = clamp_temps(r.ttr, r.trot, r.evr);
+  return r;
+}
 
 template <bool kFast, typename T>
 __device__ __forceinline__ bool chol3_sel(const T* M, T* L) {
@@ -289,17 +310,34 @@ __device__ __forceinline__ int collide_particle_t(const P_& P, const T* f, T& vx
                                                   const PhiloxRoundKeys& rk, CollideTally& t) {
   T alpha = P.alpha, nu = P.nu_ref, ttr, trot, evr;
   bool cl;
-  std::conditional_t<kFast, AlphaParts<T>, int> ap_;
-  if constexpr (kFast) {
-    ap_ = P.ap;
-    relax_fast(P, ap_.ioR, f, ttr, trot, evr, cl);
-  } else {
+  T oma2, sq, ev;                      // kFast: what goes with alpha
+  if constexpr (!kFast) {
     relax_t(P, alpha, f, ttr, trot, evr, cl);
+  } else if constexpr (sizeof(T) == 4) {
+    oma2 = P.ap.oma2;
+    sq = P.ap.sq;
+    relax_fast(P, P.ap, f, ttr, trot, evr, cl);
+  } else {
+    oma2 = P.ap.oma2;
+    sq = P.ap.sq;
+    ev = evib_fast(P.theta, f[5]);
+    relax_fast(P.ap, f, ev, ttr, trot, evr, cl);
   }
   auto relax_again = [&](bool& c2) {   // after the fix changed alpha
-    if constexpr (kFast) {
-      ap_ = alpha_parts(alpha, P.R);
-      relax_fast(P, ap_.ioR, f, ttr, trot, evr, c2);
+    if constexpr (kFast && sizeof(T) == 4) {
+      const AlphaParts<T> a = alpha_parts(P, alpha);
+      oma2 = a.oma2;
+      sq = a.sq;
+      relax_fast(P, a, f, ttr, trot, evr, c2);
+    } else if constexpr (kFast) {
+      const RelaxFixed<T> r =
+          relax_fixed<T>(alpha, P.gtr, P.gtv, P.grv, P.R, P.theta, f[3], f[4], f[5], ev);
+      oma2 = r.oma2;
+      sq = r.sq;
+      ttr = r.ttr;
+      trot = r.trot;
+      evr = r.evr;
+      c2 = r.cl;
     } else {
       relax_t(P, alpha, f, ttr, trot, evr, c2);
     }
@@ -360,11 +398,7 @@ __device__ __forceinline__ int collide_particle_t(const P_& P, const T* f, T& vx
   uint32_t j5, j6;
   particle_draws(id, step, rk, g0, g1, g2, g3, j5, j6);
   // Eq. update_ci about the interpolated bulk velocity
-  T oma2, sq;
-  if constexpr (kFast) {
-    oma2 = ap_.oma2;
-    sq = ap_.sq;
-  } else {
+  if constexpr (!kFast) {
     oma2 = T(1) - alpha * alpha;
     sq = sqrt(oma2);
   }
@@ -379,7 +413,8 @@ __device__ __forceinline__ int collide_particle_t(const P_& P, const T* f, T& vx
   // Eq. update_evib
   T eb, p_nb;
   if constexpr (kFast) {
-    eb = evr * P.iRth;
+    if constexpr (sizeof(T) == 4) eb = evr * P.iRth;
+    else eb = evr;               // in units of R theta
     p_nb = rcp_fast(T(1) + eb * oma2);
   } else {
     eb = evr / (P.R * P.theta);
@@ -737,8 +772,8 @@ moments_of_cells(long long first, long long stride, long long ny, int cpw,
       cs.Trot = se * inv / R;
       cs.Tvib = T_vib_of_level<double>(sp, cs.ebar);
     } else {
-      cs.Ttr = (P[0] + P[1] + P[2]) * (sp.iR * (1.0 / 3.0));
-      cs.Trot = se * (inv * sp.iR);
+      cs.Ttr = div_by(P[0] + P[1] + P[2], S(sp.R3), sp.iR3);
+      cs.Trot = div_by(se * inv, S(R), sp.iR);
       cs.Tvib = vib_state(sp, cs.ebar).Tvib;
     }
     if (fT) {   // the fields in the particle precision, for the stencils
@@ -896,9 +931,10 @@ __device__ void block_moments(int c, const long long* __restrict__ off, const T*
     const int k = t - 64;
     if (N >= 2)
       reinterpret_cast<double*>(&cs.Ttr)[k] =
-          (f6[k] + f6[K + k] + f6[2 * K + k]) * (inv * (sp.iR * (1.0 / 3.0)));
+          d_div_by(f6[k] * inv + f6[K + k] * inv + f6[2 * K + k] * inv, sp.R3, sp.iR3);
   } else if (t >= 96 && t < 96 + K) {
-    if (N >= 2) reinterpret_cast<double*>(&cs.Trot)[t - 96] = f4[3 * K + t - 96] * (inv * sp.iR);
+    if (N >= 2)
+      reinterpret_cast<double*>(&cs.Trot)[t - 96] = d_div_by(f4[3 * K + t - 96] * inv, sp.R, sp.iR);
   } else if (t == 31) {
     cs.off = b;
     cs.N = N;
@@ -929,7 +965,8 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
   using dual::put_part;
   __shared__ BlockTally tal;
   __shared__ CellCoeffsT<S> k;
-  __shared__ S xw, mu_ref, tauf, ip;   // (T / T_ref)^omega, mu(T_ref), tau_c p / mu, 1 / p
+  __shared__ S xw, mu_ref, tauf, p;    // (T / T_ref)^omega, mu(T_ref), tau_c p / mu, pressure
+  __shared__ double yp;                // 1 / the pressure's value
   __shared__ VibState vib;
   tally_init(tal);
   const int c = blockIdx.x, t = threadIdx.x;
@@ -963,9 +1000,9 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
     if (t < nl) {
       const Q T = lane_part(cs.Ttr, t);
       if constexpr (nl > 1)
-        put_part(xw, exp(lane_part(omega, t) * log(T * sp.iT_ref)), t);
+        put_part(xw, exp(lane_part(omega, t) * log(div_by(T, Q(sp.T_ref), sp.iT_ref))), t);
       else
-        xw = exp(sp.omega * log(T * sp.iT_ref));
+        xw = exp(sp.omega * d_log(div_by(T, sp.T_ref, sp.iT_ref)));
     } else if (t == 32) {
       vib = vib_state(sp, cs.ebar);
       k.Pr = S(cell_prandtl(vib));
@@ -976,20 +1013,20 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
     } else if (t >= 96 && t < 96 + nl) {
       const int i = t - 96;
       const double n = (double)cs.N * F_num / vol;
-      const Q p = n * kB * lane_part(cs.Ttr, i);
-      if constexpr (nl > 1) {
-        put_part(ip, rcp(p), i);
-        put_part(tauf, tau_c_factor_w<Q>(sp, lane_part(omega, i)), i);
-      } else {
-        ip = d_rcp(p);
-        tauf = sp.tauf0;
+      const Q pi = n * kB * lane_part(cs.Ttr, i);
+      put_part(p, pi, i);
+      if constexpr (nl > 1) put_part(tauf, tau_c_factor_w<Q>(sp, lane_part(omega, i)), i);
+      else tauf = sp.tauf0;
+      if (i == 0) {
+        yp = d_rcp(value(pi));
+        cs.n = n;
       }
-      if (i == 0) cs.n = n;
     }
     __syncthreads();
     CellCoeffsT<Q> q;
     const int i = t & 31;
-    if (t < 64 && i < nl) q.mu_p = lane_part(mu_ref, i) * lane_part(xw, i) * lane_part(ip, i);
+    if (t < 64 && i < nl) 
+      q.mu_p = div_by(lane_part(mu_ref, i) * lane_part(xw, i), lane_part(p, i), yp);
     if (t < nl) {
       put_part(k.mu_p, q.mu_p, t);
       q.Pr = lane_part(k.Pr, t);

@@ -4,8 +4,8 @@ collision meet, and the arguments that take CUDA's function (zeros, denormals,
 negative, very large and infinite values, NaN).
 
 Bounds, in units of the last place of the result.  Reciprocal, quotient and root end
-in one rounding of a value known to 2^-60 or better: 0.51.  The logarithm of 1 + 1/b
-rounds once at the end and has at most half a unit from its parts: 1."""
+in one rounding of a value known to 2^-60 or better: 0.51.  The logarithms round once
+at the end and have at most half a unit from their parts: 1."""
 import ctypes as C
 import subprocess
 
@@ -27,7 +27,8 @@ __global__ void run(int f, int n, const double* a, const double* b, double* own,
     case 0: own[i] = d_rcp(x); lib[i] = 1.0 / x; break;
     case 1: own[i] = d_div(x, y); lib[i] = x / y; break;
     case 2: own[i] = d_sqrt(x); lib[i] = sqrt(x); break;
-    default: own[i] = d_log1p_inv(x); lib[i] = log1p(1.0 / x);
+    case 3: own[i] = d_log1p_inv(x); lib[i] = log1p(1.0 / x); break;
+    default: own[i] = d_log(x); lib[i] = log(x);
   }
 }
 extern "C" int math_run(int f, int n, const double* a, const double* b, double* own, double* lib) {
@@ -44,11 +45,11 @@ extern "C" int math_run(int f, int n, const double* a, const double* b, double* 
   return (int)e;
 }
 """
-NAMES = ["rcp", "div", "sqrt", "log1p_inv"]
+NAMES = ["rcp", "div", "sqrt", "log1p_inv", "log"]
 W = np.longdouble
 WIDE = [lambda x, y: 1 / x, lambda x, y: x / y, lambda x, y: np.sqrt(x),
-        lambda x, y: np.log1p(1 / x)]
-BOUND = [0.51, 0.51, 0.51, 1.0]
+        lambda x, y: np.log1p(1 / x), lambda x, y: np.log(x)]
+BOUND = [0.51, 0.51, 0.51, 1.0, 1.0]
 
 
 @pytest.fixture(scope="module")
@@ -78,7 +79,7 @@ def _arguments(f, rng, n):
     return x, 2.0 ** rng.uniform(-300, 300, n) * rng.choice([-1.0, 1.0], n)
 
 
-@pytest.mark.parametrize("f", range(4), ids=NAMES)
+@pytest.mark.parametrize("f", range(5), ids=NAMES)
 def test_ordinary_arguments_within_their_bounds(math_lib, f):
     x, y = _arguments(f, np.random.default_rng(f), 200000)
     own, lib = _run(math_lib, f, x, y)
@@ -91,7 +92,7 @@ def test_ordinary_arguments_within_their_bounds(math_lib, f):
     assert rms[0] <= 1.01 * rms[1], (NAMES[f], rms)      # no less exact than CUDA's
 
 
-@pytest.mark.parametrize("f", range(4), ids=NAMES)
+@pytest.mark.parametrize("f", range(5), ids=NAMES)
 def test_other_arguments_take_the_library_value(math_lib, f):
     v = np.array([0.0, 5e-324, 1e-310, 2.2250738585072014e-308, 1e-300, 1e-200, 1.0, 3.0, 600.0,
                   700.0, 710.0, 1e200, 1e300, 8.9e307, 1.7976931348623157e308, np.inf])
