@@ -1653,8 +1653,11 @@ __global__ void pl_mom_out(int ncell, const long long* __restrict__ off,
 }
 
 // The cells' moments of a step in the FP64 form, in the same two parts: kCL
-// lanes per cell sum d = c - c_first, d d, eps and I into rec (kNAcc doubles per
-// cell), then one thread per cell forms the fields.  (A warp per cell spent
+// lanes per cell sum c, then d d about the mean, eps and I, into rec (kNAcc doubles
+// per cell: the mean, the central sums, eps, I), then one thread per cell forms the
+// fields.  The second walk reads the cell from L1; about one of its particles instead
+// of the mean, the sums are as many FP64 operations and lose a factor of up to the
+// particles' number where that one is far out.  (A warp per cell spent
 // 70 FP64 instructions on a cell of 20 particles, most of them in reductions
 // and in the mean that the whole warp divided out: 173 us for 0.77 million
 // particles in 38,400 cells.)
@@ -1667,30 +1670,40 @@ pl_cell_sums(int ncell, const long long* __restrict__ off, const double* __restr
   const int q = threadIdx.x & (CL - 1);
   const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / CL;
   const long long b = c < ncell ? off[c] : 0, e = c < ncell ? off[c + 1] : 0;
+  double m0 = 0.0, m1 = 0.0, m2 = 0.0;
+#pragma unroll 2
+  for (long long j = b + q; j < e; j += CL) {
+    m0 += cx[j]; m1 += cy[j]; m2 += cz[j];
+  }
+#pragma unroll
+  for (int o = 1; o < CL; o <<= 1) {
+    m0 += __shfl_xor_sync(0xffffffffu, m0, o);
+    m1 += __shfl_xor_sync(0xffffffffu, m1, o);
+    m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+  }
+  const double inv = e > b ? d_rcp((double)(e - b)) : 0.0;
+  m0 *= inv; m1 *= inv; m2 *= inv;
   double a[kNAcc];
 #pragma unroll
   for (int i = 0; i < kNAcc; ++i) a[i] = 0.0;
-  double r0 = 0.0, r1 = 0.0, r2 = 0.0;
-  if (b < e) { r0 = cx[b]; r1 = cy[b]; r2 = cz[b]; }
   long long sl = 0;
 #pragma unroll 2
   for (long long j = b + q; j < e; j += CL) {
-    const double d0 = cx[j] - r0, d1 = cy[j] - r1, d2 = cz[j] - r2;
-    a[0] += d0; a[1] += d1; a[2] += d2;
+    const double d0 = cx[j] - m0, d1 = cy[j] - m1, d2 = cz[j] - m2;
     a[3] = fma(d0, d0, a[3]); a[4] = fma(d1, d1, a[4]); a[5] = fma(d2, d2, a[5]);
     a[6] = fma(d0, d1, a[6]); a[7] = fma(d0, d2, a[7]); a[8] = fma(d1, d2, a[8]);
     a[9] += er[j];
     sl += lev[j];
   }
+  if (q == 0) { a[0] = m0; a[1] = m1; a[2] = m2; }
   if (sl != 0) a[10] = (double)sl;
   cl_store<CL, kNAcc>(a, c < ncell, rec + (size_t)c * kNAcc);
 }
 
 __global__ void __launch_bounds__(kBlk)
 pl_cell_fields(int ncell, const long long* __restrict__ off, const double* __restrict__ af,
-               const double* __restrict__ cx, const double* __restrict__ cy,
-               const double* __restrict__ cz, const double* __restrict__ rec,
-               ChCellT<double>* __restrict__ cells, Species sp, unsigned long long* counters,
+               const double* __restrict__ rec, ChCellT<double>* __restrict__ cells, Species sp,
+               unsigned long long* counters,
                double* __restrict__ fT, int* __restrict__ usable_c) {
   __shared__ BlockTally tal;
   tally_init(tal);
@@ -1707,11 +1720,8 @@ pl_cell_fields(int ncell, const long long* __restrict__ off, const double* __res
     usable_c[c] = cs.usable;
     const double* S = rec + (size_t)c * kNAcc;
     const double inv = N > 0 ? d_rcp((double)N) : 0.0;
-    const double m0 = S[0] * inv, m1 = S[1] * inv, m2 = S[2] * inv;
-    const double U[3] = {N > 0 ? cx[b] + m0 : 0.0, N > 0 ? cy[b] + m1 : 0.0,
-                         N > 0 ? cz[b] + m2 : 0.0};
     for (int i = 0; i < 3; ++i) {   // identity pending rescale until the cell is updated
-      cs.U[i] = U[i];
+      cs.U[i] = S[i];
       cs.Un[i] = 0.0;
       cs.Us[i] = 0.0;
     }
@@ -1720,15 +1730,14 @@ pl_cell_fields(int ncell, const long long* __restrict__ off, const double* __res
     if (!cs.active) {
       tally_add(tal, C_SKIPPED_CELLS, 1ull);
     } else {
-      const double P[6] = {fma(S[3], inv, -(m0 * m0)), fma(S[4], inv, -(m1 * m1)),
-                           fma(S[5], inv, -(m2 * m2)), fma(S[6], inv, -(m0 * m1)),
-                           fma(S[7], inv, -(m0 * m2)), fma(S[8], inv, -(m1 * m2))};
+      double P[6];
+      for (int i = 0; i < 6; ++i) P[i] = S[3 + i] * inv;
       cs.Ttr = d_div_by(P[0] + P[1] + P[2], sp.R3, sp.iR3);
       cs.Trot = d_div_by(S[9] * inv, sp.R, sp.iR);
       cs.ebar = S[10] * inv;
       cs.Tvib = vib_state(sp, cs.ebar).Tvib;
       double* o = fT + (size_t)c * kNF;
-      for (int i = 0; i < 3; ++i) o[i] = U[i];
+      for (int i = 0; i < 3; ++i) o[i] = S[i];
       o[3] = cs.Ttr; o[4] = cs.Trot; o[5] = cs.Tvib;
       for (int i = 0; i < 6; ++i) cs.Pi[i] = o[6 + i] = P[i];
     }
@@ -2085,8 +2094,7 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
     (cl == 32 ? pl_cell_sums<32> : pl_cell_sums<kCL>)<<<cell_grid(h, cl), kBlk, 0, s>>>(
         ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc);
     pl_cell_fields<<<(ncell + kBlk - 1) / kBlk, kBlk, 0, s>>>(
-        ncell, h->off, h->af, cx, cy, cz, h->macc, h->cells, env.sp, env.counters, (T*)h->fT,
-        h->usable_c);
+        ncell, h->off, h->af, h->macc, h->cells, env.sp, env.counters, (T*)h->fT, h->usable_c);
   } else {
     ch_moments<T, double><<<wb, kBlk, 0, s>>>(ncell, 32, h->off, h->af, cx, cy, cz, er, h->lv[b],
                                               h->cells, env.sp, env.counters, pend, (T*)h->fT,

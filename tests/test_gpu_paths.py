@@ -328,3 +328,39 @@ def test_host_step_reads_every_input_before_it_writes_an_overlapping_output(prec
     for a, b in zip(out[:4], ref[:4]):
         assert np.max(np.abs(a - b)) < 1e-4 * np.max(np.abs(b))
     ctx.destroy()
+
+
+@pytest.mark.parametrize("nx", [24, 184])           # a warp and four lanes per cell
+def test_plane_fields_of_cells_whose_first_particle_is_far_out(nx):
+    """The energy of an FP64 cell is kept to the rounding of its fields, which
+    central sums give whatever the particles' order: about the first particle, 20
+    thermal speeds out, they lose a factor of 200 (400 particles: variance 2, squares
+    400 in units of the thermal speed).  Central sums of 400 terms are good to some
+    3e-16 (random roundings), the others to some 3e-14; the bar lies between."""
+    w = I.cylinder_flow(nx=nx, ny=nx, ppc=1.0, cylinder=False)
+    pl = dict(w.plane, bc=(I.BC_SPECULAR,) * 4, inflow=(0,) * 4)
+    sp = w.species
+    R = 1.380649e-23 / sp["m"]
+    rng = np.random.default_rng(nx)
+    ci, cj = (a.ravel() for a in np.meshgrid(np.arange(1, 23, 3), np.arange(1, 23, 3)))
+    N, m = 400, len(ci)
+    h = ((pl["x1"] - pl["x0"]) / nx, (pl["y1"] - pl["y0"]) / nx)
+    x = np.repeat(pl["x0"] + (ci + 0.5) * h[0], N)
+    y = np.repeat(pl["y0"] + (cj + 0.5) * h[1], N)
+    s = np.sqrt(R * 200.0)
+    c = s * rng.standard_normal((3, m * N))
+    c[:, ::N] += 20.0 * s * rng.standard_normal((3, m)) / np.sqrt(3.0)
+    er, lev = rng.exponential(R * 200.0, m * N), np.zeros(m * N, dtype=np.int32)
+    ctx = usp.usp_init_plane(sp, pl, 1e-12, w.area_frac, x, y, *c, er, lev, 2 * m * N,
+                             precision=usp.USP_FP64, seed=2)
+    usp.usp_step(ctx, 1)
+    g = usp.usp_plane_get_particles(ctx)
+    W = np.longdouble
+    energy = lambda c, e, l: (0.5 * (W(c) ** 2).sum(axis=0) + W(e) +
+                              W(l) * W(R) * W(sp["theta_v"])).reshape(m, N).sum(axis=1)
+    before, after = energy(c, er, lev), energy(np.stack(g[2:5]), g[5], g[6])
+    assert np.array_equal(np.sort(g[7].reshape(m, N), axis=1),
+                          np.arange(m * N).reshape(m, N))        # every particle in its cell
+    err = np.abs(after / before - 1)
+    assert np.sqrt(np.mean(err.astype(float) ** 2)) < 3e-15, float(err.max())
+    ctx.destroy()
