@@ -1653,7 +1653,7 @@ __global__ void pl_mom_out(int ncell, const long long* __restrict__ off,
 }
 
 // The cells' moments of a step in the FP64 form, in the same two parts: kCL
-// lanes per cell sum c, then d d about the mean, eps and I, into rec (kNAcc doubles
+// lanes per cell sum c and eps, then d d about the mean and I, into rec (kNAcc doubles
 // per cell: the mean, the central sums, eps, I), then one thread per cell forms the
 // fields.  The second walk reads the cell from L1; about one of its particles instead
 // of the mean, the sums are as many FP64 operations and lose a factor of up to the
@@ -1670,19 +1670,21 @@ pl_cell_sums(int ncell, const long long* __restrict__ off, const double* __restr
   const int q = threadIdx.x & (CL - 1);
   const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / CL;
   const long long b = c < ncell ? off[c] : 0, e = c < ncell ? off[c + 1] : 0;
-  double m0 = 0.0, m1 = 0.0, m2 = 0.0;
+  double t[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 2
   for (long long j = b + q; j < e; j += CL) {
-    m0 += cx[j]; m1 += cy[j]; m2 += cz[j];
+    t[0] += cx[j]; t[1] += cy[j]; t[2] += cz[j]; t[3] += er[j];
   }
+  if constexpr (CL == kCL) {
+    cl_totals<4>(t);
+    const double mine = t[0];
 #pragma unroll
-  for (int o = 1; o < CL; o <<= 1) {
-    m0 += __shfl_xor_sync(0xffffffffu, m0, o);
-    m1 += __shfl_xor_sync(0xffffffffu, m1, o);
-    m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+    for (int i = 0; i < 4; ++i) t[i] = __shfl_sync(0xffffffffu, mine, i, kCL);
+  } else {
+    all_totals<4>(t);
   }
   const double inv = e > b ? d_rcp((double)(e - b)) : 0.0;
-  m0 *= inv; m1 *= inv; m2 *= inv;
+  const double m0 = t[0] * inv, m1 = t[1] * inv, m2 = t[2] * inv;
   double a[kNAcc];
 #pragma unroll
   for (int i = 0; i < kNAcc; ++i) a[i] = 0.0;
@@ -1692,10 +1694,9 @@ pl_cell_sums(int ncell, const long long* __restrict__ off, const double* __restr
     const double d0 = cx[j] - m0, d1 = cy[j] - m1, d2 = cz[j] - m2;
     a[3] = fma(d0, d0, a[3]); a[4] = fma(d1, d1, a[4]); a[5] = fma(d2, d2, a[5]);
     a[6] = fma(d0, d1, a[6]); a[7] = fma(d0, d2, a[7]); a[8] = fma(d1, d2, a[8]);
-    a[9] += er[j];
     sl += lev[j];
   }
-  if (q == 0) { a[0] = m0; a[1] = m1; a[2] = m2; }
+  if (q == 0) { a[0] = m0; a[1] = m1; a[2] = m2; a[9] = t[3]; }
   if (sl != 0) a[10] = (double)sl;
   cl_store<CL, kNAcc>(a, c < ncell, rec + (size_t)c * kNAcc);
 }
