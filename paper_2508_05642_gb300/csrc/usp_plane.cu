@@ -1281,12 +1281,14 @@ __global__ void __launch_bounds__(kBlk, 2) pl_collide(int ncell, const ChCellT<d
       // conversion per warp)
       const int at = halve_totals<10>(acc);
       const double sv = (double)acc[0];
-      const int sI = __reduce_add_sync(0xffffffffu, accI);
+      // the lanes' level sums by halves of their bits: 32 of them can exceed 31 bits
+      const long long sI = ((long long)__reduce_add_sync(0xffffffffu, accI >> 16) << 16) +
+                           __reduce_add_sync(0xffffffffu, accI & 0xffff);
       const int mI = __reduce_max_sync(0xffffffffu, maxI);
       ChSumsT<double>& sm = sums[c];
       if (at >= 0) sm.v[at] = sv;
       if (lane == 0) {
-        sm.I = (unsigned long long)(long long)sI;
+        sm.I = (unsigned long long)sI;
         sm.net = 0;
         sm.maxI = mI;
       }
@@ -1383,7 +1385,7 @@ pl_sample(int ncell, const long long* __restrict__ off, const double* __restrict
   double a[kNAcc];
 #pragma unroll
   for (int i = 0; i < kNAcc; ++i) a[i] = 0.0;
-  int sl = 0;   // a lane's share of a cell's levels stays far below 2^31
+  long long sl = 0;
 #pragma unroll 4
   for (long long j = b + q; j < e; j += CL) {
     const double v0 = cx[j], v1 = cy[j], v2 = cz[j];
@@ -1462,7 +1464,8 @@ pl_sample_f32(int ncell, const long long* __restrict__ off, const float* __restr
   const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kCL;
   const long long b = c < ncell ? off[c] : 0, e = c < ncell ? off[c + 1] : 0;
   // the largest |c| and |eps| of the cell by their bits (a NaN is above all)
-  int mx = 0, my = 0, mz = 0, me = 0, sl = 0;   // a lane's share of a cell's levels stays far below 2^31
+  int mx = 0, my = 0, mz = 0, me = 0;
+  long long sl = 0;
 #pragma unroll 4
   for (long long j = b + q; j < e; j += kCL) {
     mx = max(mx, __float_as_int(cx[j]) & 0x7fffffff);

@@ -364,3 +364,25 @@ def test_plane_fields_of_cells_whose_first_particle_is_far_out(nx):
     err = np.abs(after / before - 1)
     assert np.sqrt(np.mean(err.astype(float) ** 2)) < 3e-15, float(err.max())
     ctx.destroy()
+
+
+@pytest.mark.parametrize("precision,nx", [(usp.USP_FP64, 8), (usp.USP_FP64, 184), (usp.USP_FP32, 8)])
+def test_plane_averages_of_levels_beyond_31_bits(precision, nx):
+    """A cell of 64 particles at rest (no temperature, so no collision) whose levels add up
+    to 34 bits, and to more than 31 in every lane's share."""
+    w = I.cylinder_flow(nx=nx, ny=nx, ppc=1.0, cylinder=False)
+    pl = dict(w.plane, bc=(I.BC_SPECULAR,) * 4, inflow=(0,) * 4)
+    n = 64
+    at = lambda a, b: np.full(n, a + (b - a) * 2.5 / nx)      # cell (2, 2)
+    z = np.zeros(n)
+    lev = np.full(n, (1 << 30) + 12345, dtype=np.int32)
+    ctx = usp.usp_init_plane(w.species, pl, 1e-9, w.area_frac, at(pl["x0"], pl["x1"]),
+                             at(pl["y0"], pl["y1"]), z, z, z, np.full(n, 1e4), lev, 2 * n,
+                             precision=precision, seed=2)
+    usp.usp_sample(ctx, True)
+    usp.usp_step(ctx, 1)
+    acc = usp.usp_sample_read(ctx)[:nx * nx * 12].reshape(-1, 12)
+    assert np.array_equal(usp.usp_plane_get_particles(ctx)[6], lev)
+    assert acc[2 * nx + 2, 0] == n and acc[2 * nx + 2, 11] == lev.sum(dtype=np.int64)
+    assert acc[:, 11].sum() == lev.sum(dtype=np.int64)
+    ctx.destroy()
