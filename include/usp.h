@@ -24,6 +24,14 @@
  *  - Device memory is owned by the context: taken from the caller's
  *    allocator callback when one is given (released through its free
  *    callback), else from cudaMalloc.  usp_destroy releases all of it.
+ *    Beyond what a context needs, an FP64 one (also the FP64 derivative form)
+ *    of 65,536 particles or more takes 68 MB of tables at creation, and a
+ *    homogeneous FP64 one of the USP-FPM method with 512 particles per cell
+ *    or more another 28.7 kB per cell: only where the allocator grants them
+ *    beside as much memory as reading the state back takes, and never from
+ *    an allocator without a free callback.  Without them the results are the
+ *    same and a step is slower.  A context on cudaMalloc keeps a read-back
+ *    buffer of up to 64 MB from call to call.
  *  - Work is enqueued on the context's CUDA stream and returns without
  *    waiting, except where a function says it synchronises.
  *  - Every function returns USP_OK (0) or a negative usp_err.  A failing CUDA

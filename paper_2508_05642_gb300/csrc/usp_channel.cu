@@ -1216,11 +1216,11 @@ int ch_get_particles(ChannelCtx* h, const ChEnv& env, double* y, double* cx, dou
   const long long n = h->n;
   if (n == 0) return USP_OK;
   cudaStream_t s = env.stream;
-  // a small buffer is kept for the next call, a large one given back
+  // a small buffer is kept for the next call, a large one or a caller's given back
   double* tmp = h->hstage;
   if (!tmp) tmp = (double*)env.alloc(env.owner, 5 * n * sizeof(double));
   if (!tmp) return USP_ENOMEM;
-  if (n * 5 * (long long)sizeof(double) <= (64ll << 20)) h->hstage = tmp;
+  if (env.keep && n * 5 * (long long)sizeof(double) <= (64ll << 20)) h->hstage = tmp;
   const int b = h->cur;
   const int nb = (int)((n + 255) / 256);
   if (env.precision == USP_FP32)

@@ -20,6 +20,7 @@ struct ChEnv {
   int precision;              // USP_FP32 or USP_FP64
   void* (*alloc)(void* owner, size_t bytes);   // owner-tracked device allocation
   void (*release)(void* owner, void* p);       // give an allocation back early
+  bool keep;                  // small read-back buffers stay for the next call
   void* owner;
 };
 

@@ -1843,6 +1843,7 @@ void* dev_alloc(usp_ctx* c, size_t bytes) {
   if (c->cfg.alloc) {
     p = c->cfg.alloc(bytes, c->cfg.alloc_user);
   } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    (void)cudaGetLastError();   // reported by the caller, or done without
     p = nullptr;
   }
   if (p) {
@@ -1894,6 +1895,13 @@ void dev_release(usp_ctx* c, void* p) {
   else if (!c->cfg.alloc) cudaFree(p);
 }
 
+// the same for a block of `bytes` that is no longer counted
+void dev_give_back(usp_ctx* c, void* p, size_t bytes) {
+  if (!p) return;
+  dev_release(c, p);
+  c->device_bytes -= (long long)((bytes + 255) & ~(size_t)255);
+}
+
 void* env_alloc(void* owner, size_t bytes) { return dev_alloc((usp_ctx*)owner, bytes); }
 void env_release(void* owner, void* p) { dev_release((usp_ctx*)owner, p); }
 
@@ -1904,23 +1912,64 @@ PhiloxRoundKeys round_keys(const usp_ctx* c) {
   return rk;
 }
 
-// Memory for the tables of the FP64 collision draws of a context of n
-// particles, and their contents once the context has its stream.
-int alloc_draw_tables(usp_ctx* c, long long n) {
-  if ((c->precision != USP_FP64 && c->precision != USP_FP64_TANGENT) || n < kTabledParticles)
-    return USP_OK;
-  const size_t nr = (size_t)1 << kRadiusBits, na = (size_t)1 << kAngleBits;
-  c->radius = (double*)dev_alloc(c, nr * sizeof(double) + na * sizeof(double2));
-  if (!c->radius) return USP_ENOMEM;
-  c->direction = (double2*)(c->radius + nr);
-  return USP_OK;
+// The tables of an FP64 context, of the collision draws and (homogeneous, jump true) of
+// the jumps: a context has them only where its memory has them to spare, since
+// the paths without give the same numbers.  They come last, while the caller holds
+// as much as its largest later request (the read-back of the state), and they go
+// first.  An allocator without a free callback cannot give that back: no tables.
+constexpr size_t kDrawBytes = ((size_t)1 << kRadiusBits) * sizeof(double) +
+                              ((size_t)1 << kAngleBits) * sizeof(double2);
+size_t row_bytes(const usp_ctx* c) { return sizeof(float) * (size_t)c->ncell * kJR * kJK; }
+size_t guide_bytes(const usp_ctx* c) { return (size_t)c->ncell * kJR * kGB; }
+bool alloc_jump_tables(usp_ctx* c) {
+  c->tab_nb = (float*)dev_alloc(c, row_bytes(c));
+  if (c->tab_nb) c->tab_b = (float*)dev_alloc(c, row_bytes(c));
+  if (c->tab_b) c->gd_nb = (uint8_t*)dev_alloc(c, guide_bytes(c));
+  if (c->gd_nb) c->gd_b = (uint8_t*)dev_alloc(c, guide_bytes(c));
+  return c->gd_b != nullptr;
 }
-int fill_draw_tables(usp_ctx* c) {
+void drop_jump_tables(usp_ctx* c) {
+  dev_give_back(c, c->tab_nb, row_bytes(c));
+  dev_give_back(c, c->tab_b, row_bytes(c));
+  dev_give_back(c, c->gd_nb, guide_bytes(c));
+  dev_give_back(c, c->gd_b, guide_bytes(c));
+  c->tab_nb = c->tab_b = nullptr;
+  c->gd_nb = c->gd_b = nullptr;
+}
+int optional_tables(usp_ctx* c, long long n, bool jump) {
+  if ((c->precision != USP_FP64 && c->precision != USP_FP64_TANGENT) ||
+      (c->cfg.alloc && !c->cfg.free_))
+    return USP_OK;
+  if (jump && !alloc_jump_tables(c)) drop_jump_tables(c);
+  if (n < kTabledParticles) return USP_OK;
+  c->radius = (double*)dev_alloc(c, kDrawBytes);
   if (!c->radius) return USP_OK;
+  c->direction = (double2*)(c->radius + ((size_t)1 << kRadiusBits));
   draw_tables_kernel<<<1024, 256, 0, c->stream>>>(c->radius, c->direction);
   CK(cudaGetLastError());
   c->launches += 1;
   return USP_OK;
+}
+// gives them back; false: there are none
+bool drop_optional_tables(usp_ctx* c) {
+  if (c->precision == USP_FP32 || (!c->radius && !c->tab_nb)) return false;
+  cudaStreamSynchronize(c->stream);
+  drop_jump_tables(c);
+  dev_give_back(c, c->radius, kDrawBytes);
+  c->radius = nullptr;
+  c->direction = nullptr;
+  return true;
+}
+// the tables of a finished flow context, with `room` bytes held beside them
+int optional_tables_beside(usp_ctx* c, long long n, size_t room) {
+  if (n < kTabledParticles || c->precision == USP_FP32 || c->precision == USP_FP32_TANGENT ||
+      (c->cfg.alloc && !c->cfg.free_))
+    return USP_OK;
+  void* held = dev_alloc(c, room);
+  if (!held) return USP_OK;
+  const int rc = optional_tables(c, n, false);
+  dev_give_back(c, held, room);
+  return rc;
 }
 
 ChEnv make_env(usp_ctx* c) {
@@ -1935,6 +1984,7 @@ ChEnv make_env(usp_ctx* c) {
   e.precision = c->precision;
   e.alloc = env_alloc;
   e.release = env_release;
+  e.keep = !c->cfg.alloc;
   e.owner = c;
   return e;
 }
@@ -2665,14 +2715,7 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
   c->tab_b = nullptr;
   c->gd_nb = nullptr;
   c->gd_b = nullptr;
-  if (c->precision == USP_FP32 || (cfg->method == USP_METHOD_USP_FPM && n >= kTabledCell * n_cells)) {
-    c->tab_nb = (float*)dev_alloc(c, sizeof(float) * (size_t)n_cells * kJR * kJK);
-    c->tab_b = (float*)dev_alloc(c, sizeof(float) * (size_t)n_cells * kJR * kJK);
-    c->gd_nb = (uint8_t*)dev_alloc(c, (size_t)n_cells * kJR * kGB);
-    c->gd_b = (uint8_t*)dev_alloc(c, (size_t)n_cells * kJR * kGB);
-    if (!c->tab_nb || !c->tab_b || !c->gd_nb || !c->gd_b) return fail(USP_ENOMEM);
-  }
-  if (alloc_draw_tables(c, n) != USP_OK) return fail(USP_ENOMEM);
+  if (c->precision == USP_FP32 && !alloc_jump_tables(c)) return fail(USP_ENOMEM);
   c->flags = (uint32_t*)dev_alloc(c, 256);
   c->counters = (unsigned long long*)dev_alloc(c, 256);
   if (!c->cx || !c->cy || !c->cz || !c->er || !c->lev || !c->cells || !c->prm || !c->sums ||
@@ -2700,7 +2743,6 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
       cudaMemcpyAsync(c->uoff, c->h_uoff.data(), sizeof(long long) * (n_cells + 1),
                       cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
     return fail(USP_ECUDA);
-  if (fill_draw_tables(c) != USP_OK) return fail(USP_ECUDA);
   // the particle pass stages fixed tiles of kTileMax; smaller tiles (tests)
   // split cells more finely but use the same staging buffers
   const int tile = cfg->tile > 0 ? std::min(kTileMax, (cfg->tile + kAlign - 1) / kAlign * kAlign)
@@ -2733,6 +2775,8 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
   if (n > 0) {
     rc = upload_state(c, h_cx, h_cy, h_cz, h_erot, h_lev, false);
     if (rc) return fail(rc);
+    rc = optional_tables(c, n, cfg->method == USP_METHOD_USP_FPM && n >= kTabledCell * n_cells);
+    if (rc) return fail(rc);
     // the FP64 host layout of the initial upload is staged once only
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail(USP_ECUDA);
     dev_release(c, c->stage);
@@ -2742,7 +2786,9 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
   rc = c->precision == USP_FP32 ? init_params<float>(c) : init_params<double>(c);
   if (rc) return fail(rc);
   if (cfg->tile == 0 && n >= (1ll << 20)) {
-    rc = c->precision == USP_FP32 ? autotune<float>(c) : autotune<double>(c);
+    auto tune = [&] { return c->precision == USP_FP32 ? autotune<float>(c) : autotune<double>(c); };
+    rc = tune();
+    if (rc == USP_ENOMEM && drop_optional_tables(c)) rc = tune();
     if (rc) return fail(rc);
   }
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail(USP_ECUDA);
@@ -2805,16 +2851,18 @@ int usp_init_channel(usp_ctx** out, const usp_species* sp, const usp_config* cfg
   };
   c->flags = (uint32_t*)dev_alloc(c, 256);
   c->counters = (unsigned long long*)dev_alloc(c, 256);
-  if (!c->flags || !c->counters || alloc_draw_tables(c, n) != USP_OK) return fail(USP_ENOMEM);
+  if (!c->flags || !c->counters) return fail(USP_ENOMEM);
   if (cudaMemsetAsync(c->flags, 0, 256, c->stream) != cudaSuccess ||
       cudaMemsetAsync(c->counters, 0, 256, c->stream) != cudaSuccess)
     return fail(USP_ECUDA);
-  if (fill_draw_tables(c) != USP_OK) return fail(USP_ECUDA);
-  const int rc = ch_create(&c->ch, make_env(c), ch, dt, n, cfg->step0, h_y, h_cx, h_cy, h_cz,
+  int rc = ch_create(&c->ch, make_env(c), ch, dt, n, cfg->step0, h_y, h_cx, h_cy, h_cz,
                            h_erot, h_lev, h_pid);
   if (rc != USP_OK) return fail(rc);
   c->nparticles = ch_nparticles(c->ch);
   c->ncell = ch_ncell(c->ch);
+  rc = optional_tables_beside(c, n, 5 * sizeof(double) * (size_t)n);
+  if (rc == USP_OK && cudaStreamSynchronize(c->stream) != cudaSuccess) rc = USP_ECUDA;
+  if (rc != USP_OK) return fail(rc);
   *out = c;
   return USP_OK;
 }
@@ -2873,16 +2921,18 @@ int usp_init_plane(usp_ctx** out, const usp_species* sp, const usp_config* cfg,
   };
   c->flags = (uint32_t*)dev_alloc(c, 256);
   c->counters = (unsigned long long*)dev_alloc(c, 256);
-  if (!c->flags || !c->counters || alloc_draw_tables(c, n) != USP_OK) return fail(USP_ENOMEM);
+  if (!c->flags || !c->counters) return fail(USP_ENOMEM);
   if (cudaMemsetAsync(c->flags, 0, 256, c->stream) != cudaSuccess ||
       cudaMemsetAsync(c->counters, 0, 256, c->stream) != cudaSuccess)
     return fail(USP_ECUDA);
-  if (fill_draw_tables(c) != USP_OK) return fail(USP_ECUDA);
-  const int rc = pl_create(&c->pl, make_env(c), pl, dt, area_frac, n, capacity, cfg->step0, h_x,
+  int rc = pl_create(&c->pl, make_env(c), pl, dt, area_frac, n, capacity, cfg->step0, h_x,
                            h_y, h_cx, h_cy, h_cz, h_erot, h_lev, h_pid);
   if (rc != USP_OK) return fail(rc);
   c->nparticles = n;
   c->ncell = pl_ncell(c->pl);
+  rc = optional_tables_beside(c, n, 6 * sizeof(double) * (size_t)capacity);
+  if (rc == USP_OK && cudaStreamSynchronize(c->stream) != cudaSuccess) rc = USP_ECUDA;
+  if (rc != USP_OK) return fail(rc);
   *out = c;
   return USP_OK;
 }
@@ -2999,8 +3049,8 @@ int usp_get_particles(usp_ctx* c, double* hx, double* hy, double* hz, double* he
   if (c->kind != 0) return USP_ENOTSUP;
   const long long n = c->nparticles;
   if (n == 0) return USP_OK;
-  // a small buffer is kept for the next call, a large one given back
-  const bool keep = (size_t)n * 36 <= kKeptStage;
+  // a small buffer is kept for the next call, a large one or a caller's given back
+  const bool keep = !c->cfg.alloc && (size_t)n * 36 <= kKeptStage;
   double* st = (double*)(keep ? staging(c, (size_t)n * 36 + 64) : dev_alloc(c, (size_t)n * 36 + 64));
   if (!st) return USP_ENOMEM;
   double* ox = st; double* oy = st + n; double* oz = st + 2 * n; double* oe = st + 3 * n;
