@@ -84,7 +84,7 @@ struct CellSums {
   unsigned long long I;      // sum of levels after the collision
   long long net;             // net change of the level sum by the +-1 correction
   int maxI;                  // largest level after the collision
-  int top;                   // FP64 form: largest level after the correction
+  int top;                   // largest level after the correction
 };
 
 struct Tile {
@@ -997,7 +997,7 @@ __device__ __forceinline__ void build_tables(int c, F p_nb, F p_b, int maxI, Jum
 
 template <typename F>
 __global__ void __launch_bounds__(kJT)
-jumptable_kernel(int c0, int c1, const CollideParams<F>* __restrict__ prm,
+jumptable_kernel(int c0, int c1, int all, const CollideParams<F>* __restrict__ prm,
                  const CellState* __restrict__ cells, float* __restrict__ tab_nb,
                  float* __restrict__ tab_b, uint8_t* __restrict__ gd_nb,
                  uint8_t* __restrict__ gd_b) {
@@ -1006,7 +1006,7 @@ jumptable_kernel(int c0, int c1, const CollideParams<F>* __restrict__ prm,
   const CollideParams<F>& P = prm[c];
   if (!P.active) return;                     // uniform over the block
   __shared__ JumpRows rs;
-  build_tables<F>(c, P.p_nb, P.p_b, cells[c].maxI, rs, tab_nb, tab_b, gd_nb, gd_b);
+  build_tables<F>(c, P.p_nb, P.p_b, all ? kJR : cells[c].maxI, rs, tab_nb, tab_b, gd_nb, gd_b);
 }
 
 // ---------------------------------------------------------------------------
@@ -1149,9 +1149,8 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 // acceptance of draw j is decided exactly as in the one-at-a-time loop: a
 // decrement on particle k is accepted iff fewer than lev[k] earlier accepted
 // decrements in the round hit k.  The net level change goes to sums[c].net.
-// Returns the net change (every lane).  kTop: raises top to the largest level that
-// an increment reaches (a particle can be picked more than once).
-template <bool kTop>
+// Returns the net change (every lane) and raises top to the largest level that an
+// increment reaches (a particle can be picked more than once).
 __device__ __forceinline__ long long
 level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long sumI,
                int* __restrict__ lev, uint32_t* flags, unsigned long long* counters, uint32_t k0,
@@ -1221,10 +1220,9 @@ level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long
       const int order = __popc(am & lanemask_lt());
       const bool eff = accept && order < take;
       __syncwarp();
-      if (kTop && !down) {
-        if (eff) top = max(top, atomicAdd(&lv[k], 1) + 1);
-      } else if (eff) {
-        atomicAdd(&lv[k], down ? -1 : 1);
+      if (eff) {
+        if (down) atomicAdd(&lv[k], -1);
+        else top = max(top, atomicAdd(&lv[k], 1) + 1);
       }
       __syncwarp();
       long long used = 32;
@@ -1264,11 +1262,10 @@ level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long
     if (remaining != 0) atomicOr(flags, (uint32_t)F_VIB_LOOP_CAP);
     if (draws) atomicAdd(&counters[C_VIB_DRAWS], (unsigned long long)draws);
   }
-  if (kTop) top = __reduce_max_sync(0xffffffffu, top);
+  top = __reduce_max_sync(0xffffffffu, top);
   return net;
 }
 
-template <bool kTop>
 __global__ void __launch_bounds__(128, 8)
 levelfix_kernel(Species sp, int c0, int c1, const CellState* __restrict__ cells,
                 CellSums* __restrict__ sums, int* __restrict__ lev, uint32_t* flags,
@@ -1280,10 +1277,10 @@ levelfix_kernel(Species sp, int c0, int c1, const CellState* __restrict__ cells,
   if (!cs.active) return;
   int top = sums[c].maxI;
   const long long net =
-      level_fix_cell<kTop>(sp, c, cs, sums[c].I, lev, flags, counters, k0, k1, top);
+      level_fix_cell(sp, c, cs, sums[c].I, lev, flags, counters, k0, k1, top);
   if (lane == 0) {
     sums[c].net = net;
-    if (kTop) sums[c].top = top;
+    sums[c].top = top;
   }
 }
 
@@ -1343,7 +1340,7 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
   cs.s = s;
   cs.r = r;
   cs.step += 1;
-  cs.maxI = sizeof(T) == 8 ? S.top : S.maxI + 1;
+  cs.maxI = S.top;
   CollideParams<T> P;
   write_params<T>(sp, cs, P, flags, counters);
   cells[c] = cs;
@@ -1395,7 +1392,7 @@ few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
   if (w == 0) {
     int top = S.maxI;
     const long long net =
-        level_fix_cell<sizeof(T) == 8>(sp, c, cs, S.I, lev, flags, counters, k0, k1, top);
+        level_fix_cell(sp, c, cs, S.I, lev, flags, counters, k0, k1, top);
     if (lead) {
       S.net = net;
       S.top = top;
@@ -1440,7 +1437,7 @@ few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
     cs.Trot = d_div_by(e_rot_new, R, sp.iR);
     cs.s = sc;
     cs.step += 1;
-    cs.maxI = sizeof(T) == 8 ? S.top : S.maxI + 1;
+    cs.maxI = S.top;
     cell_mu_p(sp, cs.ndens, cs.Ttr, K.mu_p, xw);
   } else if (t == 32) {
     cs.ebar = sumI * invN;
@@ -2158,9 +2155,9 @@ int launch_collide(usp_ctx* c, int warp_tiles, int minb, int grid, void* cx, voi
 bool has_tables(const usp_ctx* c) { return c->tab_nb && c->sp.method == 0; }
 bool few_cells(const usp_ctx* c) { return c->ncell <= kFewCells && c->sp.method == 0; }
 
-// jump tables for the coming step
+// jump tables for the coming step (all: every row, whatever the cell's levels)
 template <typename T>
-int launch_tables_t(usp_ctx* c, const CellRange& r) {
+int launch_tables_t(usp_ctx* c, const CellRange& r, int all) {
   if (!has_tables(c) || r.c1 <= r.c0) return USP_OK;
   if (!c->jratio_ready) {
     jratio_kernel<T><<<1, 256, 0, c->stream>>>();
@@ -2168,13 +2165,14 @@ int launch_tables_t(usp_ctx* c, const CellRange& r) {
     c->jratio_ready = true;
   }
   jumptable_kernel<T><<<r.c1 - r.c0, kJT, 0, c->stream>>>(
-      r.c0, r.c1, (const CollideParams<T>*)c->prm, c->cells, c->tab_nb, c->tab_b, c->gd_nb,
+      r.c0, r.c1, all, (const CollideParams<T>*)c->prm, c->cells, c->tab_nb, c->tab_b, c->gd_nb,
       c->gd_b);
   CK(cudaGetLastError());
   return USP_OK;
 }
-int launch_tables(usp_ctx* c, const CellRange& r) {
-  return c->precision == USP_FP32 ? launch_tables_t<float>(c, r) : launch_tables_t<double>(c, r);
+int launch_tables(usp_ctx* c, const CellRange& r, int all = 0) {
+  return c->precision == USP_FP32 ? launch_tables_t<float>(c, r, all)
+                                  : launch_tables_t<double>(c, r, all);
 }
 
 // one step of the cells of r
@@ -2200,7 +2198,7 @@ int launch_step(usp_ctx* c, const CellRange& r) {
   }
   const int warps_per_block = 4;
   const int blocks = (n + warps_per_block - 1) / warps_per_block;
-  levelfix_kernel<sizeof(T) == 8><<<blocks, 32 * warps_per_block, 0, c->stream>>>(
+  levelfix_kernel<<<blocks, 32 * warps_per_block, 0, c->stream>>>(
       c->sp, r.c0, r.c1, c->cells, c->sums, c->lev, c->flags, c->counters, key0(c), key1(c));
   CK(cudaGetLastError());
   // one warp per block: the cells' FP64 work spreads over all SMs' FP64 pipes
@@ -3267,10 +3265,10 @@ int usp_load(usp_ctx* c, const void* buf, int buf_is_device) {
       CK(cudaMemcpyAsync(p[i], b, sz[i], b2d, c->stream));
       b += sz[i];
     }
-    if (c->precision != USP_FP32) {
-      const int rc = launch_tables(c, all_cells(c));
-      if (rc) return rc;
-    }
+    // the FP64 form's rows are in no file; those of a file whose writer ended them
+    // below the largest level are completed
+    const int rc = launch_tables(c, all_cells(c), 1);
+    if (rc) return rc;
   }
   c->step = h.step;
   CK(cudaStreamSynchronize(c->stream));
