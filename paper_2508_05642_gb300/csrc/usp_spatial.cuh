@@ -653,6 +653,7 @@ __global__ void ch_fix_update(int ncell, ChCellT<double>* __restrict__ cells,
 // cell are warp-wide FP32 (or working-precision) reductions, kept by lane k
 // for the k-th cell; the FP64 per-cell arithmetic then runs one cell per lane,
 // so each FP64 warp instruction serves up to 32 cells on the narrow FP64 pipe.
+// The arrays begin with particle `base`.
 template <typename T, typename S, bool kFpm = false>
 __device__ __forceinline__ void
 moments_of_cells(long long first, long long stride, long long ny, int cpw,
@@ -660,7 +661,7 @@ moments_of_cells(long long first, long long stride, long long ny, int cpw,
                  const T* __restrict__ cx, const T* __restrict__ cy, const T* __restrict__ cz,
                  const T* __restrict__ er, const int* __restrict__ lev,
                  ChCellT<S>* __restrict__ cells, const Species& sp, float* __restrict__ pend,
-                 T* __restrict__ fT, int* __restrict__ usable_c, BlockTally& tal) {
+                 T* __restrict__ fT, int* __restrict__ usable_c, BlockTally& tal, long long base = 0) {
   const int lane = threadIdx.x & 31;
   const double R = gasR(sp);
   constexpr bool f32 = sizeof(T) == 4;
@@ -682,7 +683,7 @@ moments_of_cells(long long first, long long stride, long long ny, int cpw,
     auto first = [&](int g) {
       const long long j = cell_b(g) + lane;
       if (j < cell_e(g)) {
-        nx0 = cx[j]; ny0 = cy[j]; nz0 = cz[j]; ne0 = er[j]; nl0 = lev[j];
+        nx0 = cx[j - base]; ny0 = cy[j - base]; nz0 = cz[j - base]; ne0 = er[j - base]; nl0 = lev[j - base];
       } else {
         nx0 = ny0 = nz0 = ne0 = T(0); nl0 = 0;
       }
@@ -698,7 +699,7 @@ moments_of_cells(long long first, long long stride, long long ny, int cpw,
       long long al = 0;
       if (has) { a0 += fx; a1 += fy; a2 += fz; ae += fe; al += fl; }
       for (long long j = b + 32 + lane; j < e; j += 32) {
-        a0 += cx[j]; a1 += cy[j]; a2 += cz[j]; ae += er[j]; al += lev[j];
+        a0 += cx[j - base]; a1 += cy[j - base]; a2 += cz[j - base]; ae += er[j - base]; al += lev[j - base];
       }
       T t0, t1, t2, te;
       {
@@ -723,7 +724,7 @@ moments_of_cells(long long first, long long stride, long long ny, int cpw,
         p[3] += C0 * C1; p[4] += C0 * C2; p[5] += C1 * C2;
       }
       for (long long j = b + 32 + lane; j < e; j += 32) {
-        const T C0 = cx[j] - m0, C1 = cy[j] - m1, C2 = cz[j] - m2;
+        const T C0 = cx[j - base] - m0, C1 = cy[j - base] - m1, C2 = cz[j - base] - m2;
         p[0] += C0 * C0; p[1] += C1 * C1; p[2] += C2 * C2;
         p[3] += C0 * C1; p[4] += C0 * C2; p[5] += C1 * C2;
       }
@@ -988,8 +989,8 @@ ch_prepare(const long long* __restrict__ off, const T* __restrict__ cx, const T*
       }
       __syncthreads();
       if (t < 32)
-        moments_of_cells<T, S>(c, 1, c + 1, 1, off, nullptr, st[0] - b, st[1] - b, st[2] - b,
-                               st[3] - b, sl - b, cells, sp, nullptr, (T*)nullptr, nullptr, tal);
+        moments_of_cells<T, S>(c, 1, c + 1, 1, off, nullptr, st[0], st[1], st[2], st[3], sl, cells,
+                               sp, nullptr, (T*)nullptr, nullptr, tal, b);
     } else if (t < 32) {
       moments_of_cells<T, S>(c, 1, c + 1, 1, off, nullptr, cx, cy, cz, er, lev, cells, sp, nullptr,
                              (T*)nullptr, nullptr, tal);
