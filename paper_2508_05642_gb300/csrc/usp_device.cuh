@@ -882,15 +882,15 @@ __device__ inline FpmCell fpm_cell(const Species& s, double n, double dt, const 
 // round-to-nearest one in the working precision, so the outcome is a fixed
 // function of (I, lam_up, lam_dn, the draws) up to the logarithm.
 constexpr int kGillespieCap = 4096;
-// the level, or its complement where the cap was met; k0, k1: the key
+// the level, or its complement where the cap was met
 template <typename T>
-__device__ __noinline__ int gillespie_exact(int I, T lu, T ld, uint32_t pid, uint32_t step,
-                                            uint32_t k0, uint32_t k1) {
+__device__ __forceinline__ int gillespie_exact(int I, T lu, T ld, uint32_t pid, uint32_t step,
+                                               const PhiloxRoundKeys& rk) {
   T t = T(0);
   U4 w = {0u, 0u, 0u, 0u};
 #pragma unroll 1
   for (int ev = 0; ev < kGillespieCap; ++ev) {
-    if ((ev & 1) == 0) w = philox4x32_10(pid, step, PTAG_GILLESPIE, (uint32_t)(ev >> 1), k0, k1);
+    if ((ev & 1) == 0) w = philox4x32_10(pid, step, PTAG_GILLESPIE, (uint32_t)(ev >> 1), rk);
     const T u1 = uniform_open<T>((ev & 1) ? w.z : w.x);
     const T u2 = uniform_open<T>((ev & 1) ? w.w : w.y);
     const T up = rn_mul(lu, rn_i2f(I + 1, T(0))), dn = rn_mul(ld, rn_i2f(I, T(0)));
@@ -906,14 +906,22 @@ __device__ __noinline__ int gillespie_exact(int I, T lu, T ld, uint32_t pid, uin
 // The same outcome from FP32 estimates.  What the method decides -- is the
 // step over, does the level rise -- is almost always clear of rounding: the
 // time is summed with the hardware's logarithm and reciprocal together with
-// a bound on its error (a relative 1e-6 of each waiting time, and an absolute
-// error of 1e-6 of each logarithm, over the rate), the branch is compared
-// without its division, and a particle for which either falls within its
-// bound (about one in 10^5), or whose rates are no ordinary numbers, or that makes 64
-// transitions, goes through gillespie_exact from the start.  A particle makes
+// a bound on its error (a relative 1e-6 of each waiting time, an absolute
+// error of 1e-6 of each logarithm, over the rate, and 6e-8 for each addition), the
+// branch is compared without its division, and a particle for which either falls
+// within its bound (about one in 10^5), or whose rates are no ordinary numbers, goes
+// through gillespie_exact from the start.  So do all of a cell whose rates
+// promise more transitions on average (2 lu ld / (ld - lu) at the level where they balance)
+// than kGillespieHot: the bound grows with their square, so that a warp of 32 would
+// run both loops (1.6 million particles, exact loop / estimates: FP32 540 / 430 us at 21
+// transitions a step, 1,076 / 1,690 us at 59; FP64 28.9 / 18.7 ms at 59, 61 / 73 ms
+// at 94).  A particle makes
 // a few transitions a step and a warp waits for its busiest one, so their
 // cost was the pass: a logarithm, two divisions and half a Philox block
 // each (FP64 form: some 60 FP64 operations, none now).
+template <typename T>
+constexpr float kGillespieHot = sizeof(T) == 4 ? 24.0f : 64.0f;
+constexpr int kGillespieMost = 256;
 __device__ __forceinline__ float uniform_estimate(uint32_t x, float) {
   return uniform_open<float>(x);
 }
@@ -927,8 +935,9 @@ __device__ __forceinline__ int gillespie(int I, T lu, T ld, uint32_t pid, uint32
   float t = 0.0f, err = 1e-6f;
   int J = I;
   U4 w = {0u, 0u, 0u, 0u};
+  const bool hot = !(2.0f * fu * fd <= kGillespieHot<T> * (fd - fu));
 #pragma unroll 1
-  for (int ev = 0; ev < 64; ++ev) {
+  for (int ev = hot ? kGillespieMost : 0; ev < kGillespieMost; ++ev) {
     if ((ev & 1) == 0) w = philox4x32_10(pid, step, PTAG_GILLESPIE, (uint32_t)(ev >> 1), rk);
     const float u1 = uniform_estimate((ev & 1) ? w.z : w.x, T(0));
     const float u2 = uniform_estimate((ev & 1) ? w.w : w.y, T(0));
@@ -939,14 +948,14 @@ __device__ __forceinline__ int gillespie(int I, T lu, T ld, uint32_t pid, uint32
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(rate));
     const float x = -0.693147180559945f * l2 * inv;
     t += x;
-    err = fmaf(1e-6f, x + inv, err);
+    err = fmaf(1e-6f, x + inv, err + 6e-8f);
     if (!(fabsf(t - 1.0f) > err)) break;
     if (t > 1.0f) return J;
     const float d = fmaf(u2, rate, -up);
     if (!(fabsf(d) > 2e-6f * rate)) break;
     J += d < 0.0f ? 1 : -1;
   }
-  J = gillespie_exact<T>(I, lu, ld, pid, step, rk.k0[0], rk.k1[0]);
+  J = gillespie_exact<T>(I, lu, ld, pid, step, rk);
   if (J < 0) {
     fl |= F_SAMPLER_CAP;
     J = ~J;

@@ -386,3 +386,28 @@ def test_plane_averages_of_levels_beyond_31_bits(precision, nx):
     assert acc[2 * nx + 2, 0] == n and acc[2 * nx + 2, 11] == lev.sum(dtype=np.int64)
     assert acc[:, 11].sum() == lev.sum(dtype=np.int64)
     ctx.destroy()
+
+
+@pytest.mark.parametrize("precision", [usp.USP_FP64, usp.USP_FP32])
+@pytest.mark.parametrize("steps_tau", [7.0, 9.0, 20.0, 25.0, 200.0])
+def test_gillespie_levels_of_hot_cells_match_oracle(precision, steps_tau):
+    """Cells on both sides of the mean transitions a step (21 and 27, 59 and 74) from
+    which the exact loop is run at once, and far above.  A rounding of a rate or a
+    logarithm moves a particle's time by 1e-7 of it, which turns a last transition
+    for some 1e-7 times their number of the particles: a few of 60,000."""
+    spd = I.n2_vhs_relaxation_species()
+    sp = O.species(**spd)
+    n, T = 60000, 8000.0
+    p = I.equilibrium_particles(np.random.default_rng(9), n, spd["m"], spd["theta_v"], T_tr=T,
+                                T_rot=T, T_vib=0.9 * T).astype_f32_exact()
+    form = 1 if precision == usp.USP_FP32 else 0
+    off, nd = np.array([0, n], dtype=np.int64), np.array([1e23])
+    dt = np.array([steps_tau * O.tau_c(sp, 1e23, T)])
+    st = O.State.from_arrays(p.cx, p.cy, p.cz, p.erot, p.lev)
+    O.homog_step_fpm(sp, form, 7, 0, 1, off, nd, dt, st)
+    ctx = usp.usp_init_homogeneous(spd, off, nd, dt, p.cx, p.cy, p.cz, p.erot, p.lev,
+                                   precision=precision, seed=7, method=usp.USP_METHOD_FPM)
+    usp.usp_step(ctx, 1)
+    lev = usp.usp_get_particles(ctx)[4]
+    assert np.sum(lev != st.lev) <= (0 if form == 0 else 20)
+    ctx.destroy()
