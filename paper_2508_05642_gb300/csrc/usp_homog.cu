@@ -3012,6 +3012,7 @@ int usp_step(usp_ctx* c, int nsteps) {
   int done = 0;
   while (nsteps - done >= c->graph_steps) {
     CK(cudaGraphLaunch(c->graph_exec, c->stream));
+    if (c->kind == 2) pl_stepped(c->pl);
     c->launches += kernels_per_step(c) * c->graph_steps;
     done += c->graph_steps;
   }

@@ -1861,7 +1861,7 @@ struct PlaneCtx {
   double* mout;
   long long* dstep;
   int sampling;
-  bool sorted;              // a step has left the particles in cell order
+  bool sorted;              // a step that ran has left the particles in cell order
 };
 
 namespace {
@@ -2077,7 +2077,11 @@ int pl_step_t(PlaneCtx* h, const ChEnv& env, ch_prof_fn prof) {
                                           (T*)h->st[b][4], (T*)h->st[b][5], h->lv[b], h->pd[b]);
   CHK(cudaGetLastError());
   h->cur = b;
-  h->sorted = true;
+  if (!h->sorted) {   // a captured step has not run yet
+    cudaStreamCaptureStatus cap;
+    CHK(cudaStreamIsCapturing(s, &cap));
+    h->sorted = cap == cudaStreamCaptureStatusNone;
+  }
   x = (T*)h->st[b][0]; y = (T*)h->st[b][1]; cx = (T*)h->st[b][2]; cy = (T*)h->st[b][3];
   cz = (T*)h->st[b][4]; er = (T*)h->st[b][5];
   if (prof) prof(env.owner, 0, 0);
@@ -2558,4 +2562,5 @@ int pl_leaves(const usp_plane* pp, int32_t* level, int32_t* ii, int32_t* jj) {
 
 int pl_ncell(const PlaneCtx* h) { return h->g.ncell; }
 int pl_parity(const PlaneCtx* h) { return h->cur; }
+void pl_stepped(PlaneCtx* h) { h->sorted = true; }
 void pl_destroy(PlaneCtx* h) { delete h; }

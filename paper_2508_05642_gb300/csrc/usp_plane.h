@@ -29,4 +29,5 @@ int pl_ncell(const PlaneCtx* pl);
 // cells of a plane's grid (count or USP_EINVAL; arrays may be NULL); host only
 int pl_leaves(const usp_plane* pp, int32_t* level, int32_t* ii, int32_t* jj);
 int pl_parity(const PlaneCtx* pl);
+void pl_stepped(PlaneCtx* pl);   // a graph of captured steps was launched
 void pl_destroy(PlaneCtx* pl);

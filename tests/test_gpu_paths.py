@@ -411,3 +411,33 @@ def test_gillespie_levels_of_hot_cells_match_oracle(precision, steps_tau):
     lev = usp.usp_get_particles(ctx)[4]
     assert np.sum(lev != st.lev) <= (0 if form == 0 else 20)
     ctx.destroy()
+
+
+def test_plane_moments_between_a_capture_and_its_first_replay():
+    """Steps captured into a caller's graph have not sorted the state yet: moments in
+    between are those of the state as it is, and after the replay those of the steps."""
+    torch = pytest.importorskip("torch")
+    w = I.cylinder_flow(nx=32, ny=24, ppc=5.0)
+    p = w.particles
+    dt = w.dt_over_tau_c * usp.usp_tau_c(w.species, w.plane["n_inf"], w.plane["T_inf"])
+    s = torch.cuda.Stream()
+    new = lambda **kw: usp.usp_init_plane(w.species, w.plane, dt, w.area_frac, w.x, w.y, p.cx,
+                                          p.cy, p.cz, p.erot, p.lev, w.capacity,
+                                          precision=usp.USP_FP64, seed=4, **kw)
+    ctx = new(stream=s.cuda_stream, use_graph=False)
+    before = usp.usp_moments(ctx)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        usp.usp_step(ctx, 2)            # an even number: the state's buffers alternate
+    close = lambda a, b: np.max(np.abs(a - b) / (np.max(np.abs(b), axis=1, keepdims=True) + 1e-300))
+    assert close(usp.usp_moments(ctx), before) < 1e-9      # sums by atomics
+    with torch.cuda.stream(s):
+        g.replay()
+    torch.cuda.synchronize()
+    after = usp.usp_moments(ctx)
+    ref = new()
+    usp.usp_step(ref, 2)
+    assert close(after, usp.usp_moments(ref)) < 1e-9 and close(after, before) > 1e-3
+    ctx.destroy()
+    ref.destroy()
