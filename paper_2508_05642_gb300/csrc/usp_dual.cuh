@@ -33,8 +33,6 @@ __device__ inline float vsqrt(float x) { return sqrtf(x); }
 __device__ inline double vsqrt(double x) { return sqrt_fast(x); }
 __device__ inline float vlog(float x) { return logf(x); }
 __device__ inline double vlog(double x) { return d_log(x); }
-__device__ inline float vlog1p(float x) { return log1pf(x); }
-__device__ inline double vlog1p(double x) { return ::log1p(x); }
 __device__ inline float vexp(float x) { return expf(x); }
 __device__ inline double vexp(double x) { return ::exp(x); }
 // exp(x) - 1 and its derivative
@@ -44,10 +42,6 @@ __device__ inline double vexpm1(double x, double& df) {
   df = e + 1.0;
   return e;
 }
-__device__ inline float vsinh(float x) { return sinhf(x); }
-__device__ inline double vsinh(double x) { return ::sinh(x); }
-__device__ inline float vcosh(float x) { return coshf(x); }
-__device__ inline double vcosh(double x) { return ::cosh(x); }
 __device__ inline float vcos(float x) { return cosf(x); }
 __device__ inline double vcos(double x) { return ::cos(x); }
 __device__ inline float vsin(float x) { return sinf(x); }
@@ -56,8 +50,6 @@ __device__ inline float vacos(float x) { return acosf(x); }
 __device__ inline double vacos(double x) { return ::acos(x); }
 __device__ inline float vcbrt(float x) { return cbrtf(x); }
 __device__ inline double vcbrt(double x) { return ::cbrt(x); }
-__device__ inline float vpow(float x, float y) { return powf(x, y); }
-__device__ inline double vpow(double x, double y) { return ::pow(x, y); }
 // a / b, and the same for y = 1 / b known (FP64: the value's and the derivatives'
 // quotients share it)
 __device__ inline float vdiv(float a, float b) { return a / b; }
@@ -189,13 +181,13 @@ __host__ __device__ inline Dual<V, N> operator-(const Dual<V, N>& a) {
 }
 
 #define USP_DUAL_CMP(op)                                                                       \
-  template <typename V, int N>                                                                        \
-  __host__ __device__ inline bool operator op(const Dual<V, N>& a, const Dual<V, N>& b) {            \
+  template <typename V, int N>                                                                 \
+  __host__ __device__ inline bool operator op(const Dual<V, N>& a, const Dual<V, N>& b) {      \
     return a.v op b.v;                                                                         \
   }                                                                                            \
-  template <typename V, int N>                                                                        \
+  template <typename V, int N>                                                                 \
   __host__ __device__ inline bool operator op(const Dual<V, N>& a, double b) { return a.v op b; } \
-  template <typename V, int N>                                                                        \
+  template <typename V, int N>                                                                 \
   __host__ __device__ inline bool operator op(double a, const Dual<V, N>& b) { return a op b.v; }
 USP_DUAL_CMP(<)
 USP_DUAL_CMP(>)
@@ -239,10 +231,6 @@ __device__ inline Dual<double, N> madd(const Dual<double, N>& f, const Dual<doub
 template <typename V, int N>
 __device__ inline Dual<V, N> log(const Dual<V, N>& a) { return chain(a, vlog(a.v), vdiv(V(1), a.v)); }
 template <typename V, int N>
-__device__ inline Dual<V, N> log1p(const Dual<V, N>& a) {
-  return chain(a, vlog1p(a.v), V(1) / (V(1) + a.v));
-}
-template <typename V, int N>
 __device__ inline Dual<V, N> exp(const Dual<V, N>& a) {
   const V e = vexp(a.v);
   return chain(a, e, e);
@@ -253,8 +241,6 @@ __device__ inline Dual<V, N> expm1(const Dual<V, N>& a) {
   const V e = vexpm1(a.v, df);
   return chain(a, e, df);
 }
-template <typename V, int N>
-__device__ inline Dual<V, N> sinh(const Dual<V, N>& a) { return chain(a, vsinh(a.v), vcosh(a.v)); }
 template <typename V, int N>
 __device__ inline Dual<V, N> cos(const Dual<V, N>& a) { return chain(a, vcos(a.v), -vsin(a.v)); }
 template <typename V, int N>
@@ -273,26 +259,6 @@ template <typename V, int N>
 __device__ inline Dual<V, N> fmin(const Dual<V, N>& a, const Dual<V, N>& b) { return b.v < a.v ? b : a; }
 template <typename V, int N>
 __device__ inline Dual<V, N> fmax(const Dual<V, N>& a, const Dual<V, N>& b) { return b.v > a.v ? b : a; }
-// a^b with a > 0 (both carrying derivatives)
-template <typename V, int N>
-__device__ inline Dual<V, N> pow(const Dual<V, N>& a, const Dual<V, N>& b) {
-  const V p = vpow(a.v, b.v);
-  Dual<V, N> r;
-  r.v = p;
-  const V la = vlog(a.v);
-  for (int i = 0; i < N; ++i) r.d[i] = p * (b.d[i] * la + b.v * a.d[i] / a.v);
-  return r;
-}
-template <typename V, int N>
-__device__ inline Dual<V, N> pow(const Dual<V, N>& a, double b) {
-  const V p = vpow(a.v, V(b));
-  return chain(a, p, V(b) * vpow(a.v, V(b - 1.0)));
-}
-template <typename V, int N>
-__device__ inline Dual<V, N> pow(double a, const Dual<V, N>& b) {
-  const V p = vpow(V(a), b.v);
-  return chain(b, p, p * vlog(V(a)));
-}
 template <typename V, int N>
 __device__ inline V value(const Dual<V, N>& a) { return a.v; }
 
