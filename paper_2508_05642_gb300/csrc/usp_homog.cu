@@ -1352,7 +1352,7 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
 
 // ---------------------------------------------------------------------------
 // The per-cell passes of a step in one kernel, for contexts of at most
-// kFewCells cells and the USP-FPM method: one block per cell.  A cell's update is some 400
+// one cell per SM and the USP-FPM method: one block per cell.  A cell's update is some 400
 // FP64 operations in a row, 64 cycles each (usp_math.cuh); here its
 // independent parts run on different warps, which sit on different quarters
 // of the SM, the level correction runs beside the sums' part, and the jump
@@ -1361,8 +1361,6 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
 // cells.  One cell of 20,000 particles, FP32: the three kernels took 54 us a
 // step at first (37 the update with the library's functions), 26 us so.
 // ---------------------------------------------------------------------------
-constexpr int kFewCells = 152;
-
 template <typename T>
 __global__ void __launch_bounds__(kJT)
 few_cells_kernel(Species sp, int c0, CellState* __restrict__ cells,
@@ -1785,6 +1783,7 @@ struct usp_ctx {
   float* tab_b;
   uint8_t* gd_nb;           // their guide tables
   uint8_t* gd_b;
+  int sms;                  // SMs of the device
   double* radius;           // tables of the FP64 collision draws (null: computed)
   double2* direction;
   uint32_t* flags;
@@ -2030,7 +2029,7 @@ int build_tiles(usp_ctx* c, int tile) {
   // An FP64 state of few particles is cut into tiles of one particle per lane,
   // so that its warps cover every quarter of every SM, each with half an FP64
   // lane per clock (an FP32 state keeps its tiles: its sums are FP32 per warp)
-  const bool fine = c->precision == USP_FP64 && c->nparticles <= 152ll * 4 * 32 * 4;
+  const bool fine = c->precision == USP_FP64 && c->nparticles <= 4ll * 32 * 4 * c->sms;
   rc = make_tiles(c, std::min(tile, fine ? 32 : kWT), &c->wtiles, &c->nwtiles, c->h_wfirst);
   if (rc) return rc;
   c->tile = tile;
@@ -2153,7 +2152,7 @@ int launch_collide(usp_ctx* c, int warp_tiles, int minb, int grid, void* cx, voi
 }
 
 bool has_tables(const usp_ctx* c) { return c->tab_nb && c->sp.method == 0; }
-bool few_cells(const usp_ctx* c) { return c->ncell <= kFewCells && c->sp.method == 0; }
+bool few_cells(const usp_ctx* c) { return c->ncell <= c->sms && c->sp.method == 0; }
 
 // jump tables for the coming step (all: every row, whatever the cell's levels)
 template <typename T>
@@ -2741,6 +2740,7 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
       cudaMemcpyAsync(c->uoff, c->h_uoff.data(), sizeof(long long) * (n_cells + 1),
                       cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
     return fail(USP_ECUDA);
+  c->sms = sm_count();
   // the particle pass stages fixed tiles of kTileMax; smaller tiles (tests)
   // split cells more finely but use the same staging buffers
   const int tile = cfg->tile > 0 ? std::min(kTileMax, (cfg->tile + kAlign - 1) / kAlign * kAlign)
@@ -2763,7 +2763,7 @@ int usp_init_homogeneous(usp_ctx** out, const usp_species* sp, const usp_config*
           return fail(USP_ECUDA);
         // (few tiles go one to a block, on all SMs, before a block gets a second)
         const int units = wt ? c->nwtiles : c->ntiles;
-        c->grid_by_minb[wt][mb] = std::max(1, std::min(units, sm_count() * std::max(1, per_sm)));
+        c->grid_by_minb[wt][mb] = std::max(1, std::min(units, c->sms * std::max(1, per_sm)));
       }
     }
     c->minb = 3;
