@@ -1183,6 +1183,9 @@ level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long
   // that sub-batch decremented its particle (every level of the later
   // sub-batches, after more than two decrements).
   constexpr int kSub = 4;
+  int was[kSub];   // levels before this lane's increments, looked at a round later
+#pragma unroll
+  for (int s = 0; s < kSub; ++s) was[s] = -1;
   while (remaining != 0 && draws < cap) {
     const U4 w = philox4x32_10((uint32_t)c, step, CTAG_PICK, (uint32_t)((draws >> 2) + lane),
                                k0, k1);
@@ -1199,6 +1202,8 @@ level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long
       kk[s] = (long long)(((unsigned long long)word * (unsigned long long)N) >> 32);
       vd[s] = draws + 32 * s + lane < cap;
       cur[s] = down && vd[s] ? __ldcg(&lv[kk[s]]) : 0;
+      top = max(top, was[s] + 1);
+      was[s] = -1;
     }
 #pragma unroll
     for (int s = 0; s < kSub; ++s) {
@@ -1222,7 +1227,7 @@ level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long
       __syncwarp();
       if (eff) {
         if (down) atomicAdd(&lv[k], -1);
-        else top = max(top, atomicAdd(&lv[k], 1) + 1);
+        else was[s] = atomicAdd(&lv[k], 1);
       }
       __syncwarp();
       long long used = 32;
@@ -1262,6 +1267,8 @@ level_fix_cell(const Species& sp, int c, const CellState& cs, unsigned long long
     if (remaining != 0) atomicOr(flags, (uint32_t)F_VIB_LOOP_CAP);
     if (draws) atomicAdd(&counters[C_VIB_DRAWS], (unsigned long long)draws);
   }
+#pragma unroll
+  for (int s = 0; s < kSub; ++s) top = max(top, was[s] + 1);
   top = __reduce_max_sync(0xffffffffu, top);
   return net;
 }
