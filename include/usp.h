@@ -315,8 +315,8 @@ int usp_backward(usp_ctx* ctx, const double* d_dL_dprof, double* grad3, int grad
 
 /* Checkpoints (channel and homogeneous contexts): everything a step carries
  * into the next one -- the particle state with its pending conservation
- * rescale, the per-cell records (and the jump tables of the FP32 form; those
- * of an FP64 context are built again on loading), the
+ * rescale, the per-cell records (and the jump tables of the FP32 form; a
+ * context with tables builds every row again on loading), the
  * time-average sums and sampling switch, the step counter, the status word
  * and counters -- as one opaque buffer of usp_checkpoint_bytes bytes.
  * usp_save writes it into buf; usp_load restores a context created with the
@@ -413,8 +413,8 @@ int usp_set_particles(usp_ctx* ctx, const double* h_cx, const double* h_cy, cons
  * with pinned host buffers the copies run at full link speed and hide most
  * of the arithmetic.  Where the output buffers are pinned and do not overlap
  * the inputs (or are the input buffers themselves), each run's state comes
- * down while later runs go up.  Homogeneous contexts only (USP_ENOTSUP
- * otherwise). */
+ * down while later runs go up; otherwise it comes down when all have been
+ * read.  Homogeneous contexts only (USP_ENOTSUP otherwise). */
 int usp_step_host(usp_ctx* ctx, const void* h_cx, const void* h_cy, const void* h_cz,
                   const void* h_erot, const int32_t* h_lev, int nsteps, double* h_moments,
                   void* h_cx_out, void* h_cy_out, void* h_cz_out, void* h_erot_out,

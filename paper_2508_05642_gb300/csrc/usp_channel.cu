@@ -15,7 +15,9 @@
 //   radix passes, ch_gather, ch_offsets  (otherwise) stable LSD radix sort of
 //                  (cell key, index), state permuted into cell order
 //   ch_prepare     per-cell moments (Sec. 2.A) and coefficients alpha, nu,
-//                  gamma, targets (Sec. 3.A), one warp per cell
+//                  gamma, targets (Sec. 3.A), one block of four warps per
+//                  cell (the first-order method: ch_moments and
+//                  ch_coeffs_fpm, one warp per cell)
 //   ch_collide     blocks of one cell: the first-order reconstruction of Sec.
 //                  3.B (field values and the slopes on each side of the
 //                  centroid, in shared memory), then per particle the
@@ -241,10 +243,10 @@ __global__ void ch_advect(long long n, int ny, double L, double dy, S Tw, double
 
 // ---------------------------------------------------------------------------
 // stable counting sort by cell in one pass (at most kPlaceCells cells and
-// kPlaceBlocks blocks of 256 particles): a particle's place is its cell's
-// start, plus the cell's particles in earlier blocks, plus those before it in
-// its block.  Each block sums the columns of the counts itself (at most
-// kPlaceBlocks values per cell, read coalesced from L2).
+// kPlaceBlocks blocks of 256 particles, counted by the move in blocks of kAB): a
+// particle's place is its cell's start, plus the cell's particles in earlier blocks,
+// plus those before it in its block.  Each block sums the columns of the counts
+// itself (at most 2 kPlaceBlocks values per cell, read coalesced from L2).
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256)
@@ -969,7 +971,7 @@ int ch_step_t(ChannelCtx* h, const ChEnv& env, ch_prof_fn prof) {
   h->cur = b;
   if (prof) prof(env.owner, 0, 0);
   if (prof) prof(env.owner, 1, 1);
-  // one warp per block: the cells' chains spread over all SMs
+  // a block per cell: the cells' chains spread over all SMs
   const double vol = h->area * h->dy;
   if (h->fpmrec) {
     if constexpr (std::is_same<S, double>::value) {

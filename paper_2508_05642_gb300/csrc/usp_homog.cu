@@ -344,7 +344,8 @@ __device__ __forceinline__ void collide_one(const CollideParams<T>& P, uint32_t 
 // 2 pi (2 a + 1) 2^-19, by the functions the direct path calls, so that a draw
 // is the same number either way.  The FP64 pipe of this chip has 2 lanes per SM
 // and clock; a logarithm takes 35 lane-operations, a sine-cosine pair 33, a
-// square root 10, so the two pairs of a particle were half of the FP64 collision
+// square root 10 (timed loops of the library's functions against one of
+// multiply-adds), so the two pairs of a particle were half of the FP64 collision
 // pass.  Gathers of 8 bytes from 64 MB run at 290 billion per second (one
 // 32-byte sector of L2 each), 1/8 of that time.  Filling takes 0.7 ms, the
 // work of 4 million particle-steps, hence the least count.
@@ -1366,7 +1367,7 @@ __global__ void cellupdate_kernel(Species sp, int c0, int c1, CellState* __restr
 // tables follow in the same block.  With more cells than SMs one thread per
 // cell (cellupdate_kernel) is the better split: its instructions serve 32
 // cells.  One cell of 20,000 particles, FP32: the three kernels took 54 us a
-// step at first (37 the update with the library's functions), 26 us so.
+// step at first (37 the update with the library's functions), 27 us so.
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(kJT)

@@ -142,10 +142,11 @@ __device__ __forceinline__ void relax_t(const P_& P, T alpha, const T* f, T& ttr
 
 
 // FP32 forms of relax_t / chol3_t / the jump parameters with one correctly
-// rounded reciprocal (or reciprocal square root) in place of each group of
-// divisions.  Used by the FP32 plane path, whose per-particle arithmetic is
-// compared with the oracle statistically; the other forms keep the IEEE
-// divisions operation for operation.
+// rounded reciprocal, or the hardware's reciprocal square root (rsqrtf), in place
+// of each group of divisions.  Used by the FP32 plane path, whose per-particle
+// arithmetic is compared with the oracle statistically.  The FP32 channel and its
+// derivative form keep the IEEE divisions of relax_t and chol3_t operation for
+// operation; the FP64 and FP64 derivative forms follow below.
 __device__ __forceinline__ bool chol3_fast(const float* M, float* L) {
   if (!(M[0] > 0.f)) return false;
   const float r0 = rsqrtf(M[0]);
@@ -203,7 +204,7 @@ __device__ __forceinline__ void relax_fast(const P_& P, const AlphaParts<float>&
 // relax_t and chol3_t have, but a product of a cell's factor where those divide, and
 // the vibrational energy in units of R theta.  The library's divisions, square roots and
 // expm1 were two thirds of the FP64 operations of a particle (0.77 million particles
-// on 240 x 160 cells: the plane's FP64 collision pass 1.47 ms).
+// on 240 x 160 cells: the plane's FP64 collision pass 1.47 ms, 0.74 ms so).
 __device__ __forceinline__ float rcp_fast(float x) { return __frcp_rn(x); }   // as the form always took them
 __device__ __forceinline__ double rcp_fast(double x) { return d_rcp(x); }
 template <typename T>
@@ -952,7 +953,7 @@ __device__ void block_moments(int c, const long long* __restrict__ off, const T*
 // moments and coefficients of the channel's cells, one block per cell: the
 // sums, then the parts of the coefficients that do not need one another on
 // different warps, that is on different quarters of the SM (64 cells of 200
-// particles in the derivative form: 27 us; one warp's sums and whole
+// particles in the derivative form: 25 us; one warp's sums and whole
 // derivative numbers on one thread 52 us)
 template <typename T, typename S>
 __global__ void __launch_bounds__(kPB)
