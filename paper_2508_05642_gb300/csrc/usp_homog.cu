@@ -1641,30 +1641,37 @@ __global__ void assemble_moments(Species sp, int ncell, int c0, int c1,
 // Moments of an FP64 state in one pass: raw sums of the stored particles about
 // a reference velocity (usp_sums.cuh); the pending rescale c = U + s (c* - U*),
 // eps = r eps* is applied to the finished sums.  A context's stored particles
-// have the mean U*, which is the reference; a state just uploaded (fresh)
-// takes the sampled one.  Bound by the FP64 pipe.  15.5 million particles: 1.51
-// ms for the two passes before, 0.9 ms now.
+// have the mean U*, which in FP32 is the reference; a state just uploaded (fresh)
+// takes that of usp_sums.cuh.  Bound by the FP64 pipe.  15.5 million particles: 1.51
+// ms for the two passes before, 0.93 ms now (0.90 without the references).
+template <int G>
+__global__ void __launch_bounds__(kRawBlock)
+moments_references(int c0, int c1, const CellState* __restrict__ cells,
+                   const double* __restrict__ cx, const double* __restrict__ cy,
+                   const double* __restrict__ cz, int ncell, double* __restrict__ out) {
+  const int c = c0 + blockIdx.x * (kRawBlock / G) + threadIdx.x / G;
+  if (c >= c1) return;   // uniform over the G threads
+  raw_reference<G>(cells[c].off, cells[c].N, cx, cy, cz, out + ncell + c, ncell);
+}
 __device__ __forceinline__ RawRef moments_reference(const CellState& cs, int fresh,
-                                                    const double* __restrict__ cx,
-                                                    const double* __restrict__ cy,
-                                                    const double* __restrict__ cz) {
-  if (fresh) return raw_reference(cs.off, cs.N, cx, cy, cz);
-  return RawRef{{cs.Us[0], cs.Us[1], cs.Us[2]}};
+                                                    const double* __restrict__ w, int ncell) {
+  return fresh ? RawRef{{w[0], w[ncell], w[2 * (size_t)ncell]}}
+               : RawRef{{narrow(cs.Us[0]), narrow(cs.Us[1]), narrow(cs.Us[2])}};
 }
 __global__ void __launch_bounds__(kRawBlock)
 moments_raw_kernel(int c0, int c1, int chunk_min, int fresh, const CellState* __restrict__ cells,
                    const double* __restrict__ cx, const double* __restrict__ cy,
                    const double* __restrict__ cz, const double* __restrict__ er,
                    const int* __restrict__ lev, double* __restrict__ acc, int ncell,
-                   double* __restrict__ out) {
+                   const double* __restrict__ out) {
   for (int c = c0 + blockIdx.y; c < c1; c += gridDim.y)
     raw_cell(cells[c].off, cells[c].N, chunk_min,
-             [&] { return moments_reference(cells[c], fresh, cx, cy, cz); }, cx, cy, cz, er, lev,
-             acc + (size_t)c * kMomAcc, out + ncell + c, ncell);
+             [&] { return moments_reference(cells[c], fresh, out + ncell + c, ncell); }, cx, cy, cz,
+             er, lev, acc + (size_t)c * kMomAcc);
 }
 
-// one thread per cell; the sums' kernel left the reference in the rows of U
-__global__ void assemble_raw(Species sp, int ncell, int c0, int c1,
+// one thread per cell; a fresh state's references are in the rows of U
+__global__ void assemble_raw(Species sp, int ncell, int c0, int c1, int fresh,
                              const CellState* __restrict__ cells, const double* __restrict__ acc,
                              double* __restrict__ out, double* __restrict__ levsum) {
   const int c = c0 + blockIdx.x * blockDim.x + threadIdx.x;
@@ -1676,10 +1683,10 @@ __global__ void assemble_raw(Species sp, int ncell, int c0, int c1,
     for (int f = 0; f < USP_NMOM; ++f) out[(size_t)f * ncell + c] = 0.0;
     return;
   }
-  const double w[3] = {out[ncell + c], out[2 * (size_t)ncell + c], out[3 * (size_t)ncell + c]};
+  const RawRef w = moments_reference(cs, fresh, out + ncell + c, ncell);
   const double* a = acc + (size_t)c * kMomAcc;
   if (levsum) levsum[c] = a[kRI];
-  const RawMoments m = raw_moments(a, (double)n, w);
+  const RawMoments m = raw_moments(a, (double)n, w.w);
   const double R = gasR(sp), s = cs.s, r = cs.r;
   out[c] = (double)n;
   for (int i = 0; i < 3; ++i) out[(size_t)(1 + i) * ncell + c] = cs.U[i] + s * (m.U[i] - cs.Us[i]);
@@ -2245,12 +2252,24 @@ int compute_moments(usp_ctx* c, double* levsum, const CellRange& r) {
                      sizeof(double) * kMomAcc * (r.c1 - r.c0), c->stream));
   if constexpr (sizeof(T) == 8) {
     const int n = r.c1 - r.c0;
+    const T* x = (const T*)c->cx; const T* y = (const T*)c->cy; const T* z = (const T*)c->cz;
+    const int fresh = levsum != nullptr;
+    if (fresh) {
+      if (ref_by_warp(n))
+        moments_references<32><<<(n + 7) / 8, kRawBlock, 0, c->stream>>>(r.c0, r.c1, c->cells, x, y, z,
+                                                                         c->ncell, c->mout);
+      else
+        moments_references<kRawBlock><<<n, kRawBlock, 0, c->stream>>>(r.c0, r.c1, c->cells, x, y, z,
+                                                                      c->ncell, c->mout);
+      CK(cudaGetLastError());
+      c->launches += 1;
+    }
     moments_raw_kernel<<<dim3(raw_blocks(n), std::min(n, 65535)), kRawBlock, 0, c->stream>>>(
-        r.c0, r.c1, raw_chunk(n), levsum != nullptr, c->cells, (const T*)c->cx, (const T*)c->cy, (const T*)c->cz,
-        (const T*)c->er, c->lev, c->macc, c->ncell, c->mout);
+        r.c0, r.c1, raw_chunk(n), fresh, c->cells, x, y, z, (const T*)c->er, c->lev, c->macc, c->ncell,
+        c->mout);
     CK(cudaGetLastError());
-    assemble_raw<<<(n + 63) / 64, 64, 0, c->stream>>>(c->sp, c->ncell, r.c0, r.c1, c->cells, c->macc,
-                                                      c->mout, levsum);
+    assemble_raw<<<(n + 63) / 64, 64, 0, c->stream>>>(c->sp, c->ncell, r.c0, r.c1, fresh, c->cells,
+                                                      c->macc, c->mout, levsum);
     CK(cudaGetLastError());
     c->launches += 2;
     return USP_OK;

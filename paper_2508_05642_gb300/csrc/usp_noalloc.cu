@@ -54,27 +54,36 @@ constexpr int kMaxDevices = 64;
 double* g_na_ptr[kMaxDevices] = {nullptr};
 std::mutex g_na_mutex;
 
-__global__ void na_clear(double* acc, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    acc[i] = 0.0;
+// Per cell (G threads each) its sums cleared and its reference velocity (usp_sums.cuh)
+// into the rows of U.
+template <int G>
+__global__ void __launch_bounds__(usp::kRawBlock)
+na_references(int ncell, const int64_t* __restrict__ off, const double* __restrict__ cx,
+              const double* __restrict__ cy, const double* __restrict__ cz,
+              double* __restrict__ acc, double* __restrict__ out) {
+  const int c = blockIdx.x * (usp::kRawBlock / G) + threadIdx.x / G;
+  if (c >= ncell) return;   // uniform over the G threads
+  if (threadIdx.x % G < kNaAcc) acc[(size_t)c * kNaAcc + threadIdx.x % G] = 0.0;
+  usp::raw_reference<G>(off[c], off[c + 1] - off[c], cx, cy, cz, out + ncell + c, ncell);
 }
 
-// Raw sums of every cell about its reference velocity (usp_sums.cuh), one
+// Raw sums of every cell about its reference velocity, one
 // pass; blockIdx.y walks the cells.  Bound by the FP64 pipe (22 to 26
 // operations per particle, 2 lanes per clock and SM).
 __global__ void __launch_bounds__(usp::kRawBlock)
 na_sums(int ncell, int chunk_min, const int64_t* __restrict__ off, const double* __restrict__ cx,
         const double* __restrict__ cy, const double* __restrict__ cz,
         const double* __restrict__ er, const int32_t* __restrict__ lev, double* __restrict__ acc,
-        double* __restrict__ out) {
+        const double* __restrict__ out) {
   for (int c = blockIdx.y; c < ncell; c += gridDim.y) {
-    const long long b = off[c], n = off[c + 1] - b;
-    usp::raw_cell(b, n, chunk_min, [&] { return usp::raw_reference(b, n, cx, cy, cz); }, cx, cy,
-                  cz, er, lev, acc + (size_t)c * kNaAcc, out + ncell + c, ncell);
+    const double* w = out + ncell + c;
+    usp::raw_cell(off[c], off[c + 1] - off[c], chunk_min,
+                  [&] { return usp::RawRef{{w[0], w[ncell], w[2 * (size_t)ncell]}}; }, cx, cy, cz,
+                  er, lev, acc + (size_t)c * kNaAcc);
   }
 }
 
-// one thread per cell; na_sums left the reference velocities in the rows of U
+// one thread per cell; the reference velocities are in the rows of U
 __global__ void na_assemble(NaGas gas, int ncell, const int64_t* __restrict__ off,
                             const double* __restrict__ acc, double* __restrict__ out) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -136,8 +145,12 @@ extern "C" int usp_moments_noalloc(const usp_species* sp, int n_cells, const int
   // an error left by the caller's earlier work is not this call's: report it
   // without launching (and without clearing it)
   if (cudaPeekAtLastError() != cudaSuccess) return USP_ECUDA;
-  const int nacc = kNaAcc * n_cells;
-  na_clear<<<(nacc + 255) / 256, 256, 0, st>>>(acc, nacc);
+  if (usp::ref_by_warp(n_cells))
+    na_references<32><<<(n_cells + 7) / 8, usp::kRawBlock, 0, st>>>(n_cells, d_offsets, d_cx, d_cy,
+                                                                    d_cz, acc, d_out);
+  else
+    na_references<usp::kRawBlock><<<n_cells, usp::kRawBlock, 0, st>>>(n_cells, d_offsets, d_cx, d_cy,
+                                                                      d_cz, acc, d_out);
   if (cudaGetLastError() != cudaSuccess) return USP_ECUDA;
   na_sums<<<dim3(usp::raw_blocks(n_cells), n_cells), usp::kRawBlock, 0, st>>>(
       n_cells, usp::raw_chunk(n_cells), d_offsets, d_cx, d_cy, d_cz, d_erot, d_lev, acc, d_out);

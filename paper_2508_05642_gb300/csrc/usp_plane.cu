@@ -1580,39 +1580,37 @@ pl_sample_add(int ncell, const long long* __restrict__ off,
 
 // On-demand moments of a state in cell order (every state a step has left):
 // kCL lanes per cell form the raw sums (usp_sums.cuh) about the FP32 mean of
-// kCL of its particles, then one thread per cell the moments, with the
+// its particles (left in the rows of U), then one thread per cell the moments, with the
 // pending rescale applied to the finished sums (in the first kernel that part
 // would run for 8 cells per warp: 20 FP64 instructions per cell, not 5).  6.9
 // million particles in 240,000 cells: 0.6 ms, 1.19 ms for the two passes with
 // six and fifteen FP64 atomics per particle that an unsorted state still takes.
-template <typename T>
-__device__ __forceinline__ void cl_reference(long long b, long long n, const T* __restrict__ cx,
-                                             const T* __restrict__ cy, const T* __restrict__ cz,
-                                             float* w) {
-  w[0] = w[1] = w[2] = 0.0f;
-  const int m = n < kCL ? (int)n : kCL;
-  for (int q = 0; q < m; ++q) {
-    const long long j = b + (long long)q * n / m;
-    w[0] += (float)cx[j]; w[1] += (float)cy[j]; w[2] += (float)cz[j];
-  }
-  const float im = m > 0 ? 1.0f / (float)m : 0.0f;
-  for (int i = 0; i < 3; ++i) {
-    w[i] *= im;
-    if (!(fabsf(w[i]) < 3.0e38f)) w[i] = 0.0f;
-  }
-}
-
 template <typename T, int CL>
 __global__ void __launch_bounds__(kBlk)
 pl_mom_sums(int ncell, const long long* __restrict__ off, const T* __restrict__ cx,
             const T* __restrict__ cy, const T* __restrict__ cz, const T* __restrict__ er,
-            const int* __restrict__ lev, double* __restrict__ rec) {
+            const int* __restrict__ lev, double* __restrict__ rec, double* __restrict__ out) {
   const int q = threadIdx.x & (CL - 1);
   const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / CL;
   const long long b = c < ncell ? off[c] : 0, e = c < ncell ? off[c + 1] : 0;
-  float wf[3];
-  cl_reference<T>(b, e - b, cx, cy, cz, wf);
-  const double w0 = wide(wf[0]), w1 = wide(wf[1]), w2 = wide(wf[2]);
+  float v0 = 0.0f, v1 = 0.0f, v2 = 0.0f;
+#pragma unroll 4
+  for (long long j = b + q; j < e; j += CL) {
+    v0 += narrow(cx[j]); v1 += narrow(cy[j]); v2 += narrow(cz[j]);
+  }
+#pragma unroll
+  for (int o = 1; o < CL; o <<= 1) {
+    v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+    v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+    v2 += __shfl_xor_sync(0xffffffffu, v2, o);
+  }
+  const float n = (float)max(1ll, e - b);
+  const double w0 = ref_mean(v0, n), w1 = ref_mean(v1, n), w2 = ref_mean(v2, n);
+  if (q == 0 && c < ncell) {
+    out[ncell + c] = w0;
+    out[2 * (size_t)ncell + c] = w1;
+    out[3 * (size_t)ncell + c] = w2;
+  }
   double a[kRawN];
   long long aI = 0;
 #pragma unroll
@@ -1624,21 +1622,17 @@ pl_mom_sums(int ncell, const long long* __restrict__ off, const T* __restrict__ 
   cl_store<CL, kRawN>(a, c < ncell, rec + (size_t)c * kRawN);
 }
 
-template <typename T>
 __global__ void pl_mom_out(int ncell, const long long* __restrict__ off,
-                           const ChCellT<double>* __restrict__ cells, const T* __restrict__ cx,
-                           const T* __restrict__ cy, const T* __restrict__ cz,
+                           const ChCellT<double>* __restrict__ cells,
                            const double* __restrict__ rec, double* __restrict__ out, Species sp) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
-  const long long b = off[c], n = off[c + 1] - b;
+  const long long n = off[c + 1] - off[c];
   if (n <= 0) {
     for (int f = 0; f < USP_NMOM; ++f) out[(size_t)f * ncell + c] = 0.0;
     return;
   }
-  float wf[3];
-  cl_reference<T>(b, n, cx, cy, cz, wf);
-  const double w[3] = {wide(wf[0]), wide(wf[1]), wide(wf[2])};
+  const double w[3] = {out[ncell + c], out[2 * (size_t)ncell + c], out[3 * (size_t)ncell + c]};
   const RawMoments m = raw_moments(rec + (size_t)c * kRawN, (double)n, w);
   const ChCellT<double>& cc = cells[c];
   const double R = gasR(sp), s = cc.s, r = cc.r, s2 = s * s;
@@ -2477,9 +2471,9 @@ int pl_moments(PlaneCtx* h, const ChEnv& env, double* out, int out_is_device) {
       const T* cz = (const T*)h->st[b][4]; const T* er = (const T*)h->st[b][5];
       const int cl = wide_cells(h) ? 32 : kCL;
       (cl == 32 ? pl_mom_sums<T, 32> : pl_mom_sums<T, kCL>)<<<cell_grid(h, cl), kBlk, 0, s>>>(
-          ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc);
-      pl_mom_out<T><<<(ncell + kBlk - 1) / kBlk, kBlk, 0, s>>>(ncell, h->off, h->cells, cx, cy, cz,
-                                                               h->macc, h->mout, env.sp);
+          ncell, h->off, cx, cy, cz, er, h->lv[b], h->macc, h->mout);
+      pl_mom_out<<<(ncell + kBlk - 1) / kBlk, kBlk, 0, s>>>(ncell, h->off, h->cells, h->macc, h->mout,
+                                                            env.sp);
     };
     if (env.precision == USP_FP32) sorted_moments(float());
     else sorted_moments(double());

@@ -36,32 +36,68 @@ __device__ __forceinline__ void raw_add(double* a, long long& aI, double d0, dou
   }
 }
 
-// The reference velocity of a cell of n particles: the FP32 mean of 32 of them
-// taken at equal distances (every caller of a cell gets the same one), 0 where
-// that is not finite.  It is within about 0.2 thermal speeds of the mean, so
-// the shifted sums lose no digit, and exact in FP64 whatever its value.
+// The reference velocity of a cell of n particles: the FP32 mean of all of them, or of
+// 2,048 (4,096 by a block) in runs of 8 (two sectors) at equal distances, 0 where that
+// is not finite.  It is within 1 / 45 (1 / 64) of a thermal speed of the mean, so that a
+// sum's size, and with it its rounding, stays near that of n random numbers: about the
+// mean of 32, a fifth of a thermal speed, the mean velocities of cells of 10,000 to
+// 40,000 at rest were off by 5.1e-15 of themselves, now by less than 1.5e-15.  Its
+// 24 bits leave c - w exact: about the FP64 mean all c of a binade are rounded to the
+// same side, which moves the mean of n of them by up to sqrt(n) 6e-17 of itself.
 struct RawRef {
   double w[3];
 };
-template <typename Load>
-__device__ __forceinline__ double raw_mean32(long long n, Load load) {
-  const int lane = threadIdx.x & 31;
-  const int m = n < 32 ? (int)n : 32;
-  float v = lane < m ? (float)load((long long)lane * n / m) : 0.0f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  v = __fdiv_rn(v, (float)m);
+// x rounded towards zero, by its bits: a conversion takes the FP64 pipe as long as a
+// multiply-add (0 for what FP32 has no normal number for)
+__device__ __forceinline__ float narrow(float x) { return x; }
+__device__ __forceinline__ float narrow(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t a = hi & 0x7fffffffu;
+  if (a - 0x38100000u >= 0x0fe00000u) return 0.0f;
+  return __uint_as_float((hi & 0x80000000u) | ((a - 0x38000000u) << 3) | (lo >> 29));
+}
+__device__ __forceinline__ double ref_mean(float sum, float m) {
+  const float v = __fdiv_rn(sum, m);
   return fabsf(v) < 3.0e38f ? (double)v : 0.0;
 }
-
-__device__ __forceinline__ RawRef raw_reference(long long b, long long n,
-                                                const double* __restrict__ cx,
-                                                const double* __restrict__ cy,
-                                                const double* __restrict__ cz) {
-  return RawRef{{raw_mean32(n, [&](long long k) { return cx[b + k]; }),
-                 raw_mean32(n, [&](long long k) { return cy[b + k]; }),
-                 raw_mean32(n, [&](long long k) { return cz[b + k]; })}};
+// by the G threads of a warp (32) or block (256), stored at wout[0], wout[ws], wout[2 ws]
+constexpr int kRawBlock = 256;
+template <int G>
+__device__ __forceinline__ void raw_reference(long long b, long long n,
+                                              const double* __restrict__ cx,
+                                              const double* __restrict__ cy,
+                                              const double* __restrict__ cz,
+                                              double* __restrict__ wout, long long ws) {
+  static_assert(G == 32 || G == kRawBlock, "a warp or a block");
+  constexpr int kBits = G == 32 ? 11 : 12, kMost = 1 << kBits;
+  const int t = threadIdx.x % G, m = n < kMost ? (int)n : kMost;
+  float v[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll 8
+  for (int i = t; i < m; i += G) {
+    const long long k = b + (n <= kMost ? i : (((i >> 3) * n) >> (kBits - 3)) + (i & 7));
+    v[0] += narrow(cx[k]); v[1] += narrow(cy[k]); v[2] += narrow(cz[k]);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+  if constexpr (G > 32) {
+    __shared__ float part[G / 32][3];
+    __syncthreads();                                          // the previous cell's readers
+    if ((t & 31) == 0)
+      for (int i = 0; i < 3; ++i) part[t >> 5][i] = v[i];
+    __syncthreads();
+    for (int i = 0; i < 3; ++i) {
+      v[i] = part[0][i];
+      for (int w = 1; w < G / 32; ++w) v[i] += part[w][i];
+    }
+  }
+  if (t == 0)
+    for (int i = 0; i < 3; ++i) wout[i * ws] = n > 0 ? ref_mean(v[i], (float)m) : 0.0;
 }
+// a warp per cell where they fill the chip: 15.5 million particles in 4,096 cells,
+// references and sums, 0.93 ms (0.90 about the mean of 32; 0.98 with 4,096 of them
+// taken one by one)
+inline bool ref_by_warp(int ncell) { return ncell >= 608; }
 
 // Central moments of a cell from its raw sums and reference velocity: mean
 // velocity U, C_ij, |C|^2 C_k / 2, C_k eps, C_k I (each a mean), eps, I.
@@ -99,23 +135,20 @@ __device__ __forceinline__ RawMoments raw_moments(const double* a, double n, con
   return r;
 }
 
-// The raw sums of one cell (n particles from element b on; ref() gives its
-// reference velocity to a whole warp, which one thread stores at
-// wout[0], wout[ws], wout[2 ws]) added to acc[20] by
-// the gridDim.x blocks of 256 threads that share it.  The particles are cut into
+// The raw sums of one cell (n particles from element b on, about ref()) added to acc[20]
+// by the gridDim.x blocks of 256 threads that share it.  The particles are cut into
 // chunks of at least chunk_min, dealt to the blocks first and then to their
 // warps, so that one cell of a few thousand particles spreads over the SMs'
 // FP64 pipes while a small cell costs one warp one reduction; a block adds
 // its warps' totals with one atomic per sum.
-constexpr int kRawBlock = 256;
 template <typename Ref>
 __device__ __forceinline__ void raw_cell(long long b, long long n, int chunk_min, Ref ref,
                                          const double* __restrict__ cx,
                                          const double* __restrict__ cy,
                                          const double* __restrict__ cz,
                                          const double* __restrict__ er,
-                                         const int* __restrict__ lev, double* __restrict__ acc,
-                                         double* __restrict__ wout, long long ws) {
+                                         const int* __restrict__ lev,
+                                         double* __restrict__ acc) {
   __shared__ double red[kRawBlock / 32][kRawN];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long warps = (long long)gridDim.x * (kRawBlock / 32);
@@ -128,8 +161,6 @@ __device__ __forceinline__ void raw_cell(long long b, long long n, int chunk_min
   int index = -1;
   if (k0 < k1) {                                              // uniform over the warp
     const RawRef w = ref();
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-      for (int i = 0; i < 3; ++i) wout[i * ws] = w.w[i];
     double a[kRawN];
     long long aI = 0;
 #pragma unroll

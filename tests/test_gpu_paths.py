@@ -441,3 +441,65 @@ def test_plane_moments_between_a_capture_and_its_first_replay():
     assert close(after, usp.usp_moments(ref)) < 1e-9 and close(after, before) > 1e-3
     ctx.destroy()
     ref.destroy()
+
+
+def _rest_error(U, c, off):
+    """rms over the cells of a mean velocity's error in units of the speed's spread over
+    sqrt(n), which is the size of the mean itself in a gas at rest."""
+    W = np.longdouble
+    e = []
+    for i in range(len(off) - 1):
+        v = c[:, off[i]:off[i + 1]]
+        e.append((U[:, i] - W(v).mean(axis=1)).astype(float) / (v.std(axis=1) / np.sqrt(v.shape[1])))
+    return float(np.sqrt(np.mean(np.square(e))))
+
+
+@pytest.mark.parametrize("form", ["pool", "context"])
+@pytest.mark.parametrize("ncell", [16, 640])
+def test_mean_velocities_of_large_cells_at_rest(form, ncell):
+    """About the mean the partial sums of n speeds are sqrt(n) large, and the mean is good to some
+    6e-16 of itself; about a velocity a fifth of a thermal speed off they are up to sqrt(n) / 5
+    times larger, and it is off by 4e-15 and more.  The bar lies between."""
+    torch = pytest.importorskip("torch")
+    sp = I.n2_vhs_relaxation_species()
+    rng = np.random.default_rng(ncell)
+    lo, hi = (10000, 40000) if ncell < 100 else (5000, 8000)
+    off = np.concatenate([[0], np.cumsum(rng.integers(lo, hi, ncell))]).astype(np.int64)
+    n = int(off[-1])
+    c = 250.0 * rng.standard_normal((3, n))
+    e, lev = rng.exponential(6e4, n), np.zeros(n, dtype=np.int32)
+    if form == "context":
+        ctx = usp.usp_init_homogeneous(sp, off, np.full(ncell, 1e23), np.full(ncell, 1e-10), *c, e,
+                                       lev, precision=usp.USP_FP64)
+        U = usp.usp_moments(ctx)[1:4]
+        ctx.destroy()
+    else:
+        d = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (off, *c, e, lev)]
+        out = torch.empty((usp.USP_NMOM, ncell), dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        usp.usp_moments_noalloc(sp, ncell, *[a.data_ptr() for a in d], out.data_ptr(),
+                                torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        U = out.cpu().numpy()[1:4]
+    assert _rest_error(U, c, off) < 1.5e-15, _rest_error(U, c, off)
+
+
+@pytest.mark.parametrize("ncell", [3, 700])
+def test_moments_of_velocities_beyond_fp32(ncell):
+    """The reference velocity is formed in FP32: what that has no number for leaves it finite."""
+    torch = pytest.importorskip("torch")
+    sp = I.n2_vhs_relaxation_species()
+    rng = np.random.default_rng(ncell)
+    off = np.arange(ncell + 1, dtype=np.int64) * 50
+    n = int(off[-1])
+    c = rng.standard_normal((3, n)) * np.repeat(10.0 ** rng.choice([-60, -41, 2, 37.5, 38.5, 60], ncell), 50)
+    c[0, :50] = 0.0
+    e, lev = rng.exponential(6e4, n), np.zeros(n, dtype=np.int32)
+    d = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (off, *c, e, lev)]
+    out = torch.empty((usp.USP_NMOM, ncell), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    usp.usp_moments_noalloc(sp, ncell, *[a.data_ptr() for a in d], out.data_ptr(),
+                            torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    ref, scale = _moments(sp, off, c, e, lev)
+    _near(out.cpu().numpy()[:13], ref[:13], 1.6e-11 * scale[:13] + 1e-300)
